@@ -339,8 +339,30 @@ enp_status enp_dg_create(enp_handle* out, const enp_mesh_desc* mesh, const enp_p
       e = cudaMemcpy(h->d_xvdf[a], cd.data(), sizeof(float2) * (P.ne[a] + 1), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) { enp_status s = cuda_fail(h, e, "upload coords (double-float)"); enp_dg_destroy(h); return s; }
     P.xvdf[a] = h->d_xvdf[a];
+    // (h, 2 / h) of every element: one buffer of FP64, then double-float, then FP32 values
+    const size_t ne = (size_t)P.ne[a];
+    std::vector<char> sb(ne * (sizeof(double2) + sizeof(float4) + sizeof(float2)));
+    double2* s64 = reinterpret_cast<double2*>(sb.data());
+    float4* sdf = reinterpret_cast<float4*>(s64 + ne);
+    float2* s32 = reinterpret_cast<float2*>(sdf + ne);
+    for (size_t i = 0; i < ne; ++i) {
+      const double hi = mesh->coords[a][i + 1] - mesh->coords[a][i];
+      s64[i] = make_double2(hi, 2.0 / hi);
+      const enp::df x(s64[i].x), y(s64[i].y);
+      sdf[i] = make_float4(x.hi, x.lo, y.hi, y.lo);
+      s32[i] = make_float2((float)s64[i].x, (float)s64[i].y);
+    }
+    e = cudaMalloc(&h->d_scale[a], sb.size());
+    if (e == cudaSuccess) e = cudaMemcpy(h->d_scale[a], sb.data(), sb.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) { enp_status s = cuda_fail(h, e, "upload element scales"); enp_dg_destroy(h); return s; }
+    P.xs[a] = static_cast<const double2*>(h->d_scale[a]);
+    P.xsdf[a] = reinterpret_cast<const float4*>(P.xs[a] + ne);
+    P.xsf[a] = reinterpret_cast<const float2*>(P.xsdf[a] + ne);
   }
-  for (int a = dim; a < 3; ++a) { P.xv[a] = nullptr; P.xvf[a] = nullptr; P.xvdf[a] = nullptr; }
+  for (int a = dim; a < 3; ++a) {
+    P.xv[a] = nullptr; P.xvf[a] = nullptr; P.xvdf[a] = nullptr;
+    P.xs[a] = nullptr; P.xsf[a] = nullptr; P.xsdf[a] = nullptr;
+  }
   e = cudaMalloc(&h->d_btag, tags.size());
   if (e == cudaSuccess) e = cudaMemcpy(h->d_btag, tags.data(), tags.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMalloc(&h->d_tab, sizeof(Tables));
@@ -374,7 +396,7 @@ enp_status enp_dg_create(enp_handle* out, const enp_mesh_desc* mesh, const enp_p
 enp_status enp_dg_destroy(enp_handle h) {
   if (!h) return ENP_ERR_INVALID_ARG;
   enp_solver_free(h);
-  for (int a = 0; a < 3; ++a) { cudaFree(h->d_xv[a]); cudaFree(h->d_xvf[a]); cudaFree(h->d_xvdf[a]); }
+  for (int a = 0; a < 3; ++a) { cudaFree(h->d_xv[a]); cudaFree(h->d_xvf[a]); cudaFree(h->d_xvdf[a]); cudaFree(h->d_scale[a]); }
   cudaFree(h->d_btag);
   cudaFree(h->d_tab);
   cudaFree(h->d_src);
@@ -570,9 +592,9 @@ static cudaError_t tune_mode(enp_handle h, int mode, enp::io_t<R>* u, enp::io_t<
   };
   int best_fpb = 0;
   if (mode <= enp::kVjp) {
-    const int fx = enp::fpb3d_max<R>(P.p, P.NF, mode);
+    const int fx = enp::fpb3d_max<R>(P.p, P.NF, mode), step = enp::fpb3d_step(P.p);
     float best = 1e30f;
-    for (int f = 1; f <= fx && err == cudaSuccess; ++f) {
+    for (int f = step; f <= fx && err == cudaSuccess; f += step) {
       enp::fpb3d_set<R>(P.p, P.NF, mode, f);
       float ms = 0.f;
       err = time_it(&ms);
@@ -583,7 +605,8 @@ static cudaError_t tune_mode(enp_handle h, int mode, enp::io_t<R>* u, enp::io_t<
   const int mx = enp::eb3d_max<R>(P.p, P.NF, mode);
   float best = 1e30f;
   int best_eb = 0;
-  for (int eb = 1; eb <= mx && err == cudaSuccess; ++eb) {
+  const int step = enp::eb3d_step<R>(P.p);
+  for (int eb = step; eb <= mx && err == cudaSuccess; eb += step) {
     enp::eb3d_set<R>(P.p, P.NF, mode, eb);
     float ms = 0.f;
     err = time_it(&ms);

@@ -56,6 +56,11 @@ struct OpParams {
   const double* xv[3];        // device: per-axis vertex coordinates
   const float* xvf[3];        // the same in FP32, for FP32 kernels
   const float2* xvdf[3];      // the same as double-float pairs (hi, lo)
+  // device: (h, 2 / h) of every element along each axis, formed in FP64 (in FP32
+  // the difference of two rounded vertices would be off by eps x / h)
+  const double2* xs[3];
+  const float2* xsf[3];       // the same in FP32
+  const float4* xsdf[3];      // and as double-float pairs
   const uint8_t* btag;        // device: boundary tags, side-major
   // physics (Sec. 2): mu_k = D_k / RT; migration coefficient z_k mu_k F;
   // a_k = F z_k (D_k - D_m); kappa_k so that kappa = sum_k kappa_k c_k (Eq. charge2)
@@ -84,8 +89,8 @@ struct OpParams {
   int n_theta;                // parameters of dR/dtheta: D_1..D_m, c_in_1..c_in_{m-1}, phi_app_0..3
   // hexahedra: faces of direction a are planes ia = 0..ne[a] times the cells of
   // the other two axes, numbered from foff[a] (foff[3] = all faces); the face
-  // kernel leaves per face and side the lifted face coefficients in fbuf,
-  // [batch][face][side][value, normal derivative][NF][n^2], in the kernel's type
+  // kernel leaves per face the lifted face coefficients in fbuf,
+  // [batch][face][slot][n^2] (enp_tile3d.cuh), in the kernel's type
   long long foff[4];
   void* fbuf;
   long long fbuf_stride;      // entries per operating point

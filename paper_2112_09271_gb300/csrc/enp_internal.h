@@ -35,10 +35,13 @@ ENP_DF_DECL(4)
 bool shape_supported(int dim, int p, int nf);
 
 // Elements per block of the hexahedral kernel (autotuner hooks).
+template <class R> int eb3d_step(int p);   // elements of one group: eb is a multiple of it
 template <class R> int eb3d_max(int p, int nf, int mode);
 template <class R> void eb3d_set(int p, int nf, int mode, int eb);
 template <class R> int eb3d_get(int p, int nf, int mode);
-// Faces per block of the hexahedral face kernel (modes 0..2).
+// Faces per block of the hexahedral face kernel (modes 0..2), a multiple of
+// fpb3d_step (the faces one warp takes).
+int fpb3d_step(int p);
 template <class R> int fpb3d_max(int p, int nf, int mode);
 template <class R> void fpb3d_set(int p, int nf, int mode, int fpb);
 template <class R> int fpb3d_get(int p, int nf, int mode);
@@ -71,6 +74,7 @@ struct enp_dg {
   double* d_xv[3] = {nullptr, nullptr, nullptr};
   float* d_xvf[3] = {nullptr, nullptr, nullptr};
   float2* d_xvdf[3] = {nullptr, nullptr, nullptr};
+  void* d_scale[3] = {nullptr, nullptr, nullptr};  // (h, 2 / h) per axis: FP64, double-float, FP32
   uint8_t* d_btag = nullptr;
   double* d_src = nullptr;
   double* d_dir = nullptr;

@@ -9,6 +9,7 @@
 #include "enp_operator3d.cuh"
 #include "enp_blockcols.cuh"
 #include "enp_sweep.cuh"
+#include "enp_tile3d.cuh"
 
 namespace enp {
 
@@ -37,7 +38,7 @@ static cudaError_t raise_smem_limit(SmemAttr& st, K kern, size_t bytes) {
 }
 
 // Elements per block of the hexahedral kernel, per (p, fields, mode) and
-// arithmetic type; 0 = the default (shared memory near 96 KB). One table per
+// arithmetic type; 0 = the default. One table per
 // type for the whole library (the double-float kernels span several
 // translation units).
 template <class R>
@@ -52,45 +53,47 @@ inline int (&fpb3d_table())[kMaxP + 1][4][3] {
   return t;
 }
 
+// Shared memory of one element's group and of one warp of the face kernel.
+template <int P, int NF, int MODE, class R>
+static constexpr size_t elem_bytes() {
+  if constexpr (MODE <= kVjp && std::is_same<R, float>::value) return (size_t)TileL<P, NF, MODE>::total * sizeof(R);
+  else if constexpr (MODE <= kVjp) return (size_t)TileE<P, NF, MODE>::total * sizeof(R);
+  else return (size_t)Smem3<P, NF, tpe3d<P, R>()>::total * sizeof(R);
+}
 template <int P, int NF, int MODE, class R>
 static constexpr size_t face_bytes() {
-  return (size_t)SmemF<P, NF, MODE, tpf3d<P, R>()>::total * sizeof(R);
+  return (size_t)TileF<P, NF, MODE>::total * sizeof(R);
 }
-// The default faces per block (shared memory near 96 KB) and the largest
-// feasible value (threads <= kMaxThreads3D, shared memory <= 200 KB).
+// Faces per block: as many warps as the block may hold, each tile_faces faces
+// (the warps of a block share nothing, so more only saves block launches).
+template <int P, int NF, int MODE, class R>
+static int max_fpb() { return tile_faces<P>() * (kTileThreads / 32); }
 template <int P, int NF, int MODE, class R>
 static int default_fpb() {
-  constexpr int TF = tpf3d<P, R>();
-  int f = (int)((96 * 1024) / face_bytes<P, NF, MODE, R>());
-  f = f < 1 ? 1 : f;
-  if (f * TF > kMaxThreads3D) f = kMaxThreads3D / TF;
-  return f < 1 ? 1 : f;
-}
-template <int P, int NF, int MODE, class R>
-static int max_fpb() {
-  constexpr int TF = tpf3d<P, R>();
-  int f = kMaxThreads3D / TF;
-  while (f > 1 && (size_t)f * face_bytes<P, NF, MODE, R>() > 200 * 1024) --f;
-  return f < 1 ? 1 : f;
+  return (face_lock<R>() ? 4 : 2) * tile_faces<P>();
 }
 
-template <int P, int NF, int MODE, class R>
-static int default_eb() {
-  constexpr int NT = tpe3d<P, R>();
-  constexpr size_t per_el = (size_t)Smem3<P, NF, MODE, NT>::total * sizeof(R);
-  int eb = (int)((96 * 1024) / per_el);
-  eb = eb < 1 ? 1 : eb;
-  while (eb > 1 && eb * NT > kMaxThreads3D) --eb;
-  return eb;
-}
-
+// Elements per block: groups that share nothing; two by default.
 template <int P, int NF, int MODE, class R>
 static int max_eb() {
-  constexpr int NT = tpe3d<P, R>();
-  constexpr size_t per_el = (size_t)Smem3<P, NF, MODE, NT>::total * sizeof(R);
-  int eb = kMaxThreads3D / NT;
-  while (eb > 1 && (size_t)eb * per_el > 200 * 1024) --eb;
-  return eb < 1 ? 1 : eb;
+  if constexpr (MODE <= kVjp) {
+    return kTileThreads / tile_threads<P, R>() * tile_elems<P, R>();
+  } else {
+    int eb = kMaxThreads3D / tpe3d<P, R>();
+    while (eb > 1 && (size_t)eb * elem_bytes<P, NF, MODE, R>() > 200 * 1024) --eb;
+    return eb < 1 ? 1 : eb;
+  }
+}
+template <int P, int NF, int MODE, class R>
+static int default_eb() {
+  if constexpr (MODE <= kVjp) {
+    return (tile_threads<P, R>() * 2 > kTileThreads ? 1 : 2) * tile_elems<P, R>();
+  } else {  // shared memory near 96 KB
+    int eb = (int)((96 * 1024) / elem_bytes<P, NF, MODE, R>());
+    eb = eb < 1 ? 1 : eb;
+    while (eb > 1 && eb * tpe3d<P, R>() > kMaxThreads3D) --eb;
+    return eb;
+  }
 }
 
 // Columns of the element-diagonal blocks per (element, chunk of kBlockChunk
@@ -116,8 +119,7 @@ template <int P, int NF, int MODE, class R>
 static cudaError_t launch_3d_op(const OpParams& prm, const io_t<R>* u, const io_t<R>* v,
                                 io_t<R>* out, int batch, cudaStream_t stream);
 
-// Hexahedra: the thread-per-pencil kernel with EB elements per block (the FP32
-// block columns: blockcol3d_kernel).
+// Hexahedra: R, J v, J^T w and dR/dtheta, or the block columns.
 template <int P, int NF, int MODE, class R>
 static cudaError_t launch_3d(const OpParams& prm, const io_t<R>* u, const io_t<R>* v, io_t<R>* out,
                              int batch, cudaStream_t stream) {
@@ -133,32 +135,41 @@ static cudaError_t launch_3d(const OpParams& prm, const io_t<R>* u, const io_t<R
 template <int P, int NF, int MODE, class R>
 static cudaError_t launch_3d_op(const OpParams& prm, const io_t<R>* u, const io_t<R>* v,
                                 io_t<R>* out, int batch, cudaStream_t stream) {
-  constexpr int NT = tpe3d<P, R>();
-  using S3 = Smem3<P, NF, MODE, NT>;
-  constexpr size_t per_el = (size_t)S3::total * sizeof(R);
+  constexpr size_t per_el = elem_bytes<P, NF, MODE, R>();
   int eb = eb3d_table<R>()[P][NF][MODE];
   if (eb <= 0) eb = default_eb<P, NF, MODE, R>();
-  const size_t smem = (size_t)eb * per_el;
-  auto kern = op3d_kernel<P, NF, MODE, R>;
   static SmemAttr attr;
-  cudaError_t ea = raise_smem_limit(attr, kern, (size_t)max_eb<P, NF, MODE, R>() * per_el);
-  if (ea != cudaSuccess) return ea;
-  if constexpr (S3::kFB) {
+  if constexpr (MODE <= kVjp) {
     // the faces first: each face once, both sides' terms into the face buffer
-    constexpr int TF = tpf3d<P, R>();
-    constexpr size_t per_face = face_bytes<P, NF, MODE, R>();
+    constexpr size_t per_warp = face_bytes<P, NF, MODE, R>();
+    constexpr int FW = tile_faces<P>();
     int fpb = fpb3d_table<R>()[P][NF][MODE];
     if (fpb <= 0) fpb = default_fpb<P, NF, MODE, R>();
-    auto fk = face3d_kernel<P, NF, MODE, R>;
+    const int warps = (fpb + FW - 1) / FW;
+    auto fk = tileface3d_kernel<P, NF, MODE, R>;
     static SmemAttr fattr;
-    cudaError_t ef = raise_smem_limit(fattr, fk, (size_t)max_fpb<P, NF, MODE, R>() * per_face);
-    if (ef != cudaSuccess) return ef;
-    const long long nf = prm.foff[3];
-    dim3 fgrid((unsigned)((nf + fpb - 1) / fpb), batch);
-    fk<<<fgrid, fpb * TF, fpb * per_face, stream>>>(prm, u, v);
+    cudaError_t e = raise_smem_limit(fattr, fk, (size_t)(kTileThreads / 32) * per_warp);
+    if (e != cudaSuccess) return e;
+    const long long nf = prm.foff[3], per_block = (long long)warps * FW;
+    const dim3 fgrid((unsigned)((nf + per_block - 1) / per_block), batch);
+    fk<<<fgrid, warps * 32, warps * per_warp, stream>>>(prm, u, v);
+    constexpr int EG = tile_elems<P, R>();
+    const int groups = (eb + EG - 1) / EG;
+    const dim3 grid((prm.E + groups * EG - 1) / (groups * EG), batch);
+    auto kern = [] {
+      if constexpr (std::is_same<R, float>::value) return lane3d_kernel<P, NF, MODE>;
+      else return tile3d_kernel<P, NF, MODE, R>;
+    }();
+    e = raise_smem_limit(attr, kern, (size_t)max_eb<P, NF, MODE, R>() * per_el);
+    if (e != cudaSuccess) return e;
+    kern<<<grid, groups * tile_threads<P, R>(), groups * EG * per_el, stream>>>(prm, u, v, out);
+  } else {
+    auto kern = param3d_kernel<P, NF, R>;
+    cudaError_t e = raise_smem_limit(attr, kern, (size_t)max_eb<P, NF, MODE, R>() * per_el);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((prm.E + eb - 1) / eb, batch);
+    kern<<<grid, eb * tpe3d<P, R>(), eb * per_el, stream>>>(prm, u, out);
   }
-  dim3 grid((prm.E + eb - 1) / eb, batch);
-  kern<<<grid, eb * NT, smem, stream>>>(prm, u, v, out);
   return cudaGetLastError();
 }
 
@@ -203,7 +214,8 @@ static cudaError_t launch_mode(int mode, const OpParams& prm, const Tables* t, c
       case kVjp: return launch_one<DIM, P, NF, kVjp, R>(prm, t, u, v, out, batch, s);
       case kBlockCol: return launch_one<DIM, P, NF, kBlockCol, R>(prm, t, u, v, out, batch, s);
       case kParam:
-        if constexpr (DIM == 3) return launch_one<DIM, P, NF, kParam, R>(prm, t, u, v, out, batch, s);
+        if constexpr (DIM == 3 && std::is_same<R, double>::value)
+          return launch_one<DIM, P, NF, kParam, R>(prm, t, u, v, out, batch, s);
         return cudaErrorNotSupported;
     }
     return cudaErrorInvalidValue;
@@ -257,6 +269,10 @@ cudaError_t launch_sweep_plane(const OpParams& prm, const void* binv, int storag
 
 // Elements-per-block of the hexahedral kernel: the largest feasible value for
 // (p, fields, mode), and setting the value launches use (0 = default).
+template <class R>
+int eb3d_step(int p) {
+  return p == 1 ? tile_elems<1, R>() : (p == 2 ? tile_elems<2, R>() : (p == 3 ? tile_elems<3, R>() : tile_elems<4, R>()));
+}
 template <class R>
 int eb3d_max(int p, int nf, int mode) {
 #define ENP_EBM(PP, NFF, MM) \

@@ -1,8 +1,7 @@
-// The CNP DG operator on hexahedra, thread-per-pencil layout (sm_103a).
-//
-// Same arithmetic as op_kernel (enp_operator.cuh: R(u), J(u)v, J(u)^T w and
-// block columns of Eq. NPDG / Eq. chargeDG), organised for throughput:
-//  * Q x Q threads per element, EB elements per thread block;
+// Hexahedra, thread-per-pencil layout (sm_103a): the basis tables, the pencil
+// contractions, the face stages of the downwind sweep, and the parameter
+// Jacobian dR/dtheta of Eq. NPDG / Eq. chargeDG (R, J v and J^T w:
+// enp_tile3d.cuh; block columns: enp_blockcols.cuh).
 //  * every 1D contraction is done by one thread per pencil: it loads the
 //    pencil into registers and forms all outputs with the basis table in
 //    __constant__ memory at compile-time indices (the table entries become
@@ -14,10 +13,6 @@
 #include <type_traits>
 
 #include "enp_operator.cuh"
-
-#ifndef ENP_DF_MIN_BLOCKS
-#define ENP_DF_MIN_BLOCKS 3
-#endif
 
 namespace enp {
 
@@ -201,26 +196,6 @@ __device__ __forceinline__ int face_node_pad(int a, int k, int j1, int j2) {
   return j1 + X * (j2 + N * k);
 }
 
-// Staging of global values into shared memory with asynchronous copies
-// (cp.async), so that all of a stage's loads are in flight at once without
-// holding registers. A slot of R receives the raw value of the vector type IO
-// (the same bytes for FP32 and FP64; a double into a double-float slot, whose
-// 8 bytes it fills, converted in place by stage_finish once the copies landed).
-template <class R, class IO>
-__device__ __forceinline__ void stage_copy(R* dst, const IO* src) {
-  static_assert(sizeof(IO) == sizeof(R) && (sizeof(R) == 4 || sizeof(R) == 8), "slot size");
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(sizeof(R))
-               : "memory");
-}
-__device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-// After stage_wait, by the thread that issued the copy: the slot's value as R.
-template <class R>
-__device__ __forceinline__ void stage_finish(R* slot) {
-  if constexpr (std::is_same<R, df>::value)
-    *slot = df_from_double_dev(*reinterpret_cast<const double*>(slot));
-}
-
 // The coefficients as forward tangents seeded on parameter j of
 // theta = (D_1..D_m, c_in_1..c_in_{m-1}, phi_app_0..phi_app_3).
 template <class R>
@@ -266,31 +241,26 @@ __host__ __device__ constexpr int tpe3d() {
   else return P <= 1 ? 32 : (P == 2 ? 64 : 128);   // FP32 and double-float: the FP32 pipe
 }
 
-template <int P, int NF, int MODE, int NT>
+template <int P, int NF, int NT>
 struct Smem3 {
   static constexpr int N = P + 1, Q = P + 2;
   static constexpr int NX = Pad<N>::X;                   // padded x row of nodal arrays
   static constexpr int NN = N * N * N, NQ = Q * Q * Q, FN = N * N, FQ = Q * Q;
   static constexpr int NNP = NX * N * N;                 // padded nodal array
   static constexpr int FNP = NX * N;                     // padded face-node array
-  static constexpr int NV = (MODE == kResidual || MODE == kParam) ? 1 : 2;
-  static constexpr int NA = NV * NF;                     // arrays carried through the volume
+  static constexpr int NA = NF;                          // arrays carried through the volume
   static constexpr int kX = NA * NNP;                    // element data
   static constexpr int kOut = NF * NNP;                  // rows
   static constexpr int kT1 = NA * Q * N * N;             // after the x contraction
   static constexpr int kT2 = NA * Q * Q * N;             // after the y contraction
   static constexpr int kPts = NA * 4 * NQ;               // values + 3 gradients
-  // R, J v and J^T w take their face terms from the face kernel's buffer:
-  // the six sides' lifted coefficients [6][2][NF][FN]
-  static constexpr bool kFB = MODE == kResidual || MODE == kJvp || MODE == kVjp;
-  static constexpr int kFaceLoop = NA * NNP              // neighbour data
+  static constexpr int kFace = NA * NNP              // neighbour data
                                + 2 * NA * 2 * FNP         // layer values + normal derivatives
                                + 2 * NA * 2 * Q * N       // after the first face contraction
                                + 2 * NA * 2 * FQ          // traces at face points
                                + 2 * NF * FQ              // face coefficients
                                + 2 * NF * Q * N           // transposed, first stage
                                + 2 * NF * FNP;            // transposed, at face nodes
-  static constexpr int kFace = kFB ? 6 * 2 * NF * FN : kFaceLoop;
   // T1 is dead once T2 is formed, so it shares space with the point arrays
   static constexpr int kVol = kT2 + (kPts > kT1 ? kPts : kT1);
   static constexpr int kWork = kVol > kFace ? kVol : kFace;
@@ -306,23 +276,15 @@ struct Smem3 {
 // Largest thread block of the hexahedral kernel; the elements per block (EB,
 // chosen at launch by the autotuner) satisfy EB * tpe3d <= this.
 constexpr int kMaxThreads3D = 256;
-// Resident blocks per SM the register allocation is sized for: the
-// double-float kernels are issue-bound on the FP32 pipe and need more warps in
-// flight than their natural register count allows.
-template <class R> struct MinBlocks3D { static constexpr int value = 1; };
-template <> struct MinBlocks3D<df> { static constexpr int value = ENP_DF_MIN_BLOCKS; };
-
-template <int P, int NF, int MODE, class R>
-__global__ void __launch_bounds__(kMaxThreads3D, MinBlocks3D<R>::value)
-op3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* __restrict__ v,
-            io_t<R>* __restrict__ out) {
-  using S = Smem3<P, NF, MODE, tpe3d<P, R>()>;
+// dR/dtheta_j for every parameter j (grid.y: operating points x parameters).
+template <int P, int NF, class R>
+__global__ void __launch_bounds__(kMaxThreads3D)
+param3d_kernel(const OpParams prm, const R* __restrict__ u, R* __restrict__ out) {
+  using S = Smem3<P, NF, tpe3d<P, R>()>;
   using TO = TabOff<P>;
   constexpr int N = S::N, Q = S::Q, NN = S::NN, NQ = S::NQ, FN = S::FN, FQ = S::FQ;
   constexpr int NX = S::NX, NNP = S::NNP, FNP = S::FNP;
-  constexpr int NV = S::NV, NA = S::NA, NT = tpe3d<P, R>(), PF = S::kPrefetch;
-  constexpr bool kBlk = MODE == kBlockCol;
-  constexpr int MODEc = kBlk ? kJvp : MODE;
+  constexpr int NA = S::NA, NT = tpe3d<P, R>(), PF = S::kPrefetch;
   const PhysT<R>& ph = phys<R>(prm);
   extern __shared__ __align__(16) unsigned char smem3_raw[];
   const int es = threadIdx.x / NT, tid = threadIdx.x % NT;
@@ -334,12 +296,10 @@ op3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* __
   const int e = blockIdx.x * EB + es;
   const bool valid = e < prm.E;
   const int ee = valid ? e : prm.E - 1;   // invalid slots shadow a valid element, write nothing
-  constexpr bool kPar = MODE == kParam;
-  const int col = kBlk ? (int)blockIdx.y : -1;
-  const int bidx = kBlk ? 0 : (kPar ? (int)blockIdx.y / prm.n_theta : (int)blockIdx.y);
-  const int theta_j = kPar ? (int)blockIdx.y % prm.n_theta : -1;
-  const long long boff = kBlk ? 0 : (long long)bidx * prm.batch_stride;
-  const long long ooff = kPar ? ((long long)theta_j * prm.batch + bidx) * prm.batch_stride : boff;
+  const int bidx = (int)blockIdx.y / prm.n_theta;
+  const int theta_j = (int)blockIdx.y % prm.n_theta;
+  const long long boff = (long long)bidx * prm.batch_stride;
+  const long long ooff = ((long long)theta_j * prm.batch + bidx) * prm.batch_stride;
   const long long EN = (long long)prm.E * NN;
 
   int idx[3];
@@ -362,19 +322,7 @@ op3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* __
     const int f = t / NN, i = t % NN;
     const long long gi = boff + f * EN + (long long)ee * NN + i;
     const int pi = f * NNP + padded_node<N>(i);
-    stage_copy(XA + pi, u + gi);
-    if (NV == 2) {
-      if (kBlk) XA[NF * NNP + pi] = R(t == col ? 1 : 0);
-      else stage_copy(XA + NF * NNP + pi, v + gi);
-    }
-  }
-  stage_wait();
-  if constexpr (std::is_same<R, df>::value) {
-    for (int t = tid; t < NF * NN; t += NT) {
-      const int pi = (t / NN) * NNP + padded_node<N>(t % NN);
-      stage_finish(XA + pi);
-      if (NV == 2 && !kBlk) stage_finish(XA + NF * NNP + pi);
-    }
+    XA[pi] = u[gi];
   }
   // neighbour data of a face, fetched into registers one face ahead so that the
   // global loads overlap the computation of the previous stage
@@ -389,33 +337,12 @@ op3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* __
     for (int k = 0; k < PF; ++k) {
       const int t = tid + k * NT;
       if (t < NA * NN) {
-        const int vv = t / (NF * NN), r = t % (NF * NN), f = r / NN, i = r % NN;
-        const long long gi = boff + f * EN + (long long)en * NN + i;
-        pf[k] = vv == 0 ? R(u[gi]) : (kBlk ? R(0) : R(v[gi]));
+        const int f = t / NN, i = t % NN;
+        pf[k] = u[boff + f * EN + (long long)en * NN + i];
       }
     }
   };
-  if constexpr (!S::kFB) prefetch(0);
-  if constexpr (S::kFB) {
-    // the six sides' lifted face terms are read after the volume terms: start
-    // moving them into L2 now (one 128-byte line per work item)
-    constexpr int PER = 2 * NF * FN;
-    constexpr int LINES = (PER * (int)sizeof(R) + 127) / 128 + 1;  // + 1: unaligned start
-    for (int q = tid; q < 6 * LINES; q += NT) {
-      const int s = q / LINES, l = q % LINES;
-      const int a = s >> 1, hi = s & 1;
-      const int b0 = a == 0 ? 1 : 0, b1 = a == 2 ? 1 : 2;
-      // run-time axes: selections, not indexed arrays (which would go to local memory)
-      const long long gid = pick3(prm.foff, a) + (pick3(idx, a) + hi) +
-                            (long long)(pick3(prm.ne, a) + 1) *
-                                (pick3(idx, b0) + (long long)pick3(prm.ne, b0) * pick3(idx, b1));
-      const char* src = reinterpret_cast<const char*>(reinterpret_cast<const R*>(prm.fbuf) +
-                                                      (long long)bidx * prm.fbuf_stride +
-                                                      (gid * 2 + (hi ? 0 : 1)) * PER);
-      const int off = l * 128 < PER * (int)sizeof(R) ? l * 128 : PER * (int)sizeof(R) - 1;
-      asm volatile("prefetch.global.L2 [%0];" ::"l"(src + off));
-    }
-  }
+  prefetch(0);
   __syncthreads();
 
   // ---------------------------------------------------------------- volume
@@ -459,7 +386,7 @@ op3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* __
         for (int a = 0; a < 3; ++a) g0[f][a] = V[(1 + a) * NQ + pt] * sc[a];
       }
       R oS[NF], oG[NF][3];
-      if (MODEc == kParam) {
+      {
         const PhysT<Tan<R>> pt = seed_phys<R>(ph, NF, theta_j);
         Tan<R> ct[NF], gt[NF][3], Sf[NF], Gf[NF][3];
 #pragma unroll
@@ -475,42 +402,10 @@ op3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* __
 #pragma unroll
           for (int a = 0; a < 3; ++a) oG[f][a] = Gf[f][a].d;
         }
-      } else if (MODEc == kResidual) {
-        volume_flux<NF, 3, R, R>(ph, c0, g0, uv, oS, oG);
-#pragma unroll
-        for (int f = 0; f < NF; ++f)
-          oS[f] -= prm.src ? R(prm.src[((long long)f * prm.E + ee) * NQ + pt]) : R(0);
-      } else {
-        R c1[NF], g1[NF][3];
-#pragma unroll
-        for (int f = 0; f < NF; ++f) {
-          const R* V = PT + (NF + f) * 4 * NQ;
-          c1[f] = V[pt];
-#pragma unroll
-          for (int a = 0; a < 3; ++a) g1[f][a] = V[(1 + a) * NQ + pt] * sc[a];
-        }
-        if (MODEc == kJvp) {
-          Tan<R> ct[NF], gt[NF][3], Sf[NF], Gf[NF][3];
-#pragma unroll
-          for (int f = 0; f < NF; ++f) {
-            ct[f] = Tan<R>(c0[f], c1[f]);
-#pragma unroll
-            for (int a = 0; a < 3; ++a) gt[f][a] = Tan<R>(g0[f][a], g1[f][a]);
-          }
-          volume_flux<NF, 3, Tan<R>, R>(ph, ct, gt, uv, Sf, Gf);
-#pragma unroll
-          for (int f = 0; f < NF; ++f) {
-            oS[f] = Sf[f].d;
-#pragma unroll
-            for (int a = 0; a < 3; ++a) oG[f][a] = Gf[f][a].d;
-          }
-        } else {
-          volume_flux_adjoint<NF, 3, R>(ph, c0, g0, uv, g1, oS, oG);
-        }
       }
 #pragma unroll
       for (int f = 0; f < NF; ++f) {
-        R* V = PT + ((NV - 1) * NF + f) * 4 * NQ;
+        R* V = PT + f * 4 * NQ;
         V[pt] = w * oS[f];
 #pragma unroll
         for (int a = 0; a < 3; ++a) V[(1 + a) * NQ + pt] = w * sc[a] * oG[f][a];
@@ -518,7 +413,7 @@ op3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* __
     }
   }
   __syncthreads();
-  R* PO = PT + (NV - 1) * NF * 4 * NQ;   // the NF output point arrays
+  R* PO = PT;   // the NF output point arrays
   pencil<P, Q, Q, Q, 0, 1, true, true, NF, 4 * NQ, 4 * NQ>(PO + NQ, PO, tid, NT);
   __syncthreads();
   pencil<P, Q, Q, Q, 1, 1, true, true, NF, 4 * NQ, 4 * NQ>(PO + 2 * NQ, PO, tid, NT);
@@ -534,45 +429,6 @@ op3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* __
   __syncthreads();
 
   // ---------------------------------------------------------------- faces
-  if constexpr (S::kFB) {
-    // the lifted coefficients of the six sides, left by the face kernel: side
-    // (a, hi) of this element is the lower element (0) of face plane
-    // idx[a] + 1 when hi, the upper one (1) of plane idx[a] otherwise
-    R* FS = WK;  // [6][2][NF][FN]
-    const R* fb = reinterpret_cast<const R*>(prm.fbuf) + (long long)bidx * prm.fbuf_stride;
-    constexpr int PER = 2 * NF * FN;
-#pragma unroll
-    for (int s = 0; s < 6; ++s) {
-      const int a = s >> 1, hi = s & 1;
-      const int b0 = a == 0 ? 1 : 0, b1 = a == 2 ? 1 : 2;
-      const long long gid = prm.foff[a] + (idx[a] + hi) +
-                            (long long)(prm.ne[a] + 1) * (idx[b0] + (long long)prm.ne[b0] * idx[b1]);
-      const R* src = fb + (gid * 2 + (hi ? 0 : 1)) * PER;
-      for (int r = tid; r < PER; r += NT) stage_copy(FS + s * PER + r, src + r);
-    }
-    stage_wait();
-    __syncthreads();
-    // each row gathers its six face terms in side order (no two threads write
-    // one row)
-    for (int t = tid; t < NF * NN; t += NT) {
-      const int f = t / NN, i = t % NN;
-      const int c3[3] = {i % N, (i / N) % N, i / (N * N)};
-      R acc = RO[f * NNP + padded_node<N>(i)];
-#pragma unroll
-      for (int s = 0; s < 6; ++s) {
-        const int a = s >> 1, hi = s & 1;
-        const int k = c3[a];
-        const int j = a == 0 ? c3[1] + N * c3[2] : (a == 1 ? c3[0] + N * c3[2] : c3[0] + N * c3[1]);
-        const R sv = FS[((s * 2 + 0) * NF + f) * FN + j];
-        const R tv = FS[((s * 2 + 1) * NF + f) * FN + j];
-        R add = ctab<P, R>(TO::dL + hi * N + k) * tv;
-        if (k == (hi ? N - 1 : 0)) add += sv;
-        acc += add;
-      }
-      RO[f * NNP + padded_node<N>(i)] = acc;
-    }
-    __syncthreads();
-  } else {
   R* XN = WK;                                  // [NA][NNP] neighbour data
   R* FL = XN + NA * NNP;                       // [2 sides][NA][2][FNP] layer values, derivatives
   R* F1 = FL + 2 * NA * 2 * FNP;               // [2][NA][2][Q][N]
@@ -613,7 +469,7 @@ op3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* __
       }
     }
     if (s < 5) prefetch(s + 1);
-    const bool active = !(tag == kWall || (tag == kInlet && MODEc != kResidual && MODEc != kParam));
+    const bool active = tag != kWall;
     __syncthreads();
     // layer values and reference normal derivatives at the face nodes
     const int lay = hi ? N - 1 : 0, layo = hi ? 0 : N - 1;
@@ -662,16 +518,16 @@ op3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* __
       velocity(ph, xp, uv);
       const R un = uv[a] * nrm;
       const R w = ctab<P, R>(TO::W + k1) * ctab<P, R>(TO::W + k2) * area;
-      auto trv = [&](int side, int vv, int f, int comp) -> R {
-        return TR[(((side * NA) + vv * NF + f) * 2 + comp) * FQ + pt];
+      auto trv = [&](int side, int f, int comp) -> R {
+        return TR[((side * NA + f) * 2 + comp) * FQ + pt];
       };
       R cm[NF], dm[NF], cp[NF], dp[NF], g[NF];
 #pragma unroll
       for (int f = 0; f < NF; ++f) {
-        cm[f] = trv(0, 0, f, 0);
-        dm[f] = trv(0, 0, f, 1) * sca;
-        cp[f] = boundary ? R(0) : trv(1, 0, f, 0);
-        dp[f] = boundary ? R(0) : trv(1, 0, f, 1) * scn;
+        cm[f] = trv(0, f, 0);
+        dm[f] = trv(0, f, 1) * sca;
+        cp[f] = boundary ? R(0) : trv(1, f, 0);
+        dp[f] = boundary ? R(0) : trv(1, f, 1) * scn;
         g[f] = (tag == kDirichlet && prm.dirv)
                    ? R(prm.dirv[((long long)f * prm.NBF + bface) * prm.Nfq + pt]) : R(0);
       }
@@ -679,7 +535,7 @@ op3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* __
 #pragma unroll
       for (int f = 0; f < NF; ++f) { oS[f] = R(0); oT[f] = R(0); }
       if (active) {
-        if (MODEc == kParam) {
+        {
           const PhysT<Tan<R>> pt = seed_phys<R>(ph, NF, theta_j);
           const Tan<R> phit(phiapp, (tag >= kElectrode0 && theta_j == 2 * NF - 1 + tag - kElectrode0)
                                         ? R(1) : R(0));
@@ -695,51 +551,6 @@ op3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* __
             face_interior_flux<NF, Tan<R>, R, Tan<R>>(pt, tm, tdm, tp, tdp, un, delta, Sf, Tf);
 #pragma unroll
           for (int f = 0; f < NF; ++f) { oS[f] = Sf[f].d; oT[f] = Tf[f].d; }
-        } else if (MODEc == kResidual) {
-          if (boundary) face_boundary_flux<NF, R, R>(ph, tag, cm, dm, g, un, delta, xp, phiapp, oS, oT);
-          else face_interior_flux<NF, R, R>(ph, cm, dm, cp, dp, un, delta, oS, oT);
-        } else {
-          R cm1[NF], dm1[NF], cp1[NF], dp1[NF];
-#pragma unroll
-          for (int f = 0; f < NF; ++f) {
-            cm1[f] = trv(0, 1, f, 0);
-            dm1[f] = trv(0, 1, f, 1) * sca;
-            cp1[f] = boundary ? R(0) : trv(1, 1, f, 0);
-            dp1[f] = boundary ? R(0) : trv(1, 1, f, 1) * scn;
-          }
-          if (MODEc == kJvp) {
-            Tan<R> tm[NF], tdm[NF], tp[NF], tdp[NF], Sf[NF], Tf[NF];
-#pragma unroll
-            for (int f = 0; f < NF; ++f) {
-              tm[f] = Tan<R>(cm[f], cm1[f]); tdm[f] = Tan<R>(dm[f], dm1[f]);
-              tp[f] = Tan<R>(cp[f], cp1[f]); tdp[f] = Tan<R>(dp[f], dp1[f]);
-            }
-            if (boundary) face_boundary_flux<NF, Tan<R>, R>(ph, tag, tm, tdm, g, un, delta, xp, phiapp, Sf, Tf);
-            else face_interior_flux<NF, Tan<R>, R>(ph, tm, tdm, tp, tdp, un, delta, Sf, Tf);
-#pragma unroll
-            for (int f = 0; f < NF; ++f) { oS[f] = Sf[f].d; oT[f] = Tf[f].d; }
-          } else {
-            R Sh[NF], Th[NF], acm[NF], adm[NF], acp[NF], adp[NF];
-#pragma unroll
-            for (int f = 0; f < NF; ++f) { Sh[f] = cm1[f]; Th[f] = dm1[f]; acm[f] = adm[f] = acp[f] = adp[f] = R(0); }
-            if (boundary) {
-              face_boundary_adjoint<NF, R>(ph, tag, cm, dm, g, un, delta, xp, phiapp, Sh, Th, acm, adm);
-            } else {
-              face_interior_adjoint<NF, R>(ph, cm, dm, cp, dp, un, delta, Sh, Th, acm, adm, acp, adp);
-              R ncm[NF], ndm[NF], ncp[NF], ndp[NF], bcm[NF], bdm[NF], bcp[NF], bdp[NF];
-#pragma unroll
-              for (int f = 0; f < NF; ++f) {
-                ncm[f] = cp[f]; ndm[f] = -dp[f]; ncp[f] = cm[f]; ndp[f] = -dm[f];
-                Sh[f] = cp1[f]; Th[f] = -dp1[f];
-                bcm[f] = bdm[f] = bcp[f] = bdp[f] = R(0);
-              }
-              face_interior_adjoint<NF, R>(ph, ncm, ndm, ncp, ndp, -un, delta, Sh, Th, bcm, bdm, bcp, bdp);
-#pragma unroll
-              for (int f = 0; f < NF; ++f) { acm[f] += bcp[f]; adm[f] -= bdp[f]; }
-            }
-#pragma unroll
-            for (int f = 0; f < NF; ++f) { oS[f] = acm[f]; oT[f] = adm[f]; }
-          }
         }
       }
 #pragma unroll
@@ -771,26 +582,17 @@ op3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* __
     }
     __syncthreads();
   }
-  }  // face loop of the block-column and parameter modes
 
   if (valid) {
-    if (kBlk) {
-      const long long nb = NF * NN;
-      for (int t = tid; t < NF * NN; t += NT)
-        out[((long long)e * nb + t) * nb + col] = to_io(RO[(t / NN) * NNP + padded_node<N>(t % NN)]);
-    } else {
-      for (int t = tid; t < NF * NN; t += NT) {
-        const int f = t / NN, i = t % NN;
-        out[ooff + f * EN + (long long)e * NN + i] = to_io(RO[f * NNP + padded_node<N>(i)]);
-      }
+    for (int t = tid; t < NF * NN; t += NT) {
+      const int f = t / NN, i = t % NN;
+      out[ooff + f * EN + (long long)e * NN + i] = RO[f * NNP + padded_node<N>(i)];
     }
   }
 }
 
-
 // ---------------------------------------------------------------------------
-// Face kernel of R, J v and J^T w: each face of the mesh once, for both of its
-// sides. Threads per face: Q x Q for FP64; for FP32 and double-float the
+// Face stages of the downwind sweep. Threads per face: Q x Q for FP64; for FP32 and double-float the
 // fewest threads that cover the Q x Q face points in about one pass of the
 // pointwise fluxes (16, 16, 32 and 48 at p = 1..4), so that the costliest
 // stage keeps its lanes busy; faces per block make up the block.
@@ -1040,92 +842,6 @@ __device__ __forceinline__ void face3d_stages(const OpParams& prm, R* base, int 
   __syncthreads();
   pencil<P, Q, N, 1, 0, 0, true, false, 4 * NF, Q * N, FNP, R, Q, NX>(G1, G2, tid, NT);
   __syncthreads();
-}
-
-template <int P, int NF, int MODE, class R>
-__global__ void __launch_bounds__(kMaxThreads3D, MinBlocks3D<R>::value)
-face3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* __restrict__ v) {
-  constexpr int NT = tpf3d<P, R>();
-  using S = SmemF<P, NF, MODE, NT>;
-  constexpr int N = S::N, NN = S::NN, FN = S::FN;
-  constexpr int NX = S::NX, NNP = S::NNP, FNP = S::FNP, NA = S::NA;
-  extern __shared__ __align__(16) unsigned char smemf_raw[];
-  const int fs = threadIdx.x / NT, tid = threadIdx.x % NT;
-  R* base = reinterpret_cast<R*>(smemf_raw) + fs * S::total;
-  R* XS = base;                  // [2][NA][NNP]
-  const int FPB = blockDim.x / NT;
-  const long long nf = prm.foff[3];
-  const long long graw = (long long)blockIdx.x * FPB + fs;
-  const bool valid = graw < nf;
-  const long long g = valid ? graw : nf - 1;     // idle slots shadow a face, write nothing
-  const int bidx = blockIdx.y;
-  const long long boff = (long long)bidx * prm.batch_stride;
-  const long long EN = (long long)prm.E * NN;
-
-  const int a = (g >= prm.foff[1]) + (g >= prm.foff[2]);
-  const long long fi = g - prm.foff[a];
-  const int na0 = prm.ne[a] + 1;
-  const int ia = (int)(fi % na0);
-  const long long rr = fi / na0;
-  const int nb0 = prm.ne[a == 0 ? 1 : 0];
-  const int j0 = (int)(rr % nb0), j1 = (int)(rr / nb0);
-  const int b0 = a == 0 ? 1 : 0, b1 = a == 2 ? 1 : 2;
-  const long long gid = prm.foff[a] + ia + (long long)(prm.ne[a] + 1) * (j0 + (long long)prm.ne[b0] * j1);
-  const bool hasL = ia > 0, hasU = ia < prm.ne[a];
-  const int stride[3] = {1, prm.ne[0], prm.ne[0] * prm.ne[1]};
-  const int sa = pick3(stride, a);
-  const int eU = ia * sa + j0 * pick3(stride, b0) + j1 * pick3(stride, b1);  // valid when hasU
-  const int eL = eU - sa;                                                   // valid when hasL
-
-  // both elements' data (a missing side is zero and never read); node-outer, so
-  // the padded offset is formed once per node
-  {
-    const long long gL = boff + (long long)(hasL ? eL : 0) * NN;
-    const long long gU = boff + (long long)(hasU ? eU : 0) * NN;
-    for (int i = tid; i < NN; i += NT) {
-      const int pi = padded_node<N>(i);
-#pragma unroll
-      for (int f = 0; f < NF; ++f) {
-        const long long o = f * EN + i;
-        if (hasL) stage_copy(XS + f * NNP + pi, u + gL + o);
-        else XS[f * NNP + pi] = R(0);
-        if (hasU) stage_copy(XS + (NA + f) * NNP + pi, u + gU + o);
-        else XS[(NA + f) * NNP + pi] = R(0);
-        if (NA > NF) {
-          if (hasL) stage_copy(XS + (NF + f) * NNP + pi, v + gL + o);
-          else XS[(NF + f) * NNP + pi] = R(0);
-          if (hasU) stage_copy(XS + (NA + NF + f) * NNP + pi, v + gU + o);
-          else XS[(NA + NF + f) * NNP + pi] = R(0);
-        }
-      }
-    }
-    stage_wait();
-    if constexpr (std::is_same<R, df>::value) {
-      for (int i = tid; i < NN; i += NT) {
-        const int pi = padded_node<N>(i);
-#pragma unroll
-        for (int f = 0; f < NF; ++f) {
-          if (hasL) stage_finish(XS + f * NNP + pi);
-          if (hasU) stage_finish(XS + (NA + f) * NNP + pi);
-          if (NA > NF) {
-            if (hasL) stage_finish(XS + (NF + f) * NNP + pi);
-            if (hasU) stage_finish(XS + (NA + NF + f) * NNP + pi);
-          }
-        }
-      }
-    }
-  }
-  __syncthreads();
-  face3d_stages<P, NF, MODE, R, NT>(prm, base, tid, NT, a, ia, j0, j1, bidx);
-  const R* G2 = face3d_g2<P, NF, MODE, R, NT>(base);
-  if (valid) {
-    R* fb = reinterpret_cast<R*>(prm.fbuf) + (long long)bidx * prm.fbuf_stride +
-            gid * 2 * 2 * NF * FN;
-    for (int w = tid; w < 2 * 2 * NF * FN; w += NT) {
-      const int c = w / FN, j = w % FN;   // c = (side * 2 + S/T) * NF + f
-      fb[w] = G2[c * FNP + (j % N) + NX * (j / N)];
-    }
-  }
 }
 
 }  // namespace enp

@@ -24,7 +24,12 @@ cudaError_t enp::prepare_tables_df(int p, const Tables& t) {
   return cudaErrorInvalidConfiguration;
 }
 
+int enp::fpb3d_step(int p) {
+  return p == 1 ? tile_faces<1>() : (p == 2 ? tile_faces<2>() : (p == 3 ? tile_faces<3>() : tile_faces<4>()));
+}
+
 // Launch-shape hooks of the autotuner (shape arithmetic only, no kernels here).
+template int enp::eb3d_step<enp::df>(int);
 template int enp::eb3d_max<enp::df>(int, int, int);
 template void enp::eb3d_set<enp::df>(int, int, int, int);
 template int enp::eb3d_get<enp::df>(int, int, int);
