@@ -34,6 +34,13 @@ ENP_DF_DECL(4)
 
 bool shape_supported(int dim, int p, int nf);
 
+// dtheta[b][j] = <w_b, dR_b/dtheta_j> on hexahedra, device [batch][n_theta];
+// part: device workspace of batch x kPvjpPartials doubles.
+cudaError_t upload_tables_param(int p, const Tables& t);
+constexpr int kPvjpPartials = 2 * 608 * 14;
+cudaError_t launch_param_vjp(const OpParams& prm, const double* u, const double* w, double* part,
+                             double* dtheta, int batch, cudaStream_t s);
+
 // Elements per block of the hexahedral kernel (autotuner hooks).
 template <class R> int eb3d_step(int p);   // elements of one group: eb is a multiple of it
 template <class R> int eb3d_max(int p, int nf, int mode);

@@ -1384,14 +1384,14 @@ struct SolverState {
   // reductions
   double* part = nullptr;
   size_t part_count = 0;
+  double* pvjp = nullptr;         // block sums of the parameter adjoint
+  size_t pvjp_count = 0;
   double* dsmall = nullptr;       // device small vectors
   size_t dsmall_count = 0;
   // Krylov workspace
   void* V = nullptr;
   void* Z = nullptr;
   size_t krylov_bytes = 0;
-  double* dRdtheta = nullptr;     // parameter Jacobian workspace [n_theta][batch][n]
-  size_t dRdtheta_count = 0;
   // CUDA graph of one FGMRES restart cycle, on handle-owned copies of the inputs
   cudaStream_t gstream = nullptr;
   cudaGraphExec_t gexec = nullptr;
@@ -1779,7 +1779,7 @@ void enp_solver_free(enp_handle h) {
   cudaFree(S.nbuf); cudaFree(S.nsmall);
   cudaFree(S.blocks); cudaFree(S.binv); cudaFree(S.gj_work); cudaFree(S.d_flag);
   cudaFree(S.blocks32); cudaFree(S.u32);
-  cudaFree(S.part); cudaFree(S.dsmall); cudaFree(S.V); cudaFree(S.dRdtheta);
+  cudaFree(S.part); cudaFree(S.pvjp); cudaFree(S.dsmall); cudaFree(S.V);
   for (auto& L : S.levels) {
     cudaFree(L.A); cudaFree(L.A32); cudaFree(L.x); cudaFree(L.b); cudaFree(L.r);
   }
@@ -3129,16 +3129,18 @@ __global__ void sum_over_batch_kernel(const double* __restrict__ v, int B, int n
 
 // <w_b, dR_b/dtheta_j> for every operating point into S.dsmall[b][j] (device).
 static enp_status param_dots(enp_handle h, const double* u, const double* w, size_t extra) {
+  if (h->prm.dim != 3) {
+    h->err = "dR/dtheta is built for hexahedra";
+    return ENP_ERR_UNSUPPORTED;
+  }
   SolverState& S = state_of(h);
   const int nt = h->prm.n_theta, B = h->batch;
-  const long long n = h->n_dof;
-  cudaError_t e = ensure(&S.dRdtheta, S.dRdtheta_count, (size_t)nt * B * n);
-  if (e != cudaSuccess) return cuda_err(h, e, "cudaMalloc parameter Jacobian");
-  enp_status st = enp_param_jacobian(h, u, S.dRdtheta);
-  if (st != ENP_OK) return st;
+  // a buffer of its own: captured FGMRES cycles hold the address of S.part
+  cudaError_t e = ensure(&S.pvjp, S.pvjp_count, (size_t)B * enp::kPvjpPartials);
+  if (e != cudaSuccess) return cuda_err(h, e, "cudaMalloc partials");
   if ((e = small(h, (size_t)B * nt + extra)) != cudaSuccess) return cuda_err(h, e, "cudaMalloc small");
-  if ((e = multidot<double>(h, S.dRdtheta, (long long)B * n, nt, w, S.dsmall)) != cudaSuccess)
-    return cuda_err(h, e, "parameter dots");
+  if ((e = enp::launch_param_vjp(h->prm, u, w, S.pvjp, S.dsmall, B, h->stream)) != cudaSuccess)
+    return cuda_err(h, e, "parameter adjoint");
   return ENP_OK;
 }
 

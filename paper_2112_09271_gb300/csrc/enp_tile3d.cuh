@@ -149,13 +149,17 @@ constexpr int kTileThreads = 128;   // largest block of either kernel
 
 template <int P, int NF, int MODE>
 struct Slots {
-  static constexpr bool JAC = MODE != kResidual;
-  static constexpr int NA = JAC ? 2 * NF : NF;       // arrays interpolated to the points
-  static constexpr int NG = JAC ? NF + 1 : NF;       // of them with gradients (listed first)
-  static constexpr int NSL = MODE == kVjp ? 3 * NF : 2 * NF + 1;   // face coefficient arrays
+  static constexpr bool JAC = MODE == kJvp || MODE == kVjp;
+  static constexpr int NA = MODE == kResidual ? NF : 2 * NF;   // arrays interpolated to the points
+  static constexpr int NG = JAC ? NF + 1 : NA;                 // of them with gradients (listed first)
+  // face coefficient arrays (none for <w, dR/dtheta>, kParam, which sums at the points)
+  static constexpr int NSL = MODE == kParam ? 0 : (MODE == kVjp ? 3 * NF : 2 * NF + 1);
   // array s: vector (0 u, 1 v) and field
-  __device__ static __forceinline__ int vec(int s) { return JAC && s >= 1 && s <= NF ? 1 : 0; }
+  __device__ static __forceinline__ int vec(int s) {
+    return MODE == kParam ? s >= NF : (JAC && s >= 1 && s <= NF ? 1 : 0);
+  }
   __device__ static __forceinline__ int field(int s) {
+    if (MODE == kParam) return s < NF ? s : s - NF;
     return !JAC ? s : (s == 0 ? 0 : (s <= NF ? s - 1 : s - NF));
   }
 };
@@ -395,32 +399,18 @@ __device__ __forceinline__ void add_face_terms(const OpParams& prm, const R* __r
   }
 }
 
-// ------------------------------------------- element kernel, pooled pencils
-// FP64 and double-float, whose pencils cost 100 to 300 issue slots: every stage
-// is one pool, so that the lanes stay full (94 % at p = 3) at the price of one
-// index computation per pencil.
+// The pooled stages from the nodal values of one element to the values and
+// reference gradients at its points: region A [NA] values, [NG] z gradients;
+// region B [NG][2] x and y gradients. Ends with a barrier of the group.
 template <int P, int NF, int MODE, class R>
-__global__ void __launch_bounds__(kTileThreads, 5)
-tile3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* __restrict__ v,
-              io_t<R>* __restrict__ out) {
+__device__ __forceinline__ void tile_points(const io_t<R>* __restrict__ ue,
+                                            const io_t<R>* __restrict__ ve, long long EN, R* A,
+                                            R* Bq, int tid) {
   using S = TileE<P, NF, MODE>;
   using SL = Slots<P, NF, MODE>;
   using TO = TabOff<P>;
-  constexpr int N = S::N, Q = S::Q, QP = S::QP, AQ = S::AQ, NN = N * N * N, FN = N * N, FQ = Q * Q;
+  constexpr int N = S::N, Q = S::Q, QP = S::QP, AQ = S::AQ, FN = N * N, FQ = Q * Q;
   constexpr int NA = S::NA, NG = S::NG, T = tile_threads<P, R>();
-  extern __shared__ __align__(16) unsigned char tile_raw[];
-  const int grp = threadIdx.x / T, tid = threadIdx.x % T;
-  const int eraw = blockIdx.x * (blockDim.x / T) + grp;
-  if (!tile_lock<P, R>() && eraw >= prm.E) return;
-  const bool valid = eraw < prm.E;
-  const int e = valid ? eraw : prm.E - 1;
-  R* A = reinterpret_cast<R*>(tile_raw) + grp * S::total;
-  R* Bq = A + S::kA;
-  const int bidx = blockIdx.y;
-  const long long boff = (long long)bidx * prm.batch_stride;
-  const long long EN = (long long)prm.E * NN;
-  const io_t<R>* ue = u + boff + (long long)e * NN;
-  const io_t<R>* ve = SL::JAC ? v + boff + (long long)e * NN : nullptr;
   // x: nodal lines from global memory
 #pragma unroll 1
   for (int w = tid; w < NA * FN; w += T) {
@@ -461,6 +451,35 @@ tile3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* 
     line<P, TO::Dq, false, Q, Q, R>(A + s * AQ + o, is, Bq + (2 * s + d) * AQ + o, is);
   }
   group_sync<tile_lock<P, R>()>();
+}
+
+// ------------------------------------------- element kernel, pooled pencils
+// FP64 and double-float, whose pencils cost 100 to 300 issue slots: every stage
+// is one pool, so that the lanes stay full (94 % at p = 3) at the price of one
+// index computation per pencil.
+template <int P, int NF, int MODE, class R>
+__global__ void __launch_bounds__(kTileThreads, 5)
+tile3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* __restrict__ v,
+              io_t<R>* __restrict__ out) {
+  using S = TileE<P, NF, MODE>;
+  using SL = Slots<P, NF, MODE>;
+  using TO = TabOff<P>;
+  constexpr int N = S::N, Q = S::Q, QP = S::QP, AQ = S::AQ, NN = N * N * N, FN = N * N, FQ = Q * Q;
+  constexpr int NA = S::NA, NG = S::NG, T = tile_threads<P, R>();
+  extern __shared__ __align__(16) unsigned char tile_raw[];
+  const int grp = threadIdx.x / T, tid = threadIdx.x % T;
+  const int eraw = blockIdx.x * (blockDim.x / T) + grp;
+  if (!tile_lock<P, R>() && eraw >= prm.E) return;
+  const bool valid = eraw < prm.E;
+  const int e = valid ? eraw : prm.E - 1;
+  R* A = reinterpret_cast<R*>(tile_raw) + grp * S::total;
+  R* Bq = A + S::kA;
+  const int bidx = blockIdx.y;
+  const long long boff = (long long)bidx * prm.batch_stride;
+  const long long EN = (long long)prm.E * NN;
+  const io_t<R>* ue = u + boff + (long long)e * NN;
+  const io_t<R>* ve = SL::JAC ? v + boff + (long long)e * NN : nullptr;
+  tile_points<P, NF, MODE, R>(ue, ve, EN, A, Bq, tid);
 
   // point fluxes: those of field f replace x, y in region B slots 2f, 2f + 1, z
   // in region A slot NA + f; the value coefficient (R with sources, J^T w) in
@@ -1059,27 +1078,21 @@ __device__ __forceinline__ void face_point(const OpParams& prm, const FaceAt& F,
   }
 }
 
+// The stages from both elements' nodal values to the traces at the points of
+// the warp's nw faces (from face g0): region A [face][side][NTR][Q][QP], values
+// of the NA arrays, then physical normal derivatives along +axis of the first NG.
+// B: scratch. Ends with a barrier.
 template <int P, int NF, int MODE, class R>
-__global__ void __launch_bounds__(kTileThreads, FaceBlocks<R>::value)
-tileface3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* __restrict__ v) {
+__device__ __forceinline__ void face_traces(const OpParams& prm, const io_t<R>* __restrict__ u,
+                                            const io_t<R>* __restrict__ v, long long boff,
+                                            long long g0, int nw, const FaceAt& F0, int lane, R* A,
+                                            R* B) {
   using S = TileF<P, NF, MODE>;
   using SL = Slots<P, NF, MODE>;
   using TO = TabOff<P>;
-  constexpr int N = S::N, Q = S::Q, QP = S::QP, NX = S::NX, FN = S::FN, FQ = S::FQ;
-  constexpr int NN = N * N * N, NA = SL::NA, NG = SL::NG, NTR = S::NTR, NSL = SL::NSL, FW = S::NF_;
-  extern __shared__ __align__(16) unsigned char tile_raw[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  R* A = reinterpret_cast<R*>(tile_raw) + warp * S::total;
-  R* B = A + S::kA;
-  const long long nf = prm.foff[3];
-  const long long g0 = ((long long)blockIdx.x * (blockDim.x >> 5) + warp) * FW;
-  if (!face_lock<R>() && g0 >= nf) return;
-  const int nw = g0 >= nf ? 0 : (int)(nf - g0 < FW ? nf - g0 : FW);   // faces of this warp
-  const int bidx = blockIdx.y;
-  const long long boff = (long long)bidx * prm.batch_stride;
+  constexpr int N = S::N, Q = S::Q, QP = S::QP, NX = S::NX, FN = S::FN, NN = N * N * N;
+  constexpr int NA = SL::NA, NG = SL::NG, NTR = S::NTR, FW = S::NF_;
   const long long EN = (long long)prm.E * NN;
-
-  const FaceAt F0 = face_at(prm, g0);
   // layer values, and physical normal derivatives along +axis, of both elements
   // (node (k along a, (j1, j2) in the face) at base(j1, j2) + k * fs); a side
   // that does not exist is skipped, and its traces are never used
@@ -1137,6 +1150,29 @@ tileface3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<
       line<P, TO::B, false, N, Q, R>(B + g * (N * QP) + k1, QP, A + g * (Q * QP) + k1, QP);
   }
   group_sync<face_lock<R>()>();
+}
+
+template <int P, int NF, int MODE, class R>
+__global__ void __launch_bounds__(kTileThreads, FaceBlocks<R>::value)
+tileface3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* __restrict__ v) {
+  using S = TileF<P, NF, MODE>;
+  using SL = Slots<P, NF, MODE>;
+  using TO = TabOff<P>;
+  constexpr int N = S::N, Q = S::Q, QP = S::QP, FN = S::FN, FQ = S::FQ;
+  constexpr int NTR = S::NTR, NSL = SL::NSL, FW = S::NF_;
+  extern __shared__ __align__(16) unsigned char tile_raw[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  R* A = reinterpret_cast<R*>(tile_raw) + warp * S::total;
+  R* B = A + S::kA;
+  const long long nf = prm.foff[3];
+  const long long g0 = ((long long)blockIdx.x * (blockDim.x >> 5) + warp) * FW;
+  if (!face_lock<R>() && g0 >= nf) return;
+  const int nw = g0 >= nf ? 0 : (int)(nf - g0 < FW ? nf - g0 : FW);   // faces of this warp
+  const int bidx = blockIdx.y;
+  const long long boff = (long long)bidx * prm.batch_stride;
+
+  const FaceAt F0 = face_at(prm, g0);
+  face_traces<P, NF, MODE, R>(prm, u, v, boff, g0, nw, F0, lane, A, B);
 #pragma unroll 1
   for (int w = lane; w < nw * FQ; w += 32) {
     const int fi = w / FQ, pt = w - fi * FQ;
@@ -1149,6 +1185,9 @@ tileface3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<
         [&](int slot, R val) { c0[slot * (Q * QP)] = val; });
   }
   group_sync<face_lock<R>()>();
+  // lane (sub, k1): line k1 of every K-th array
+  constexpr int K = 32 / Q;
+  const int sub = lane / Q, k1 = lane - sub * Q;
   if (sub < K) {
 #pragma unroll 1
     for (int g = sub; g < nw * NSL; g += K)

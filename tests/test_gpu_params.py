@@ -115,3 +115,30 @@ def test_param_vjp_total_sums_the_operating_points_on_the_device():
     th = torch.zeros(op.n_theta, dtype=torch.float64, device="cuda", requires_grad=True)
     fn(u, th).backward(w)
     assert np.array_equal(th.grad.cpu().numpy(), total)
+
+
+@pytest.mark.parametrize("dirichlet", [False, True])
+@pytest.mark.parametrize("cfg,p,n", [("cube_n2_p2", 1, (1, 1, 1)), ("channel_n1", 2, (5, 3, 1)),
+                                     ("channel_n1", 3, (2, 2, 3)), ("cube_n2_p2", 4, (3, 2, 1))])
+def test_param_vjp_equals_the_jacobian_times_w(cfg, p, n, dirichlet):
+    """<w, dR/dtheta> summed at the points against the parameter Jacobian's rows:
+    meshes that fill no thread block evenly, two and three fields, every boundary
+    kind, a reaction order other than one and an eliminated oxidant (channel)."""
+    import dataclasses
+
+    import torch
+    enp = _enp()
+    base = W.config(cfg, p=p)
+    coords = [c[-1] * np.linspace(0, 1, k + 1) ** 1.2 for c, k in zip(base.coords, n)]
+    tags = W.box_tags(3, list(n), coords, W.DIRICHLET if dirichlet else W.WALL)
+    if not dirichlet:
+        tags[0][:], tags[1][:] = W.INLET, W.OUTLET
+        tags[2][:], tags[3][:] = W.ELECTRODE0, W.ELECTRODE0 + 1
+    P = dataclasses.replace(base, n_el=list(n), coords=coords, tags=tags, bv_gamma=1.5)
+    op = enp.Operator(P)
+    if dirichlet:
+        op.set_sources(None, _cuda(W.random_dirichlet(P, 9)))
+    u, w = _cuda(W.random_state(P, 3)), _cuda(W.random_vector(P, 4))
+    ref = (op.param_jacobian(u) @ w).cpu().numpy()
+    d = op.param_vjp(u, w)[0]
+    assert np.abs(d - ref).max() <= 1e-12 * np.abs(ref).max()
