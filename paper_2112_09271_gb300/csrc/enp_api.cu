@@ -389,6 +389,8 @@ enp_status enp_dg_create(enp_handle* out, const enp_mesh_desc* mesh, const enp_p
   if (e == cudaSuccess) e = enp::prepare_tables<float>(P.p, h->htab);
   if (e == cudaSuccess && dim == 3) e = enp::prepare_tables_df(P.p, h->htab);
   if (e == cudaSuccess && dim == 3) e = enp::upload_tables_param(P.p, h->htab);
+  if (e == cudaSuccess && dim == 3) e = enp::upload_tables_sweep<float>(P.p, h->htab);
+  if (e == cudaSuccess && dim == 3) e = enp::upload_tables_sweep<double>(P.p, h->htab);
   if (e != cudaSuccess) { enp_status s = cuda_fail(h, e, "upload constant tables"); enp_dg_destroy(h); return s; }
   *out = h;
   return ENP_OK;

@@ -58,16 +58,16 @@ template <class R> int fpb3d_get(int p, int nf, int mode);
 template <class R>
 cudaError_t prepare_tables(int p, const Tables& t);
 
-// One element plane k (along axis a, flow direction dir = +-1) of the downwind
-// block Gauss-Seidel sweep for every operating point: z_e = Binv_e (x_e -
-// J_(e,up) z_up), the upstream face term evaluated in the same launch
-// (upstream = 0 for the first plane). binv: the transposed block inverses in
-// `storage` (0 FP64, 1 FP32, 2 BF16), one set per point or one shared set;
-// upc: the linearisation point (hexahedra).
+// The downwind block Gauss-Seidel sweep along axis a (flow direction dir = +-1)
+// for every operating point: z_e = Binv_e (x_e - J_(e,up) z_up) down every line
+// of elements (hexahedra). binv: the transposed block inverses in `storage`
+// (0 FP64, 1 FP32, 2 BF16), one set per point or one shared set; upc: the
+// linearisation point. x and z do not overlap.
 template <class TV>
-cudaError_t launch_sweep_plane(const OpParams& prm, const void* binv, int storage, const TV* x,
-                               TV* z, const TV* upc, int batch, cudaStream_t s, int a, int k,
-                               int dir, int upstream, int shared_blocks);
+cudaError_t launch_sweep(const OpParams& prm, const void* binv, int storage, const TV* x, TV* z,
+                         const TV* upc, int batch, cudaStream_t s, int a, int dir,
+                         int shared_blocks);
+template <class TV> cudaError_t upload_tables_sweep(int p, const Tables& t);
 
 }  // namespace enp
 

@@ -8,7 +8,6 @@
 #include "enp_operator.cuh"
 #include "enp_operator3d.cuh"
 #include "enp_blockcols.cuh"
-#include "enp_sweep.cuh"
 #include "enp_tile3d.cuh"
 
 namespace enp {
@@ -227,43 +226,6 @@ static cudaError_t launch_nf(int mode, const OpParams& prm, const Tables* t, con
                              const io_t<R>* v, io_t<R>* out, int batch, cudaStream_t s) {
   if (prm.NF == 2) return launch_mode<DIM, P, 2, R>(mode, prm, t, u, v, out, batch, s);
   if (prm.NF == 3) return launch_mode<DIM, P, 3, R>(mode, prm, t, u, v, out, batch, s);
-  return cudaErrorInvalidConfiguration;
-}
-
-// One plane of the downwind block Gauss-Seidel sweep (sweep_fused_kernel).
-template <int P, int NF, class TV>
-static cudaError_t launch_sweep_pn(const OpParams& prm, const void* binv, int storage, const TV* x,
-                                   TV* z, const TV* upc, int batch, cudaStream_t stream, int a,
-                                   int k, int dir, int upstream, int shared_blocks) {
-  using SS = SweepSmem<P, NF, TV>;
-  auto kern = sweep_fused_kernel<P, NF, TV>;
-  static SmemAttr attr;
-  cudaError_t e = raise_smem_limit(attr, kern, SS::bytes);
-  if (e != cudaSuccess) return e;
-  const int nplane = prm.ne[a == 0 ? 1 : 0] * prm.ne[a == 2 ? 1 : 2];
-  const dim3 grid((unsigned)nplane, (unsigned)batch);
-  kern<<<grid, SS::NT, SS::bytes, stream>>>(prm, binv, storage, x, z, upc, a, k, dir, upstream,
-                                            shared_blocks);
-  return cudaGetLastError();
-}
-
-template <class TV>
-cudaError_t launch_sweep_plane(const OpParams& prm, const void* binv, int storage, const TV* x,
-                               TV* z, const TV* upc, int batch, cudaStream_t s, int a, int k,
-                               int dir, int upstream, int shared_blocks) {
-  if (prm.dim != 3 || storage < 0 || storage > 2 || (dir != 1 && dir != -1))
-    return cudaErrorInvalidConfiguration;
-#define ENP_SW(PP)                                                                              \
-  case PP:                                                                                      \
-    if (prm.NF == 2)                                                                            \
-      return launch_sweep_pn<PP, 2, TV>(prm, binv, storage, x, z, upc, batch, s, a, k, dir,     \
-                                        upstream, shared_blocks);                               \
-    if (prm.NF == 3)                                                                            \
-      return launch_sweep_pn<PP, 3, TV>(prm, binv, storage, x, z, upc, batch, s, a, k, dir,     \
-                                        upstream, shared_blocks);                               \
-    return cudaErrorInvalidConfiguration;
-  switch (prm.p) { ENP_SW(1) ENP_SW(2) ENP_SW(3) ENP_SW(4) }
-#undef ENP_SW
   return cudaErrorInvalidConfiguration;
 }
 

@@ -1,6 +1,5 @@
 // Hexahedra, thread-per-pencil layout (sm_103a): the basis tables, the pencil
-// contractions, the face stages of the downwind sweep, and the parameter
-// Jacobian dR/dtheta of Eq. NPDG / Eq. chargeDG (R, J v and J^T w:
+// contractions, and the parameter Jacobian dR/dtheta of Eq. NPDG / Eq. chargeDG (R, J v and J^T w:
 // enp_tile3d.cuh; block columns: enp_blockcols.cuh).
 //  * every 1D contraction is done by one thread per pencil: it loads the
 //    pencil into registers and forms all outputs with the basis table in
@@ -589,259 +588,6 @@ param3d_kernel(const OpParams prm, const R* __restrict__ u, R* __restrict__ out)
       out[ooff + f * EN + (long long)e * NN + i] = RO[f * NNP + padded_node<N>(i)];
     }
   }
-}
-
-// ---------------------------------------------------------------------------
-// Face stages of the downwind sweep. Threads per face: Q x Q for FP64; for FP32 and double-float the
-// fewest threads that cover the Q x Q face points in about one pass of the
-// pointwise fluxes (16, 16, 32 and 48 at p = 1..4), so that the costliest
-// stage keeps its lanes busy; faces per block make up the block.
-template <int P, class R>
-__host__ __device__ constexpr int tpf3d() {
-  if constexpr (std::is_same<R, double>::value) return (P + 2) * (P + 2);
-  else return P <= 2 ? 16 : (P == 3 ? 32 : 48);
-}
-
-template <int P, int NF, int MODE, int NT>
-struct SmemF {
-  static constexpr int N = P + 1, Q = P + 2;
-  static constexpr int NX = Pad<N>::X;
-  static constexpr int NN = N * N * N, FN = N * N, FQ = Q * Q;
-  static constexpr int NNP = NX * N * N, FNP = NX * N;
-  static constexpr int NV = MODE == kResidual ? 1 : 2;
-  static constexpr int NA = NV * NF;
-  // Two regions, reused stage by stage: A holds both elements' data X, then
-  // (once FL is formed) the interpolation F1 and the traces TR, then (once the
-  // fluxes are formed) the transposed contractions G1 and G2; B holds FL, then
-  // (once F1 is formed) the face coefficients FC.
-  static constexpr int kX = 2 * NA * NNP;              // both elements' data
-  static constexpr int kF1 = 2 * NA * 2 * Q * N;       // after the first face contraction
-  static constexpr int kTR = 2 * NA * 2 * FQ;          // traces at the face points
-  static constexpr int kG1 = 2 * 2 * NF * Q * N;
-  static constexpr int kG2 = 2 * 2 * NF * FNP;
-  static constexpr int kA0 = kX > kF1 + kTR ? kX : kF1 + kTR;
-  static constexpr int kA = kA0 > kG1 + kG2 ? kA0 : kG1 + kG2;
-  static constexpr int kFL = 2 * NA * 2 * FNP;         // layer values + normal derivatives
-  static constexpr int kFC = 2 * 2 * NF * FQ;          // [side][S, T][NF] at face points
-  static constexpr int kB = kFL > kFC ? kFL : kFC;
-  static constexpr int raw = kA + kB;
-  static constexpr int total = raw + ((NT - raw % 32) % 32 + 32) % 32;
-};
-
-// The stages of one face after both elements' data are in XS (the first
-// region of `base`): layer values and normal derivatives, the 2D interpolation
-// to the face points, the pointwise fluxes, and the transposed 2D contraction
-// back to the face nodes. On return (after a barrier) the lifted coefficients
-// of both sides are at face3d_g2(base): [side][S, T][NF][FNP]. All threads of
-// the block take part in every barrier.
-template <int P, int NF, int MODE, class R, int NTS>
-__device__ __forceinline__ R* face3d_g2(R* base) {
-  using S = SmemF<P, NF, MODE, NTS>;
-  return base + S::kG1;
-}
-template <int P, int NF, int MODE, class R, int NTS>
-__device__ __forceinline__ void face3d_stages(const OpParams& prm, R* base, int tid, int NT, int a,
-                                              int ia, int j0, int j1, int bidx) {
-  using S = SmemF<P, NF, MODE, NTS>;
-  using TO = TabOff<P>;
-  constexpr int N = S::N, Q = S::Q, FN = S::FN, FQ = S::FQ;
-  constexpr int NX = S::NX, NNP = S::NNP, FNP = S::FNP, NA = S::NA;
-  const PhysT<R>& ph = phys<R>(prm);
-  R* XS = base;                  // [2][NA][NNP]
-  R* F1 = base;                  // [2][NA][2][Q][N] (over XS, once FL is formed)
-  R* TR = F1 + S::kF1;           // [2][NA][2][FQ]
-  R* G1 = base;                  // [2][2][NF][N][Q] (over F1 and TR, once FC is formed)
-  R* G2 = G1 + S::kG1;           // [2][2][NF][FNP]
-  R* FL = base + S::kA;          // [2][NA][2][FNP]
-  R* FC = FL;                    // [2][2][NF][FQ] (over FL, once F1 is formed)
-  const int b0 = a == 0 ? 1 : 0, b1 = a == 2 ? 1 : 2;
-  const bool hasL = ia > 0, hasU = ia < prm.ne[a];
-  const R lo0 = vertex<R>(prm, b0, j0), lo1 = vertex<R>(prm, b1, j1);
-  const R h0 = vertex<R>(prm, b0, j0 + 1) - lo0, h1 = vertex<R>(prm, b1, j1 + 1) - lo1;
-  const R xa = vertex<R>(prm, a, ia);
-  const R hL = hasL ? xa - vertex<R>(prm, a, ia - 1) : R(1);
-  const R hU = hasU ? vertex<R>(prm, a, ia + 1) - xa : R(1);
-  const R diagL = sqrtv(hL * hL + h0 * h0 + h1 * h1), diagU = sqrtv(hU * hU + h0 * h0 + h1 * h1);
-  // face-layer values and reference normal derivatives: the lower element at
-  // its upper face (layer N-1, derivative at xi = +1), the upper element at its
-  // lower face (layer 0, derivative at xi = -1)
-  // node (k along a, face node (j1, j2)) of a padded element array sits at
-  // fbase(j1, j2) + k * fstr
-  const int fstr = a == 0 ? 1 : (a == 1 ? NX : NX * N);
-  for (int w = tid; w < 2 * NA * FN; w += NT) {
-    const int sa = w / FN, j = w % FN;          // sa = side * NA + arr
-    const int side = sa >= NA ? 1 : 0, arr = sa - side * NA;
-    const int jn1 = j % N, jn2 = j / N;
-    const int fbase = a == 0 ? NX * (jn1 + N * jn2) : (a == 1 ? jn1 + NX * N * jn2 : jn1 + NX * jn2);
-    const R* X = XS + (side * NA + arr) * NNP + fbase;
-    const int lay = side == 0 ? N - 1 : 0, dsel = side == 0 ? 1 : 0;
-    R d = R(0);
-#pragma unroll
-    for (int k = 0; k < N; ++k) d = mad(ctab<P, R>(TO::dL + dsel * N + k), X[k * fstr], d);
-    R* o = FL + ((side * NA + arr) * 2) * FNP;
-    const int jp = jn1 + NX * jn2;
-    o[jp] = X[lay * fstr];
-    o[FNP + jp] = d;
-  }
-  __syncthreads();
-  pencil<P, N, N, 1, 0, 0, false, false, 4 * NA, FNP, Q * N, R, NX>(FL, F1, tid, NT);
-  __syncthreads();
-  pencil<P, Q, N, 1, 1, 0, false, false, 4 * NA, Q * N, FQ>(F1, TR, tid, NT);
-  __syncthreads();
-
-  {
-    const R area = R(0.25) * h0 * h1;
-    const R scL = R(2) / hL, scU = R(2) / hU;
-    const bool interior = hasL && hasU;
-    // boundary face: the one element's own side and outward normal
-    const int bside = hasL ? 0 : 1;
-    const R nrm = bside == 0 ? R(1) : R(-1);
-    const R sca = (bside == 0 ? scL : scU) * nrm;
-    int tag = kInterior, bface = -1;
-    if (!interior) {
-      bface = prm.side_off[2 * a + (bside == 0 ? 1 : 0)] + j0 + prm.ne[b0] * j1;
-      tag = prm.btag[bface];
-    }
-    const bool active = interior || !(tag == kWall || (tag == kInlet && MODE != kResidual));
-    const R delta = ph.cip * R(P * P) /
-                    (interior ? R(0.5) * (diagL + diagU) : (bside == 0 ? diagL : diagU));
-    const R phiapp = (tag >= kElectrode0)
-        ? (prm.phiapp_batch ? R(prm.phiapp_batch[bidx * 4 + (tag - kElectrode0)])
-                            : ph.phiapp[tag - kElectrode0])
-        : R(0);
-#pragma unroll 1
-    for (int pt = tid; pt < FQ; pt += NT) {
-      const int k1 = pt % Q, k2 = pt / Q;
-      const R xb0 = lo0 + R(0.5) * (ctab<P, R>(TO::X + k1) + R(1)) * h0;
-      const R xb1 = lo1 + R(0.5) * (ctab<P, R>(TO::X + k2) + R(1)) * h1;
-      // (x, y, z) of the point by selection (a, b0, b1 are run-time axes)
-      R xp[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) xp[c] = c == a ? xa : (c == b0 ? xb0 : xb1);
-      R uv[3];
-      velocity(ph, xp, uv);
-      const R ua = pick3(uv, a);
-      const R w = ctab<P, R>(TO::W + k1) * ctab<P, R>(TO::W + k2) * area;
-      const R* T0p = TR + pt;
-      auto tr = [&](int side, int vv, int f, int comp) -> R {
-        return T0p[(((side * NA) + vv * NF + f) * 2 + comp) * FQ];
-      };
-      R oSL[NF], oTL[NF], oSU[NF], oTU[NF];
-#pragma unroll
-      for (int f = 0; f < NF; ++f) { oSL[f] = oTL[f] = oSU[f] = oTU[f] = R(0); }
-      if (interior) {
-        // the lower element's view: outward normal +e_a, derivatives along it
-        const R un = ua;
-        R cm[NF], dm[NF], cp[NF], dp[NF];
-#pragma unroll
-        for (int f = 0; f < NF; ++f) {
-          cm[f] = tr(0, 0, f, 0); dm[f] = tr(0, 0, f, 1) * scL;
-          cp[f] = tr(1, 0, f, 0); dp[f] = tr(1, 0, f, 1) * scU;
-        }
-        if (MODE == kResidual) {
-          face_interior_flux2<NF, R, R>(ph, cm, dm, cp, dp, un, delta, oSL, oTL, oTU);
-#pragma unroll
-          for (int f = 0; f < NF; ++f) oSU[f] = -oSL[f];
-        } else {
-          R cm1[NF], dm1[NF], cp1[NF], dp1[NF];
-#pragma unroll
-          for (int f = 0; f < NF; ++f) {
-            cm1[f] = tr(0, 1, f, 0); dm1[f] = tr(0, 1, f, 1) * scL;
-            cp1[f] = tr(1, 1, f, 0); dp1[f] = tr(1, 1, f, 1) * scU;
-          }
-          if (MODE == kJvp) {
-            Tan<R> tm[NF], tdm[NF], tp[NF], tdp[NF], Sf[NF], Tf[NF], TfP[NF];
-#pragma unroll
-            for (int f = 0; f < NF; ++f) {
-              tm[f] = Tan<R>(cm[f], cm1[f]); tdm[f] = Tan<R>(dm[f], dm1[f]);
-              tp[f] = Tan<R>(cp[f], cp1[f]); tdp[f] = Tan<R>(dp[f], dp1[f]);
-            }
-            face_interior_flux2<NF, Tan<R>, R>(ph, tm, tdm, tp, tdp, un, delta, Sf, Tf, TfP);
-#pragma unroll
-            for (int f = 0; f < NF; ++f) {
-              oSL[f] = Sf[f].d; oTL[f] = Tf[f].d; oSU[f] = -Sf[f].d; oTU[f] = TfP[f].d;
-            }
-          } else {
-            // J^T w: the rows of each side, differentiated with respect to both
-            // sides' states; the upper side's rows seen from the upper element
-            // (normal and normal derivatives flip)
-            R acm[NF], adm[NF], acp[NF], adp[NF], bcm[NF], bdm[NF], bcp[NF], bdp[NF];
-            R ncm[NF], ndm[NF], ncp[NF], ndp[NF], Sh[NF], Th[NF];
-#pragma unroll
-            for (int f = 0; f < NF; ++f) {
-              acm[f] = adm[f] = acp[f] = adp[f] = bcm[f] = bdm[f] = bcp[f] = bdp[f] = R(0);
-              Sh[f] = cm1[f]; Th[f] = dm1[f];
-            }
-            face_interior_adjoint<NF, R>(ph, cm, dm, cp, dp, un, delta, Sh, Th, acm, adm, acp, adp);
-#pragma unroll
-            for (int f = 0; f < NF; ++f) {
-              ncm[f] = cp[f]; ndm[f] = -dp[f]; ncp[f] = cm[f]; ndp[f] = -dm[f];
-              Sh[f] = cp1[f]; Th[f] = -dp1[f];
-            }
-            face_interior_adjoint<NF, R>(ph, ncm, ndm, ncp, ndp, -un, delta, Sh, Th, bcm, bdm, bcp, bdp);
-#pragma unroll
-            for (int f = 0; f < NF; ++f) {
-              oSL[f] = acm[f] + bcp[f]; oTL[f] = adm[f] - bdp[f];
-              oSU[f] = bcm[f] + acp[f]; oTU[f] = bdm[f] - adp[f];
-            }
-          }
-        }
-      } else if (active) {
-        const R un = ua * nrm;
-        R cm[NF], dm[NF], g[NF], oS[NF], oT[NF];
-#pragma unroll
-        for (int f = 0; f < NF; ++f) {
-          cm[f] = tr(bside, 0, f, 0);
-          dm[f] = tr(bside, 0, f, 1) * sca;
-          g[f] = (tag == kDirichlet && prm.dirv)
-                     ? R(prm.dirv[((long long)f * prm.NBF + bface) * prm.Nfq + pt]) : R(0);
-          oS[f] = R(0); oT[f] = R(0);
-        }
-        if (MODE == kResidual) {
-          face_boundary_flux<NF, R, R>(ph, tag, cm, dm, g, un, delta, xp, phiapp, oS, oT);
-        } else {
-          R cm1[NF], dm1[NF];
-#pragma unroll
-          for (int f = 0; f < NF; ++f) { cm1[f] = tr(bside, 1, f, 0); dm1[f] = tr(bside, 1, f, 1) * sca; }
-          if (MODE == kJvp) {
-            Tan<R> tm[NF], tdm[NF], Sf[NF], Tf[NF];
-#pragma unroll
-            for (int f = 0; f < NF; ++f) { tm[f] = Tan<R>(cm[f], cm1[f]); tdm[f] = Tan<R>(dm[f], dm1[f]); }
-            face_boundary_flux<NF, Tan<R>, R>(ph, tag, tm, tdm, g, un, delta, xp, phiapp, Sf, Tf);
-#pragma unroll
-            for (int f = 0; f < NF; ++f) { oS[f] = Sf[f].d; oT[f] = Tf[f].d; }
-          } else {
-            R acm[NF], adm[NF];
-#pragma unroll
-            for (int f = 0; f < NF; ++f) acm[f] = adm[f] = R(0);
-            face_boundary_adjoint<NF, R>(ph, tag, cm, dm, g, un, delta, xp, phiapp, cm1, dm1, acm, adm);
-#pragma unroll
-            for (int f = 0; f < NF; ++f) { oS[f] = acm[f]; oT[f] = adm[f]; }
-          }
-        }
-#pragma unroll
-        for (int f = 0; f < NF; ++f) {
-          if (bside == 0) { oSL[f] = oS[f]; oTL[f] = oT[f]; }
-          else { oSU[f] = oS[f]; oTU[f] = oT[f]; }
-        }
-      }
-      // weights, and the normal derivative of each side's test functions along
-      // its own outward normal (+e_a for the lower side, -e_a for the upper)
-#pragma unroll
-      for (int f = 0; f < NF; ++f) {
-        FC[((0 * 2 + 0) * NF + f) * FQ + pt] = w * oSL[f];
-        FC[((0 * 2 + 1) * NF + f) * FQ + pt] = w * scL * oTL[f];
-        FC[((1 * 2 + 0) * NF + f) * FQ + pt] = w * oSU[f];
-        FC[((1 * 2 + 1) * NF + f) * FQ + pt] = -(w * scU * oTU[f]);
-      }
-    }
-  }
-  __syncthreads();
-  // transposed 2D contraction back to the face nodes, both sides
-  pencil<P, Q, Q, 1, 1, 0, true, false, 4 * NF, FQ, Q * N>(FC, G1, tid, NT);
-  __syncthreads();
-  pencil<P, Q, N, 1, 0, 0, true, false, 4 * NF, Q * N, FNP, R, Q, NX>(G1, G2, tid, NT);
-  __syncthreads();
 }
 
 }  // namespace enp

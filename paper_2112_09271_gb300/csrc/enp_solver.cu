@@ -2082,28 +2082,14 @@ static cudaError_t bj_apply_plain(enp_handle h, const TV* x, TV* y) {
 }
 
 // Downwind block Gauss-Seidel: z = (D + L)^-1 x with D the element blocks and L
-// the couplings of each element to its upstream neighbour along the flow axis;
-// the element planes are solved in flow order, one launch per plane, each
-// element evaluating its upstream face term from the plane solved before.
+// the couplings of each element to its upstream neighbour along the flow axis.
 template <class TV>
 static cudaError_t sweep_apply(enp_handle h, const TV* x, TV* z) {
   SolverState& S = state_of(h);
-  const OpParams& P = h->prm;
-  const int B = h->batch;
-  const long long ntot = h->n_dof * B;
-  cudaError_t e = cudaMemsetAsync(z, 0, sizeof(TV) * ntot, h->stream);
-  if (e != cudaSuccess) return e;
-  const int a = S.sweep_axis, dir = S.sweep_dir;
-  const int nk = P.ne[a];
   const TV* upc = std::is_same<TV, double>::value ? reinterpret_cast<const TV*>(S.upc64)
                                                   : reinterpret_cast<const TV*>(S.upc32);
-  for (int step = 0; step < nk; ++step) {
-    const int k = dir > 0 ? step : nk - 1 - step;
-    if ((e = enp::launch_sweep_plane<TV>(P, S.binv, S.storage, x, z, upc, B, h->stream, a, k, dir,
-                                         step > 0 ? 1 : 0, S.pc_shared_built)) != cudaSuccess)
-      return e;
-  }
-  return cudaSuccess;
+  return enp::launch_sweep<TV>(h->prm, S.binv, S.storage, x, z, upc, h->batch, h->stream,
+                               S.sweep_axis, S.sweep_dir, S.pc_shared_built);
 }
 
 extern "C" enp_status enp_set_shared_blocks(enp_handle h, int point) {

@@ -841,28 +841,198 @@ __device__ __forceinline__ FaceAt face_at(const OpParams& prm, long long g) {
   return f;
 }
 
-// The flux coefficients of one face point. tr(side, t): trace t (values of the
-// NA arrays, then physical normal derivatives along +axis of the first NG) of
-// the lower (0) or upper (1) side; put(slot, value).
+// Sizes and position of a face: in-plane corner and lengths, plane coordinate,
+// the two elements' lengths along the axis (1 where there is none).
+template <class R>
+struct FaceGeo {
+  R lo0, lo1, h0, h1, xa, hL, hU;
+  __device__ __forceinline__ void in_plane(const OpParams& prm, int a, int j0, int j1) {
+    const int b0 = a == 0 ? 1 : 0, b1 = a == 2 ? 1 : 2;
+    lo0 = vertex<R>(prm, b0, j0);
+    lo1 = vertex<R>(prm, b1, j1);
+    h0 = elem_size<R>(prm, b0, j0);
+    h1 = elem_size<R>(prm, b1, j1);
+  }
+  __device__ __forceinline__ void along(const OpParams& prm, int a, int ia, bool hasL, bool hasU) {
+    xa = vertex<R>(prm, a, ia);
+    hL = hasL ? elem_size<R>(prm, a, ia - 1) : R(1);
+    hU = hasU ? elem_size<R>(prm, a, ia) : R(1);
+  }
+};
+
+// The flux coefficients at a point of an interior face: ua the velocity along
+// +axis, w the weight, delta the penalty. tr(side, t): trace t (values of the NA
+// arrays, then physical normal derivatives along +axis of the first NG) of the
+// lower (0) or upper (1) side; put(slot, value).
 template <int P, int NF, int MODE, class R, class TR, class PUT>
-__device__ __forceinline__ void face_point(const OpParams& prm, const FaceAt& F, int bidx, int pt,
-                                           TR tr, PUT put) {
+__device__ __forceinline__ void face_interior_point(const PhysT<R>& ph, R ua, R w, R delta, TR tr,
+                                                    PUT put) {
+  constexpr int NA = Slots<P, NF, MODE>::NA;
+  const R hw = halfv(w);
+  if constexpr (MODE == kResidual) {
+    const R pm = tr(0, 0), pp = tr(1, 0), dm = tr(0, NA), dp = tr(1, NA);
+    const R jphi = pm - pp;
+    R kapm, kapp;
+    Dot<R> t0, s0;
+    Dot<R> km, kp;
+#pragma unroll
+    for (int k = 0; k < NF - 1; ++k) {
+      const R cm = tr(0, k + 1), cp = tr(1, k + 1);
+      const R jc = cm - cp, dd = tr(0, NA + k + 1) + tr(1, NA + k + 1);
+      Dot<R> qmd(ua), qpd(ua);
+      qmd.fma(-ph.mig[k], dm);
+      qpd.fma(-ph.mig[k], dp);
+      const R qm = qmd.get(), qp = qpd.get();
+      const R qa = halfv(qm + qp);
+      // 2 S = D (2 delta jc - dd) + cm qm + cp qp + |qa| jc
+      Dot<R> x(delta + delta, jc);
+      x.add(-dd);
+      Dot<R> sk(ph.D[k], x.get());
+      sk.fma(cm, qm);
+      sk.fma(cp, qp);
+      sk.fma(absv(qa), jc);
+      put(k + 1, hw * sk.get());
+      put(NF + k + 1, -(hw * (ph.D[k] * jc)));
+      acc(km, k == 0, ph.kcoef[k], cm);
+      acc(kp, k == 0, ph.kcoef[k], cp);
+      acc(t0, k == 0, ph.acoef[k], jc);
+      acc(s0, k == 0, ph.acoef[k], dd);
+    }
+    kapm = km.get(); kapp = kp.get();
+    Dot<R> tL = t0, tU = t0;
+    tL.fma(kapm, jphi);
+    tU.fma(kapp, jphi);
+    put(NF, -(hw * tL.get()));
+    put(2 * NF, -(hw * tU.get()));
+    s0.fma(kapm, dm);
+    s0.fma(kapp, dp);
+    s0.fma(-(delta * jphi), kapm + kapp);
+    put(0, -(hw * s0.get()));
+  } else if constexpr (MODE == kJvp) {
+    const R jphi0 = tr(0, 0) - tr(1, 0), jphi1 = tr(0, 1) - tr(1, 1);
+    const R d0m = tr(0, NA), d0p = tr(1, NA), d1m = tr(0, NA + 1), d1p = tr(1, NA + 1);
+    const R e1 = halfv(d1m + d1p);
+    Dot<R> t0, s0;
+    Dot<R> k0m, k0p, k1m, k1p;
+#pragma unroll
+    for (int k = 0; k < NF - 1; ++k) {
+      const R c0m = tr(0, NF + 1 + k), c0p = tr(1, NF + 1 + k);
+      const R c1m = tr(0, 2 + k), c1p = tr(1, 2 + k);
+      const R jc0 = c0m - c0p, jc1 = c1m - c1p;
+      const R dd = tr(0, NA + 2 + k) + tr(1, NA + 2 + k);
+      Dot<R> qmd(ua), qpd(ua);
+      qmd.fma(-ph.mig[k], d0m);
+      qpd.fma(-ph.mig[k], d0p);
+      const R qm = qmd.get(), qp = qpd.get();
+      const R qa = halfv(qm + qp);
+      const R sg = qa > R(0) ? jc0 : (qa < R(0) ? -jc0 : R(0));
+      // 2 S' = D (2 delta jc' - dd') + cm' qm + cp' qp + |qa| jc'
+      //        - mig (cm dm' + cp dp' + sign(qa) jc (dm' + dp') / 2)
+      Dot<R> x(delta + delta, jc1);
+      x.add(-dd);
+      Dot<R> y(c0m, d1m);
+      y.fma(c0p, d1p);
+      y.fma(sg, e1);
+      Dot<R> sk(ph.D[k], x.get());
+      sk.fma(c1m, qm);
+      sk.fma(c1p, qp);
+      sk.fma(absv(qa), jc1);
+      sk.fma(-ph.mig[k], y.get());
+      put(k + 1, hw * sk.get());
+      put(NF + k + 1, -(hw * (ph.D[k] * jc1)));
+      acc(k0m, k == 0, ph.kcoef[k], c0m);
+      acc(k0p, k == 0, ph.kcoef[k], c0p);
+      acc(k1m, k == 0, ph.kcoef[k], c1m);
+      acc(k1p, k == 0, ph.kcoef[k], c1p);
+      acc(t0, k == 0, ph.acoef[k], jc1);
+      acc(s0, k == 0, ph.acoef[k], dd);
+    }
+    const R a0m = k0m.get(), a0p = k0p.get(), a1m = k1m.get(), a1p = k1p.get();
+    Dot<R> tL = t0, tU = t0;
+    tL.fma(a1m, jphi0);
+    tL.fma(a0m, jphi1);
+    tU.fma(a1p, jphi0);
+    tU.fma(a0p, jphi1);
+    put(NF, -(hw * tL.get()));
+    put(2 * NF, -(hw * tU.get()));
+    s0.fma(a1m, d0m);
+    s0.fma(a0m, d1m);
+    s0.fma(a1p, d0p);
+    s0.fma(a0p, d1p);
+    Dot<R> pen(a1m + a1p, jphi0);
+    pen.fma(a0m + a0p, jphi1);
+    s0.fma(-delta, pen.get());
+    put(0, -(hw * s0.get()));
+  } else {
+    // adjoint: the functional S_f (wm_f - wp_f) + T_f (dwm_f + dwp_f) (the
+    // potential's T with each side's own kappa), differentiated by both states
+    const R jphi = tr(0, 0) - tr(1, 0), dm = tr(0, NA), dp = tr(1, NA);
+    const R jw0 = tr(0, 1) - tr(1, 1), vm0 = tr(0, NA + 1), vp0 = tr(1, NA + 1);
+    const R vs = vm0 + vp0;
+    const R dj = delta * jphi;
+    Dot<R> km, kp, am, ap;
+#pragma unroll
+    for (int k = 0; k < NF - 1; ++k) {
+      const R cm = tr(0, NF + 1 + k), cp = tr(1, NF + 1 + k), jc = cm - cp;
+      const R jw = tr(0, 2 + k) - tr(1, 2 + k), vw = tr(0, NA + 2 + k) + tr(1, NA + 2 + k);
+      Dot<R> qmd(ua), qpd(ua);
+      qmd.fma(-ph.mig[k], dm);
+      qpd.fma(-ph.mig[k], dp);
+      const R qm = qmd.get(), qp = qpd.get();
+      const R qa = halfv(qm + qp), aq = absv(qa);
+      const R sg = qa > R(0) ? jc : (qa < R(0) ? -jc : R(0));
+      const R dj2 = ph.D[k] * (delta + delta);
+      // 2 x (derivatives with respect to cm, cp)
+      Dot<R> xm(dj2 + qm + aq, jw), xp_(-dj2 + qp - aq, jw);
+      Dot<R> dv(ph.D[k], vw);
+      dv.fma(ph.acoef[k], vs);
+      const R dvv = dv.get();
+      Dot<R> ym(dj - dm, jw0), yp(dj - dp, jw0);
+      ym.fma(-jphi, vm0);
+      yp.fma(-jphi, vp0);
+      xm.add(-dvv);
+      xm.fma(ph.kcoef[k], ym.get());
+      xp_.add(dvv);
+      xp_.fma(ph.kcoef[k], yp.get());
+      put(k + 1, hw * xm.get());
+      put(2 * NF + k + 1, hw * xp_.get());
+      Dot<R> tk(ph.D[k], jw);
+      tk.fma(ph.acoef[k], jw0);
+      put(NF + k + 1, -(hw * tk.get()));
+      const R mj = ph.mig[k] * jw, hs = halfv(sg);
+      acc(am, k == 0, mj, cm + hs);
+      acc(ap, k == 0, mj, cp + hs);
+      acc(km, k == 0, ph.kcoef[k], cm);
+      acc(kp, k == 0, ph.kcoef[k], cp);
+    }
+    const R kapm = km.get(), kapp = kp.get();
+    Dot<R> x0(kapm, vm0);
+    x0.fma(kapp, vp0);
+    x0.fma(-(delta * jw0), kapm + kapp);
+    put(0, -(hw * x0.get()));
+    am.fma(kapm, jw0);
+    ap.fma(kapp, jw0);
+    put(NF, -(hw * am.get()));
+    put(2 * NF, -(hw * ap.get()));
+  }
+}
+
+// The flux coefficients of one face point (tr and put as above).
+template <int P, int NF, int MODE, class R, class TR, class PUT>
+__device__ __forceinline__ void face_point(const OpParams& prm, const FaceAt& F,
+                                           const FaceGeo<R>& G, int bidx, int pt, TR tr, PUT put) {
   using SL = Slots<P, NF, MODE>;
   using TO = TabOff<P>;
   constexpr int Q = P + 2, NA = SL::NA;
   const PhysT<R>& ph = phys<R>(prm);
   const int a = F.a, b0 = a == 0 ? 1 : 0, b1 = a == 2 ? 1 : 2;
   const int k1 = pt % Q, k2 = pt / Q;
-  const R lo0 = vertex<R>(prm, b0, F.j0), lo1 = vertex<R>(prm, b1, F.j1);
-  const R h0 = elem_size<R>(prm, b0, F.j0), h1 = elem_size<R>(prm, b1, F.j1);
-  const R xa = vertex<R>(prm, a, F.ia);
-  const R hL = F.hasL ? elem_size<R>(prm, a, F.ia - 1) : R(1);
-  const R hU = F.hasU ? elem_size<R>(prm, a, F.ia) : R(1);
+  const R h0 = G.h0, h1 = G.h1, xa = G.xa, hL = G.hL, hU = G.hU;
   const R hh = h0 * h0 + h1 * h1;
   R xp[3], uv[3];
   {
-    const R xb0 = lo0 + halfv((ctab<P, R>(TO::X + k1) + R(1)) * h0);
-    const R xb1 = lo1 + halfv((ctab<P, R>(TO::X + k2) + R(1)) * h1);
+    const R xb0 = G.lo0 + halfv((ctab<P, R>(TO::X + k1) + R(1)) * h0);
+    const R xb1 = G.lo1 + halfv((ctab<P, R>(TO::X + k2) + R(1)) * h1);
 #pragma unroll
     for (int c = 0; c < 3; ++c) xp[c] = c == a ? xa : (c == b0 ? xb0 : xb1);
   }
@@ -871,153 +1041,7 @@ __device__ __forceinline__ void face_point(const OpParams& prm, const FaceAt& F,
   const R w = ctab<P, R>(TO::W + k1) * ctab<P, R>(TO::W + k2) * (R(0.25f) * h0 * h1);
   if (F.hasL && F.hasU) {
     const R delta = ph.cip * R(P * P) / halfv(sqrtv(hL * hL + hh) + sqrtv(hU * hU + hh));
-    const R hw = halfv(w);
-    if constexpr (MODE == kResidual) {
-      const R pm = tr(0, 0), pp = tr(1, 0), dm = tr(0, NA), dp = tr(1, NA);
-      const R jphi = pm - pp;
-      R kapm, kapp;
-      Dot<R> t0, s0;
-      Dot<R> km, kp;
-#pragma unroll
-      for (int k = 0; k < NF - 1; ++k) {
-        const R cm = tr(0, k + 1), cp = tr(1, k + 1);
-        const R jc = cm - cp, dd = tr(0, NA + k + 1) + tr(1, NA + k + 1);
-        Dot<R> qmd(ua), qpd(ua);
-        qmd.fma(-ph.mig[k], dm);
-        qpd.fma(-ph.mig[k], dp);
-        const R qm = qmd.get(), qp = qpd.get();
-        const R qa = halfv(qm + qp);
-        // 2 S = D (2 delta jc - dd) + cm qm + cp qp + |qa| jc
-        Dot<R> x(delta + delta, jc);
-        x.add(-dd);
-        Dot<R> sk(ph.D[k], x.get());
-        sk.fma(cm, qm);
-        sk.fma(cp, qp);
-        sk.fma(absv(qa), jc);
-        put(k + 1, hw * sk.get());
-        put(NF + k + 1, -(hw * (ph.D[k] * jc)));
-        acc(km, k == 0, ph.kcoef[k], cm);
-        acc(kp, k == 0, ph.kcoef[k], cp);
-        acc(t0, k == 0, ph.acoef[k], jc);
-        acc(s0, k == 0, ph.acoef[k], dd);
-      }
-      kapm = km.get(); kapp = kp.get();
-      Dot<R> tL = t0, tU = t0;
-      tL.fma(kapm, jphi);
-      tU.fma(kapp, jphi);
-      put(NF, -(hw * tL.get()));
-      put(2 * NF, -(hw * tU.get()));
-      s0.fma(kapm, dm);
-      s0.fma(kapp, dp);
-      s0.fma(-(delta * jphi), kapm + kapp);
-      put(0, -(hw * s0.get()));
-    } else if constexpr (MODE == kJvp) {
-      const R jphi0 = tr(0, 0) - tr(1, 0), jphi1 = tr(0, 1) - tr(1, 1);
-      const R d0m = tr(0, NA), d0p = tr(1, NA), d1m = tr(0, NA + 1), d1p = tr(1, NA + 1);
-      const R e1 = halfv(d1m + d1p);
-      Dot<R> t0, s0;
-      Dot<R> k0m, k0p, k1m, k1p;
-#pragma unroll
-      for (int k = 0; k < NF - 1; ++k) {
-        const R c0m = tr(0, NF + 1 + k), c0p = tr(1, NF + 1 + k);
-        const R c1m = tr(0, 2 + k), c1p = tr(1, 2 + k);
-        const R jc0 = c0m - c0p, jc1 = c1m - c1p;
-        const R dd = tr(0, NA + 2 + k) + tr(1, NA + 2 + k);
-        Dot<R> qmd(ua), qpd(ua);
-        qmd.fma(-ph.mig[k], d0m);
-        qpd.fma(-ph.mig[k], d0p);
-        const R qm = qmd.get(), qp = qpd.get();
-        const R qa = halfv(qm + qp);
-        const R sg = qa > R(0) ? jc0 : (qa < R(0) ? -jc0 : R(0));
-        // 2 S' = D (2 delta jc' - dd') + cm' qm + cp' qp + |qa| jc'
-        //        - mig (cm dm' + cp dp' + sign(qa) jc (dm' + dp') / 2)
-        Dot<R> x(delta + delta, jc1);
-        x.add(-dd);
-        Dot<R> y(c0m, d1m);
-        y.fma(c0p, d1p);
-        y.fma(sg, e1);
-        Dot<R> sk(ph.D[k], x.get());
-        sk.fma(c1m, qm);
-        sk.fma(c1p, qp);
-        sk.fma(absv(qa), jc1);
-        sk.fma(-ph.mig[k], y.get());
-        put(k + 1, hw * sk.get());
-        put(NF + k + 1, -(hw * (ph.D[k] * jc1)));
-        acc(k0m, k == 0, ph.kcoef[k], c0m);
-        acc(k0p, k == 0, ph.kcoef[k], c0p);
-        acc(k1m, k == 0, ph.kcoef[k], c1m);
-        acc(k1p, k == 0, ph.kcoef[k], c1p);
-        acc(t0, k == 0, ph.acoef[k], jc1);
-        acc(s0, k == 0, ph.acoef[k], dd);
-      }
-      const R a0m = k0m.get(), a0p = k0p.get(), a1m = k1m.get(), a1p = k1p.get();
-      Dot<R> tL = t0, tU = t0;
-      tL.fma(a1m, jphi0);
-      tL.fma(a0m, jphi1);
-      tU.fma(a1p, jphi0);
-      tU.fma(a0p, jphi1);
-      put(NF, -(hw * tL.get()));
-      put(2 * NF, -(hw * tU.get()));
-      s0.fma(a1m, d0m);
-      s0.fma(a0m, d1m);
-      s0.fma(a1p, d0p);
-      s0.fma(a0p, d1p);
-      Dot<R> pen(a1m + a1p, jphi0);
-      pen.fma(a0m + a0p, jphi1);
-      s0.fma(-delta, pen.get());
-      put(0, -(hw * s0.get()));
-    } else {
-      // adjoint: the functional S_f (wm_f - wp_f) + T_f (dwm_f + dwp_f) (the
-      // potential's T with each side's own kappa), differentiated by both states
-      const R jphi = tr(0, 0) - tr(1, 0), dm = tr(0, NA), dp = tr(1, NA);
-      const R jw0 = tr(0, 1) - tr(1, 1), vm0 = tr(0, NA + 1), vp0 = tr(1, NA + 1);
-      const R vs = vm0 + vp0;
-      const R dj = delta * jphi;
-      Dot<R> km, kp, am, ap;
-#pragma unroll
-      for (int k = 0; k < NF - 1; ++k) {
-        const R cm = tr(0, NF + 1 + k), cp = tr(1, NF + 1 + k), jc = cm - cp;
-        const R jw = tr(0, 2 + k) - tr(1, 2 + k), vw = tr(0, NA + 2 + k) + tr(1, NA + 2 + k);
-        Dot<R> qmd(ua), qpd(ua);
-        qmd.fma(-ph.mig[k], dm);
-        qpd.fma(-ph.mig[k], dp);
-        const R qm = qmd.get(), qp = qpd.get();
-        const R qa = halfv(qm + qp), aq = absv(qa);
-        const R sg = qa > R(0) ? jc : (qa < R(0) ? -jc : R(0));
-        const R dj2 = ph.D[k] * (delta + delta);
-        // 2 x (derivatives with respect to cm, cp)
-        Dot<R> xm(dj2 + qm + aq, jw), xp_(-dj2 + qp - aq, jw);
-        Dot<R> dv(ph.D[k], vw);
-        dv.fma(ph.acoef[k], vs);
-        const R dvv = dv.get();
-        Dot<R> ym(dj - dm, jw0), yp(dj - dp, jw0);
-        ym.fma(-jphi, vm0);
-        yp.fma(-jphi, vp0);
-        xm.add(-dvv);
-        xm.fma(ph.kcoef[k], ym.get());
-        xp_.add(dvv);
-        xp_.fma(ph.kcoef[k], yp.get());
-        put(k + 1, hw * xm.get());
-        put(2 * NF + k + 1, hw * xp_.get());
-        Dot<R> tk(ph.D[k], jw);
-        tk.fma(ph.acoef[k], jw0);
-        put(NF + k + 1, -(hw * tk.get()));
-        const R mj = ph.mig[k] * jw, hs = halfv(sg);
-        acc(am, k == 0, mj, cm + hs);
-        acc(ap, k == 0, mj, cp + hs);
-        acc(km, k == 0, ph.kcoef[k], cm);
-        acc(kp, k == 0, ph.kcoef[k], cp);
-      }
-      const R kapm = km.get(), kapp = kp.get();
-      Dot<R> x0(kapm, vm0);
-      x0.fma(kapp, vp0);
-      x0.fma(-(delta * jw0), kapm + kapp);
-      put(0, -(hw * x0.get()));
-      am.fma(kapm, jw0);
-      ap.fma(kapp, jw0);
-      put(NF, -(hw * am.get()));
-      put(2 * NF, -(hw * ap.get()));
-    }
+    face_interior_point<P, NF, MODE, R>(ph, ua, w, delta, tr, put);
     return;
   }
   // boundary face: the one element's own side and outward normal
@@ -1180,8 +1204,11 @@ tileface3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<
     const R* t0 = A + fi * 2 * NTR * (Q * QP) + o;
     R* c0 = B + fi * NSL * (Q * QP) + o;
     const FaceAt F = FW == 1 ? F0 : face_at(prm, g0 + fi);
+    FaceGeo<R> G;
+    G.in_plane(prm, F.a, F.j0, F.j1);
+    G.along(prm, F.a, F.ia, F.hasL, F.hasU);
     face_point<P, NF, MODE, R>(
-        prm, F, bidx, pt, [&](int side, int t) -> R { return t0[(side * NTR + t) * (Q * QP)]; },
+        prm, F, G, bidx, pt, [&](int side, int t) -> R { return t0[(side * NTR + t) * (Q * QP)]; },
         [&](int slot, R val) { c0[slot * (Q * QP)] = val; });
   }
   group_sync<face_lock<R>()>();

@@ -266,3 +266,40 @@ def test_sweep_automatic_mode(n_along, same_as):
         zs[mode] = op.block_jacobi_apply(r).cpu().numpy()
     np.testing.assert_array_equal(zs[2], zs[same_as])
     assert np.linalg.norm(zs[2] - zs[1 - same_as]) > 0
+
+
+@pytest.mark.parametrize("direction", [1, -1])
+@pytest.mark.parametrize("fields", [2, 3])
+@pytest.mark.parametrize("p", [1, 2, 3, 4])
+def test_sweep_every_block_size(p, fields, direction):
+    """Every degree and field count (the block is split over 1 to 4 threads per
+    row, and held in registers wholly or in part), both flow directions, each
+    storage of the inverses, on lines of three elements with the inlet upstream.
+    FP64 inverses: 1e-10 as above. FP32 and BF16: a stored inverse is off by the
+    storage's unit roundoff, and one inverted in FP32 by its roundoff times the
+    block's condition number kappa (of the oracle's blocks), three elements deep."""
+    import scipy.sparse.linalg as spla
+    enp = _enp()
+    base = W.config("cube_n2_p2" if fields == 2 else "channel_n1", p=p)
+    n = [3, 1, 2]
+    coords = [c[-1] * np.linspace(0, 1, k + 1) ** 1.2 for c, k in zip(base.coords, n)]
+    tags = W.box_tags(3, n, coords, W.WALL)
+    tags[0][:], tags[1][:] = (W.INLET, W.OUTLET) if direction > 0 else (W.OUTLET, W.INLET)
+    tags[2][:] = W.ELECTRODE0
+    vp = list(base.vel_params)
+    vp[4] *= direction
+    P = dataclasses.replace(base, n_el=n, coords=coords, tags=tags, vel_params=vp)
+    u, r = W.random_state(P, 2), W.random_vector(P, 5)
+    orc = oracle.Oracle(P)
+    ref = spla.spsolve(_lower_block_system(orc, P, u, 0, direction).tocsc(), r)
+    kappa = max(np.linalg.cond(b) for b in orc.block_diagonal(u))
+    op = enp.Operator(P)
+    op.set_sweep(1)
+    for storage, unit in ((enp.BJ_F64, 0.0), (enp.BJ_F32, 2.0 ** -24), (enp.BJ_BF16, 2.0 ** -9)):
+        tol = 1e-10 if storage == enp.BJ_F64 else 3 * kappa * (unit + 10 * 2.0 ** -24)
+        op.block_jacobi_setup(_cuda(u), storage)
+        z = op.block_jacobi_apply(_cuda(r)).cpu().numpy()
+        assert np.linalg.norm(z - ref) <= tol * np.linalg.norm(ref)
+        if storage != enp.BJ_F64:
+            z = op.block_jacobi_apply_f32(_cuda(r).float()).cpu().numpy()
+            assert np.linalg.norm(z - ref) <= tol * np.linalg.norm(ref)
