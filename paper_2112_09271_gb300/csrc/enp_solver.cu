@@ -429,71 +429,122 @@ __global__ void coarse_pack32(const double* __restrict__ A, float* __restrict__ 
   }
 }
 
-__device__ __forceinline__ float stencil_off(const float* __restrict__ a, const float* __restrict__ x,
-                                             int i, int nx, int ny, int nz, int ix, int iy, int iz) {
+// A cell's packed stencil, as two 16-byte loads.
+struct Cell7 {
+  float4 lo, hi;   // (self, -x, +x, -y), (+y, -z, +z, 1 / self)
+  __device__ __forceinline__ Cell7(const float* __restrict__ A, int i) {
+    const float4* p = reinterpret_cast<const float4*>(A) + 2 * (long long)i;
+    lo = __ldg(p);
+    hi = __ldg(p + 1);
+  }
+};
+// Values that other blocks of the cluster write are read past L1 (CG).
+template <bool CG>
+__device__ __forceinline__ float ld(const float* p) {
+  return CG ? __ldcg(p) : *p;
+}
+
+// Off-diagonal part of row i with x given by a function of the cell.
+template <class X>
+__device__ __forceinline__ float stencil_off(const Cell7& a, X x, int i, int nx, int ny, int nz,
+                                             int ix, int iy, int iz) {
   float s = 0.0f;
-  if (ix > 0) s += a[1] * x[i - 1];
-  if (ix < nx - 1) s += a[2] * x[i + 1];
-  if (iy > 0) s += a[3] * x[i - nx];
-  if (iy < ny - 1) s += a[4] * x[i + nx];
-  if (iz > 0) s += a[5] * x[i - nx * ny];
-  if (iz < nz - 1) s += a[6] * x[i + nx * ny];
+  if (ix > 0) s += a.lo.y * x(i - 1);
+  if (ix < nx - 1) s += a.lo.z * x(i + 1);
+  if (iy > 0) s += a.lo.w * x(i - nx);
+  if (iy < ny - 1) s += a.hi.x * x(i + nx);
+  if (iz > 0) s += a.hi.y * x(i - nx * ny);
+  if (iz < nz - 1) s += a.hi.z * x(i + nx * ny);
   return s;
 }
 
 // The per-cell steps of the V-cycle, shared by the grid-wide kernels (large
-// levels) and the one-block kernel (small levels), so both give the same bits.
+// levels) and the cluster kernel (small levels), so both give the same bits.
 // Ab, xb, bb: one operating point's packed stencil, iterate and right-hand side.
 
 // Gauss-Seidel update of cell i if it has parity `colour` (red-black).
-__device__ __forceinline__ void gs_cell(const float* __restrict__ Ab, float* __restrict__ xb,
-                                        const float* __restrict__ bb, int nx, int ny, int nz,
-                                        int colour, int i) {
+template <bool CG>
+__device__ __forceinline__ void gs_cell(const float* __restrict__ Ab, float* xb, const float* bb,
+                                        int nx, int ny, int nz, int colour, int i) {
   const int ix = i % nx, iy = (i / nx) % ny, iz = i / (nx * ny);
   if (((ix + iy + iz) & 1) != colour) return;
-  const float* a = Ab + (long long)i * kPack;
-  if (a[7] == 0.0f) return;
-  xb[i] = (bb[i] - stencil_off(a, xb, i, nx, ny, nz, ix, iy, iz)) * a[7];
+  const Cell7 a(Ab, i);
+  if (a.hi.w == 0.0f) return;
+  xb[i] = (ld<CG>(bb + i) - stencil_off(a, [&](int j) { return ld<CG>(xb + j); }, i, nx, ny, nz, ix,
+                                        iy, iz)) * a.hi.w;
 }
 
-__device__ __forceinline__ float residual_cell(const float* __restrict__ Ab,
-                                               const float* __restrict__ xb,
-                                               const float* __restrict__ bb, int nx, int ny,
-                                               int nz, int i) {
+// The first sweep from x = 0, both colours at once: a cell of colour 0 sees zero
+// neighbours, one of colour 1 its neighbours' updates, formed again here.
+template <bool CG>
+__device__ __forceinline__ void gs_first_cell(const float* __restrict__ Ab, float* xb,
+                                              const float* bb, int nx, int ny, int nz, int i) {
   const int ix = i % nx, iy = (i / nx) % ny, iz = i / (nx * ny);
-  const float* a = Ab + (long long)i * kPack;
-  return bb[i] - a[0] * xb[i] - stencil_off(a, xb, i, nx, ny, nz, ix, iy, iz);
+  const Cell7 a(Ab, i);
+  float v = 0.0f;
+  if (a.hi.w != 0.0f) {
+    v = ld<CG>(bb + i);
+    if ((ix + iy + iz) & 1)
+      v -= stencil_off(a, [&](int j) { return ld<CG>(bb + j) * __ldg(Ab + (long long)j * kPack + 7); },
+                       i, nx, ny, nz, ix, iy, iz);
+    v *= a.hi.w;
+  }
+  xb[i] = v;
 }
 
-// sum of the fine values over the 2 x 2 x 2 aggregate of coarse cell C
-__device__ __forceinline__ float restrict_cell(const float* __restrict__ rf, int fx, int fy,
-                                               int fz, int cx, int cy, int C) {
+template <bool CG>
+__device__ __forceinline__ float residual_cell(const float* __restrict__ Ab, const float* xb,
+                                               const float* bb, int nx, int ny, int nz, int ix,
+                                               int iy, int iz) {
+  const int i = ix + nx * (iy + ny * iz);
+  const Cell7 a(Ab, i);
+  return ld<CG>(bb + i) - a.lo.x * ld<CG>(xb + i) -
+         stencil_off(a, [&](int j) { return ld<CG>(xb + j); }, i, nx, ny, nz, ix, iy, iz);
+}
+
+// sum of the fine residual b - A x over the 2 x 2 x 2 aggregate of coarse cell C
+template <bool CG>
+__device__ __forceinline__ float restrict_cell(const float* __restrict__ Ab, const float* xb,
+                                               const float* bb, int fx, int fy, int fz, int cx,
+                                               int cy, int C) {
   const int jx = C % cx, jy = (C / cx) % cy, jz = C / (cx * cy);
   float s = 0.0f;
-  for (int dz = 0; dz < 2; ++dz)
-    for (int dy = 0; dy < 2; ++dy)
-      for (int dx = 0; dx < 2; ++dx) {
-        const int ix = 2 * jx + dx, iy = 2 * jy + dy, iz = 2 * jz + dz;
-        if (ix < fx && iy < fy && iz < fz) s += rf[ix + fx * (iy + fy * iz)];
-      }
+#pragma unroll
+  for (int d = 0; d < 8; ++d) {
+    const int ix = 2 * jx + (d & 1), iy = 2 * jy + ((d >> 1) & 1), iz = 2 * jz + (d >> 2);
+    if (ix < fx && iy < fy && iz < fz) s += residual_cell<CG>(Ab, xb, bb, fx, fy, fz, ix, iy, iz);
+  }
   return s;
 }
 
-// the coarse value of the aggregate that holds fine cell i
-__device__ __forceinline__ float prolong_cell(const float* __restrict__ xc, int cx, int cy,
-                                              int fx, int fy, int i) {
+// x_i += omega times the coarse value of its aggregate, for the cells that keep
+// it: the post-smoothing starts by overwriting the cells of colour 1 (those with
+// a zero diagonal excepted).
+template <bool CG>
+__device__ __forceinline__ void prolong_cell(const float* __restrict__ Ab, const float* xc, int cx,
+                                             int cy, float* xb, int fx, int fy, float omega, int i) {
   const int ix = i % fx, iy = (i / fx) % fy, iz = i / (fx * fy);
-  return xc[ix / 2 + cx * (iy / 2 + cy * (iz / 2))];
+  if (((ix + iy + iz) & 1) && __ldg(Ab + (long long)i * kPack + 7) != 0.0f) return;
+  xb[i] = ld<CG>(xb + i) + omega * ld<CG>(xc + ix / 2 + cx * (iy / 2 + cy * (iz / 2)));
 }
 
-// One half-sweep of red-black Gauss-Seidel on cells of parity `colour`.
-__global__ void coarse_gs(const float* __restrict__ A, float* __restrict__ x,
-                          const float* __restrict__ bvec, int nx, int ny, int nz, int colour) {
+__global__ void coarse_gs_first(const float* __restrict__ A, float* __restrict__ x,
+                                const float* __restrict__ bvec, int nx, int ny, int nz) {
   const int b = blockIdx.y;
   const int N = nx * ny * nz;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x)
-    gs_cell(A + (long long)b * N * kPack, x + (long long)b * N, bvec + (long long)b * N, nx, ny,
-            nz, colour, i);
+    gs_first_cell<false>(A + (long long)b * N * kPack, x + (long long)b * N, bvec + (long long)b * N,
+                         nx, ny, nz, i);
+}
+
+// One half-sweep of red-black Gauss-Seidel on cells of parity `colour`.
+__global__ void coarse_gs(const float* __restrict__ A, float* x, const float* __restrict__ bvec,
+                          int nx, int ny, int nz, int colour) {
+  const int b = blockIdx.y;
+  const int N = nx * ny * nz;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x)
+    gs_cell<false>(A + (long long)b * N * kPack, x + (long long)b * N, bvec + (long long)b * N, nx,
+                   ny, nz, colour, i);
 }
 
 // r = b - A x
@@ -503,34 +554,37 @@ __global__ void coarse_residual(const float* __restrict__ A, const float* __rest
   const int b = blockIdx.y;
   const int N = nx * ny * nz;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x)
-    r[(long long)b * N + i] = residual_cell(A + (long long)b * N * kPack, x + (long long)b * N,
-                                            bvec + (long long)b * N, nx, ny, nz, i);
+    r[(long long)b * N + i] =
+        residual_cell<false>(A + (long long)b * N * kPack, x + (long long)b * N,
+                             bvec + (long long)b * N, nx, ny, nz, i % nx, (i / nx) % ny, i / (nx * ny));
 }
 
 // b_c = sum of the fine residual over each 2 x 2 x 2 aggregate
-__global__ void coarse_restrict(const float* __restrict__ rf, int fx, int fy, int fz,
+__global__ void coarse_restrict(const float* __restrict__ A, const float* __restrict__ x,
+                                const float* __restrict__ bvec, int fx, int fy, int fz,
                                 float* __restrict__ bc, int cx, int cy, int cz) {
   const int b = blockIdx.y;
   const int Nc = cx * cy * cz, Nf = fx * fy * fz;
   for (int C = blockIdx.x * blockDim.x + threadIdx.x; C < Nc; C += gridDim.x * blockDim.x)
-    bc[(long long)b * Nc + C] = restrict_cell(rf + (long long)b * Nf, fx, fy, fz, cx, cy, C);
+    bc[(long long)b * Nc + C] =
+        restrict_cell<false>(A + (long long)b * Nf * kPack, x + (long long)b * Nf,
+                             bvec + (long long)b * Nf, fx, fy, fz, cx, cy, C);
 }
 
-// x_f += omega x_c on every fine cell of the aggregate
-__global__ void coarse_prolong(const float* __restrict__ xc, int cx, int cy, int cz,
-                               float* __restrict__ xf, int fx, int fy, int fz, float omega) {
+__global__ void coarse_prolong(const float* __restrict__ A, const float* __restrict__ xc, int cx,
+                               int cy, int cz, float* xf, int fx, int fy, int fz, float omega) {
   const int b = blockIdx.y;
   const int Nc = cx * cy * cz, Nf = fx * fy * fz;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < Nf; i += gridDim.x * blockDim.x)
-    xf[(long long)b * Nf + i] += omega * prolong_cell(xc + (long long)b * Nc, cx, cy, fx, fy, i);
+    prolong_cell<false>(A + (long long)b * Nf * kPack, xc + (long long)b * Nc, cx, cy,
+                        xf + (long long)b * Nf, fx, fy, omega, i);
 }
 
 // The coarsest level (at most kCoarsestCells cells) is solved with its dense
 // inverse, computed in FP64 at setup by the block Gauss-Jordan kernel below and
 // stored in FP32. If that matrix is singular to working accuracy (a potential
 // fixed by no boundary condition), it is smoothed instead: x = 0, then
-// `sweeps` red-black Gauss-Seidel sweeps inside one thread block per operating
-// point, with the stencil, x and b held in shared memory.
+// red-black Gauss-Seidel sweeps.
 constexpr int kCoarsestCells = 128;
 
 // dense[b][i][j] = the FP64 stencil rows of a level as a dense n x n matrix
@@ -556,59 +610,25 @@ __global__ void coarse_dense(const double* __restrict__ A, int nx, int ny, int n
   }
 }
 
-// Row r of inv * b with the inverse stored transposed (M[c][r]).
-__device__ __forceinline__ float dense_row(const float* __restrict__ M,
-                                           const float* __restrict__ bb, int N, int r) {
-  float s = 0.0f;
-  for (int c = 0; c < N; ++c) s += M[(long long)c * N + r] * bb[c];
-  return s;
-}
-
-// x_b = inv_b r_b, one block per operating point.
-__global__ void __launch_bounds__(kCoarsestCells)
-coarse_dense_apply(const float* __restrict__ invT, const float* __restrict__ rhs, int N,
-                   float* __restrict__ x) {
-  const int b = blockIdx.x;
-  for (int r = threadIdx.x; r < N; r += blockDim.x)
-    x[(long long)b * N + r] = dense_row(invT + (long long)b * N * N, rhs + (long long)b * N, N, r);
-}
-
-__global__ void __launch_bounds__(kCoarsestCells)
-coarse_solve_small(const float* __restrict__ A, float* __restrict__ x,
-                   const float* __restrict__ bvec, int nx, int ny, int nz, int sweeps) {
-  __shared__ float sA[kCoarsestCells * kPack];
-  __shared__ float sx[kCoarsestCells];
-  __shared__ float sb[kCoarsestCells];
-  const int b = blockIdx.x;
-  const int N = nx * ny * nz;  // <= kCoarsestCells, checked by the host
-  const float* Ab = A + (long long)b * N * kPack;
-  for (int i = threadIdx.x; i < kPack * N; i += blockDim.x) sA[i] = Ab[i];
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    sx[i] = 0.0f;
-    sb[i] = bvec[(long long)b * N + i];
-  }
-  __syncthreads();
-  for (int sw = 0; sw < sweeps; ++sw)
-    for (int colour = 0; colour < 2; ++colour) {
-      for (int i = threadIdx.x; i < N; i += blockDim.x) gs_cell(sA, sx, sb, nx, ny, nz, colour, i);
-      __syncthreads();
-    }
-  for (int i = threadIdx.x; i < N; i += blockDim.x) x[(long long)b * N + i] = sx[i];
-}
-
-// The small levels of the V-cycle (at most kTailCells cells) run in one
-// thread block per operating point, with a barrier between steps, instead of
-// one launch per half-sweep: levels l0 .. nl-2 are smoothed, their residuals
-// restricted, the coarsest solved (its inverse, or smoothing), and the
-// corrections prolonged and post-smoothed, as in the grid-wide kernels.
-constexpr int kTailCells = 8192;
+// The levels of at most kTailCells cells run in one launch, one cluster of
+// thread blocks per operating point, with a cluster barrier between steps
+// instead of a launch per half-sweep; those of at most kSoloCells cells in the
+// cluster's first block, from its shared memory, while the others wait at one
+// barrier. A step of the level reads its stencils (32 bytes a cell) from L2 and
+// costs a launch or a barrier: with one launch per half-sweep above 8192 cells
+// the V-cycle of 192 x 48 x 16 cells took 170 us, 125 in this form (a cluster for
+// that many cells too: 220, eight SMs are too few).
+constexpr int kTailCells = 32768;
+constexpr int kTailCtas = 8;
 constexpr int kTailThreads = 1024;
-constexpr int kMaxLevels = 16;
+constexpr int kSoloCells = 2048;
+constexpr int kSoloFloats = 4 * kSoloCells;   // x and b of the solo levels (each at most half the one above)
+constexpr int kMaxLevels = 32;      // 2^30 cells in a row have 24
 
 struct LevelDev {
   int nx, ny, nz, n;
   const float* A;
-  float *x, *b, *r;
+  float *x, *b;
 };
 
 struct VcycleTail {
@@ -619,79 +639,142 @@ struct VcycleTail {
   float omega;       // over-correction of the prolongated coarse values
 };
 
-__global__ void __launch_bounds__(kTailThreads) coarse_vcycle_tail(const VcycleTail T) {
-  const int b = blockIdx.x;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int l = T.l0; l < T.nl - 1; ++l) {
-    const LevelDev L = T.L[l], C = T.L[l + 1];
-    const int N = L.n;
-    const float* Ab = L.A + (long long)b * N * kPack;
-    float* xb = L.x + (long long)b * N;
-    const float* bb = L.b + (long long)b * N;
-    float* rb = L.r + (long long)b * N;
-    for (int i = tid; i < N; i += nt) xb[i] = 0.0f;
-    __syncthreads();
-    for (int sw = 0; sw < T.smooth; ++sw)
-      for (int colour = 0; colour < 2; ++colour) {
-        for (int i = tid; i < N; i += nt) gs_cell(Ab, xb, bb, L.nx, L.ny, L.nz, colour, i);
-        __syncthreads();
-      }
-    for (int i = tid; i < N; i += nt) rb[i] = residual_cell(Ab, xb, bb, L.nx, L.ny, L.nz, i);
-    __syncthreads();
-    for (int c = tid; c < C.n; c += nt)
-      C.b[(long long)b * C.n + c] = restrict_cell(rb, L.nx, L.ny, L.nz, C.nx, C.ny, c);
-    __syncthreads();
-  }
-  {
-    const LevelDev L = T.L[T.nl - 1];
-    const int N = L.n;
-    float* xb = L.x + (long long)b * N;
-    const float* bb = L.b + (long long)b * N;
-    if (T.inv) {
-      for (int r = tid; r < N; r += nt) xb[r] = dense_row(T.inv + (long long)b * N * N, bb, N, r);
-    } else {
-      const float* Ab = L.A + (long long)b * N * kPack;
-      for (int i = tid; i < N; i += nt) xb[i] = 0.0f;
-      __syncthreads();
-      for (int sw = 0; sw < T.coarsest_sweeps; ++sw)
-        for (int colour = 0; colour < 2; ++colour) {
-          for (int i = tid; i < N; i += nt) gs_cell(Ab, xb, bb, L.nx, L.ny, L.nz, colour, i);
-          __syncthreads();
-        }
+// Down (pre-smooth, restrict the residual into bc) and up (prolong, post-smooth)
+// on one level; tid, nt: the threads that share it, sync: their barrier.
+template <bool CG, class SYNC>
+__device__ __forceinline__ void vcycle_down(const LevelDev& L, const LevelDev& C, const float* Ab,
+                                            float* xb, const float* bb, float* bc, int smooth,
+                                            int tid, int nt, SYNC sync) {
+  for (int i = tid; i < L.n; i += nt) gs_first_cell<CG>(Ab, xb, bb, L.nx, L.ny, L.nz, i);
+  sync();
+  for (int sw = 1; sw < smooth; ++sw)
+    for (int colour = 0; colour < 2; ++colour) {
+      for (int i = tid; i < L.n; i += nt) gs_cell<CG>(Ab, xb, bb, L.nx, L.ny, L.nz, colour, i);
+      sync();
     }
-    __syncthreads();
+  for (int c = tid; c < C.n; c += nt)
+    bc[c] = restrict_cell<CG>(Ab, xb, bb, L.nx, L.ny, L.nz, C.nx, C.ny, c);
+  sync();
+}
+template <bool CG, class SYNC>
+__device__ __forceinline__ void vcycle_up(const LevelDev& L, const LevelDev& C, const float* Ab,
+                                          float* xb, const float* bb, const float* xc, float omega,
+                                          int smooth, int tid, int nt, SYNC sync) {
+  for (int i = tid; i < L.n; i += nt)
+    prolong_cell<CG>(Ab, xc, C.nx, C.ny, xb, L.nx, L.ny, omega, i);
+  sync();
+  for (int sw = 0; sw < smooth; ++sw)
+    for (int colour = 1; colour >= 0; --colour) {
+      for (int i = tid; i < L.n; i += nt) gs_cell<CG>(Ab, xb, bb, L.nx, L.ny, L.nz, colour, i);
+      sync();
+    }
+}
+
+__global__ void __cluster_dims__(kTailCtas, 1, 1) __launch_bounds__(kTailThreads)
+coarse_vcycle_tail(const VcycleTail T) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  __shared__ float solo[kSoloFloats];
+  const int b = blockIdx.y, rank = (int)cluster.block_rank();
+  const int ct = rank * kTailThreads + threadIdx.x, cn = kTailCtas * kTailThreads;
+  auto csync = [&] { cluster.sync(); };
+  int s0 = T.l0;      // first solo level: every level below it fits as well
+  while (s0 < T.nl - 1 && T.L[s0].n > kSoloCells) ++s0;
+  for (int l = T.l0; l < s0; ++l) {
+    const LevelDev &L = T.L[l], &C = T.L[l + 1];
+    vcycle_down<true>(L, C, L.A + (long long)b * L.n * kPack, L.x + (long long)b * L.n,
+                      L.b + (long long)b * L.n, C.b + (long long)b * C.n, T.smooth, ct, cn, csync);
   }
-  for (int l = T.nl - 2; l >= T.l0; --l) {
-    const LevelDev L = T.L[l], C = T.L[l + 1];
-    const int N = L.n;
-    const float* Ab = L.A + (long long)b * N * kPack;
-    float* xb = L.x + (long long)b * N;
-    const float* bb = L.b + (long long)b * N;
-    for (int i = tid; i < N; i += nt)
-      xb[i] += T.omega * prolong_cell(C.x + (long long)b * C.n, C.nx, C.ny, L.nx, L.ny, i);
+  if (rank == 0) {
+    const int tid = threadIdx.x, nt = kTailThreads;
+    auto bsync = [] { __syncthreads(); };
+    // x and b of the solo levels, one after the other
+    for (int i = tid; i < T.L[s0].n; i += nt)
+      solo[T.L[s0].n + i] = __ldcg(T.L[s0].b + (long long)b * T.L[s0].n + i);
     __syncthreads();
-    for (int sw = 0; sw < T.smooth; ++sw)
-      for (int colour = 1; colour >= 0; --colour) {
-        for (int i = tid; i < N; i += nt) gs_cell(Ab, xb, bb, L.nx, L.ny, L.nz, colour, i);
+    float* p = solo;
+    for (int l = s0; l < T.nl - 1; ++l) {
+      const LevelDev &L = T.L[l], &C = T.L[l + 1];
+      float* pc = p + 2 * L.n;
+      vcycle_down<false>(L, C, L.A + (long long)b * L.n * kPack, p, p + L.n, pc + C.n, T.smooth, tid,
+                         nt, bsync);
+      p = pc;
+    }
+    {
+      const LevelDev& L = T.L[T.nl - 1];
+      const int N = L.n;
+      if (T.inv) {
+        // eight threads per row, every eighth column each, summed in a fixed tree
+        const float* M = T.inv + (long long)b * N * N;
+        const int part = tid & 7;
+        for (int r0 = 0; r0 < N; r0 += nt / 8) {
+          const int r = r0 + tid / 8;
+          float s = 0.0f;
+          if (r < N)
+            for (int c = part; c < N; c += 8) s += __ldg(M + (long long)c * N + r) * p[N + c];
+          s += __shfl_xor_sync(0xffffffffu, s, 1);
+          s += __shfl_xor_sync(0xffffffffu, s, 2);
+          s += __shfl_xor_sync(0xffffffffu, s, 4);
+          if (r < N && part == 0) p[r] = s;
+        }
+      } else {
+        const float* Ab = L.A + (long long)b * N * kPack;
+        for (int i = tid; i < N; i += nt) p[i] = 0.0f;
         __syncthreads();
+        for (int sw = 0; sw < T.coarsest_sweeps; ++sw)
+          for (int colour = 0; colour < 2; ++colour) {
+            for (int i = tid; i < N; i += nt) gs_cell<false>(Ab, p, p + N, L.nx, L.ny, L.nz, colour, i);
+            __syncthreads();
+          }
       }
+      __syncthreads();
+    }
+    for (int l = T.nl - 2; l >= s0; --l) {
+      const LevelDev &L = T.L[l], &C = T.L[l + 1];
+      float* pf = p - 2 * L.n;
+      vcycle_up<false>(L, C, L.A + (long long)b * L.n * kPack, pf, pf + L.n, p, T.omega, T.smooth,
+                       tid, nt, bsync);
+      p = pf;
+    }
+    for (int i = tid; i < T.L[s0].n; i += nt) T.L[s0].x[(long long)b * T.L[s0].n + i] = p[i];
+  }
+  cluster.sync();
+  for (int l = s0 - 1; l >= T.l0; --l) {
+    const LevelDev &L = T.L[l], &C = T.L[l + 1];
+    vcycle_up<true>(L, C, L.A + (long long)b * L.n * kPack, L.x + (long long)b * L.n,
+                    L.b + (long long)b * L.n, C.x + (long long)b * C.n, T.omega, T.smooth, ct, cn,
+                    csync);
   }
 }
 
-// b0[K] = sum over the Phi nodes of element K of r (P^T r), summed in FP64;
-// one warp per element
+// b0[K] = sum over the Phi nodes of element K of r (P^T r), one lane per element:
+// FP64 vectors summed in FP64, FP32 ones as a double-float pair (TwoSum), which
+// rounds to the same FP32 value and keeps off the FP64 pipe (a warp per element
+// with an FP64 shuffle tree took 77 us on 147,456 elements, 9.6 now).
 template <class TV>
 __global__ void coarse_from_fine(const TV* __restrict__ r, float* __restrict__ b0, int E, int Np,
                                  long long bstride) {
   const int b = blockIdx.y;
-  const int lane = threadIdx.x & 31;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int K = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; K < E; K += nw) {
+  for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < E; K += gridDim.x * blockDim.x) {
     const TV* row = r + b * bstride + (long long)K * Np;
-    double s = 0.0;
-    for (int i = lane; i < Np; i += 32) s += (double)row[i];
-    s = warp_sum(s);
-    if (lane == 0) b0[(long long)b * E + K] = (float)s;
+    float out;
+    if constexpr (std::is_same<TV, float>::value) {
+      float s = row[0], t = 0.0f;
+#pragma unroll 4
+      for (int i = 1; i < Np; ++i) {
+        float s2, err;
+        two_sum(s, row[i], s2, err);
+        s = s2;
+        t = __fadd_rn(t, err);
+      }
+      out = __fadd_rn(s, t);
+    } else {
+      double s = row[0];
+#pragma unroll 4
+      for (int i = 1; i < Np; ++i) s += row[i];
+      out = (float)s;
+    }
+    b0[(long long)b * E + K] = out;
   }
 }
 
@@ -702,15 +785,15 @@ __global__ void axpy_f32(const float* __restrict__ x, float* __restrict__ acc, l
     acc[t] += x[t];
 }
 
-// z[Phi nodes of K] += x0[K] (P x0)
+// z[Phi nodes of K] += x0[K] (P x0); blockDim.x is a multiple of Np and a block
+// takes whole elements, so that no index is divided in 64 bits
 template <class TV>
 __global__ void coarse_to_fine(const float* __restrict__ x0, TV* __restrict__ z, int E, int Np,
                                long long bstride) {
   const int b = blockIdx.y;
-  const long long n = (long long)E * Np;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
-       t += (long long)gridDim.x * blockDim.x)
-    z[b * bstride + t] += (TV)x0[(long long)b * E + t / Np];
+  const int per = blockDim.x / Np, k = threadIdx.x / Np, i = threadIdx.x % Np;
+  for (int K = blockIdx.x * per + k; K < E; K += gridDim.x * per)
+    z[b * bstride + (long long)K * Np + i] += (TV)x0[(long long)b * E + K];
 }
 
 // ------------------------------------------------------------------ block inverse
@@ -1432,7 +1515,7 @@ struct SolverState {
   float* cb_keep = nullptr;       // [B][n0] level-0 right-hand side (cycles > 1)
   size_t cx_acc_count = 0, cb_keep_count = 0;
   bool coarse_ready = false;
-  struct Level { int nx, ny, nz, n; double* A; float *A32, *x, *b, *r; };  // A: FP64 stencil
+  struct Level { int nx, ny, nz, n; double* A; float *A32, *x, *b; };  // A: FP64 stencil
   std::vector<Level> levels;      // level 0: the element grid
   bool coarse_direct = false;     // coarsest level solved by its dense inverse
   double* cdense = nullptr;       // [B][n][n] coarsest matrix
@@ -1597,12 +1680,11 @@ cudaError_t coarse_levels(enp_handle h) {
   int nx = P.ne[0], ny = P.ne[1], nz = P.ne[2];
   const int B = h->batch;
   while (true) {
-    SolverState::Level L{nx, ny, nz, nx * ny * nz, nullptr, nullptr, nullptr, nullptr, nullptr};
+    SolverState::Level L{nx, ny, nz, nx * ny * nz, nullptr, nullptr, nullptr, nullptr};
     cudaError_t e = cudaMalloc(&L.A, sizeof(double) * 7 * (size_t)L.n * B);
     if (e == cudaSuccess) e = cudaMalloc(&L.A32, sizeof(float) * enp::kPack * (size_t)L.n * B);
     if (e == cudaSuccess) e = cudaMalloc(&L.x, sizeof(float) * (size_t)L.n * B);
     if (e == cudaSuccess) e = cudaMalloc(&L.b, sizeof(float) * (size_t)L.n * B);
-    if (e == cudaSuccess) e = cudaMalloc(&L.r, sizeof(float) * (size_t)L.n * B);
     S.levels.push_back(L);
     if (e != cudaSuccess) return e;
     if (L.n <= enp::kCoarsestCells) break;
@@ -1693,42 +1775,33 @@ void vcycle(enp_handle h, size_t l) {
   SolverState& S = state_of(h);
   const int B = h->batch;
   auto& L = S.levels[l];
-  if (L.n <= enp::kTailCells && S.levels.size() <= (size_t)enp::kMaxLevels) {
+  if (L.n <= enp::kTailCells) {
     // this level and all below it in one launch
     enp::VcycleTail T{};
     T.l0 = (int)l;
     T.nl = (int)S.levels.size();
     for (size_t k = 0; k < S.levels.size(); ++k) {
       const auto& Q = S.levels[k];
-      T.L[k] = enp::LevelDev{Q.nx, Q.ny, Q.nz, Q.n, Q.A32, Q.x, Q.b, Q.r};
+      T.L[k] = enp::LevelDev{Q.nx, Q.ny, Q.nz, Q.n, Q.A32, Q.x, Q.b};
     }
     T.inv = S.coarse_direct ? S.cinv : nullptr;
     T.smooth = S.coarse_smooth;
     T.omega = S.coarse_omega;
     T.coarsest_sweeps = kCoarsestSweeps;
-    enp::coarse_vcycle_tail<<<B, enp::kTailThreads, 0, h->stream>>>(T);
-    return;
-  }
-  if (l + 1 == S.levels.size()) {
-    if (S.coarse_direct)
-      enp::coarse_dense_apply<<<B, enp::kCoarsestCells, 0, h->stream>>>(S.cinv, L.b, L.n, L.x);
-    else
-      enp::coarse_solve_small<<<B, enp::kCoarsestCells, 0, h->stream>>>(L.A32, L.x, L.b, L.nx,
-                                                                      L.ny, L.nz, kCoarsestSweeps);
+    enp::coarse_vcycle_tail<<<dim3(enp::kTailCtas, B), enp::kTailThreads, 0, h->stream>>>(T);
     return;
   }
   const dim3 g(grid_for(L.n), B);
-  cudaMemsetAsync(L.x, 0, sizeof(float) * (size_t)L.n * B, h->stream);
-  for (int sw = 0; sw < S.coarse_smooth; ++sw) {
+  enp::coarse_gs_first<<<g, 256, 0, h->stream>>>(L.A32, L.x, L.b, L.nx, L.ny, L.nz);
+  for (int sw = 1; sw < S.coarse_smooth; ++sw) {
     enp::coarse_gs<<<g, 256, 0, h->stream>>>(L.A32, L.x, L.b, L.nx, L.ny, L.nz, 0);
     enp::coarse_gs<<<g, 256, 0, h->stream>>>(L.A32, L.x, L.b, L.nx, L.ny, L.nz, 1);
   }
   auto& C = S.levels[l + 1];
-  enp::coarse_residual<<<g, 256, 0, h->stream>>>(L.A32, L.x, L.b, L.r, L.nx, L.ny, L.nz);
-  enp::coarse_restrict<<<dim3(grid_for(C.n), B), 256, 0, h->stream>>>(L.r, L.nx, L.ny, L.nz, C.b,
-                                                                      C.nx, C.ny, C.nz);
+  enp::coarse_restrict<<<dim3(grid_for(C.n), B), 256, 0, h->stream>>>(
+      L.A32, L.x, L.b, L.nx, L.ny, L.nz, C.b, C.nx, C.ny, C.nz);
   vcycle(h, l + 1);
-  enp::coarse_prolong<<<g, 256, 0, h->stream>>>(C.x, C.nx, C.ny, C.nz, L.x, L.nx, L.ny, L.nz,
+  enp::coarse_prolong<<<g, 256, 0, h->stream>>>(L.A32, C.x, C.nx, C.ny, C.nz, L.x, L.nx, L.ny, L.nz,
                                                 S.coarse_omega);
   for (int sw = 0; sw < S.coarse_smooth; ++sw) {
     enp::coarse_gs<<<g, 256, 0, h->stream>>>(L.A32, L.x, L.b, L.nx, L.ny, L.nz, 1);
@@ -1743,8 +1816,8 @@ cudaError_t coarse_apply(enp_handle h, const TV* r, TV* z) {
   const OpParams& P = h->prm;
   const int B = h->batch;
   auto& L0 = S.levels[0];
-  enp::coarse_from_fine<TV><<<dim3(grid_for(32LL * P.E), B), 256, 0, h->stream>>>(r, L0.b, P.E, P.Np,
-                                                                               P.batch_stride);
+  enp::coarse_from_fine<TV><<<dim3(grid_for(P.E, 128), B), 128, 0, h->stream>>>(r, L0.b, P.E, P.Np,
+                                                                             P.batch_stride);
   vcycle(h, 0);
   if (S.coarse_cycles > 1) {
     // further cycles on the level-0 residual: x += V(b - A0 x); the buffers
@@ -1763,7 +1836,8 @@ cudaError_t coarse_apply(enp_handle h, const TV* r, TV* z) {
     }
     cudaMemcpyAsync(L0.x, S.cx_acc, sizeof(float) * n0, cudaMemcpyDeviceToDevice, h->stream);
   }
-  enp::coarse_to_fine<TV><<<dim3(grid_for((long long)P.E * P.Np), B), 256, 0, h->stream>>>(
+  const int tf = std::max(1, 256 / P.Np) * P.Np;   // whole elements per block (Np <= 125)
+  enp::coarse_to_fine<TV><<<dim3(grid_for((long long)P.E * P.Np, tf), B), tf, 0, h->stream>>>(
       L0.x, z, P.E, P.Np, P.batch_stride);
   return cudaGetLastError();
 }
@@ -1781,7 +1855,7 @@ void enp_solver_free(enp_handle h) {
   cudaFree(S.blocks32); cudaFree(S.u32);
   cudaFree(S.part); cudaFree(S.pvjp); cudaFree(S.dsmall); cudaFree(S.V);
   for (auto& L : S.levels) {
-    cudaFree(L.A); cudaFree(L.A32); cudaFree(L.x); cudaFree(L.b); cudaFree(L.r);
+    cudaFree(L.A); cudaFree(L.A32); cudaFree(L.x); cudaFree(L.b);
   }
   cudaFree(S.cwork); cudaFree(S.cdense); cudaFree(S.cinv);
   cudaFree(S.cx_acc); cudaFree(S.cb_keep);

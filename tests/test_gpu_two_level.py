@@ -243,3 +243,80 @@ def test_two_level_graph_equals_eager_batched():
         xs.append(x.cpu().numpy())
         its.append(st["iterations"])
     np.testing.assert_array_equal(xs[0], xs[1])
+
+
+def _vcycle(A, b, smooth=2, omega=1.8):
+    """One V-cycle in FP64 on the packed stencil A [nz, ny, nx, 7]."""
+    def off(t):
+        o = np.zeros_like(t)
+        o[:, :, 1:] += A[:, :, 1:, 1] * t[:, :, :-1]
+        o[:, :, :-1] += A[:, :, :-1, 2] * t[:, :, 1:]
+        o[:, 1:] += A[:, 1:, :, 3] * t[:, :-1]
+        o[:, :-1] += A[:, :-1, :, 4] * t[:, 1:]
+        o[1:] += A[1:, :, :, 5] * t[:-1]
+        o[:-1] += A[:-1, :, :, 6] * t[1:]
+        return o
+
+    n = b.size
+    if n <= 128:
+        M = np.empty((n, n))
+        for i in range(n):
+            e = np.zeros(n)
+            e[i] = 1.0
+            e = e.reshape(b.shape)
+            M[:, i] = (A[..., 0] * e + off(e)).reshape(-1)
+        return np.linalg.solve(M, b.reshape(-1)).reshape(b.shape)
+    iz, iy, ix = np.indices(b.shape)
+    par = (ix + iy + iz) % 2
+    x = np.zeros_like(b)
+    for c in (0, 1) * smooth:
+        x = np.where(par == c, (b - off(x)) / A[..., 0], x)
+    res = b - A[..., 0] * x - off(x)
+    c = tuple((k + 1) // 2 for k in b.shape)
+    Ac, bc = np.zeros(c + (7,)), np.zeros(c)
+    np.add.at(bc, (iz // 2, iy // 2, ix // 2), res)
+    inside = {1: ix % 2 == 1, 2: ix % 2 == 0, 3: iy % 2 == 1, 4: iy % 2 == 0, 5: iz % 2 == 1,
+              6: iz % 2 == 0}
+    at = (iz // 2, iy // 2, ix // 2)
+    np.add.at(Ac[..., 0], at, A[..., 0])
+    for d in range(1, 7):
+        np.add.at(Ac[..., 0], at, np.where(inside[d], A[..., d], 0.0))
+        np.add.at(Ac[..., d], at, np.where(inside[d], 0.0, A[..., d]))
+    x = x + omega * _vcycle(Ac, bc, smooth, omega)[at]
+    for c in (1, 0) * smooth:
+        x = np.where(par == c, (b - off(x)) / A[..., 0], x)
+    return x
+
+
+@pytest.mark.parametrize("smooth", [1, 2])
+@pytest.mark.parametrize("n", [(5, 5, 5), (12, 11, 10), (13, 13, 13), (33, 32, 32)])
+def test_vcycle_of_every_level_size(n, smooth):
+    """The coarse correction against a V-cycle in FP64 on the exported stencil: the
+    coarsest level alone, levels in one block's shared memory (up to 2,048 cells),
+    in the cluster (up to 32,768) and in grid-wide launches, odd sizes among them.
+    FP32 arithmetic and an inverse stored in FP32: unit roundoff 6e-8 times a
+    condition number of the coarsest matrix of at most some 1e3, so 2e-4."""
+    import dataclasses
+    enp = _enp()
+    base = W.config("cube_n2_p2", p=1)
+    coords = [np.linspace(0.0, 1.0, k + 1) for k in n]
+    tags = W.box_tags(3, list(n), coords, W.WALL)
+    tags[0][:], tags[1][:] = W.INLET, W.OUTLET
+    tags[2][:], tags[3][:] = W.ELECTRODE0, W.ELECTRODE0 + 1
+    P = dataclasses.replace(base, n_el=list(n), coords=coords, tags=tags)
+    op = enp.Operator(P)
+    u, r = _cuda(W.random_state(P, 1)), W.random_vector(P, 2)
+    op.set_coarse_options(cycles=1, smooth=smooth, omega=1.8)
+    op.set_preconditioner(1)
+    op.block_jacobi_setup(u, enp.BJ_F64)
+    with_ = op.block_jacobi_apply(_cuda(r)).cpu().numpy()
+    A = op.coarse_operator().cpu().numpy().reshape(n[2], n[1], n[0], 7)
+    op.set_preconditioner(0)
+    op.block_jacobi_setup(u, enp.BJ_F64)
+    plain = op.block_jacobi_apply(_cuda(r)).cpu().numpy()
+    d = (with_ - plain).reshape(P.n_fields, P.E, P.Np)
+    assert not d[1:].any()
+    b = r.reshape(P.n_fields, P.E, P.Np)[0].sum(-1).reshape(n[2], n[1], n[0])
+    ref = _vcycle(A, b, smooth).reshape(-1)
+    assert np.linalg.norm(d[0, :, 0] - ref) <= 2e-4 * np.linalg.norm(ref)
+    assert np.abs(d[0] - d[0, :, :1]).max() <= 1e-12 * np.abs(with_).max()
