@@ -23,7 +23,8 @@ _CSRC = os.path.join(_HERE, "csrc")
 _BUILD = os.path.join(_HERE, "_build")
 LIB_PATH = os.path.join(_BUILD, "libenp_dg.so")
 SOURCES = ["enp_api.cu", "op_f64.cu", "op_f32.cu", "op_df.cu", "op_df_p1.cu", "op_df_p2.cu",
-           "op_df_p3.cu", "op_df_p4.cu", "op_param.cu", "op_sweep_f32.cu",
+           "op_df_p3.cu", "op_df_p4.cu", "op_param.cu", "op_blocks_f32.cu",
+           "op_blocks_f64.cu", "op_sweep_f32.cu",
            "op_sweep_f64.cu", "enp_solver.cu", "enp_noalloc.cu"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", ARCH, "-Xcompiler", "-fPIC",

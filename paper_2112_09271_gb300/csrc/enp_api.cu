@@ -389,6 +389,8 @@ enp_status enp_dg_create(enp_handle* out, const enp_mesh_desc* mesh, const enp_p
   if (e == cudaSuccess) e = enp::prepare_tables<float>(P.p, h->htab);
   if (e == cudaSuccess && dim == 3) e = enp::prepare_tables_df(P.p, h->htab);
   if (e == cudaSuccess && dim == 3) e = enp::upload_tables_param(P.p, h->htab);
+  if (e == cudaSuccess && dim == 3) e = enp::upload_tables_assemble<float>(P.p, h->htab);
+  if (e == cudaSuccess && dim == 3) e = enp::upload_tables_assemble<double>(P.p, h->htab);
   if (e == cudaSuccess && dim == 3) e = enp::upload_tables_sweep<float>(P.p, h->htab);
   if (e == cudaSuccess && dim == 3) e = enp::upload_tables_sweep<double>(P.p, h->htab);
   if (e != cudaSuccess) { enp_status s = cuda_fail(h, e, "upload constant tables"); enp_dg_destroy(h); return s; }
@@ -561,7 +563,7 @@ enp_status enp_param_jacobian(enp_handle h, const double* u, double* dRdtheta) {
 
 // Time every feasible elements-per-block value of the hexahedral kernel for
 // each operator mode on this handle's mesh (three launches each, CUDA events)
-// and keep the fastest. The block-column pass follows the J v choice.
+// and keep the fastest.
 template <class R>
 static cudaError_t tune_launch(int mode, const OpParams& P, const Tables* t, enp::io_t<R>* u,
                                enp::io_t<R>* v, enp::io_t<R>* out, cudaStream_t s) {
@@ -616,7 +618,6 @@ static cudaError_t tune_mode(enp_handle h, int mode, enp::io_t<R>* u, enp::io_t<
     if (err == cudaSuccess && ms < best) { best = ms; best_eb = eb; }
   }
   enp::eb3d_set<R>(P.p, P.NF, mode, best_eb);
-  if (mode == enp::kJvp) enp::eb3d_set<R>(P.p, P.NF, enp::kBlockCol, best_eb);
   if (chosen) *chosen = best_eb;
   if (chosen_fpb) *chosen_fpb = best_fpb;
   cudaEventDestroy(e0);

@@ -16,8 +16,7 @@ template <class R>
 cudaError_t launch_op(int mode, const OpParams& prm, const Tables* tabs, const io_t<R>* u,
                       const io_t<R>* v, io_t<R>* out, int batch, cudaStream_t stream);
 
-// The double-float hexahedral operator: R, J v, J^T w and block columns of
-// degree prm.p (op_df.cu), compiled one degree per translation unit
+// The double-float hexahedral operator: R, J v and J^T w of degree prm.p (op_df.cu), compiled one degree per translation unit
 // (op_df_p1.cu .. op_df_p4.cu), each with its own constant tables.
 cudaError_t launch_op_df(int mode, const OpParams& prm, const double* u, const double* v,
                          double* out, int batch, cudaStream_t stream);
@@ -33,6 +32,12 @@ ENP_DF_DECL(4)
 #undef ENP_DF_DECL
 
 bool shape_supported(int dim, int p, int nf);
+
+// The element-diagonal blocks of J(u) of one operating point on hexahedra,
+// blocks[e][row][col] (R = double or float).
+template <class R>
+cudaError_t launch_assemble(const OpParams& prm, const io_t<R>* u, io_t<R>* blocks, cudaStream_t s);
+template <class R> cudaError_t upload_tables_assemble(int p, const Tables& t);
 
 // dtheta[b][j] = <w_b, dR_b/dtheta_j> on hexahedra, device [batch][n_theta];
 // part: device workspace of batch x kPvjpPartials doubles.

@@ -1,13 +1,12 @@
 // Run-time dispatch from (dim, p, fields, mode) to a compiled operator kernel.
-// For kBlockCol, `batch` is the number of block columns (NF * Np): grid.y runs
-// over the columns.
+// For kBlockCol (quads), `batch` is the number of block columns (NF * Np): grid.y
+// runs over the columns.
 #pragma once
 #include <mutex>
 
 #include "enp_internal.h"
 #include "enp_operator.cuh"
 #include "enp_operator3d.cuh"
-#include "enp_blockcols.cuh"
 #include "enp_tile3d.cuh"
 
 namespace enp {
@@ -95,42 +94,7 @@ static int default_eb() {
   }
 }
 
-// Columns of the element-diagonal blocks per (element, chunk of kBlockChunk
-// columns), the state's point values and face traces formed once per chunk.
-constexpr int kBlockChunk = 16;
-template <int P, int NF, class R>
-static cudaError_t launch_blockcols(const OpParams& prm, const io_t<R>* u, io_t<R>* out,
-                                    cudaStream_t stream) {
-  constexpr int NT = tpe3d<P, R>();
-  constexpr size_t smem = (size_t)SmemB<P, NF, NT, kBlockChunk>::total * sizeof(R);
-  static_assert(smem <= 200 * 1024, "block-column kernel shared memory");
-  auto k = blockcol3d_kernel<P, NF, kBlockChunk, R>;
-  static SmemAttr attr;
-  cudaError_t e = raise_smem_limit(attr, k, smem);
-  if (e != cudaSuccess) return e;
-  constexpr int nb = NF * (P + 1) * (P + 1) * (P + 1);
-  const dim3 grid((unsigned)prm.E, (nb + kBlockChunk - 1) / kBlockChunk);
-  k<<<grid, NT, smem, stream>>>(prm, u, out);
-  return cudaGetLastError();
-}
-
-template <int P, int NF, int MODE, class R>
-static cudaError_t launch_3d_op(const OpParams& prm, const io_t<R>* u, const io_t<R>* v,
-                                io_t<R>* out, int batch, cudaStream_t stream);
-
-// Hexahedra: R, J v, J^T w and dR/dtheta, or the block columns.
-template <int P, int NF, int MODE, class R>
-static cudaError_t launch_3d(const OpParams& prm, const io_t<R>* u, const io_t<R>* v, io_t<R>* out,
-                             int batch, cudaStream_t stream) {
-  if constexpr (MODE == kBlockCol) {
-    (void)v;
-    (void)batch;  // the nb columns
-    return launch_blockcols<P, NF, R>(prm, u, out, stream);
-  } else {
-    return launch_3d_op<P, NF, MODE, R>(prm, u, v, out, batch, stream);
-  }
-}
-
+// Hexahedra: R, J v, J^T w and dR/dtheta (the blocks: enp_assemble.cuh).
 template <int P, int NF, int MODE, class R>
 static cudaError_t launch_3d_op(const OpParams& prm, const io_t<R>* u, const io_t<R>* v,
                                 io_t<R>* out, int batch, cudaStream_t stream) {
@@ -177,7 +141,7 @@ static cudaError_t launch_one(const OpParams& prm, const Tables* tabs, const io_
                               const io_t<R>* v, io_t<R>* out, int batch, cudaStream_t stream) {
   if constexpr (DIM == 3) {
     (void)tabs;
-    return launch_3d<P, NF, MODE, R>(prm, u, v, out, batch, stream);
+    return launch_3d_op<P, NF, MODE, R>(prm, u, v, out, batch, stream);
   } else {
   using M = WarpSmem<DIM, P, NF, MODE>;
   constexpr size_t per_warp = (size_t)M::total * sizeof(R);
@@ -197,13 +161,12 @@ template <int DIM, int P, int NF, class R>
 static cudaError_t launch_mode(int mode, const OpParams& prm, const Tables* t, const io_t<R>* u,
                                const io_t<R>* v, io_t<R>* out, int batch, cudaStream_t s) {
   if constexpr (std::is_same<R, df>::value) {
-    // double-float: the residual, J v, J^T w and block columns (dR/dtheta
-    // stays with the FP64 kernels)
+    // double-float: the residual, J v and J^T w (the element blocks and dR/dtheta
+    // stay with the FP64 kernels)
     switch (mode) {
       case kResidual: return launch_one<DIM, P, NF, kResidual, R>(prm, t, u, v, out, batch, s);
       case kJvp: return launch_one<DIM, P, NF, kJvp, R>(prm, t, u, v, out, batch, s);
       case kVjp: return launch_one<DIM, P, NF, kVjp, R>(prm, t, u, v, out, batch, s);
-      case kBlockCol: return launch_one<DIM, P, NF, kBlockCol, R>(prm, t, u, v, out, batch, s);
     }
     return cudaErrorNotSupported;
   } else {
@@ -211,7 +174,9 @@ static cudaError_t launch_mode(int mode, const OpParams& prm, const Tables* t, c
       case kResidual: return launch_one<DIM, P, NF, kResidual, R>(prm, t, u, v, out, batch, s);
       case kJvp: return launch_one<DIM, P, NF, kJvp, R>(prm, t, u, v, out, batch, s);
       case kVjp: return launch_one<DIM, P, NF, kVjp, R>(prm, t, u, v, out, batch, s);
-      case kBlockCol: return launch_one<DIM, P, NF, kBlockCol, R>(prm, t, u, v, out, batch, s);
+      case kBlockCol:
+        if constexpr (DIM == 2) return launch_one<DIM, P, NF, kBlockCol, R>(prm, t, u, v, out, batch, s);
+        return cudaErrorNotSupported;
       case kParam:
         if constexpr (DIM == 3 && std::is_same<R, double>::value)
           return launch_one<DIM, P, NF, kParam, R>(prm, t, u, v, out, batch, s);
@@ -239,8 +204,8 @@ template <class R>
 int eb3d_max(int p, int nf, int mode) {
 #define ENP_EBM(PP, NFF, MM) \
   if (p == PP && nf == NFF && mode == MM && (MM != kParam || !std::is_same<R, df>::value)) return max_eb<PP, NFF, MM, R>();
-#define ENP_EBM_P(PP) ENP_EBM(PP, 2, 0) ENP_EBM(PP, 2, 1) ENP_EBM(PP, 2, 2) ENP_EBM(PP, 2, 3) ENP_EBM(PP, 2, 4) \
-  ENP_EBM(PP, 3, 0) ENP_EBM(PP, 3, 1) ENP_EBM(PP, 3, 2) ENP_EBM(PP, 3, 3) ENP_EBM(PP, 3, 4)
+#define ENP_EBM_P(PP) ENP_EBM(PP, 2, 0) ENP_EBM(PP, 2, 1) ENP_EBM(PP, 2, 2) ENP_EBM(PP, 2, 4) \
+  ENP_EBM(PP, 3, 0) ENP_EBM(PP, 3, 1) ENP_EBM(PP, 3, 2) ENP_EBM(PP, 3, 4)
   ENP_EBM_P(1) ENP_EBM_P(2) ENP_EBM_P(3) ENP_EBM_P(4)
 #undef ENP_EBM_P
 #undef ENP_EBM
@@ -292,8 +257,8 @@ template <class R>
 cudaError_t launch_op(int mode, const OpParams& prm, const Tables* t, const io_t<R>* u,
                       const io_t<R>* v, io_t<R>* out, int batch, cudaStream_t s) {
   if constexpr (std::is_same<R, double>::value) {
-    // R, J v, J^T w and block columns in double-float arithmetic on hexahedra
-    if (prm.arith == kArithDF && prm.dim == 3 && mode != kParam)
+    // R, J v and J^T w in double-float arithmetic on hexahedra
+    if (prm.arith == kArithDF && prm.dim == 3 && mode <= kVjp)
       return launch_op_df(mode, prm, u, v, out, batch, s);
   }
   if (prm.dim == 3) {

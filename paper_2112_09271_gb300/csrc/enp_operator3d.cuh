@@ -1,6 +1,6 @@
 // Hexahedra, thread-per-pencil layout (sm_103a): the basis tables, the pencil
 // contractions, and the parameter Jacobian dR/dtheta of Eq. NPDG / Eq. chargeDG (R, J v and J^T w:
-// enp_tile3d.cuh; block columns: enp_blockcols.cuh).
+// enp_tile3d.cuh; the element blocks: enp_assemble.cuh).
 //  * every 1D contraction is done by one thread per pencil: it loads the
 //    pencil into registers and forms all outputs with the basis table in
 //    __constant__ memory at compile-time indices (the table entries become

@@ -1,9 +1,8 @@
 // Element block-Jacobi preconditioner, Krylov and Newton solvers, c_m recovery.
 //
 //  * block setup: the element-diagonal blocks of J(u) (volume terms plus this
-//    element's own-side face terms, all fields coupled), one column per grid.y
-//    of the J v kernel, then batched Gauss-Jordan inversion with partial
-//    pivoting; the inverse is stored transposed in FP64, FP32 or BF16.
+//    element's own-side face terms, all fields coupled; enp_assemble.cuh), then
+//    batched Gauss-Jordan inversion with partial pivoting; the inverse is stored transposed in FP64, FP32 or BF16.
 //  * block apply: y_e = B_e^{-1} x_e, one thread block per element, threads over
 //    rows, reading the stored inverse once (an HBM-bound batched GEMV).
 //  * FGMRES(m) with right preconditioning (flexible: the preconditioner may
@@ -1582,6 +1581,14 @@ cudaError_t apply_residual(enp_handle h, const double* u, double* r, int B) {
   return e;
 }
 
+// The element-diagonal blocks of J(u) of one operating point, [E][nb][nb]
+// (hexahedra: assembled as matrices; quads: a J v pass per column).
+template <class R>
+cudaError_t element_blocks(enp_handle h, const OpParams& P, const R* u, R* blocks) {
+  if (P.dim == 3) return enp::launch_assemble<R>(P, u, blocks, h->stream);
+  return enp::launch_op<R>(enp::kBlockCol, P, h->d_tab, u, nullptr, blocks, P.NF * P.Np, h->stream);
+}
+
 // Partials of <V_i, w>_b (i < nd) into S.part; *nparts = the partials per dot.
 template <class T>
 cudaError_t dot_partials(enp_handle h, const T* V, long long vstride, int nd, const T* w,
@@ -1929,9 +1936,8 @@ enp_status enp_block_diagonal(enp_handle h, const double* u, double* blocks) {
   for (int b = 0; b < h->batch; ++b) {
     OpParams Pb = P;
     if (P.phiapp_batch) Pb.phiapp_batch = P.phiapp_batch + 4 * b;
-    cudaError_t e = enp::launch_op<double>(enp::kBlockCol, Pb, h->d_tab, u + b * P.batch_stride,
-                                           nullptr, blocks + b * bsz, nb, h->stream);
-    if (e != cudaSuccess) return cuda_err(h, e, "block columns");
+    cudaError_t e = element_blocks<double>(h, Pb, u + b * P.batch_stride, blocks + b * bsz);
+    if (e != cudaSuccess) return cuda_err(h, e, "element blocks");
   }
   return ENP_OK;
 }
@@ -2007,18 +2013,16 @@ enp_status enp_block_jacobi_setup(enp_handle h, const double* u, int storage) {
     const int b = shared ? S.pc_shared : set;
     OpParams Pb = P;
     if (P.phiapp_batch) Pb.phiapp_batch = P.phiapp_batch + 4 * b;
-    // assemble operating point b's blocks: column j of every block per grid.y
+    // assemble operating point b's blocks
     if (f64) {
-      e = enp::launch_op<double>(enp::kBlockCol, Pb, h->d_tab, u + b * P.batch_stride, nullptr,
-                                 S.blocks, nb, h->stream);
-      if (e != cudaSuccess) return cuda_err(h, e, "block columns");
+      e = element_blocks<double>(h, Pb, u + b * P.batch_stride, S.blocks);
+      if (e != cudaSuccess) return cuda_err(h, e, "element blocks");
       if (S.potential_only)
         enp::block_species_identity<double><<<grid_for((long long)(nb - P.Np) * nb * nblk), 256, 0,
                                               h->stream>>>(S.blocks, nblk, nb, P.Np);
     } else {
-      e = enp::launch_op<float>(enp::kBlockCol, Pb, h->d_tab, S.u32 + b * P.batch_stride, nullptr,
-                                S.blocks32, nb, h->stream);
-      if (e != cudaSuccess) return cuda_err(h, e, "FP32 block columns");
+      e = element_blocks<float>(h, Pb, S.u32 + b * P.batch_stride, S.blocks32);
+      if (e != cudaSuccess) return cuda_err(h, e, "FP32 element blocks");
       if (S.potential_only)
         enp::block_species_identity<float><<<grid_for((long long)(nb - P.Np) * nb * nblk), 256, 0,
                                              h->stream>>>(S.blocks32, nblk, nb, P.Np);
