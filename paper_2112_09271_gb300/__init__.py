@@ -23,7 +23,7 @@ _CSRC = os.path.join(_HERE, "csrc")
 _BUILD = os.path.join(_HERE, "_build")
 LIB_PATH = os.path.join(_BUILD, "libenp_dg.so")
 SOURCES = ["enp_api.cu", "op_f64.cu", "op_f32.cu", "op_df.cu", "op_df_p1.cu", "op_df_p2.cu",
-           "op_df_p3.cu", "op_df_p4.cu", "op_param.cu", "op_blocks_f32.cu",
+           "op_df_p3.cu", "op_df_p4.cu", "op_param.cu", "op_inverse.cu", "op_blocks_f32.cu",
            "op_blocks_f64.cu", "op_sweep_f32.cu",
            "op_sweep_f64.cu", "enp_solver.cu", "enp_noalloc.cu"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"

@@ -39,6 +39,13 @@ template <class R>
 cudaError_t launch_assemble(const OpParams& prm, const io_t<R>* u, io_t<R>* blocks, cudaStream_t s);
 template <class R> cudaError_t upload_tables_assemble(int p, const Tables& t);
 
+// Inverses of nblk element blocks (FP32, destroyed) by elimination of the species
+// (enp_blockinv.cuh), transposed, stored as 1 = FP32 or 2 = BF16. *singular is set
+// (device) where a field block has no safe pivot: the result is then not usable.
+bool elimination_available(int dim, int p);
+cudaError_t launch_elimination(float* blocks, void* out, int storage, int p, int nf,
+                               long long nblk, int* singular, cudaStream_t s);
+
 // dtheta[b][j] = <w_b, dR_b/dtheta_j> on hexahedra, device [batch][n_theta];
 // part: device workspace of batch x kPvjpPartials doubles.
 cudaError_t upload_tables_param(int p, const Tables& t);

@@ -2009,6 +2009,12 @@ enp_status enp_block_jacobi_setup(enp_handle h, const double* u, int storage) {
     if (e != cudaSuccess) return cuda_err(h, e, "cudaMalloc inversion work");
   }
   const size_t smem = in_smem ? smem_full : telt * 2 * nb + sizeof(int) * nb;
+  // FP32 inversions eliminate the species first; if a field block of any element
+  // has no safe pivot, all sets are formed again and inverted with the pivot
+  // search over the whole block
+  bool elim = !f64 && enp::elimination_available(P.dim, P.p);
+  int flag = 0;
+  while (true) {
   for (int set = 0; set < nsets; ++set) {
     const int b = shared ? S.pc_shared : set;
     OpParams Pb = P;
@@ -2068,7 +2074,9 @@ enp_status enp_block_jacobi_setup(enp_handle h, const double* u, int storage) {
   else ENP_GJR(TS, 16, 12, 6)
     const bool regs = !f64 && nb <= 192;
     const bool clus = !f64 && !regs && nb <= enp::kGjcCols;
-    if (regs) {
+    if (elim) {
+      e = enp::launch_elimination(S.blocks32, out, storage, P.p, P.NF, nblk, S.d_flag, h->stream);
+    } else if (regs) {
       if (storage == 1) ENP_GJR_ANY(float)
       else ENP_GJR_ANY(__nv_bfloat16)
     } else if (clus) {
@@ -2089,10 +2097,13 @@ enp_status enp_block_jacobi_setup(enp_handle h, const double* u, int storage) {
     if (e != cudaSuccess) break;
   }
   if (e != cudaSuccess) return cuda_err(h, e, "block inversion");
-  int flag = 0;
   e = cudaMemcpyAsync(&flag, S.d_flag, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return cuda_err(h, e, "block inversion sync");
+  if (!flag || !elim) break;
+  elim = false;
+  cudaMemsetAsync(S.d_flag, 0, sizeof(int), h->stream);
+  }
   if (flag) {
     h->err = "singular or non-finite element block";
     return ENP_ERR_NONFINITE;
