@@ -193,34 +193,73 @@ struct ElimShape {
   static constexpr int KC = 16;
   static constexpr int LD = NP + 4;
 };
+__device__ __forceinline__ void copy4(float* dst, const float* src, bool ok) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  const int size = ok ? 4 : 0;     // 0: zeros, nothing read
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(size) : "memory");
+}
+__device__ __forceinline__ void copy16(float* dst, const float* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
 // c += A B (A, B: global, leading dimension ld; written by this block before, if
-// at all, so no read-only loads). Barriers on both sides.
+// at all, so no read-only loads). As, Bs: two buffers each; the next chunk is
+// copied while this one is multiplied (loads through registers left the products
+// waiting on memory 80 % of the time). Barriers on both sides.
 template <int n>
 __device__ __forceinline__ void elim_gemm(float (&c)[ElimShape<n>::TM][ElimShape<n>::TM],
                                           const float* A, const float* B, int ld, float* As,
                                           float* Bs) {
   using S = ElimShape<n>;
   constexpr int TM = S::TM, T = S::T, NP = S::NP, NT = S::NT, KC = S::KC, LD = S::LD;
+  constexpr int NCH = (n + KC - 1) / KC;
   const int tid = threadIdx.x, r0 = (tid % T) * TM, c0 = (tid / T) * TM;
-#pragma unroll 1
-  for (int k0 = 0; k0 < n; k0 += KC) {
-    __syncthreads();
+  auto fetch = [&](int ch) {
+    const int k0 = ch * KC;
+    float *a = As + (ch & 1) * (KC * LD), *b = Bs + (ch & 1) * (KC * LD);
+#pragma unroll 4
     for (int t = tid; t < NP * KC; t += NT) {
       const int i = t / KC, k = t % KC;
-      As[k * LD + i] = (i < n && k0 + k < n) ? A[(long long)i * ld + k0 + k] : 0.f;
+      const bool ok = i < n && k0 + k < n;
+      copy4(a + k * LD + i, ok ? A + (long long)i * ld + k0 + k : A, ok);
     }
-    for (int t = tid; t < NP * KC; t += NT) {
-      const int k = t / NP, j = t % NP;
-      Bs[k * LD + j] = (j < n && k0 + k < n) ? B[(long long)(k0 + k) * ld + j] : 0.f;
+    if constexpr (n % KC == 0) {   // rows of 16-byte multiples: n, ld and the offsets are multiples of 4
+#pragma unroll 4
+      for (int t = tid; t < n / 4 * KC; t += NT) {
+        const int k = t / (n / 4), j = t % (n / 4) * 4;
+        copy16(b + k * LD + j, B + (long long)(k0 + k) * ld + j);
+      }
+    } else {
+#pragma unroll 4
+      for (int t = tid; t < NP * KC; t += NT) {
+        const int k = t / NP, j = t % NP;
+        const bool ok = j < n && k0 + k < n;
+        copy4(b + k * LD + j, ok ? B + (long long)(k0 + k) * ld + j : B, ok);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  __syncthreads();
+  fetch(0);
+#pragma unroll 1
+  for (int ch = 0; ch < NCH; ++ch) {
+    if (ch + 1 < NCH) {
+      fetch(ch + 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
     __syncthreads();
-#pragma unroll
+    const float *as = As + (ch & 1) * (KC * LD) + r0, *bs = Bs + (ch & 1) * (KC * LD) + c0;
+    // four at a time: three to four products are inlined in a kernel, and whole
+    // chunks of straight-line code (16 KB each) outran the instruction cache
+#pragma unroll 4
     for (int k = 0; k < KC; ++k) {
       float a[TM], b[TM];
 #pragma unroll
       for (int q = 0; q < TM; q += 4) {
-        const float4 x = *reinterpret_cast<const float4*>(As + k * LD + r0 + q);
-        const float4 y = *reinterpret_cast<const float4*>(Bs + k * LD + c0 + q);
+        const float4 x = *reinterpret_cast<const float4*>(as + k * LD + q);
+        const float4 y = *reinterpret_cast<const float4*>(bs + k * LD + q);
         a[q] = x.x; a[q + 1] = x.y; a[q + 2] = x.z; a[q + 3] = x.w;
         b[q] = y.x; b[q + 1] = y.y; b[q + 2] = y.z; b[q + 3] = y.w;
       }
@@ -229,8 +268,69 @@ __device__ __forceinline__ void elim_gemm(float (&c)[ElimShape<n>::TM][ElimShape
 #pragma unroll
         for (int j = 0; j < TM; ++j) c[i][j] = fmaf(a[i], b[j], c[i][j]);
     }
+    __syncthreads();
   }
-  __syncthreads();
+}
+// A thread's tile of a row-major matrix (leading dimension ld) in and out; whole
+// 16-byte groups where the tile rows are such (n and ld multiples of 4).
+template <int n, int TM>
+__device__ __forceinline__ void tile_load(float (&c)[TM][TM], const float* p, int ld, int r0, int c0) {
+#pragma unroll
+  for (int i = 0; i < TM; ++i) {
+    if constexpr (n % TM == 0 && n % 4 == 0) {
+#pragma unroll
+      for (int j = 0; j < TM; j += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(p + (long long)(r0 + i) * ld + c0 + j);
+        c[i][j] = v.x; c[i][j + 1] = v.y; c[i][j + 2] = v.z; c[i][j + 3] = v.w;
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < TM; ++j)
+        c[i][j] = (r0 + i < n && c0 + j < n) ? p[(long long)(r0 + i) * ld + c0 + j] : 0.f;
+    }
+  }
+}
+template <int n, int TM>
+__device__ __forceinline__ void tile_store(float* p, const float (&c)[TM][TM], int ld, int r0, int c0) {
+#pragma unroll
+  for (int i = 0; i < TM; ++i) {
+    if constexpr (n % TM == 0 && n % 4 == 0) {
+#pragma unroll
+      for (int j = 0; j < TM; j += 4)
+        *reinterpret_cast<float4*>(p + (long long)(r0 + i) * ld + c0 + j) =
+            make_float4(c[i][j], c[i][j + 1], c[i][j + 2], c[i][j + 3]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < TM; ++j)
+        if (r0 + i < n && c0 + j < n) p[(long long)(r0 + i) * ld + c0 + j] = c[i][j];
+    }
+  }
+}
+// The tile times sign, transposed, as TS.
+template <int n, int TM, class TS>
+__device__ __forceinline__ void tile_emit(TS* o, float sign, const float (&c)[TM][TM], int ld, int r0,
+                                          int c0) {
+#pragma unroll
+  for (int j = 0; j < TM; ++j) {
+    TS* q = o + (long long)(c0 + j) * ld + r0;
+    if constexpr (n % TM == 0 && TM == 8 && n % 8 == 0) {
+      if constexpr (sizeof(TS) == 4) {
+#pragma unroll
+        for (int i = 0; i < TM; i += 4)
+          *reinterpret_cast<float4*>(q + i) = make_float4(sign * c[i][j], sign * c[i + 1][j],
+                                                          sign * c[i + 2][j], sign * c[i + 3][j]);
+      } else {
+        union { __nv_bfloat16 h[8]; uint4 u; } v;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v.h[i] = (__nv_bfloat16)(sign * c[i][j]);
+        *reinterpret_cast<uint4*>(q) = v.u;
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+        if (r0 + i < n && c0 + j < n) q[i] = (TS)(sign * c[i][j]);
+    }
+  }
 }
 template <int TM>
 __device__ __forceinline__ void tile_zero(float (&c)[TM][TM]) {
@@ -242,84 +342,58 @@ __device__ __forceinline__ void tile_zero(float (&c)[TM][TM]) {
 
 // With A_kk^-1 in place: X_k over A_k0, Y_k over A_0k, S over A_00.
 template <int n, int NF>
-__global__ void __launch_bounds__(ElimShape<n>::NT)
+__global__ void __launch_bounds__(ElimShape<n>::NT, 384 / ElimShape<n>::NT > 0 ? 384 / ElimShape<n>::NT : 1)
 elim_schur_kernel(float* blocks) {
   using S = ElimShape<n>;
   constexpr int TM = S::TM, T = S::T, nb = NF * n;
-  __shared__ __align__(16) float As[S::KC * S::LD], Bs[S::KC * S::LD];
+  __shared__ __align__(16) float As[2 * S::KC * S::LD], Bs[2 * S::KC * S::LD];
   float* E = blocks + (long long)blockIdx.x * nb * nb;
   const int r0 = ((int)threadIdx.x % T) * TM, c0 = ((int)threadIdx.x / T) * TM;
   auto at = [&](int f, int g) { return E + (long long)f * n * nb + g * n; };
-  auto store = [&](float* p, const float (&c)[TM][TM]) {
-#pragma unroll
-    for (int i = 0; i < TM; ++i)
-#pragma unroll
-      for (int j = 0; j < TM; ++j)
-        if (r0 + i < n && c0 + j < n) p[(long long)(r0 + i) * nb + c0 + j] = c[i][j];
-  };
   float s[TM][TM], c[TM][TM];
   tile_zero(s);
 #pragma unroll 1
   for (int k = 1; k < NF; ++k) {
     tile_zero(c);
     elim_gemm<n>(c, at(k, k), at(k, 0), nb, As, Bs);
-    store(at(k, 0), c);                         // X_k
+    tile_store<n>(at(k, 0), c, nb, r0, c0);     // X_k
     __syncthreads();
     elim_gemm<n>(s, at(0, k), at(k, 0), nb, As, Bs);
     tile_zero(c);
     elim_gemm<n>(c, at(0, k), at(k, k), nb, As, Bs);
-    store(at(0, k), c);                         // Y_k
+    tile_store<n>(at(0, k), c, nb, r0, c0);     // Y_k
   }
-  float* a00 = at(0, 0);
+  tile_load<n>(c, at(0, 0), nb, r0, c0);
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < TM; ++j)
-      if (r0 + i < n && c0 + j < n) {
-        const long long o = (long long)(r0 + i) * nb + c0 + j;
-        a00[o] -= s[i][j];
-      }
+    for (int j = 0; j < TM; ++j) c[i][j] -= s[i][j];
+  tile_store<n>(at(0, 0), c, nb, r0, c0);
 }
 
 // With S^-1 in place: the inverse, transposed, out[e][c][r] in type TS.
 template <int n, int NF, class TS>
-__global__ void __launch_bounds__(ElimShape<n>::NT)
+__global__ void __launch_bounds__(ElimShape<n>::NT, 512 / ElimShape<n>::NT)
 elim_finish_kernel(float* blocks, TS* __restrict__ out) {
   using S = ElimShape<n>;
   constexpr int TM = S::TM, T = S::T, nb = NF * n;
-  __shared__ __align__(16) float As[S::KC * S::LD], Bs[S::KC * S::LD];
+  __shared__ __align__(16) float As[2 * S::KC * S::LD], Bs[2 * S::KC * S::LD];
   float* E = blocks + (long long)blockIdx.x * nb * nb;
   TS* O = out + (long long)blockIdx.x * nb * nb;
   const int r0 = ((int)threadIdx.x % T) * TM, c0 = ((int)threadIdx.x / T) * TM;
   auto at = [&](int f, int g) { return E + (long long)f * n * nb + g * n; };
   auto emit = [&](int f, int g, float sign, const float (&c)[TM][TM]) {
-    TS* o = O + (long long)g * n * nb + f * n;
-#pragma unroll
-    for (int j = 0; j < TM; ++j)
-#pragma unroll
-      for (int i = 0; i < TM; ++i)
-        if (r0 + i < n && c0 + j < n) o[(long long)(c0 + j) * nb + r0 + i] = (TS)(sign * c[i][j]);
+    tile_emit<n>(O + (long long)g * n * nb + f * n, sign, c, nb, r0, c0);
   };
   float c[TM][TM];
-  const float* t00 = at(0, 0);
-#pragma unroll
-  for (int i = 0; i < TM; ++i)
-#pragma unroll
-    for (int j = 0; j < TM; ++j)
-      c[i][j] = (r0 + i < n && c0 + j < n) ? t00[(long long)(r0 + i) * nb + c0 + j] : 0.f;
+  tile_load<n>(c, at(0, 0), nb, r0, c0);
   emit(0, 0, 1.f, c);
 #pragma unroll 1
   for (int k = 1; k < NF; ++k) {
     tile_zero(c);
     elim_gemm<n>(c, at(k, 0), at(0, 0), nb, As, Bs);
     emit(k, 0, -1.f, c);
-    // X_k S^-1 over X_k
-    float* p = at(k, 0);
-#pragma unroll
-    for (int i = 0; i < TM; ++i)
-#pragma unroll
-      for (int j = 0; j < TM; ++j)
-        if (r0 + i < n && c0 + j < n) p[(long long)(r0 + i) * nb + c0 + j] = c[i][j];
+    tile_store<n>(at(k, 0), c, nb, r0, c0);     // X_k S^-1 over X_k
     __syncthreads();
   }
 #pragma unroll 1
@@ -329,12 +403,8 @@ elim_finish_kernel(float* blocks, TS* __restrict__ out) {
     emit(0, l, -1.f, c);
 #pragma unroll 1
     for (int k = 1; k < NF; ++k) {
-      const float* d = at(k, k);
-#pragma unroll
-      for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int j = 0; j < TM; ++j)
-          c[i][j] = (k == l && r0 + i < n && c0 + j < n) ? d[(long long)(r0 + i) * nb + c0 + j] : 0.f;
+      if (k == l) tile_load<n>(c, at(k, k), nb, r0, c0);
+      else tile_zero(c);
       elim_gemm<n>(c, at(k, 0), at(0, l), nb, As, Bs);
       emit(k, l, 1.f, c);
     }
