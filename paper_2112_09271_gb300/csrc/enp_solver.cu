@@ -1319,6 +1319,60 @@ __global__ void bj_apply_kernel(const TS* __restrict__ BT, const TV* __restrict_
   }
 }
 
+// The same with V consecutive rows per load (V sizeof(TS) bytes): blockDim.x =
+// n / V row groups times S column sets, each thread summing its V rows over every
+// S-th column, the sets added through shared memory in order. A row per thread
+// reads 64 bytes a warp and column from BF16 inverses (8,000 blocks of 192: 178
+// us, 3.3 TB/s; 99 us, 6.0 TB/s so; FP32 212 and 182 us); V = 8 (BF16) or 4 (FP32) where n is a multiple, 2
+// where it is even.
+template <class TS, int V> struct alignas(V * sizeof(TS)) RowVec { TS v[V]; };
+template <class TS, class TA, class TV, int V>
+__global__ void __launch_bounds__(256)
+bj_apply_rows_kernel(const TS* __restrict__ BT, const TV* __restrict__ x, TV* __restrict__ y, int n,
+                     int Np, long long EN, long long bstride, int shared_blocks) {
+  extern __shared__ __align__(16) unsigned char xsm_raw[];
+  TA* xs = reinterpret_cast<TA*>(xsm_raw);        // [n]
+  TA* ps = xs + n;                                // [S][n]
+  const long long e = blockIdx.x;
+  const int b = blockIdx.y;
+  const long long E = EN / Np;
+  const TV* xb = x + b * bstride + e * Np;
+  for (int c = threadIdx.x; c < n; c += blockDim.x) xs[c] = (TA)xb[c / Np * EN + c % Np];
+  const int rg = n / V, S = blockDim.x / rg, g = threadIdx.x % rg, set = threadIdx.x / rg;
+  const RowVec<TS, V>* B = reinterpret_cast<const RowVec<TS, V>*>(
+      BT + ((long long)(shared_blocks ? 0 : b) * E + e) * (long long)n * n) + g;
+  __syncthreads();
+  TA acc[V];
+#pragma unroll
+  for (int q = 0; q < V; ++q) acc[q] = TA(0);
+  int c = set;
+  for (; c + 7 * S < n; c += 8 * S) {
+    RowVec<TS, V> t[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) t[k] = B[(long long)(c + k * S) * rg];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const TA xc = xs[c + k * S];
+#pragma unroll
+      for (int q = 0; q < V; ++q) acc[q] += (TA)t[k].v[q] * xc;
+    }
+  }
+  for (; c < n; c += S) {
+    const RowVec<TS, V> t = B[(long long)c * rg];
+#pragma unroll
+    for (int q = 0; q < V; ++q) acc[q] += (TA)t.v[q] * xs[c];
+  }
+#pragma unroll
+  for (int q = 0; q < V; ++q) ps[set * n + g * V + q] = acc[q];
+  __syncthreads();
+  TV* yb = y + b * bstride + e * Np;
+  for (int r = threadIdx.x; r < n; r += blockDim.x) {
+    TA s = ps[r];
+    for (int q = 1; q < S; ++q) s += ps[q * n + r];
+    yb[r / Np * EN + r % Np] = (TV)s;
+  }
+}
+
 // ------------------------------------------------- graph-driven Newton iteration
 // Device-side control of a Newton solve whose iterations run as one CUDA graph
 // launch with conditional WHILE nodes (the FGMRES restart cycles, the
@@ -2146,28 +2200,38 @@ static cudaError_t bj_apply_any(enp_handle h, const TV* x, TV* y) {
   return e;
 }
 
+template <class TS, class TA, class TV>
+static cudaError_t bj_launch(enp_handle h, const TV* x, TV* y) {
+  SolverState& S = state_of(h);
+  const OpParams& P = h->prm;
+  const int n = S.nb;
+  const long long EN = (long long)P.E * P.Np;
+  const dim3 g(P.E, h->batch);
+  const TS* B = (const TS*)S.binv;
+  constexpr int W = 16 / sizeof(TS);     // rows of a 16-byte load
+  // blocks of 96 rows and more, whose columns fill several warps' wide loads;
+  // the inverses' base is cudaMalloc's, so n alone decides the alignment
+  auto rows = [&](auto V) {
+    constexpr int v = decltype(V)::value;
+    const int rg = n / v, sets = std::max(1, std::min(256 / rg, 8));
+    enp::bj_apply_rows_kernel<TS, TA, TV, v><<<g, rg * sets, sizeof(TA) * n * (1 + sets), h->stream>>>(
+        B, x, y, n, P.Np, EN, P.batch_stride, S.pc_shared_built);
+    return cudaGetLastError();
+  };
+  if (n >= 96 && n % W == 0) return rows(std::integral_constant<int, W>());
+  if (n >= 96 && n % 2 == 0) return rows(std::integral_constant<int, 2>());
+  const int threads = std::min(256, ((n + 31) / 32) * 32);
+  enp::bj_apply_kernel<TS, TA, TV><<<g, threads, sizeof(TA) * n, h->stream>>>(
+      B, x, y, n, P.NF, P.Np, EN, P.batch_stride, S.pc_shared_built);
+  return cudaGetLastError();
+}
+
 template <class TV>
 static cudaError_t bj_apply_plain(enp_handle h, const TV* x, TV* y) {
   SolverState& S = state_of(h);
-  const OpParams& P = h->prm;
-  const int nb = S.nb;
-  const long long EN = (long long)P.E * P.Np;
-  dim3 g(P.E, h->batch);
-  int threads = std::min(256, ((nb + 31) / 32) * 32);
-  if (S.storage == 0) {
-    size_t sm = sizeof(double) * nb;
-    enp::bj_apply_kernel<double, double, TV><<<g, threads, sm, h->stream>>>(
-        (const double*)S.binv, x, y, nb, P.NF, P.Np, EN, P.batch_stride, S.pc_shared_built);
-  } else if (S.storage == 1) {
-    size_t sm = sizeof(float) * nb;
-    enp::bj_apply_kernel<float, float, TV><<<g, threads, sm, h->stream>>>(
-        (const float*)S.binv, x, y, nb, P.NF, P.Np, EN, P.batch_stride, S.pc_shared_built);
-  } else {
-    size_t sm = sizeof(float) * nb;
-    enp::bj_apply_kernel<__nv_bfloat16, float, TV><<<g, threads, sm, h->stream>>>(
-        (const __nv_bfloat16*)S.binv, x, y, nb, P.NF, P.Np, EN, P.batch_stride, S.pc_shared_built);
-  }
-  return cudaGetLastError();
+  if (S.storage == 0) return bj_launch<double, double, TV>(h, x, y);
+  if (S.storage == 1) return bj_launch<float, float, TV>(h, x, y);
+  return bj_launch<__nv_bfloat16, float, TV>(h, x, y);
 }
 
 // Downwind block Gauss-Seidel: z = (D + L)^-1 x with D the element blocks and L
