@@ -18,8 +18,8 @@ constexpr int kMaxP = 4;
 constexpr int kMaxN = kMaxP + 1;
 constexpr int kMaxQ = kMaxP + 2;
 
-// kBlockCol: column blockIdx.y of every element-diagonal block of J(u): the
-// J v pass with v = the local unit vector e_col in every element and the
+// kBlockCol (quadrilaterals): column blockIdx.y of every element-diagonal block
+// of J(u): the J v pass with v = the local unit vector e_col in every element and the
 // neighbour's tangent set to zero, written to blk[e][row][col].
 // kParam: dR/dtheta_j for every parameter j (grid.y = batch * n_theta), the
 // residual evaluated with forward-tangent coefficients seeded on theta_j.
@@ -159,35 +159,5 @@ template <class R> __device__ __forceinline__ R valof(Tan<R> x) { return x.v; }
 
 __device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a, b, c); }
-
-// Apply a small dense matrix along one direction of a 3D array held in shared
-// memory by one warp. Input extents (E0, E1, E2), E0 fastest; the contracted
-// direction DIR has extent COLS in the input and ROWS in the output.
-//   TRANS = false: out(r) = sum_c M[r * COLS + c] in(c)      (M stored ROWS x COLS)
-//   TRANS = true:  out(r) = sum_c M[c * ROWS + r] in(c)      (M stored COLS x ROWS)
-//   ACC:           out += instead of out =
-template <int E0, int E1, int E2, int DIR, int ROWS, bool TRANS, bool ACC, class R>
-__device__ __forceinline__ void apply1d(const R* __restrict__ M, const R* __restrict__ in,
-                                        R* __restrict__ out, int lane) {
-  constexpr int O0 = DIR == 0 ? ROWS : E0;
-  constexpr int O1 = DIR == 1 ? ROWS : E1;
-  constexpr int O2 = DIR == 2 ? ROWS : E2;
-  constexpr int COLS = DIR == 0 ? E0 : (DIR == 1 ? E1 : E2);
-  constexpr int NOUT = O0 * O1 * O2;
-  constexpr int IS = DIR == 0 ? 1 : (DIR == 1 ? E0 : E0 * E1);  // input stride along DIR
-#pragma unroll 1
-  for (int o = lane; o < NOUT; o += 32) {
-    const int i0 = o % O0, i1 = (o / O0) % O1, i2 = o / (O0 * O1);
-    const int r = DIR == 0 ? i0 : (DIR == 1 ? i1 : i2);
-    const int base = (DIR == 0 ? 0 : i0) + E0 * ((DIR == 1 ? 0 : i1) + E1 * (DIR == 2 ? 0 : i2));
-    R acc = ACC ? out[o] : R(0);
-#pragma unroll
-    for (int c = 0; c < COLS; ++c) {
-      const R m = TRANS ? M[c * ROWS + r] : M[r * COLS + c];
-      acc = mad(m, in[base + c * IS], acc);
-    }
-    out[o] = acc;
-  }
-}
 
 }  // namespace enp

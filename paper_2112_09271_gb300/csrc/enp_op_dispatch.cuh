@@ -95,6 +95,11 @@ static int default_eb() {
 }
 
 // Hexahedra: R, J v, J^T w and dR/dtheta (the blocks: enp_assemble.cuh).
+
+}  // namespace enp
+#include "enp_quad2d.cuh"
+namespace enp {
+
 template <int P, int NF, int MODE, class R>
 static cudaError_t launch_3d_op(const OpParams& prm, const io_t<R>* u, const io_t<R>* v,
                                 io_t<R>* out, int batch, cudaStream_t stream) {
@@ -143,17 +148,8 @@ static cudaError_t launch_one(const OpParams& prm, const Tables* tabs, const io_
     (void)tabs;
     return launch_3d_op<P, NF, MODE, R>(prm, u, v, out, batch, stream);
   } else {
-  using M = WarpSmem<DIM, P, NF, MODE>;
-  constexpr size_t per_warp = (size_t)M::total * sizeof(R);
-  constexpr int WPB = per_warp * 4 <= 96 * 1024 ? 4 : (per_warp * 2 <= 110 * 1024 ? 2 : 1);
-  const size_t smem = ((size_t)TabSmem<P>::total + (size_t)WPB * M::total) * sizeof(R);
-  auto kern = op_kernel<DIM, P, NF, MODE, WPB, R>;
-  static SmemAttr attr;
-  cudaError_t ea = raise_smem_limit(attr, kern, smem);
-  if (ea != cudaSuccess) return ea;
-  dim3 grid((prm.E + WPB - 1) / WPB, batch);
-  kern<<<grid, WPB * 32, smem, stream>>>(prm, tabs, u, v, out);
-  return cudaGetLastError();
+    (void)tabs;
+    return launch_quad<P, NF, MODE, R>(prm, u, v, out, batch, stream);
   }
 }
 

@@ -206,7 +206,7 @@ template <class R> struct FaceBlocks { static constexpr int value = std::is_same
 // val(s) and grad(s, a) of array s, putg(f, a, x) the coefficient of the
 // reference derivative of field f's test function along a, putv(f, x) of its
 // value (J^T w). s2[a] = w (2/h_a)^2 and adv[a] = -w (2/h_a) u_a carry the weight.
-template <int NF, int MODE, class R, class VAL, class GRAD, class PUTG, class PUTV>
+template <int NF, int MODE, class R, int DIM = 3, class VAL, class GRAD, class PUTG, class PUTV>
 __device__ __forceinline__ void point_flux(const PhysT<R>& ph, const R* s2, const R* adv, VAL val,
                                            GRAD grad, PUTG putg, PUTV putv) {
   if constexpr (MODE == kResidual) {
@@ -220,7 +220,7 @@ __device__ __forceinline__ void point_flux(const PhysT<R>& ph, const R* s2, cons
     }
     const R kap = kd.get();
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
+    for (int a = 0; a < DIM; ++a) {
       R g[NF];
 #pragma unroll
       for (int f = 0; f < NF; ++f) g[f] = grad(f, a);
@@ -253,7 +253,7 @@ __device__ __forceinline__ void point_flux(const PhysT<R>& ph, const R* s2, cons
     }
     const R kap0 = k0.get(), kap1 = k1.get();
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
+    for (int a = 0; a < DIM; ++a) {
       const R g0 = grad(0, a);
       R t1[NF];
 #pragma unroll
@@ -286,7 +286,7 @@ __device__ __forceinline__ void point_flux(const PhysT<R>& ph, const R* s2, cons
     const R kap0 = k0.get();
     Dot<R> gw0, ch[NF - 1], cm[NF - 1];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
+    for (int a = 0; a < DIM; ++a) {
       const R sg0 = s2[a] * grad(0, a);
       R W[NF];
 #pragma unroll
@@ -1017,44 +1017,20 @@ __device__ __forceinline__ void face_interior_point(const PhysT<R>& ph, R ua, R 
   }
 }
 
-// The flux coefficients of one face point (tr and put as above).
+// The same at a point pt of a boundary face of the element on `side`: tag and
+// index of the face, ua the velocity along +axis at xp.
 template <int P, int NF, int MODE, class R, class TR, class PUT>
-__device__ __forceinline__ void face_point(const OpParams& prm, const FaceAt& F,
-                                           const FaceGeo<R>& G, int bidx, int pt, TR tr, PUT put) {
+__device__ __forceinline__ void face_boundary_point(const OpParams& prm, int tag, int bface, int side,
+                                                    R ua, R w, R delta, const R* xp, int bidx, int pt,
+                                                    TR tr, PUT put) {
   using SL = Slots<P, NF, MODE>;
-  using TO = TabOff<P>;
-  constexpr int Q = P + 2, NA = SL::NA;
+  constexpr int NA = SL::NA;
   const PhysT<R>& ph = phys<R>(prm);
-  const int a = F.a, b0 = a == 0 ? 1 : 0, b1 = a == 2 ? 1 : 2;
-  const int k1 = pt % Q, k2 = pt / Q;
-  const R h0 = G.h0, h1 = G.h1, xa = G.xa, hL = G.hL, hU = G.hU;
-  const R hh = h0 * h0 + h1 * h1;
-  R xp[3], uv[3];
-  {
-    const R xb0 = G.lo0 + halfv((ctab<P, R>(TO::X + k1) + R(1)) * h0);
-    const R xb1 = G.lo1 + halfv((ctab<P, R>(TO::X + k2) + R(1)) * h1);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) xp[c] = c == a ? xa : (c == b0 ? xb0 : xb1);
-  }
-  velocity(ph, xp, uv);
-  const R ua = pick3(uv, a);
-  const R w = ctab<P, R>(TO::W + k1) * ctab<P, R>(TO::W + k2) * (R(0.25f) * h0 * h1);
-  if (F.hasL && F.hasU) {
-    const R delta = ph.cip * R(P * P) / halfv(sqrtv(hL * hL + hh) + sqrtv(hU * hU + hh));
-    face_interior_point<P, NF, MODE, R>(ph, ua, w, delta, tr, put);
-    return;
-  }
-  // boundary face: the one element's own side and outward normal
-  const int side = F.hasL ? 0 : 1;
   const R nrm = side == 0 ? R(1) : R(-1);
-  const int bface = prm.side_off[2 * a + (side == 0 ? 1 : 0)] + F.j0 + pick3(prm.ne, b0) * F.j1;
-  const int tag = prm.btag[bface];
   R oS[NF], oT[NF];
 #pragma unroll
   for (int f = 0; f < NF; ++f) { oS[f] = R(0); oT[f] = R(0); }
   if (!(tag == kWall || (tag == kInlet && MODE != kResidual))) {
-    const R hs = side == 0 ? hL : hU;
-    const R delta = ph.cip * R(P * P) / sqrtv(hs * hs + hh);
     const R phiapp = (tag >= kElectrode0)
         ? (prm.phiapp_batch ? R(prm.phiapp_batch[bidx * 4 + (tag - kElectrode0)])
                             : ph.phiapp[tag - kElectrode0])
@@ -1100,6 +1076,39 @@ __device__ __forceinline__ void face_point(const OpParams& prm, const FaceAt& F,
     put(NF + f, t);
     if (f == 0) put(2 * NF, t);
   }
+}
+
+// The flux coefficients of one face point (tr and put as above).
+template <int P, int NF, int MODE, class R, class TR, class PUT>
+__device__ __forceinline__ void face_point(const OpParams& prm, const FaceAt& F,
+                                           const FaceGeo<R>& G, int bidx, int pt, TR tr, PUT put) {
+  using TO = TabOff<P>;
+  constexpr int Q = P + 2;
+  const PhysT<R>& ph = phys<R>(prm);
+  const int a = F.a, b0 = a == 0 ? 1 : 0, b1 = a == 2 ? 1 : 2;
+  const int k1 = pt % Q, k2 = pt / Q;
+  const R h0 = G.h0, h1 = G.h1, xa = G.xa, hL = G.hL, hU = G.hU;
+  const R hh = h0 * h0 + h1 * h1;
+  R xp[3], uv[3];
+  {
+    const R xb0 = G.lo0 + halfv((ctab<P, R>(TO::X + k1) + R(1)) * h0);
+    const R xb1 = G.lo1 + halfv((ctab<P, R>(TO::X + k2) + R(1)) * h1);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) xp[c] = c == a ? xa : (c == b0 ? xb0 : xb1);
+  }
+  velocity(ph, xp, uv);
+  const R ua = pick3(uv, a);
+  const R w = ctab<P, R>(TO::W + k1) * ctab<P, R>(TO::W + k2) * (R(0.25f) * h0 * h1);
+  if (F.hasL && F.hasU) {
+    const R delta = ph.cip * R(P * P) / halfv(sqrtv(hL * hL + hh) + sqrtv(hU * hU + hh));
+    face_interior_point<P, NF, MODE, R>(ph, ua, w, delta, tr, put);
+    return;
+  }
+  const int side = F.hasL ? 0 : 1;
+  const int bface = prm.side_off[2 * a + (side == 0 ? 1 : 0)] + F.j0 + pick3(prm.ne, b0) * F.j1;
+  const R hs = side == 0 ? hL : hU;
+  face_boundary_point<P, NF, MODE, R>(prm, prm.btag[bface], bface, side, ua, w,
+                                      ph.cip * R(P * P) / sqrtv(hs * hs + hh), xp, bidx, pt, tr, put);
 }
 
 // The stages from both elements' nodal values to the traces at the points of

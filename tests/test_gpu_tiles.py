@@ -57,3 +57,32 @@ def test_ragged_groups(p, fields, n):
     jv = op.jvp_f32(ud.float(), vd.float()).cpu().numpy()
     u32, v32 = (x.float().double().cpu().numpy() for x in (ud, vd))
     assert _rel(jv, orc.jvp(u32, v32), fields) < 2e-5
+
+
+@pytest.mark.parametrize("n", [(1, 1), (5, 3), (2, 7)])
+@pytest.mark.parametrize("fields", [2, 3])
+@pytest.mark.parametrize("p", [1, 2, 3])
+def test_quads(p, fields, n):
+    """Quadrilaterals: one element, odd meshes, every degree and field count, with
+    every boundary kind (Dirichlet on one side), FP64 and FP32."""
+    import torch
+    import paper_2112_09271_gb300 as enp
+    enp.build()
+    base = W.config("cube_n2_p2" if fields == 2 else "channel_n1", p=p)
+    coords = [c[-1] * np.linspace(0, 1, k + 1) ** 1.2 for c, k in zip(base.coords, n)]
+    tags = W.box_tags(2, list(n), coords, W.WALL)
+    tags[0][:], tags[1][:] = W.INLET, W.OUTLET
+    tags[2][:], tags[3][:] = W.ELECTRODE0, W.DIRICHLET
+    P = dataclasses.replace(base, dim=2, n_el=list(n) + [1], coords=coords, tags=tags)
+    src, dirv = W.random_sources(P, 5), W.random_dirichlet(P, 6)
+    orc = oracle.Oracle(P, src=src, dirichlet=dirv)
+    op = enp.Operator(P)
+    op.set_sources(torch.tensor(src, device="cuda"), torch.tensor(dirv, device="cuda"))
+    u, v, w = W.random_state(P, 1), W.random_vector(P, 2), W.random_vector(P, 3)
+    ud, vd, wd = (torch.tensor(x, device="cuda") for x in (u, v, w))
+    for g, r in ((op.residual(ud), orc.residual(u)), (op.jvp(ud, vd), orc.jvp(u, v)),
+                 (op.vjp(ud, wd), orc.vjp_entries(u, w, np.arange(P.n_dof)))):
+        assert _rel(g.cpu().numpy(), r, fields) < 1e-12
+    jv = op.jvp_f32(ud.float(), vd.float()).cpu().numpy()
+    u32, v32 = (x.float().double().cpu().numpy() for x in (ud, vd))
+    assert _rel(jv, orc.jvp(u32, v32), fields) < 2e-5
