@@ -87,15 +87,17 @@ __device__ __forceinline__ T warp_reduce8(T (&v)[8], int lane) {
 constexpr int kDotGroup = 8;
 
 template <class T, int W>
-__global__ void __launch_bounds__(kRedThreads)
-multidot_partial(const T* __restrict__ V, long long vstride, int nd, const T* __restrict__ w,
-                 long long n, long long bstride, double* __restrict__ part) {
+__device__ __forceinline__ void multidot_block(const T* __restrict__ V, long long vstride, int nd,
+                                               const T* __restrict__ w, long long n,
+                                               long long bstride, double* __restrict__ part) {
   __shared__ double red[kRedThreads / 32][kDotGroup];
   const int b = blockIdx.y;
   const T* wb = w + b * bstride;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long nu = n / W;
-  for (int i0 = 0; i0 < nd; i0 += kDotGroup) {
+  // the groups are shared over grid.z (short vectors leave the chip idle otherwise);
+  // each sum is the same whichever block forms it
+  for (int i0 = blockIdx.z * kDotGroup; i0 < nd; i0 += gridDim.z * kDotGroup) {
     const int ni = min(kDotGroup, nd - i0);
     const T* V0 = V + i0 * vstride + b * bstride;
     T acc[kDotGroup];
@@ -126,6 +128,13 @@ multidot_partial(const T* __restrict__ V, long long vstride, int nd, const T* __
   }
 }
 
+template <class T, int W>
+__global__ void __launch_bounds__(kRedThreads)
+multidot_partial(const T* __restrict__ V, long long vstride, int nd, const T* __restrict__ w,
+                 long long n, long long bstride, double* __restrict__ part) {
+  multidot_block<T, W>(V, vstride, nd, w, n, bstride, part);
+}
+
 // out[b][i] = sum over blocks of part[b][i][:], in block order.
 static __global__ void finish_partials(const double* __restrict__ part, int nparts, int count,
                                 double* __restrict__ out) {
@@ -149,11 +158,11 @@ inline int vec_width(long long n, long long vstride, const void* a, const void* 
   return ok ? W : 1;
 }
 
-// Blocks of a reduction over n entries in units of W: about two units per
-// thread, at most kRedBlocks. Depends on n only (not on the batch), so a point
+// Blocks of a reduction over n entries in units of W: one unit per thread, at most
+// kRedBlocks. Depends on n only (not on the batch), so a point
 // of a batch is reduced exactly as it is alone.
 inline int red_blocks(long long n, int W) {
   const long long nu = n / W;
-  const long long g = (nu + 2LL * enp::kRedThreads - 1) / (2LL * enp::kRedThreads);
+  const long long g = (nu + enp::kRedThreads - 1) / enp::kRedThreads;
   return (int)std::max(1LL, std::min<long long>(g, enp::kRedBlocks));
 }

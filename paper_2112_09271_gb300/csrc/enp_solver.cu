@@ -49,53 +49,6 @@ __global__ void recover_cm_kernel(const double* __restrict__ u, double* __restri
 }
 
 
-// w[b] -= sum_i V_i[b] h[b][i]  (h on the device, [batch][nd], nd <= 256),
-// in the vector's precision with the coefficients staged once per block, W
-// entries per 16-byte load. With NORM, also the partial sums of ||w_new||^2
-// per block, part[b][block] (thread sums in the vector's precision, then FP64).
-template <class T, int W, bool NORM>
-__global__ void __launch_bounds__(kRedThreads)
-multi_axpy(const T* __restrict__ V, long long vstride, int nd, const double* __restrict__ h,
-           T* __restrict__ w, long long n, long long bstride, double* __restrict__ part) {
-  __shared__ T hs[256];
-  __shared__ double red[kRedThreads / 32];
-  const int b = blockIdx.y;
-  for (int i = threadIdx.x; i < nd; i += blockDim.x) hs[i] = (T)h[b * nd + i];
-  __syncthreads();
-  const long long nu = n / W;
-  T nrm = T(0);
-  for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < nu;
-       u += (long long)gridDim.x * blockDim.x) {
-    T acc[W];
-    load_vec<T, W>(w + b * bstride + u * W, acc);
-    const T* Vu = V + b * bstride + u * W;
-#pragma unroll 4
-    for (int i = 0; i < nd; ++i) {
-      T vv[W];
-      load_vec<T, W>(Vu + i * vstride, vv);
-      const T hi = hs[i];
-#pragma unroll
-      for (int c = 0; c < W; ++c) acc[c] -= hi * vv[c];
-    }
-    store_vec<T, W>(w + b * bstride + u * W, acc);
-    if (NORM) {
-#pragma unroll
-      for (int c = 0; c < W; ++c) nrm += acc[c] * acc[c];
-    }
-  }
-  if (NORM) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const double s = warp_sum((double)nrm);
-    if (lane == 0) red[warp] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int wv = 0; wv < kRedThreads / 32; ++wv) t += red[wv];
-      part[(long long)b * gridDim.x + blockIdx.x] = t;
-    }
-  }
-}
-
 // y[b] = sum_{i<nd} V_i[b] c[b * cstride + i] (+ y[b] if accumulate), nd <= 256
 template <class T, class TY>
 __global__ void combine(const T* __restrict__ V, long long vstride, int nd,
@@ -209,6 +162,7 @@ __global__ void convert_kernel(const TX* __restrict__ x, TY* __restrict__ y, lon
 struct KrylovDev {
   double *H, *g, *cs, *sn, *hcol, *dh, *hn2, *inv, *beta, *bn2, *tol, *resn, *coef;
   int* jconv;   // -2 done before the cycle, -1 running, j converged at iteration j
+  int* count;   // blocks done, per point (zero between kernels)
 };
 
 __global__ void krylov_tolerance(KrylovDev K, int B, double rtol, double atol) {
@@ -233,42 +187,63 @@ __global__ void krylov_cycle_init(KrylovDev K, int B, int m, int* any_running, i
   if (!done) atomicOr(any_running, 1);
 }
 
-// One warp per (b, i): dh[b][i] = the partials of <V_i, w>_b summed in block
-// order (as finish_partials), added into the Hessenberg column (first pass:
-// stored).
-__global__ void krylov_hcol_finish(KrylovDev K, const double* __restrict__ part, int nparts,
-                                   int B, int m, int nd, int first) {
-  const int t = blockIdx.x;
-  if (t >= B * nd) return;
-  double s = 0.0;
-  for (int k = threadIdx.x; k < nparts; k += 32) s += part[(long long)t * nparts + k];
-  s = warp_sum(s);
+// Whether this block is the last of operating point blockIdx.y's to get here, all
+// of whose global writes before are then visible to it (the counter returns to 0).
+__device__ __forceinline__ bool last_block(int* counter, int blocks) {
+  __shared__ int s_last;
+  __threadfence();
+  __syncthreads();
   if (threadIdx.x == 0) {
-    const int b = t / nd, i = t % nd;
-    K.dh[t] = s;
-    K.hcol[(long long)b * (m + 1) + i] = first ? s : K.hcol[(long long)b * (m + 1) + i] + s;
+    s_last = atomicAdd(counter, 1) == blocks - 1;
+    if (s_last) *counter = 0;
+  }
+  __syncthreads();
+  if (s_last) __threadfence();
+  return s_last;
+}
+
+// One Gram-Schmidt pass' dot products: the partials of <V_i, w>_b, and, by the last
+// block of every point, dh[b][i] = their sum in block order (as finish_partials),
+// added into the Hessenberg column (first pass: stored).
+template <class T, int W>
+__global__ void __launch_bounds__(kRedThreads)
+arnoldi_dots(KrylovDev K, const T* __restrict__ V, long long vstride, int nd,
+             const T* __restrict__ w, long long n, long long bstride, double* part, int m,
+             int first) {
+  multidot_block<T, W>(V, vstride, nd, w, n, bstride, part);
+  const int b = blockIdx.y, nparts = gridDim.x;
+  if (!last_block(K.count + b, gridDim.x * gridDim.z)) return;
+  const int lane = threadIdx.x & 31;
+  for (int i = threadIdx.x >> 5; i < nd; i += kRedThreads / 32) {
+    const double* p = part + ((long long)b * nd + i) * nparts;
+    double s = 0.0;
+    for (int k = lane; k < nparts; k += 32) s += __ldcg(p + k);
+    s = warp_sum(s);
+    if (lane == 0) {
+      K.dh[(long long)b * nd + i] = s;
+      double* h = K.hcol + (long long)b * (m + 1) + i;
+      *h = first ? s : *h + s;
+    }
   }
 }
 
-// Iteration j of Arnoldi with Givens rotations, one warp per running point:
-// ||w||^2 summed from its partials in block order; the new Hessenberg column
-// and the earlier rotations staged in shared memory by the warp, then rotated
-// by lane 0 with the running entry in a register.
-__global__ void krylov_norm_givens(KrylovDev K, const double* __restrict__ part, int nparts, int B,
-                                   int m, int j, int* nonfinite) {
+// Arnoldi iteration j with Givens rotations for point b, by one block: ||w||^2
+// from its partials in block order, the new Hessenberg column rotated by the
+// earlier rotations (a chain of one fused multiply-add each) and by its own.
+__device__ __forceinline__ void norm_givens(KrylovDev K, const double* part, int nparts, int b,
+                                            int m, int j, int* nonfinite) {
   __shared__ double s_h[256], s_cs[256], s_sn[256];  // m <= 255
-  const int b = blockIdx.x;
-  if (b >= B) return;
-  const int lane = threadIdx.x;
-  double s = 0.0;
-  for (int k = lane; k < nparts; k += 32) s += part[(long long)b * nparts + k];
-  s = warp_sum(s);
   const double* hc = K.hcol + (long long)b * (m + 1);
   double* cs = K.cs + (long long)b * m;
   double* sn = K.sn + (long long)b * m;
-  for (int r = lane; r <= j; r += 32) s_h[r] = hc[r];
-  for (int r = lane; r < j; r += 32) { s_cs[r] = cs[r]; s_sn[r] = sn[r]; }
-  __syncwarp();
+  for (int r = threadIdx.x; r <= j; r += blockDim.x) s_h[r] = hc[r];
+  for (int r = threadIdx.x; r < j; r += blockDim.x) { s_cs[r] = cs[r]; s_sn[r] = sn[r]; }
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  const int lane = threadIdx.x;
+  double s = 0.0;
+  for (int k = lane; k < nparts; k += 32) s += __ldcg(part + (long long)b * nparts + k);
+  s = warp_sum(s);
   if (lane != 0) return;
   K.hn2[b] = s;
   const double hn = sqrt(s);
@@ -276,6 +251,7 @@ __global__ void krylov_norm_givens(KrylovDev K, const double* __restrict__ part,
   double* H = K.H + (long long)b * (m + 1) * m;
   double* g = K.g + (long long)b * (m + 1);
   double a = s_h[0];  // entry r of the column, already rotated by rotations < r
+#pragma unroll 4
   for (int r = 0; r < j; ++r) {
     const double c = s_h[r + 1], cr = s_cs[r], sr = s_sn[r];
     H[(long long)r * m + j] = cr * a + sr * c;
@@ -298,22 +274,90 @@ __global__ void krylov_norm_givens(KrylovDev K, const double* __restrict__ part,
   K.inv[b] = (hn > 0 && K.jconv[b] == -1) ? 1.0 / hn : 0.0;
 }
 
+// w[b] -= sum_i V_i[b] h[b][i]  (h on the device, [batch][nd], nd <= 256),
+// in the vector's precision with the coefficients staged once per block, W
+// entries per 16-byte load. With NORM (the second Gram-Schmidt pass of iteration
+// nd - 1), also the partial sums of ||w_new||^2 per block, part[b][block] (thread
+// sums in the vector's precision, then FP64), and the Givens update by the last
+// block of every point.
+template <class T, int W, bool NORM>
+__global__ void __launch_bounds__(kRedThreads)
+multi_axpy(KrylovDev K, const T* __restrict__ V, long long vstride, int nd,
+           const double* __restrict__ h, T* __restrict__ w, long long n, long long bstride,
+           double* part, int m, int* nonfinite) {
+  __shared__ T hs[256];
+  __shared__ double red[kRedThreads / 32];
+  const int b = blockIdx.y;
+  for (int i = threadIdx.x; i < nd; i += blockDim.x) hs[i] = (T)h[b * nd + i];
+  __syncthreads();
+  const long long nu = n / W;
+  T nrm = T(0);
+  for (long long u = blockIdx.x * (long long)blockDim.x + threadIdx.x; u < nu;
+       u += (long long)gridDim.x * blockDim.x) {
+    T acc[W];
+    load_vec<T, W>(w + b * bstride + u * W, acc);
+    const T* Vu = V + b * bstride + u * W;
+#pragma unroll 8
+    for (int i = 0; i < nd; ++i) {
+      T vv[W];
+      load_vec<T, W>(Vu + i * vstride, vv);
+      const T hi = hs[i];
+#pragma unroll
+      for (int c = 0; c < W; ++c) acc[c] -= hi * vv[c];
+    }
+    store_vec<T, W>(w + b * bstride + u * W, acc);
+    if (NORM) {
+#pragma unroll
+      for (int c = 0; c < W; ++c) nrm += acc[c] * acc[c];
+    }
+  }
+  if (NORM) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double s = warp_sum((double)nrm);
+    if (lane == 0) red[warp] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double t = 0.0;
+      for (int wv = 0; wv < kRedThreads / 32; ++wv) t += red[wv];
+      part[(long long)b * gridDim.x + blockIdx.x] = t;
+    }
+    if (last_block(K.count + b, gridDim.x)) norm_givens(K, part, gridDim.x, b, m, nd - 1, nonfinite);
+  }
+}
+
 // Back substitution for the update coefficients of every point (columns beyond
-// its convergence iteration are zero).
+// its convergence iteration are zero), one warp per point: right-hand sides in the
+// lanes, each solved value subtracted from all of them at once.
 __global__ void krylov_solve_upper(KrylovDev K, int B, int m, int jm) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  constexpr int R = 8;   // m <= 255
+  const int b = blockIdx.x, lane = threadIdx.x;
   if (b >= B) return;
   const int jc = K.jconv[b];
   const int ji = jc == -2 ? 0 : (jc >= 0 ? jc + 1 : jm);
   const double* H = K.H + (long long)b * (m + 1) * m;
   const double* g = K.g + (long long)b * (m + 1);
   double* y = K.coef + (long long)b * m;
-  for (int r = m - 1; r >= ji; --r) y[r] = 0.0;
-  for (int r = ji - 1; r >= 0; --r) {
-    double s = g[r];
-    for (int c = r + 1; c < ji; ++c) s -= H[(long long)r * m + c] * y[c];
-    const double d = H[(long long)r * m + r];
-    y[r] = d != 0.0 ? s / d : 0.0;
+  double s[R];
+#pragma unroll
+  for (int q = 0; q < R; ++q) {
+    const int r = lane + 32 * q;
+    s[q] = r < ji ? g[r] : 0.0;
+    if (r >= ji && r < m) y[r] = 0.0;
+  }
+  for (int c = ji - 1; c >= 0; --c) {
+    const double d = H[(long long)c * m + c];
+    double mine = 0.0;
+#pragma unroll
+    for (int q = 0; q < R; ++q)
+      if (c / 32 == q) mine = s[q];
+    const double v = __shfl_sync(0xffffffffu, mine, c & 31);
+    const double yc = d != 0.0 ? v / d : 0.0;
+    if (lane == 0) y[c] = yc;
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      const int r = lane + 32 * q;
+      if (r < c) s[q] -= H[(long long)r * m + c] * yc;
+    }
   }
 }
 
@@ -1520,6 +1564,7 @@ struct SolverState {
   // reductions
   double* part = nullptr;
   size_t part_count = 0;
+  int* kcount = nullptr;          // [B] blocks done, zero between kernels (KrylovDev::count)
   double* pvjp = nullptr;         // block sums of the parameter adjoint
   size_t pvjp_count = 0;
   double* dsmall = nullptr;       // device small vectors
@@ -1664,32 +1709,6 @@ cudaError_t dot_partials(enp_handle h, const T* V, long long vstride, int nd, co
   return cudaGetLastError();
 }
 
-// w -= sum_i V_i h_i (h: device [B][nd]); with part, also the partials of
-// ||w_new||^2 into part (their count per point in *nparts).
-template <class T>
-cudaError_t axpy_many(enp_handle h, const T* V, long long vstride, int nd, const double* hc, T* w,
-                      double* part, int* nparts) {
-  const long long n = h->n_dof;
-  const int B = h->batch;
-  const int W = vec_width<T>(n, vstride, V, w);
-  const int nb = red_blocks(n, W);
-  const dim3 g(nb, B);
-  constexpr int WV = 16 / sizeof(T);
-  if (part) {
-    if (W == 1)
-      enp::multi_axpy<T, 1, true><<<g, enp::kRedThreads, 0, h->stream>>>(V, vstride, nd, hc, w, n, n, part);
-    else
-      enp::multi_axpy<T, WV, true><<<g, enp::kRedThreads, 0, h->stream>>>(V, vstride, nd, hc, w, n, n, part);
-    *nparts = nb;
-  } else {
-    if (W == 1)
-      enp::multi_axpy<T, 1, false><<<g, enp::kRedThreads, 0, h->stream>>>(V, vstride, nd, hc, w, n, n, nullptr);
-    else
-      enp::multi_axpy<T, WV, false><<<g, enp::kRedThreads, 0, h->stream>>>(V, vstride, nd, hc, w, n, n, nullptr);
-  }
-  return cudaGetLastError();
-}
-
 template <class T>
 cudaError_t multidot(enp_handle h, const T* V, long long vstride, int nd, const T* w,
                      double* out) {
@@ -1701,29 +1720,49 @@ cudaError_t multidot(enp_handle h, const T* V, long long vstride, int nd, const 
 }
 
 // Gram-Schmidt of w against V_0..V_j, twice (classical, CGS2), then ||w||^2
-// and the Givens update of Arnoldi iteration j: seven launches, the partial
-// sums finished inside the kernels that consume them.
+// and the Givens update of Arnoldi iteration j: four launches, the partial sums
+// finished by the last block of the kernel that forms them.
+template <class TV, int W>
+cudaError_t arnoldi_launch(enp_handle h, const enp::KrylovDev& K, TV* V, long long vs, int j, TV* w,
+                           int m, int* nonfinite) {
+  SolverState& S = state_of(h);
+  const long long n = h->n_dof;
+  const int B = h->batch, nd = j + 1, nb = red_blocks(n, W);
+  // short vectors: the groups of eight dot products in blocks of their own
+  const int groups = (nd + enp::kDotGroup - 1) / enp::kDotGroup;
+  const int gz = std::max(1, std::min(groups, 608 / (nb * B)));
+  const dim3 g(nb, B), gd(nb, B, gz);
+  for (int pass = 0; pass < 2; ++pass) {
+    enp::arnoldi_dots<TV, W><<<gd, enp::kRedThreads, 0, h->stream>>>(K, V, vs, nd, w, n, n, S.part, m,
+                                                                    pass == 0);
+    if (pass == 0)
+      enp::multi_axpy<TV, W, false><<<g, enp::kRedThreads, 0, h->stream>>>(K, V, vs, nd, K.dh, w, n, n,
+                                                                          S.part, m, nonfinite);
+    else
+      enp::multi_axpy<TV, W, true><<<g, enp::kRedThreads, 0, h->stream>>>(K, V, vs, nd, K.dh, w, n, n,
+                                                                         S.part, m, nonfinite);
+  }
+  return cudaGetLastError();
+}
 template <class TV>
 cudaError_t arnoldi_orthogonalise(enp_handle h, const enp::KrylovDev& K, TV* V, long long vs,
                                   int j, TV* w, int m, int* nonfinite) {
   SolverState& S = state_of(h);
-  const int B = h->batch;
-  const int nd = j + 1;
-  cudaError_t e = cudaSuccess;
-  int np = 0;
-  for (int pass = 0; pass < 2; ++pass) {
-    if ((e = dot_partials<TV>(h, V, vs, nd, w, &np)) != cudaSuccess) return e;
-    enp::krylov_hcol_finish<<<B * nd, 32, 0, h->stream>>>(K, S.part, np, B, m, nd, pass == 0);
-    if ((e = axpy_many<TV>(h, V, vs, nd, K.dh, w, pass == 1 ? S.part : nullptr, &np)) !=
-        cudaSuccess)
-      return e;
-  }
-  enp::krylov_norm_givens<<<B, 32, 0, h->stream>>>(K, S.part, np, B, m, j, nonfinite);
-  return cudaGetLastError();
+  cudaError_t e = ensure(&S.part, S.part_count, (size_t)h->batch * (j + 1) * enp::kRedBlocks);
+  if (e != cudaSuccess) return e;
+  constexpr int W = 16 / sizeof(TV);
+  return vec_width<TV>(h->n_dof, vs, V, w) == 1
+             ? arnoldi_launch<TV, 1>(h, K, V, vs, j, w, m, nonfinite)
+             : arnoldi_launch<TV, W>(h, K, V, vs, j, w, m, nonfinite);
 }
 
 cudaError_t small(enp_handle h, size_t count) {
   SolverState& S = state_of(h);
+  if (!S.kcount) {
+    cudaError_t e = cudaMalloc(&S.kcount, sizeof(int) * h->batch);
+    if (e == cudaSuccess) e = cudaMemsetAsync(S.kcount, 0, sizeof(int) * h->batch, h->stream);
+    if (e != cudaSuccess) return e;
+  }
   return ensure(&S.dsmall, S.dsmall_count, count);
 }
 
@@ -1914,7 +1953,7 @@ void enp_solver_free(enp_handle h) {
   cudaFree(S.nbuf); cudaFree(S.nsmall);
   cudaFree(S.blocks); cudaFree(S.binv); cudaFree(S.gj_work); cudaFree(S.d_flag);
   cudaFree(S.blocks32); cudaFree(S.u32);
-  cudaFree(S.part); cudaFree(S.pvjp); cudaFree(S.dsmall); cudaFree(S.V);
+  cudaFree(S.part); cudaFree(S.pvjp); cudaFree(S.kcount); cudaFree(S.dsmall); cudaFree(S.V);
   for (auto& L : S.levels) {
     cudaFree(L.A); cudaFree(L.A32); cudaFree(L.x); cudaFree(L.b);
   }
@@ -2395,6 +2434,7 @@ static enp_status fgmres_any(enp_handle h, const TV* ulin, const TV* b, TV* x,
   int* flags = reinterpret_cast<int*>(q); q += B;   // jconv
   int* dflag = reinterpret_cast<int*>(q);           // [0] any running, [1] non-finite
   K.jconv = flags;
+  K.count = S.kcount;
   const int gx = grid_for(n);
   dim3 gv(gx, B);
   const int tb = std::min(B, 256), gbk = (B + tb - 1) / tb;
@@ -2461,7 +2501,7 @@ static enp_status fgmres_any(enp_handle h, const TV* ulin, const TV* b, TV* x,
     }
     if (nonfinite) break;
     const int jm = j;
-    enp::krylov_solve_upper<<<gbk, tb, 0, h->stream>>>(K, B, m, jm);
+    enp::krylov_solve_upper<<<B, 32, 0, h->stream>>>(K, B, m, jm);
     enp::combine<TV, TV><<<gv, 256, 0, h->stream>>>(Z, vs, jm, K.coef, m, x, n, n, 1);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_err(h, e, "fgmres update");
     all_done = cycle_done;
@@ -2559,6 +2599,7 @@ static enp_status fgmres_graph(enp_handle h, const TV* ulin, const TV* b, TV* x,
   int* flags = reinterpret_cast<int*>(q); q += B;
   int* dflag = reinterpret_cast<int*>(q);
   K.jconv = flags;
+  K.count = S.kcount;
   const int gx = grid_for(n);
   dim3 gv(gx, B);
   const int tb = std::min(B, 256), gbk = (B + tb - 1) / tb;
@@ -2602,7 +2643,7 @@ static enp_status fgmres_graph(enp_handle h, const TV* ulin, const TV* b, TV* x,
       arnoldi_orthogonalise<TV>(h, K, V, vs, j, w, m, dflag + 1);
       enp::scale_copy<TV, TV><<<gv, 256, 0, h->stream>>>(w, K.inv, 0.0, w, n, n);
     }
-    enp::krylov_solve_upper<<<gbk, tb, 0, h->stream>>>(K, B, m, m);
+    enp::krylov_solve_upper<<<B, 32, 0, h->stream>>>(K, B, m, m);
     enp::combine<TV, TV><<<gv, 256, 0, h->stream>>>(Z, vs, m, K.coef, m, xg, n, n, 1);
     e = cudaStreamEndCapture(h->stream, &graph);
     if (e == cudaSuccess) e = cudaGraphInstantiate(&S.gexec, graph, 0);
@@ -2881,6 +2922,7 @@ static enp_status newton_device(enp_handle h, double* u_user, const enp_newton_o
       K.resn = q; q += B;
       int* dflag = reinterpret_cast<int*>(q + B);
       K.jconv = reinterpret_cast<int*>(q);
+      K.count = S.kcount;
       TV* V = (TV*)S.V;
       TV* Z = (TV*)((char*)S.V + vbytes * (m + 1));
       const long long vs = ntot;
@@ -2936,7 +2978,7 @@ static enp_status newton_device(enp_handle h, double* u_user, const enp_newton_o
           arnoldi_orthogonalise<TV>(h, K, V, vs, j, w, m, dflag + 1);
           enp::scale_copy<TV, TV><<<gv, 256, 0, s2s>>>(w, K.inv, 0.0, w, n, n);
         }
-        enp::krylov_solve_upper<<<gbk, tb, 0, s2s>>>(K, B, m, m);
+        enp::krylov_solve_upper<<<B, 32, 0, s2s>>>(K, B, m, m);
         enp::combine<TV, TV><<<gv, 256, 0, s2s>>>(Z, vs, m, K.coef, m, xk, n, n, 1);
         enp::ng_krylov_count<<<1, 256, 0, s2s>>>(K, A, dflag, B, m, o->krylov.max_it, hK);
         if ((er = end_while(s2s)) != cudaSuccess) return er;
