@@ -718,6 +718,7 @@ coarse_vcycle_tail(const VcycleTail T) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   __shared__ float solo[kSoloFloats];
+  asm volatile("griddepcontrol.launch_dependents;");   // the block apply, see wait_for_tail
   const int b = blockIdx.y, rank = (int)cluster.block_rank();
   const int ct = rank * kTailThreads + threadIdx.x, cn = kTailCtas * kTailThreads;
   auto csync = [&] { cluster.sync(); };
@@ -1328,6 +1329,18 @@ gj_invert_cluster(const float* __restrict__ blocks, TS* __restrict__ out, int n,
   }
 }
 
+// The block apply may be launched beside the V-cycle's tail kernel: the tail lets
+// it start at once (let_next_start), and its last block ends only when the tail has
+// (wait_for_tail; no wait where it was launched alone), so that what follows in
+// the stream sees both. A 40x20x10 channel at p = 3 (blocks 98 us, tail 43 us, of
+// 330 us an iteration) then takes 248 ms a Newton solve (277 ms one after the
+// other), eight reactors of 24x6x2 at p = 2 28.0 ms (29.3 ms). A branch on a second
+// stream gains the same on the channel, but slows later graph launches by 5 %.
+__device__ __forceinline__ void wait_for_tail() {
+  if (blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // y_e = Binv_e x_e with the inverse stored transposed (BT[c][r]); accumulation in TA.
 template <class TS, class TA, class TV>
 __global__ void bj_apply_kernel(const TS* __restrict__ BT, const TV* __restrict__ x,
@@ -1361,6 +1374,7 @@ __global__ void bj_apply_kernel(const TS* __restrict__ BT, const TV* __restrict_
     const int f = r / Np, i = r % Np;
     y[b * bstride + f * EN + e * Np + i] = (TV)s;
   }
+  wait_for_tail();
 }
 
 // The same with V consecutive rows per load (V sizeof(TS) bytes): blockDim.x =
@@ -1415,6 +1429,7 @@ bj_apply_rows_kernel(const TS* __restrict__ BT, const TV* __restrict__ x, TV* __
     for (int q = 1; q < S; ++q) s += ps[q * n + r];
     yb[r / Np * EN + r % Np] = (TV)s;
   }
+  wait_for_tail();
 }
 
 // ------------------------------------------------- graph-driven Newton iteration
@@ -1871,7 +1886,9 @@ cudaError_t coarse_setup(enp_handle h, const double* u) {
   return cudaSuccess;
 }
 
-void vcycle(enp_handle h, size_t l) {
+// `beside` is launched next to the tail kernel and joined by what follows.
+template <class BESIDE>
+void vcycle(enp_handle h, size_t l, BESIDE beside) {
   SolverState& S = state_of(h);
   const int B = h->batch;
   auto& L = S.levels[l];
@@ -1889,6 +1906,7 @@ void vcycle(enp_handle h, size_t l) {
     T.omega = S.coarse_omega;
     T.coarsest_sweeps = kCoarsestSweeps;
     enp::coarse_vcycle_tail<<<dim3(enp::kTailCtas, B), enp::kTailThreads, 0, h->stream>>>(T);
+    beside();
     return;
   }
   const dim3 g(grid_for(L.n), B);
@@ -1900,7 +1918,7 @@ void vcycle(enp_handle h, size_t l) {
   auto& C = S.levels[l + 1];
   enp::coarse_restrict<<<dim3(grid_for(C.n), B), 256, 0, h->stream>>>(
       L.A32, L.x, L.b, L.nx, L.ny, L.nz, C.b, C.nx, C.ny, C.nz);
-  vcycle(h, l + 1);
+  vcycle(h, l + 1, beside);
   enp::coarse_prolong<<<g, 256, 0, h->stream>>>(L.A32, C.x, C.nx, C.ny, C.nz, L.x, L.nx, L.ny, L.nz,
                                                 S.coarse_omega);
   for (int sw = 0; sw < S.coarse_smooth; ++sw) {
@@ -1909,16 +1927,17 @@ void vcycle(enp_handle h, size_t l) {
   }
 }
 
-// z += P V(P^T r): the coarse correction of the two-level preconditioner.
-template <class TV>
-cudaError_t coarse_apply(enp_handle h, const TV* r, TV* z) {
+// z += P V(P^T r): the coarse correction of the two-level preconditioner. beside()
+// is launched next to the first V-cycle's tail and may form the z to add to.
+template <class TV, class BESIDE>
+cudaError_t coarse_apply(enp_handle h, const TV* r, TV* z, BESIDE beside) {
   SolverState& S = state_of(h);
   const OpParams& P = h->prm;
   const int B = h->batch;
   auto& L0 = S.levels[0];
   enp::coarse_from_fine<TV><<<dim3(grid_for(P.E, 128), B), 128, 0, h->stream>>>(r, L0.b, P.E, P.Np,
                                                                              P.batch_stride);
-  vcycle(h, 0);
+  vcycle(h, 0, beside);
   if (S.coarse_cycles > 1) {
     // further cycles on the level-0 residual: x += V(b - A0 x); the buffers
     // were allocated by the setup (no allocation here: this may be captured)
@@ -1931,7 +1950,7 @@ cudaError_t coarse_apply(enp_handle h, const TV* r, TV* z) {
     for (int c = 1; c < S.coarse_cycles; ++c) {
       enp::coarse_residual<<<g0, 256, 0, h->stream>>>(L0.A32, S.cx_acc, S.cb_keep, L0.b, L0.nx,
                                                       L0.ny, L0.nz);
-      vcycle(h, 0);
+      vcycle(h, 0, [] {});
       enp::axpy_f32<<<grid_for((long long)n0), 256, 0, h->stream>>>(L0.x, S.cx_acc, (long long)n0);
     }
     cudaMemcpyAsync(L0.x, S.cx_acc, sizeof(float) * n0, cudaMemcpyDeviceToDevice, h->stream);
@@ -2224,54 +2243,74 @@ enp_status enp_block_jacobi_setup(enp_handle h, const double* u, int storage) {
 
 // Apply the stored block inverse to a vector of type TV (double or float).
 template <class TV>
-static cudaError_t bj_apply_plain(enp_handle h, const TV* x, TV* y);
+static cudaError_t bj_apply_plain(enp_handle h, const TV* x, TV* y, bool beside);
 
 // The preconditioner: block-Jacobi, plus the coarse potential correction when
 // the two-level preconditioner is enabled and set up.
 template <class TV>
 static cudaError_t sweep_apply(enp_handle h, const TV* x, TV* z);
 
-template <class TV>
-static cudaError_t bj_apply_any(enp_handle h, const TV* x, TV* y) {
-  SolverState& S = state_of(h);
-  cudaError_t e = S.sweep_ready ? sweep_apply<TV>(h, x, y) : bj_apply_plain<TV>(h, x, y);
-  if (e == cudaSuccess && S.coarse && S.coarse_ready) e = coarse_apply<TV>(h, x, y);
-  return e;
-}
-
+// beside: start with the kernel launched before (the V-cycle's tail), not after it.
 template <class TS, class TA, class TV>
-static cudaError_t bj_launch(enp_handle h, const TV* x, TV* y) {
+static cudaError_t bj_launch(enp_handle h, const TV* x, TV* y, bool beside) {
   SolverState& S = state_of(h);
   const OpParams& P = h->prm;
   const int n = S.nb;
   const long long EN = (long long)P.E * P.Np;
-  const dim3 g(P.E, h->batch);
   const TS* B = (const TS*)S.binv;
+  cudaLaunchAttribute early{};
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(P.E, h->batch);
+  cfg.stream = h->stream;
+  cfg.attrs = &early;
+  cfg.numAttrs = beside ? 1 : 0;
   constexpr int W = 16 / sizeof(TS);     // rows of a 16-byte load
   // blocks of 96 rows and more, whose columns fill several warps' wide loads;
   // the inverses' base is cudaMalloc's, so n alone decides the alignment
   auto rows = [&](auto V) {
     constexpr int v = decltype(V)::value;
     const int rg = n / v, sets = std::max(1, std::min(256 / rg, 8));
-    enp::bj_apply_rows_kernel<TS, TA, TV, v><<<g, rg * sets, sizeof(TA) * n * (1 + sets), h->stream>>>(
-        B, x, y, n, P.Np, EN, P.batch_stride, S.pc_shared_built);
-    return cudaGetLastError();
+    cfg.blockDim = dim3(rg * sets);
+    cfg.dynamicSmemBytes = sizeof(TA) * n * (1 + sets);
+    return cudaLaunchKernelEx(&cfg, enp::bj_apply_rows_kernel<TS, TA, TV, v>, B, x, y, n, P.Np, EN,
+                              P.batch_stride, S.pc_shared_built);
   };
   if (n >= 96 && n % W == 0) return rows(std::integral_constant<int, W>());
   if (n >= 96 && n % 2 == 0) return rows(std::integral_constant<int, 2>());
-  const int threads = std::min(256, ((n + 31) / 32) * 32);
-  enp::bj_apply_kernel<TS, TA, TV><<<g, threads, sizeof(TA) * n, h->stream>>>(
-      B, x, y, n, P.NF, P.Np, EN, P.batch_stride, S.pc_shared_built);
-  return cudaGetLastError();
+  cfg.blockDim = dim3(std::min(256, ((n + 31) / 32) * 32));
+  cfg.dynamicSmemBytes = sizeof(TA) * n;
+  return cudaLaunchKernelEx(&cfg, enp::bj_apply_kernel<TS, TA, TV>, B, x, y, n, P.NF, P.Np, EN,
+                            P.batch_stride, S.pc_shared_built);
 }
 
 template <class TV>
-static cudaError_t bj_apply_plain(enp_handle h, const TV* x, TV* y) {
+static cudaError_t bj_apply_plain(enp_handle h, const TV* x, TV* y, bool beside) {
   SolverState& S = state_of(h);
-  if (S.storage == 0) return bj_launch<double, double, TV>(h, x, y);
-  if (S.storage == 1) return bj_launch<float, float, TV>(h, x, y);
-  return bj_launch<__nv_bfloat16, float, TV>(h, x, y);
+  if (S.storage == 0) return bj_launch<double, double, TV>(h, x, y, beside);
+  if (S.storage == 1) return bj_launch<float, float, TV>(h, x, y, beside);
+  return bj_launch<__nv_bfloat16, float, TV>(h, x, y, beside);
 }
+
+// The blocks and the V-cycle read x and each other's results not at all; the tail
+// of the V-cycle is a chain of short steps on eight SMs per point, so the blocks
+// stream beside it. A sweep goes before the coarse correction.
+template <class TV>
+static cudaError_t bj_apply_any(enp_handle h, const TV* x, TV* y) {
+  SolverState& S = state_of(h);
+  const bool coarse = S.coarse && S.coarse_ready;
+  cudaError_t e = cudaSuccess;
+  if (coarse && !S.sweep_ready) {
+    const cudaError_t ec =
+        coarse_apply<TV>(h, x, y, [&] { e = bj_apply_plain<TV>(h, x, y, true); });
+    return e != cudaSuccess ? e : ec;
+  }
+  e = S.sweep_ready ? sweep_apply<TV>(h, x, y) : bj_apply_plain<TV>(h, x, y, false);
+  if (e == cudaSuccess && coarse) e = coarse_apply<TV>(h, x, y, [] {});
+  return e;
+}
+
 
 // Downwind block Gauss-Seidel: z = (D + L)^-1 x with D the element blocks and L
 // the couplings of each element to its upstream neighbour along the flow axis.
