@@ -160,4 +160,13 @@ template <class R> __device__ __forceinline__ R valof(Tan<R> x) { return x.v; }
 __device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a, b, c); }
 
+// A kernel launched beside the one before it in the stream (programmatic launch; the
+// earlier kernel lets it start with griddepcontrol.launch_dependents) shares no
+// data with it, and its last block ends only when the earlier kernel has, so that
+// what follows in the stream sees both. No wait where it was launched alone.
+__device__ __forceinline__ void wait_for_launch_before() {
+  if (blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 }  // namespace enp

@@ -74,11 +74,12 @@ cudaError_t prepare_tables(int p, const Tables& t);
 // for every operating point: z_e = Binv_e (x_e - J_(e,up) z_up) down every line
 // of elements (hexahedra). binv: the transposed block inverses in `storage`
 // (0 FP64, 1 FP32, 2 BF16), one set per point or one shared set; upc: the
-// linearisation point. x and z do not overlap.
+// linearisation point. x and z do not overlap. beside: start with the kernel
+// launched before on s, whose results it does not read, and end after it.
 template <class TV>
 cudaError_t launch_sweep(const OpParams& prm, const void* binv, int storage, const TV* x, TV* z,
                          const TV* upc, int batch, cudaStream_t s, int a, int dir,
-                         int shared_blocks);
+                         int shared_blocks, bool beside);
 template <class TV> cudaError_t upload_tables_sweep(int p, const Tables& t);
 
 }  // namespace enp

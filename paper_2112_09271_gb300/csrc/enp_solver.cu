@@ -718,7 +718,7 @@ coarse_vcycle_tail(const VcycleTail T) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   __shared__ float solo[kSoloFloats];
-  asm volatile("griddepcontrol.launch_dependents;");   // the block apply, see wait_for_tail
+  asm volatile("griddepcontrol.launch_dependents;");   // see wait_for_launch_before
   const int b = blockIdx.y, rank = (int)cluster.block_rank();
   const int ct = rank * kTailThreads + threadIdx.x, cn = kTailCtas * kTailThreads;
   auto csync = [&] { cluster.sync(); };
@@ -1329,18 +1329,6 @@ gj_invert_cluster(const float* __restrict__ blocks, TS* __restrict__ out, int n,
   }
 }
 
-// The block apply may be launched beside the V-cycle's tail kernel: the tail lets
-// it start at once (let_next_start), and its last block ends only when the tail has
-// (wait_for_tail; no wait where it was launched alone), so that what follows in
-// the stream sees both. A 40x20x10 channel at p = 3 (blocks 98 us, tail 43 us, of
-// 330 us an iteration) then takes 248 ms a Newton solve (277 ms one after the
-// other), eight reactors of 24x6x2 at p = 2 28.0 ms (29.3 ms). A branch on a second
-// stream gains the same on the channel, but slows later graph launches by 5 %.
-__device__ __forceinline__ void wait_for_tail() {
-  if (blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-
 // y_e = Binv_e x_e with the inverse stored transposed (BT[c][r]); accumulation in TA.
 template <class TS, class TA, class TV>
 __global__ void bj_apply_kernel(const TS* __restrict__ BT, const TV* __restrict__ x,
@@ -1374,7 +1362,7 @@ __global__ void bj_apply_kernel(const TS* __restrict__ BT, const TV* __restrict_
     const int f = r / Np, i = r % Np;
     y[b * bstride + f * EN + e * Np + i] = (TV)s;
   }
-  wait_for_tail();
+  wait_for_launch_before();
 }
 
 // The same with V consecutive rows per load (V sizeof(TS) bytes): blockDim.x =
@@ -1429,7 +1417,7 @@ bj_apply_rows_kernel(const TS* __restrict__ BT, const TV* __restrict__ x, TV* __
     for (int q = 1; q < S; ++q) s += ps[q * n + r];
     yb[r / Np * EN + r % Np] = (TV)s;
   }
-  wait_for_tail();
+  wait_for_launch_before();
 }
 
 // ------------------------------------------------- graph-driven Newton iteration
@@ -2248,7 +2236,7 @@ static cudaError_t bj_apply_plain(enp_handle h, const TV* x, TV* y, bool beside)
 // The preconditioner: block-Jacobi, plus the coarse potential correction when
 // the two-level preconditioner is enabled and set up.
 template <class TV>
-static cudaError_t sweep_apply(enp_handle h, const TV* x, TV* z);
+static cudaError_t sweep_apply(enp_handle h, const TV* x, TV* z, bool beside);
 
 // beside: start with the kernel launched before (the V-cycle's tail), not after it.
 template <class TS, class TA, class TV>
@@ -2293,34 +2281,35 @@ static cudaError_t bj_apply_plain(enp_handle h, const TV* x, TV* y, bool beside)
   return bj_launch<__nv_bfloat16, float, TV>(h, x, y, beside);
 }
 
-// The blocks and the V-cycle read x and each other's results not at all; the tail
-// of the V-cycle is a chain of short steps on eight SMs per point, so the blocks
-// stream beside it. A sweep goes before the coarse correction.
+// The block part and the V-cycle read x and nothing of each other's; the tail of
+// the V-cycle is a chain of short steps on eight SMs per point, so the block part
+// runs beside it. A 40x20x10 channel at p = 3 (blocks 98 us, tail 43 us, of 330 us an
+// iteration) then takes 248 ms a Newton solve (277 ms one after the other), eight
+// reactors of 24x6x2 at p = 2 28.0 ms (29.3 ms); a sweep over 192x48x16 elements at
+// p = 2 with its correction 436 us (499 us). A branch on a second stream gains the
+// same on the channel, but slows later graph launches by 5 %.
 template <class TV>
 static cudaError_t bj_apply_any(enp_handle h, const TV* x, TV* y) {
   SolverState& S = state_of(h);
-  const bool coarse = S.coarse && S.coarse_ready;
+  auto block_part = [&](bool beside) {
+    return S.sweep_ready ? sweep_apply<TV>(h, x, y, beside) : bj_apply_plain<TV>(h, x, y, beside);
+  };
+  if (!(S.coarse && S.coarse_ready)) return block_part(false);
   cudaError_t e = cudaSuccess;
-  if (coarse && !S.sweep_ready) {
-    const cudaError_t ec =
-        coarse_apply<TV>(h, x, y, [&] { e = bj_apply_plain<TV>(h, x, y, true); });
-    return e != cudaSuccess ? e : ec;
-  }
-  e = S.sweep_ready ? sweep_apply<TV>(h, x, y) : bj_apply_plain<TV>(h, x, y, false);
-  if (e == cudaSuccess && coarse) e = coarse_apply<TV>(h, x, y, [] {});
-  return e;
+  const cudaError_t ec = coarse_apply<TV>(h, x, y, [&] { e = block_part(true); });
+  return e != cudaSuccess ? e : ec;
 }
 
 
 // Downwind block Gauss-Seidel: z = (D + L)^-1 x with D the element blocks and L
 // the couplings of each element to its upstream neighbour along the flow axis.
 template <class TV>
-static cudaError_t sweep_apply(enp_handle h, const TV* x, TV* z) {
+static cudaError_t sweep_apply(enp_handle h, const TV* x, TV* z, bool beside) {
   SolverState& S = state_of(h);
   const TV* upc = std::is_same<TV, double>::value ? reinterpret_cast<const TV*>(S.upc64)
                                                   : reinterpret_cast<const TV*>(S.upc32);
   return enp::launch_sweep<TV>(h->prm, S.binv, S.storage, x, z, upc, h->batch, h->stream,
-                               S.sweep_axis, S.sweep_dir, S.pc_shared_built);
+                               S.sweep_axis, S.sweep_dir, S.pc_shared_built, beside);
 }
 
 extern "C" enp_status enp_set_shared_blocks(enp_handle h, int point) {

@@ -294,13 +294,14 @@ sweep_line_kernel(const OpParams prm, const TS* __restrict__ binv, const TV* __r
       __syncthreads();
     }
   }
+  wait_for_launch_before();
 }
 
 // The sweep over every line of elements along axis a, for every operating point.
 template <int P, int NF, class TV, class TS>
 static cudaError_t launch_sweep_typed(const OpParams& prm, const void* binv, const TV* x, TV* z,
                                       const TV* upc, int batch, cudaStream_t stream, int a, int dir,
-                                      int shared_blocks) {
+                                      int shared_blocks, bool beside) {
   using TA = typename std::conditional<sizeof(TS) == 8, double, float>::type;
   constexpr size_t bytes = SweepSmem<P, NF, TV, TA>::bytes;
   auto kern = sweep_line_kernel<P, NF, TV, TS>;
@@ -308,31 +309,40 @@ static cudaError_t launch_sweep_typed(const OpParams& prm, const void* binv, con
   cudaError_t e = raise_smem_limit(attr, kern, bytes);
   if (e != cudaSuccess) return e;
   const int lines = prm.ne[a == 0 ? 1 : 0] * prm.ne[a == 2 ? 1 : 2];
-  kern<<<dim3((unsigned)lines, (unsigned)batch), SweepShape<P, NF>::NT, bytes, stream>>>(
-      prm, static_cast<const TS*>(binv), x, z, upc, a, dir, shared_blocks);
-  return cudaGetLastError();
+  cudaLaunchAttribute early{};
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)lines, (unsigned)batch);
+  cfg.blockDim = dim3(SweepShape<P, NF>::NT);
+  cfg.dynamicSmemBytes = bytes;
+  cfg.stream = stream;
+  cfg.attrs = &early;
+  cfg.numAttrs = beside ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, prm, static_cast<const TS*>(binv), x, z, upc, a, dir,
+                            shared_blocks);
 }
 template <int P, int NF, class TV>
 static cudaError_t launch_sweep_pn(const OpParams& prm, const void* binv, int storage, const TV* x,
                                    TV* z, const TV* upc, int batch, cudaStream_t s, int a, int dir,
-                                   int shared_blocks) {
-  if (storage == 0) return launch_sweep_typed<P, NF, TV, double>(prm, binv, x, z, upc, batch, s, a, dir, shared_blocks);
-  if (storage == 1) return launch_sweep_typed<P, NF, TV, float>(prm, binv, x, z, upc, batch, s, a, dir, shared_blocks);
-  return launch_sweep_typed<P, NF, TV, __nv_bfloat16>(prm, binv, x, z, upc, batch, s, a, dir, shared_blocks);
+                                   int shared_blocks, bool beside) {
+  if (storage == 0) return launch_sweep_typed<P, NF, TV, double>(prm, binv, x, z, upc, batch, s, a, dir, shared_blocks, beside);
+  if (storage == 1) return launch_sweep_typed<P, NF, TV, float>(prm, binv, x, z, upc, batch, s, a, dir, shared_blocks, beside);
+  return launch_sweep_typed<P, NF, TV, __nv_bfloat16>(prm, binv, x, z, upc, batch, s, a, dir, shared_blocks, beside);
 }
 
 template <class TV>
 cudaError_t launch_sweep(const OpParams& prm, const void* binv, int storage, const TV* x, TV* z,
                          const TV* upc, int batch, cudaStream_t s, int a, int dir,
-                         int shared_blocks) {
+                         int shared_blocks, bool beside) {
   if (prm.dim != 3 || storage < 0 || storage > 2 || (dir != 1 && dir != -1))
     return cudaErrorInvalidConfiguration;
 #define ENP_SW(PP)                                                                                  \
   case PP:                                                                                          \
     if (prm.NF == 2)                                                                                \
-      return launch_sweep_pn<PP, 2, TV>(prm, binv, storage, x, z, upc, batch, s, a, dir, shared_blocks); \
+      return launch_sweep_pn<PP, 2, TV>(prm, binv, storage, x, z, upc, batch, s, a, dir, shared_blocks, beside); \
     if (prm.NF == 3)                                                                                \
-      return launch_sweep_pn<PP, 3, TV>(prm, binv, storage, x, z, upc, batch, s, a, dir, shared_blocks); \
+      return launch_sweep_pn<PP, 3, TV>(prm, binv, storage, x, z, upc, batch, s, a, dir, shared_blocks, beside); \
     return cudaErrorInvalidConfiguration;
   switch (prm.p) { ENP_SW(1) ENP_SW(2) ENP_SW(3) ENP_SW(4) }
 #undef ENP_SW
