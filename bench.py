@@ -68,7 +68,7 @@ TRAFFIC = {
 }
 
 KERNEL_SOURCES = {
-    "operator": ("enp_operator.cuh", "enp_operator3d.cuh", "enp_common.cuh"),
+    "operator": ("enp_operator.cuh", "enp_tile3d.cuh", "enp_common.cuh"),
 }
 
 
@@ -80,11 +80,12 @@ def _function_text(src, signature):
 
 
 def _solver_apply_text():
-    """The block apply's own source: its kernel and its host launcher."""
+    """The block apply's own source: its kernels and their host launcher."""
     with open(os.path.join(ROOT, "paper_2112_09271_gb300", "csrc", "enp_solver.cu")) as fh:
         src = fh.read()
     return (_function_text(src, "__global__ void bj_apply_kernel(") +
-            _function_text(src, "static cudaError_t bj_apply_plain(enp_handle h, const TV* x, TV* y) {"))
+            _function_text(src, "bj_apply_rows_kernel(const TS*") +
+            _function_text(src, "static cudaError_t bj_launch("))
 
 
 def _kernel_hash(kind=None):
@@ -109,18 +110,23 @@ def _family(op_name):
 def contraction_flops(dim, p, nf, mode):
     """Floating-point operations (2 per multiply-add) of the sum-factorised
     contractions of one element for one operator application (mode 'res', 'jvp'
-    or 'vjp'): the volume, and the dim faces the element owns (every face once),
-    each with the traces of both sides and the test contractions of both sides,
-    all counted as interior. Pointwise physics is excluded."""
+    or 'vjp') as the kernels form them: the volume, and the dim faces the element
+    owns (every face once), all counted as interior. Hexahedra: only the arrays the
+    physics reads are interpolated (`na` values, the first `ng` with gradients), and
+    a face leaves `ns` coefficient arrays. Pointwise physics is excluded."""
     n, q = p + 1, p + 2
     if dim == 3:
-        interp = q * n ** 3 + q * q * n * n + q ** 3 * n + 3 * q ** 4
-        trace = n ** 3 + 2 * (q * n * n + q * q * n)
-        ftest = 2 * (q * q * n + q * n * n) + n ** 3
-    else:
-        interp = q * n * n + q * q * n + 2 * q ** 3
-        trace = n * n + 2 * q * n
-        ftest = 2 * q * n + n * n
+        na = nf if mode == "res" else 2 * nf
+        ng = nf if mode == "res" else nf + 1
+        ns = 3 * nf if mode == "vjp" else 2 * nf + 1
+        interp = q * n ** 3 + q * q * n * n + q ** 3 * n
+        vol = na * interp + ng * (q ** 3 * n + 2 * q ** 4) + nf * (interp + q ** 3 * n + 2 * q ** 4)
+        line = q * n * n + q * q * n
+        faces = dim * (2 * (ng * n ** 3 + (na + ng) * line) + ns * line + 2 * nf * n ** 3)
+        return 2 * (vol + faces)
+    interp = q * n * n + q * q * n + 2 * q ** 3
+    trace = n * n + 2 * q * n
+    ftest = 2 * q * n + n * n
     nv = 1 if mode == "res" else 2
     vol = nf * (nv * interp + interp)
     faces = dim * nf * (2 * nv * trace + 2 * ftest)
@@ -529,7 +535,7 @@ def main():
     ap.add_argument("--only", default=None,
                     help="time one operator alone (for profiling): residual_f64, jvp_f64, "
                          "vjp_f64, residual_df32, jvp_df32, vjp_df32, jvp_f32, bj_apply_f32, "
-                         "bj_setup_f32 (block-Jacobi setup: FP32 block columns and inversion); "
+                         "bj_setup_f32 (block-Jacobi setup: FP32 element blocks and inversion); "
                          "no autotune, solves or e2e; or "
                          "fgmres_f64 / fgmres_f32: FGMRES(50) cycles with the two-level "
                          "preconditioner on the solve workload; precond_f32: block-Jacobi "
@@ -616,7 +622,8 @@ def main():
     op_l = 2 if prob.dim == 3 else 1   # hexahedra: a face launch, then an element launch
     launches = {nm: op_l for nm in fp64_ops + ["jvp_f32"]}
     launches.update({"bj_apply_f32": 1, "recover_cm": 1, "inner_product": 2,
-                     "bj_setup_f32": 3})  # FP32 copy of u, block columns, inversion
+                     # FP32 copy of u, assembly, and the inversion (by elimination: four)
+                     "bj_setup_f32": 6 if prob.dim == 3 and prob.p > 1 else 3})
     launches_per_step = sum(launches[nm] for nm in ops)
     ip_out = np.zeros(1)
 
@@ -711,11 +718,11 @@ def main():
         peak = DF32_PEAK_TFLOPS
         peak_kind = ("derived: 152 SMs x 128 FP32 lanes x 2.07 GHz / 12 FP32 instructions per "
                      "double-float multiply-add x 2 flop")
-        kname = f"face3d_kernel + op3d_kernel <p={prob.p},NF={prob.n_fields},jvp,df> (double-float)"
+        kname = f"tileface3d_kernel + tile3d_kernel <p={prob.p},NF={prob.n_fields},jvp,df> (double-float)"
     else:
         peak = FP64_PEAK_TFLOPS
         peak_kind = "derived: 152 SMs x 2 FP64 FMA/clk x 2.07 GHz (measured FMA loop 1.20)"
-        kname = f"face3d_kernel + op3d_kernel <p={prob.p},NF={prob.n_fields},jvp,double>"
+        kname = f"tileface3d_kernel + tile3d_kernel <p={prob.p},NF={prob.n_fields},jvp,double>"
     achieved = fl / dom_s / 1e12
     hbm_frac = hbm_bytes / dom_s / 1e9 / hbm
     roof = {"bound": "alu", "kernel": kname + " (one operator application = the two launches, "
