@@ -317,57 +317,58 @@ enp_status enp_dg_create(enp_handle* out, const enp_mesh_desc* mesh, const enp_p
   build_tables(P.p, h->htab);
 
   cudaError_t e;
-  for (int a = 0; a < dim; ++a) {
-    e = cudaMalloc(&h->d_xv[a], sizeof(double) * (P.ne[a] + 1));
-    if (e != cudaSuccess) { enp_status s = cuda_fail(h, e, "cudaMalloc coords"); enp_dg_destroy(h); return s; }
-    e = cudaMemcpy(h->d_xv[a], mesh->coords[a], sizeof(double) * (P.ne[a] + 1), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) { enp_status s = cuda_fail(h, e, "upload coords"); enp_dg_destroy(h); return s; }
-    P.xv[a] = h->d_xv[a];
-    std::vector<float> cf(mesh->coords[a], mesh->coords[a] + P.ne[a] + 1);
-    e = cudaMalloc(&h->d_xvf[a], sizeof(float) * (P.ne[a] + 1));
-    if (e == cudaSuccess)
-      e = cudaMemcpy(h->d_xvf[a], cf.data(), sizeof(float) * (P.ne[a] + 1), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) { enp_status s = cuda_fail(h, e, "upload coords (FP32)"); enp_dg_destroy(h); return s; }
-    P.xvf[a] = h->d_xvf[a];
-    std::vector<float2> cd(P.ne[a] + 1);
-    for (int i = 0; i <= P.ne[a]; ++i) {
-      const enp::df x(mesh->coords[a][i]);
-      cd[i] = make_float2(x.hi, x.lo);
+  // The geometry of every axis in one buffer and one copy: (h, 2 / h) of each element
+  // (FP64, double-float, FP32) and the vertices (the same). A buffer and a copy for
+  // each of them took 12 of either, some 130 us of creating a handle.
+  {
+    std::vector<char> geo;
+    size_t at[3][6];
+    auto put = [&](size_t bytes) {       // room for one array, 16-byte aligned
+      const size_t o = (geo.size() + 15) / 16 * 16;
+      geo.resize(o + bytes);
+      return o;
+    };
+    for (int a = 0; a < dim; ++a) {
+      const size_t ne = (size_t)P.ne[a];
+      const double* x = mesh->coords[a];
+      at[a][0] = put(ne * sizeof(double2));
+      at[a][1] = put(ne * sizeof(float4));
+      at[a][2] = put(ne * sizeof(float2));
+      at[a][3] = put((ne + 1) * sizeof(double));
+      at[a][4] = put((ne + 1) * sizeof(float2));
+      at[a][5] = put((ne + 1) * sizeof(float));
+      for (size_t i = 0; i < ne; ++i) {
+        const double hi = x[i + 1] - x[i];
+        const double2 s64 = make_double2(hi, 2.0 / hi);
+        const enp::df u(s64.x), v(s64.y);
+        reinterpret_cast<double2*>(geo.data() + at[a][0])[i] = s64;
+        reinterpret_cast<float4*>(geo.data() + at[a][1])[i] = make_float4(u.hi, u.lo, v.hi, v.lo);
+        reinterpret_cast<float2*>(geo.data() + at[a][2])[i] = make_float2((float)s64.x, (float)s64.y);
+      }
+      for (size_t i = 0; i <= ne; ++i) {
+        const enp::df u(x[i]);
+        reinterpret_cast<double*>(geo.data() + at[a][3])[i] = x[i];
+        reinterpret_cast<float2*>(geo.data() + at[a][4])[i] = make_float2(u.hi, u.lo);
+        reinterpret_cast<float*>(geo.data() + at[a][5])[i] = (float)x[i];
+      }
     }
-    e = cudaMalloc(&h->d_xvdf[a], sizeof(float2) * (P.ne[a] + 1));
-    if (e == cudaSuccess)
-      e = cudaMemcpy(h->d_xvdf[a], cd.data(), sizeof(float2) * (P.ne[a] + 1), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) { enp_status s = cuda_fail(h, e, "upload coords (double-float)"); enp_dg_destroy(h); return s; }
-    P.xvdf[a] = h->d_xvdf[a];
-    // (h, 2 / h) of every element: one buffer of FP64, then double-float, then FP32 values
-    const size_t ne = (size_t)P.ne[a];
-    std::vector<char> sb(ne * (sizeof(double2) + sizeof(float4) + sizeof(float2)));
-    double2* s64 = reinterpret_cast<double2*>(sb.data());
-    float4* sdf = reinterpret_cast<float4*>(s64 + ne);
-    float2* s32 = reinterpret_cast<float2*>(sdf + ne);
-    for (size_t i = 0; i < ne; ++i) {
-      const double hi = mesh->coords[a][i + 1] - mesh->coords[a][i];
-      s64[i] = make_double2(hi, 2.0 / hi);
-      const enp::df x(s64[i].x), y(s64[i].y);
-      sdf[i] = make_float4(x.hi, x.lo, y.hi, y.lo);
-      s32[i] = make_float2((float)s64[i].x, (float)s64[i].y);
+    e = cudaMalloc(&h->d_geo, geo.size());
+    if (e == cudaSuccess) e = cudaMemcpy(h->d_geo, geo.data(), geo.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) { enp_status s = cuda_fail(h, e, "upload geometry"); enp_dg_destroy(h); return s; }
+    for (int a = 0; a < 3; ++a) {
+      const char* g = static_cast<const char*>(h->d_geo);
+      const bool has = a < dim;
+      P.xs[a] = has ? reinterpret_cast<const double2*>(g + at[a][0]) : nullptr;
+      P.xsdf[a] = has ? reinterpret_cast<const float4*>(g + at[a][1]) : nullptr;
+      P.xsf[a] = has ? reinterpret_cast<const float2*>(g + at[a][2]) : nullptr;
+      P.xv[a] = has ? reinterpret_cast<const double*>(g + at[a][3]) : nullptr;
+      P.xvdf[a] = has ? reinterpret_cast<const float2*>(g + at[a][4]) : nullptr;
+      P.xvf[a] = has ? reinterpret_cast<const float*>(g + at[a][5]) : nullptr;
     }
-    e = cudaMalloc(&h->d_scale[a], sb.size());
-    if (e == cudaSuccess) e = cudaMemcpy(h->d_scale[a], sb.data(), sb.size(), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) { enp_status s = cuda_fail(h, e, "upload element scales"); enp_dg_destroy(h); return s; }
-    P.xs[a] = static_cast<const double2*>(h->d_scale[a]);
-    P.xsdf[a] = reinterpret_cast<const float4*>(P.xs[a] + ne);
-    P.xsf[a] = reinterpret_cast<const float2*>(P.xsdf[a] + ne);
-  }
-  for (int a = dim; a < 3; ++a) {
-    P.xv[a] = nullptr; P.xvf[a] = nullptr; P.xvdf[a] = nullptr;
-    P.xs[a] = nullptr; P.xsf[a] = nullptr; P.xsdf[a] = nullptr;
   }
   e = cudaMalloc(&h->d_btag, tags.size());
   if (e == cudaSuccess) e = cudaMemcpy(h->d_btag, tags.data(), tags.size(), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMalloc(&h->d_tab, sizeof(Tables));
-  if (e == cudaSuccess) e = cudaMemcpy(h->d_tab, &h->htab, sizeof(Tables), cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) { enp_status s = cuda_fail(h, e, "upload tables"); enp_dg_destroy(h); return s; }
+  if (e != cudaSuccess) { enp_status s = cuda_fail(h, e, "upload face tags"); enp_dg_destroy(h); return s; }
   P.btag = h->d_btag;
   P.fbuf = nullptr;
   P.fbuf_stride = 0;
@@ -401,9 +402,8 @@ enp_status enp_dg_create(enp_handle* out, const enp_mesh_desc* mesh, const enp_p
 enp_status enp_dg_destroy(enp_handle h) {
   if (!h) return ENP_ERR_INVALID_ARG;
   enp_solver_free(h);
-  for (int a = 0; a < 3; ++a) { cudaFree(h->d_xv[a]); cudaFree(h->d_xvf[a]); cudaFree(h->d_xvdf[a]); cudaFree(h->d_scale[a]); }
+  cudaFree(h->d_geo);
   cudaFree(h->d_btag);
-  cudaFree(h->d_tab);
   cudaFree(h->d_src);
   cudaFree(h->d_dir);
   cudaFree(h->d_phiapp);
@@ -528,7 +528,7 @@ enp_status enp_quadrature_points(enp_handle h, double* xq, double* xbq) {
 
 static enp_status run_op_f64(enp_handle h, int mode, const double* u, const double* v, double* out) {
   if (!h || !u || !out || (mode != 0 && !v)) return fail(h, ENP_ERR_INVALID_ARG, "null argument");
-  cudaError_t e = enp::launch_op<double>(mode, h->prm, h->d_tab, u, v, out, h->batch, h->stream);
+  cudaError_t e = enp::launch_op<double>(mode, h->prm, u, v, out, h->batch, h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "operator launch");
   return ENP_OK;
 }
@@ -539,7 +539,7 @@ enp_status enp_vjp(enp_handle h, const double* u, const double* w, double* jtw) 
 
 enp_status enp_jvp_f32(enp_handle h, const float* u, const float* v, float* jv) {
   if (!h || !u || !v || !jv) return fail(h, ENP_ERR_INVALID_ARG, "null argument");
-  cudaError_t e = enp::launch_op<float>(1, h->prm, h->d_tab, u, v, jv, h->batch, h->stream);
+  cudaError_t e = enp::launch_op<float>(1, h->prm, u, v, jv, h->batch, h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "operator launch (f32)");
   return ENP_OK;
 }
@@ -553,7 +553,7 @@ enp_status enp_param_count(enp_handle h, int* n_theta) {
 enp_status enp_param_jacobian(enp_handle h, const double* u, double* dRdtheta) {
   if (!h || !u || !dRdtheta) return fail(h, ENP_ERR_INVALID_ARG, "null argument");
   if (h->prm.dim != 3) return fail(h, ENP_ERR_UNSUPPORTED, "dR/dtheta is built for hexahedra");
-  cudaError_t e = enp::launch_op<double>(enp::kParam, h->prm, h->d_tab, u, nullptr, dRdtheta,
+  cudaError_t e = enp::launch_op<double>(enp::kParam, h->prm, u, nullptr, dRdtheta,
                                          h->batch * h->prm.n_theta, h->stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "parameter Jacobian launch");
   return ENP_OK;
@@ -565,10 +565,10 @@ enp_status enp_param_jacobian(enp_handle h, const double* u, double* dRdtheta) {
 // each operator mode on this handle's mesh (three launches each, CUDA events)
 // and keep the fastest.
 template <class R>
-static cudaError_t tune_launch(int mode, const OpParams& P, const Tables* t, enp::io_t<R>* u,
+static cudaError_t tune_launch(int mode, const OpParams& P, enp::io_t<R>* u,
                                enp::io_t<R>* v, enp::io_t<R>* out, cudaStream_t s) {
   if constexpr (std::is_same<R, enp::df>::value) return enp::launch_op_df(mode, P, u, v, out, 1, s);
-  else return enp::launch_op<R>(mode, P, t, u, v, out, 1, s);
+  else return enp::launch_op<R>(mode, P, u, v, out, 1, s);
 }
 
 // The tile shapes of one operator mode: faces per block of the face kernel
@@ -585,10 +585,10 @@ static cudaError_t tune_mode(enp_handle h, int mode, enp::io_t<R>* u, enp::io_t<
   cudaEventCreate(&e1);
   cudaError_t err = cudaSuccess;
   auto time_it = [&](float* ms) -> cudaError_t {
-    cudaError_t er = tune_launch<R>(mode, P, h->d_tab, u, v, out, h->stream);
+    cudaError_t er = tune_launch<R>(mode, P, u, v, out, h->stream);
     if (er != cudaSuccess) return er;
     cudaEventRecord(e0, h->stream);
-    for (int r = 0; r < 3; ++r) tune_launch<R>(mode, P, h->d_tab, u, v, out, h->stream);
+    for (int r = 0; r < 3; ++r) tune_launch<R>(mode, P, u, v, out, h->stream);
     cudaEventRecord(e1, h->stream);
     er = cudaEventSynchronize(e1);
     *ms = 0.f;

@@ -13,7 +13,7 @@ namespace enp {
 // double). With prm.arith == kArithDF, launch_op<double> on hexahedra runs the
 // double-float kernels.
 template <class R>
-cudaError_t launch_op(int mode, const OpParams& prm, const Tables* tabs, const io_t<R>* u,
+cudaError_t launch_op(int mode, const OpParams& prm, const io_t<R>* u,
                       const io_t<R>* v, io_t<R>* out, int batch, cudaStream_t stream);
 
 // The double-float hexahedral operator: R, J v and J^T w of degree prm.p (op_df.cu), compiled one degree per translation unit
@@ -90,11 +90,7 @@ void enp_solver_free(struct enp_dg* h);
 struct enp_dg {
   enp::OpParams prm{};
   enp::Tables htab{};
-  enp::Tables* d_tab = nullptr;
-  double* d_xv[3] = {nullptr, nullptr, nullptr};
-  float* d_xvf[3] = {nullptr, nullptr, nullptr};
-  float2* d_xvdf[3] = {nullptr, nullptr, nullptr};
-  void* d_scale[3] = {nullptr, nullptr, nullptr};  // (h, 2 / h) per axis: FP64, double-float, FP32
+  void* d_geo = nullptr;     // vertices and element scales of every axis
   uint8_t* d_btag = nullptr;
   double* d_src = nullptr;
   double* d_dir = nullptr;

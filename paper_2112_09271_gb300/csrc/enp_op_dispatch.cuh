@@ -142,40 +142,38 @@ static cudaError_t launch_3d_op(const OpParams& prm, const io_t<R>* u, const io_
 }
 
 template <int DIM, int P, int NF, int MODE, class R>
-static cudaError_t launch_one(const OpParams& prm, const Tables* tabs, const io_t<R>* u,
+static cudaError_t launch_one(const OpParams& prm, const io_t<R>* u,
                               const io_t<R>* v, io_t<R>* out, int batch, cudaStream_t stream) {
   if constexpr (DIM == 3) {
-    (void)tabs;
     return launch_3d_op<P, NF, MODE, R>(prm, u, v, out, batch, stream);
   } else {
-    (void)tabs;
     return launch_quad<P, NF, MODE, R>(prm, u, v, out, batch, stream);
   }
 }
 
 template <int DIM, int P, int NF, class R>
-static cudaError_t launch_mode(int mode, const OpParams& prm, const Tables* t, const io_t<R>* u,
+static cudaError_t launch_mode(int mode, const OpParams& prm, const io_t<R>* u,
                                const io_t<R>* v, io_t<R>* out, int batch, cudaStream_t s) {
   if constexpr (std::is_same<R, df>::value) {
     // double-float: the residual, J v and J^T w (the element blocks and dR/dtheta
     // stay with the FP64 kernels)
     switch (mode) {
-      case kResidual: return launch_one<DIM, P, NF, kResidual, R>(prm, t, u, v, out, batch, s);
-      case kJvp: return launch_one<DIM, P, NF, kJvp, R>(prm, t, u, v, out, batch, s);
-      case kVjp: return launch_one<DIM, P, NF, kVjp, R>(prm, t, u, v, out, batch, s);
+      case kResidual: return launch_one<DIM, P, NF, kResidual, R>(prm, u, v, out, batch, s);
+      case kJvp: return launch_one<DIM, P, NF, kJvp, R>(prm, u, v, out, batch, s);
+      case kVjp: return launch_one<DIM, P, NF, kVjp, R>(prm, u, v, out, batch, s);
     }
     return cudaErrorNotSupported;
   } else {
     switch (mode) {
-      case kResidual: return launch_one<DIM, P, NF, kResidual, R>(prm, t, u, v, out, batch, s);
-      case kJvp: return launch_one<DIM, P, NF, kJvp, R>(prm, t, u, v, out, batch, s);
-      case kVjp: return launch_one<DIM, P, NF, kVjp, R>(prm, t, u, v, out, batch, s);
+      case kResidual: return launch_one<DIM, P, NF, kResidual, R>(prm, u, v, out, batch, s);
+      case kJvp: return launch_one<DIM, P, NF, kJvp, R>(prm, u, v, out, batch, s);
+      case kVjp: return launch_one<DIM, P, NF, kVjp, R>(prm, u, v, out, batch, s);
       case kBlockCol:
-        if constexpr (DIM == 2) return launch_one<DIM, P, NF, kBlockCol, R>(prm, t, u, v, out, batch, s);
+        if constexpr (DIM == 2) return launch_one<DIM, P, NF, kBlockCol, R>(prm, u, v, out, batch, s);
         return cudaErrorNotSupported;
       case kParam:
         if constexpr (DIM == 3 && std::is_same<R, double>::value)
-          return launch_one<DIM, P, NF, kParam, R>(prm, t, u, v, out, batch, s);
+          return launch_one<DIM, P, NF, kParam, R>(prm, u, v, out, batch, s);
         return cudaErrorNotSupported;
     }
     return cudaErrorInvalidValue;
@@ -183,10 +181,10 @@ static cudaError_t launch_mode(int mode, const OpParams& prm, const Tables* t, c
 }
 
 template <int DIM, int P, class R>
-static cudaError_t launch_nf(int mode, const OpParams& prm, const Tables* t, const io_t<R>* u,
+static cudaError_t launch_nf(int mode, const OpParams& prm, const io_t<R>* u,
                              const io_t<R>* v, io_t<R>* out, int batch, cudaStream_t s) {
-  if (prm.NF == 2) return launch_mode<DIM, P, 2, R>(mode, prm, t, u, v, out, batch, s);
-  if (prm.NF == 3) return launch_mode<DIM, P, 3, R>(mode, prm, t, u, v, out, batch, s);
+  if (prm.NF == 2) return launch_mode<DIM, P, 2, R>(mode, prm, u, v, out, batch, s);
+  if (prm.NF == 3) return launch_mode<DIM, P, 3, R>(mode, prm, u, v, out, batch, s);
   return cudaErrorInvalidConfiguration;
 }
 
@@ -250,7 +248,7 @@ cudaError_t prepare_tables(int p, const Tables& t) {
 }
 
 template <class R>
-cudaError_t launch_op(int mode, const OpParams& prm, const Tables* t, const io_t<R>* u,
+cudaError_t launch_op(int mode, const OpParams& prm, const io_t<R>* u,
                       const io_t<R>* v, io_t<R>* out, int batch, cudaStream_t s) {
   if constexpr (std::is_same<R, double>::value) {
     // R, J v and J^T w in double-float arithmetic on hexahedra
@@ -259,17 +257,17 @@ cudaError_t launch_op(int mode, const OpParams& prm, const Tables* t, const io_t
   }
   if (prm.dim == 3) {
     switch (prm.p) {
-      case 1: return launch_nf<3, 1, R>(mode, prm, t, u, v, out, batch, s);
-      case 2: return launch_nf<3, 2, R>(mode, prm, t, u, v, out, batch, s);
-      case 3: return launch_nf<3, 3, R>(mode, prm, t, u, v, out, batch, s);
-      case 4: return launch_nf<3, 4, R>(mode, prm, t, u, v, out, batch, s);
+      case 1: return launch_nf<3, 1, R>(mode, prm, u, v, out, batch, s);
+      case 2: return launch_nf<3, 2, R>(mode, prm, u, v, out, batch, s);
+      case 3: return launch_nf<3, 3, R>(mode, prm, u, v, out, batch, s);
+      case 4: return launch_nf<3, 4, R>(mode, prm, u, v, out, batch, s);
     }
   }
   if (prm.dim == 2) {
     switch (prm.p) {
-      case 1: return launch_nf<2, 1, R>(mode, prm, t, u, v, out, batch, s);
-      case 2: return launch_nf<2, 2, R>(mode, prm, t, u, v, out, batch, s);
-      case 3: return launch_nf<2, 3, R>(mode, prm, t, u, v, out, batch, s);
+      case 1: return launch_nf<2, 1, R>(mode, prm, u, v, out, batch, s);
+      case 2: return launch_nf<2, 2, R>(mode, prm, u, v, out, batch, s);
+      case 3: return launch_nf<2, 3, R>(mode, prm, u, v, out, batch, s);
     }
   }
   return cudaErrorInvalidConfiguration;
@@ -283,6 +281,6 @@ cudaError_t launch_op(int mode, const OpParams& prm, const Tables* t, const io_t
   cudaError_t enp::launch_df_p##PP(int mode, const OpParams& prm, const double* u,             \
                                    const double* v, double* out, int batch, cudaStream_t s) { \
     if (prm.dim != 3) return cudaErrorInvalidConfiguration;                                   \
-    return launch_nf<3, PP, df>(mode, prm, nullptr, u, v, out, batch, s);                     \
+    return launch_nf<3, PP, df>(mode, prm, u, v, out, batch, s);                              \
   }                                                                                           \
   cudaError_t enp::upload_tables_df_p##PP(const Tables& t) { return upload_const_tables(PP, t); }

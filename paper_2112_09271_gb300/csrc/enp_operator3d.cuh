@@ -16,17 +16,21 @@
 namespace enp {
 
 constexpr int kTabSz = 128;  // per degree: B (Q*N), Dq (Q*Q), dL (2N), wq (Q), xq (Q), BD (Q*N)
-static __constant__ double c_tabd[kMaxP + 1][kTabSz];
-static __constant__ float c_tabf[kMaxP + 1][kTabSz];
-static __constant__ float2 c_tabdf[kMaxP + 1][kTabSz];   // (hi, lo) double-float pairs
+// One struct per degree, so that a table set is one copy (there is one set per
+// translation unit with hexahedral kernels).
+struct ConstTab {
+  double d[kTabSz];
+  float2 df[kTabSz];   // (hi, lo) double-float pairs
+  float f[kTabSz];
+};
+static __constant__ ConstTab c_tab[kMaxP + 1];
 
 // Upload the tables of degree p to this translation unit's constant banks on
 // the current device.
 static inline cudaError_t upload_const_tables(int p, const Tables& t) {
   const int n = p + 1, q = p + 2;
-  double d[kTabSz] = {0};
-  float f[kTabSz] = {0};
-  float2 w[kTabSz];
+  ConstTab c{};
+  double* d = c.d;
   int o = 0;
   for (int i = 0; i < q * n; ++i) d[o++] = t.B[i];
   for (int i = 0; i < q * q; ++i) d[o++] = t.Dq[i];
@@ -42,21 +46,18 @@ static inline cudaError_t upload_const_tables(int p, const Tables& t) {
       d[o++] = sacc;
     }
   for (int i = 0; i < kTabSz; ++i) {
-    f[i] = (float)d[i];
+    c.f[i] = (float)d[i];
     const df x(d[i]);
-    w[i] = make_float2(x.hi, x.lo);
+    c.df[i] = make_float2(x.hi, x.lo);
   }
-  cudaError_t e = cudaMemcpyToSymbol(c_tabd, d, sizeof(d), sizeof(d) * p);
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_tabf, f, sizeof(f), sizeof(f) * p);
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_tabdf, w, sizeof(w), sizeof(w) * p);
-  return e;
+  return cudaMemcpyToSymbol(c_tab, &c, sizeof(c), sizeof(c) * p);
 }
 
 template <int P, class R>
 __device__ __forceinline__ R ctab(int i) {
-  if constexpr (std::is_same<R, double>::value) return c_tabd[P][i];
-  else if constexpr (std::is_same<R, df>::value) return df(c_tabdf[P][i].x, c_tabdf[P][i].y);
-  else return c_tabf[P][i];
+  if constexpr (std::is_same<R, double>::value) return c_tab[P].d[i];
+  else if constexpr (std::is_same<R, df>::value) return df(c_tab[P].df[i].x, c_tab[P].df[i].y);
+  else return c_tab[P].f[i];
 }
 template <int P> struct TabOff {
   static constexpr int N = P + 1, Q = P + 2;
@@ -89,7 +90,7 @@ __device__ __forceinline__ void pencil_rows(const R* __restrict__ src, int is, R
         int idx;
         if (TAB == 0) idx = T::B + (TRANS ? k * T::N + r : r * T::N + k);
         else idx = T::Dq + (TRANS ? k * T::Q + r : r * T::Q + k);
-        const float2 m = c_tabdf[P][idx];
+        const float2 m = c_tab[P].df[idx];
         const float p = __fmul_rn(m.x, x[k].hi);
         float e = __fmaf_rn(m.x, x[k].hi, -p);
         e = __fmaf_rn(m.x, x[k].lo, e);

@@ -1659,7 +1659,7 @@ cudaError_t ensure(P** p, size_t& have, size_t want_count) {
 // the species rows are the identity.
 template <class TV>
 cudaError_t apply_jv(enp_handle h, const OpParams& P, const TV* ulin, const TV* v, TV* out, int B) {
-  cudaError_t e = enp::launch_op<TV>(enp::kJvp, P, h->d_tab, ulin, v, out, B, h->stream);
+  cudaError_t e = enp::launch_op<TV>(enp::kJvp, P, ulin, v, out, B, h->stream);
   if (e == cudaSuccess && state_of(h).potential_only) {
     const long long EN = (long long)P.E * P.Np;
     enp::species_rows_copy<TV><<<grid_for((P.NF - 1) * EN * B), 256, 0, h->stream>>>(
@@ -1673,7 +1673,7 @@ cudaError_t apply_jv(enp_handle h, const OpParams& P, const TV* ulin, const TV* 
 // rows are c_k - c_k^in.
 cudaError_t apply_residual(enp_handle h, const double* u, double* r, int B) {
   const OpParams& P = h->prm;
-  cudaError_t e = enp::launch_op<double>(enp::kResidual, P, h->d_tab, u, nullptr, r, B, h->stream);
+  cudaError_t e = enp::launch_op<double>(enp::kResidual, P, u, nullptr, r, B, h->stream);
   if (e == cudaSuccess && state_of(h).potential_only) {
     const long long EN = (long long)P.E * P.Np;
     enp::species_rows_offset<<<grid_for((P.NF - 1) * EN * B), 256, 0, h->stream>>>(
@@ -1688,7 +1688,7 @@ cudaError_t apply_residual(enp_handle h, const double* u, double* r, int B) {
 template <class R>
 cudaError_t element_blocks(enp_handle h, const OpParams& P, const R* u, R* blocks) {
   if (P.dim == 3) return enp::launch_assemble<R>(P, u, blocks, h->stream);
-  return enp::launch_op<R>(enp::kBlockCol, P, h->d_tab, u, nullptr, blocks, P.NF * P.Np, h->stream);
+  return enp::launch_op<R>(enp::kBlockCol, P, u, nullptr, blocks, P.NF * P.Np, h->stream);
 }
 
 // Partials of <V_i, w>_b (i < nd) into S.part; *nparts = the partials per dot.
@@ -1816,7 +1816,7 @@ cudaError_t coarse_setup(enp_handle h, const double* u) {
     for (int c = 0; c < 7; ++c) {
       enp::coarse_colour_vector<T><<<dim3(gx, B), 256, 0, h->stream>>>(v, P.ne[0], P.ne[1], P.ne[2],
                                                                         P.Np, P.batch_stride, P.E, c);
-      cudaError_t er = enp::launch_op<T>(enp::kJvp, P, h->d_tab, uu, v, jv, B, h->stream);
+      cudaError_t er = enp::launch_op<T>(enp::kJvp, P, uu, v, jv, B, h->stream);
       if (er != cudaSuccess) return er;
       enp::coarse_gather<T><<<dim3(grid_for(P.E), B), 256, 0, h->stream>>>(
           jv, L0.A, P.ne[0], P.ne[1], P.ne[2], P.Np, P.batch_stride, c);
