@@ -130,7 +130,18 @@ static cudaError_t launch_3d_op(const OpParams& prm, const io_t<R>* u, const io_
     }();
     e = raise_smem_limit(attr, kern, (size_t)max_eb<P, NF, MODE, R>() * per_el);
     if (e != cudaSuccess) return e;
-    kern<<<grid, groups * tile_threads<P, R>(), groups * EG * per_el, stream>>>(prm, u, v, out);
+    // beside the face kernel: its volume stages need nothing of the faces
+    cudaLaunchAttribute early{};
+    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(groups * tile_threads<P, R>());
+    cfg.dynamicSmemBytes = groups * EG * per_el;
+    cfg.stream = stream;
+    cfg.attrs = &early;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, prm, u, v, out);
   } else {
     auto kern = param3d_kernel<P, NF, R>;
     cudaError_t e = raise_smem_limit(attr, kern, (size_t)max_eb<P, NF, MODE, R>() * per_el);

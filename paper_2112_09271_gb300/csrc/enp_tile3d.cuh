@@ -351,10 +351,35 @@ struct ElemGeo {
   __device__ __forceinline__ R weight(R w) const { return w * (area[0] * halfv(h[0])); }
 };
 
+// A load of what the kernel before wrote while this one was already running: an
+// ordinary (coherent) load, and not moved above wait_for_faces.
+__device__ __forceinline__ float load_after_wait(const float* p) {
+  float x;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(x) : "l"(p));
+  return x;
+}
+__device__ __forceinline__ double load_after_wait(const double* p) {
+  double x;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(x) : "l"(p));
+  return x;
+}
+__device__ __forceinline__ df load_after_wait(const df* p) {
+  float hi, lo;
+  asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(hi), "=f"(lo) : "l"(p));
+  return df(hi, lo);
+}
+
+// The element kernel starts as soon as every block of the face kernel has (programmatic
+// launch): its volume stages read u and v only. The face terms are there after this.
+// One after the other, the face kernel's last wave and a launch stood between the two:
+// double-float J v on 24 x 6 x 2 elements, p = 2, eight points 41.0 -> 36.9 us, FP32 on
+// 61 x 15 x 5, p = 4, two points 82.0 -> 77.8 us, on 64 x 32 x 16, p = 3 192.6 -> 188.4 us.
+__device__ __forceinline__ void wait_for_faces() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Adds the six face terms of field f to the row of N nodes r = iy + N iz, in
 // side order, from the face kernel's coefficients.
 template <int P, int NF, int MODE, class R>
-__device__ __forceinline__ void add_face_terms(const OpParams& prm, const R* __restrict__ fb,
+__device__ __forceinline__ void add_face_terms(const OpParams& prm, const R* fb,
                                                const int* idx, const R* sc, int f, int r,
                                                Dot<R> (&acc)[P + 1]) {
   using SL = Slots<P, NF, MODE>;
@@ -372,8 +397,8 @@ __device__ __forceinline__ void add_face_terms(const OpParams& prm, const R* __r
     const R* Tp = F + (!hi && f == 0 ? 2 * NF : NF + f) * FN;
     const bool neg = !hi && !(MODE == kVjp && f > 0);
     if (a == 0) {
-      const R tv = sc[0] * Tp[r];
-      R sv = Sp[r];
+      const R tv = sc[0] * load_after_wait(Tp + r);
+      R sv = load_after_wait(Sp + r);
       if (neg) sv = -sv;
       acc[hi ? N - 1 : 0].add(sv);
 #pragma unroll
@@ -383,11 +408,11 @@ __device__ __forceinline__ void add_face_terms(const OpParams& prm, const R* __r
       const int j = N * (a == 1 ? iz : iy);
       const R cf = ctab<P, R>(TO::dL + hi * N + k) * sc[a];
 #pragma unroll
-      for (int n = 0; n < N; ++n) acc[n].fma(cf, Tp[j + n]);
+      for (int n = 0; n < N; ++n) acc[n].fma(cf, load_after_wait(Tp + j + n));
       if (k == (hi ? N - 1 : 0)) {
 #pragma unroll
         for (int n = 0; n < N; ++n) {
-          const R sv = Sp[j + n];
+          const R sv = load_after_wait(Sp + j + n);
           acc[n].add(neg ? -sv : sv);
         }
       }
@@ -562,6 +587,7 @@ tile3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* 
     line<P, TO::B, true, Q, N, R>(A + f * AQ + iz * (Q * QP) + qx, QP, Bq + g * (N * QP) + qx, QP);
   }
   group_sync<tile_lock<P, R>()>();
+  wait_for_faces();
   // x^T: one row of N nodes per lane; the six face terms; store
   const R* fb = reinterpret_cast<const R*>(prm.fbuf) + (long long)bidx * prm.fbuf_stride;
 #pragma unroll 1
@@ -769,6 +795,7 @@ lane3d_kernel(const OpParams prm, const float* __restrict__ u, const float* __re
                                   A_ + S::kA + (f * N + iz) * (N * QP) + qx, QP);
   });
   group_sync<tile_lock<P, R>()>();
+  wait_for_faces();
   const R* fb = reinterpret_cast<const R*>(prm.fbuf) + (long long)bidx * prm.fbuf_stride;
   // x^T: one row of N nodes per lane; the six face terms; store
   constexpr int KX = T / (FN * EG) < 1 ? 1 : (T / (FN * EG) > NF ? NF : T / (FN * EG));
@@ -1197,6 +1224,7 @@ tileface3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   R* A = reinterpret_cast<R*>(tile_raw) + warp * S::total;
   R* B = A + S::kA;
+  asm volatile("griddepcontrol.launch_dependents;");   // see wait_for_faces
   const long long nf = prm.foff[3];
   const long long g0 = ((long long)blockIdx.x * (blockDim.x >> 5) + warp) * FW;
   if (!face_lock<R>() && g0 >= nf) return;
