@@ -62,9 +62,9 @@ DF32_PEAK_TFLOPS = 152 * 128 * 2.07e9 / 12 * 2 / 1e12
 # of the sources that kernel is built from (stale -> reported null): the
 # operator kernels from the operator headers, the block apply from the solver.
 TRAFFIC = {
-    ("5d4d7cdd78a5", "jvp_df32", "channel64_p3"): 699.86e6,  # face + element kernel
-    ("5d4d7cdd78a5", "jvp_f32", "channel64_p3"): 243.07e6,   # face + element kernel
-    ("33fe528c30dc", "bj_apply_f32", "channel64_p3"): 4933.98e6,
+    ("e4205d55fbb1", "jvp_df32", "channel64_p3"): 538.70e6,  # face + element kernel
+    ("e4205d55fbb1", "jvp_f32", "channel64_p3"): 166.23e6,   # face + element kernel
+    ("90522817d8ea", "bj_apply_f32", "channel64_p3"): 4931.24e6,
 }
 
 KERNEL_SOURCES = {
@@ -737,7 +737,7 @@ def main():
     nb = prob.n_fields * prob.Np
     bj_bytes = prob.E * (nb * nb * 4 + 2 * nb * 8)  # FP32 inverse + FP64 x in, y out
     bj_s = t_ops["bj_apply_f32"] / args.steps * 1e-3
-    roof_hbm = {"bound": "hbm", "kernel": "bj_apply_kernel<float,float,double>",
+    roof_hbm = {"bound": "hbm", "kernel": "bj_apply_rows_kernel<float,float,double,4>",
                 "achieved": bj_bytes / bj_s / 1e9, "peak": hbm, "unit": "GB/s",
                 "frac": bj_bytes / bj_s / 1e9 / hbm, "peak_kind": hbm_kind,
                 "bytes_per_launch": bj_bytes,
