@@ -318,8 +318,9 @@ enp_status enp_dg_create(enp_handle* out, const enp_mesh_desc* mesh, const enp_p
 
   cudaError_t e;
   // The geometry of every axis in one buffer and one copy: (h, 2 / h) of each element
-  // (FP64, double-float, FP32) and the vertices (the same). A buffer and a copy for
-  // each of them took 12 of either, some 130 us of creating a handle.
+  // (FP64, double-float, FP32) and the vertices (the same). With a buffer and a copy
+  // for each of them, and three copies per set of constant tables, creating a handle
+  // took 1.03 ms, 0.15 ms longer than before the element scales.
   {
     std::vector<char> geo;
     size_t at[3][6];
