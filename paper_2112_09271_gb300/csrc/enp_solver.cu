@@ -791,34 +791,38 @@ coarse_vcycle_tail(const VcycleTail T) {
   }
 }
 
-// b0[K] = sum over the Phi nodes of element K of r (P^T r), one lane per element:
-// FP64 vectors summed in FP64, FP32 ones as a double-float pair (TwoSum), which
-// rounds to the same FP32 value and keeps off the FP64 pipe (a warp per element
-// with an FP64 shuffle tree took 77 us on 147,456 elements, 9.6 now).
+// b0[K] = sum over the Phi nodes of element K of r (P^T r), one lane per element,
+// to FP64 accuracy or better. FP64 vectors are summed in FP64. FP32 ones by cascaded
+// TwoSum (Ogita, Rump, Oishi 2005, three terms: 72 bits before the last, FP64
+// additions), off the FP64 pipe: on 147,456 elements, p = 2, an FP64 addition and
+// conversion per entry take 11 us more, a warp per element with an FP64 shuffle
+// tree 77 us in all, 9.1 us here. A sum that leaves FP32's range is formed again in FP64.
 template <class TV>
 __global__ void coarse_from_fine(const TV* __restrict__ r, float* __restrict__ b0, int E, int Np,
                                  long long bstride) {
   const int b = blockIdx.y;
   for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < E; K += gridDim.x * blockDim.x) {
     const TV* row = r + b * bstride + (long long)K * Np;
-    float out;
+    double out = 0.0;
+    bool done = false;
     if constexpr (std::is_same<TV, float>::value) {
-      float s = row[0], t = 0.0f;
-#pragma unroll 4
+      float s = row[0], t = 0.0f, c = 0.0f;
+#pragma unroll 8
       for (int i = 1; i < Np; ++i) {
-        float s2, err;
-        two_sum(s, row[i], s2, err);
-        s = s2;
-        t = __fadd_rn(t, err);
+        float e1, e2;
+        two_sum(s, row[i], s, e1);
+        two_sum(t, e1, t, e2);
+        c = __fadd_rn(c, e2);
       }
-      out = __fadd_rn(s, t);
-    } else {
-      double s = row[0];
-#pragma unroll 4
-      for (int i = 1; i < Np; ++i) s += row[i];
-      out = (float)s;
+      out = (double)s + ((double)t + (double)c);
+      done = isfinite(out);
     }
-    b0[(long long)b * E + K] = out;
+    if (!done) {
+      out = (double)row[0];
+#pragma unroll 4
+      for (int i = 1; i < Np; ++i) out += (double)row[i];
+    }
+    b0[(long long)b * E + K] = (float)out;
   }
 }
 

@@ -320,3 +320,29 @@ def test_vcycle_of_every_level_size(n, smooth):
     ref = _vcycle(A, b, smooth).reshape(-1)
     assert np.linalg.norm(d[0, :, 0] - ref) <= 2e-4 * np.linalg.norm(ref)
     assert np.abs(d[0] - d[0, :, :1]).max() <= 1e-12 * np.abs(with_).max()
+
+
+# one element's potential residuals whose sum needs 53 bits, and whose partial sums
+# pass FP32's range: FP64 forms both exactly, in any order
+@pytest.mark.parametrize("values,total", [
+    ([1.0, 2.0 ** -26, 2.0 ** -52, -1.0, -2.0 ** -26], 2.0 ** -52),
+    ([3e38, 3e38, -3e38, -3e38], 0.0)])
+def test_coarse_right_hand_side_is_summed_in_fp64(values, total):
+    """FP32 vectors: P^T r is summed in FP64, so a residual in one element equals, in
+    every other element (where the block part is zero), bit for bit the coarse
+    correction of a residual that is that sum at one node."""
+    enp = _enp()
+    P = W.config("cube_n5_p2")
+    op = enp.Operator(P)
+    op.set_preconditioner(1)
+    op.set_sweep(0)
+    op.block_jacobi_setup(_cuda(W.random_state(P, 2)), enp.BJ_F32)
+    K = P.E // 2
+    z = []
+    for v in (values, [total]):
+        r = np.zeros((P.n_fields, P.E, P.Np), np.float32)
+        r[0, K, :len(v)] = v
+        z.append(op.block_jacobi_apply_f32(_cuda(r.reshape(-1))).cpu().numpy().reshape(r.shape))
+    others = np.arange(P.E) != K
+    assert (np.abs(z[1][0, others]).max() > 0) == (total != 0)
+    np.testing.assert_array_equal(z[0][:, others], z[1][:, others])
