@@ -23,6 +23,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <initializer_list>
 #include <string>
 #include <vector>
 
@@ -1585,8 +1586,7 @@ struct SolverState {
   cudaGraphExec_t gexec = nullptr;
   void* gbuf = nullptr;           // [3][B][n] of the Krylov type: u_lin, b, x
   size_t gbuf_bytes = 0;
-  const void* gkey[4] = {nullptr, nullptr, nullptr, nullptr};
-  int gkey_i[4] = {0, 0, 0, 0};
+  std::vector<char> gkey;         // capture_key of gexec
   // graph-driven Newton iteration (enp_newton_opts.device_loop): the graph, the
   // streams its nested bodies were captured on, handle-owned copies of the
   // Newton vectors, the device control block, and the key it was captured for
@@ -1600,7 +1600,7 @@ struct SolverState {
   // preconditioner generation: bumped whenever its configuration changes or a
   // buffer it reads is reallocated, so that a captured FGMRES cycle is replayed
   // only with the preconditioner it was captured with
-  unsigned long long pc_gen = 1, gkey_gen = 0;
+  unsigned long long pc_gen = 1;
   // two-level preconditioner: element-mean potential correction
   int sweep_mode = 2;             // downwind block Gauss-Seidel: 0 off, 1 on, 2 automatic
   bool potential_only = false;    // the potential rows alone (enp_initial_guess)
@@ -2567,6 +2567,25 @@ static enp_status fgmres_any(enp_handle h, const TV* ulin, const TV* b, TV* x,
   return ENP_OK;
 }
 
+// What a captured sequence of operator and preconditioner applications and Arnoldi
+// iterations bakes in: the operator parameters, which the kernels receive by value,
+// every buffer and setting of the preconditioner, and the caller's own pointers and
+// sizes. A graph is replayed only under the key it was captured with.
+static std::vector<char> capture_key(enp_handle h, std::initializer_list<double> own) {
+  const SolverState& S = state_of(h);
+  std::vector<double> kv = {
+      (double)(uintptr_t)S.V, (double)(uintptr_t)S.dsmall, (double)(uintptr_t)S.part,
+      (double)(uintptr_t)S.kcount, (double)(uintptr_t)S.binv, (double)S.storage, (double)S.nb,
+      (double)S.pc_gen, (double)S.pc_shared_built, (double)S.potential_only, (double)S.sweep_ready,
+      (double)S.coarse, (double)S.coarse_ready, (double)S.coarse_direct};
+  kv.insert(kv.end(), own);
+  const size_t nkv = sizeof(double) * kv.size();
+  std::vector<char> key(nkv + sizeof(OpParams));
+  std::memcpy(key.data(), kv.data(), nkv);
+  std::memcpy(key.data() + nkv, &h->prm, sizeof(OpParams));
+  return key;
+}
+
 // FGMRES with each restart cycle (r0, m Arnoldi iterations, update) captured
 // once in a CUDA graph and replayed: one launch and one host read per cycle.
 // The inputs are copied into handle-owned buffers so that the graph's pointers
@@ -2649,11 +2668,9 @@ static enp_status fgmres_graph(enp_handle h, const TV* ulin, const TV* b, TV* x,
   auto apply_A = [&](const TV* in, TV* outv) -> cudaError_t {
     return apply_jv<TV>(h, P, ug, in, outv, B);
   };
-  const bool same = S.gexec && S.gkey[0] == (const void*)S.V && S.gkey[1] == S.binv &&
-                    S.gkey[2] == (const void*)S.gbuf && S.gkey[3] == (const void*)S.dsmall &&
-                    S.gkey_i[0] == m && S.gkey_i[1] == S.storage && S.gkey_i[2] == (int)sizeof(TV) &&
-                    S.gkey_i[3] == B && S.gkey_gen == S.pc_gen;
-  if (!same) {
+  const std::vector<char> key = capture_key(
+      h, {(double)(uintptr_t)S.gbuf, (double)m, (double)sizeof(TV)});
+  if (!S.gexec || S.gkey != key) {
     if (S.gexec) { cudaGraphExecDestroy(S.gexec); S.gexec = nullptr; }
     cudaGraph_t graph = nullptr;
     if ((e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeRelaxed)) != cudaSuccess) {
@@ -2681,9 +2698,7 @@ static enp_status fgmres_graph(enp_handle h, const TV* ulin, const TV* b, TV* x,
     if (e == cudaSuccess) e = cudaGraphInstantiate(&S.gexec, graph, 0);
     if (graph) cudaGraphDestroy(graph);
     if (e != cudaSuccess) { S.gexec = nullptr; cudaEventDestroy(ev); return fail_cuda(e, "capture FGMRES cycle"); }
-    S.gkey[0] = S.V; S.gkey[1] = S.binv; S.gkey[2] = S.gbuf; S.gkey[3] = S.dsmall;
-    S.gkey_i[0] = m; S.gkey_i[1] = S.storage; S.gkey_i[2] = (int)sizeof(TV); S.gkey_i[3] = B;
-    S.gkey_gen = S.pc_gen;
+    S.gkey = key;
   }
   std::vector<int> hj(B);
   int hflag[2] = {0, 0};
@@ -2924,17 +2939,10 @@ static enp_status newton_device(enp_handle h, double* u_user, const enp_newton_o
     if ((e = small(h, nsmallk)) != cudaSuccess) return cuda_err(h, e, "cudaMalloc small");
     if ((e = ensure(&S.part, S.part_count, (size_t)B * (m + 1) * enp::kRedBlocks)) != cudaSuccess)
       return cuda_err(h, e, "cudaMalloc partials");
-    // the capture key: every pointer and setting the captured sequence bakes in,
-    // including the operator parameters the kernels receive by value
-    const double kv[] = {
-        (double)(uintptr_t)S.V, (double)(uintptr_t)S.binv, (double)(uintptr_t)S.dsmall,
-        (double)(uintptr_t)S.part, (double)(uintptr_t)S.nbuf, (double)(uintptr_t)S.nsmall,
-        (double)m, (double)S.storage, (double)sizeof(TV), (double)B, (double)S.pc_gen,
-        (double)S.potential_only, o->krylov.rtol, o->krylov.atol, (double)o->krylov.max_it,
-        (double)o->max_it, o->armijo_c, (double)o->max_backtracks, (double)per_setup};
-    std::vector<char> key(sizeof(kv) + sizeof(OpParams));
-    std::memcpy(key.data(), kv, sizeof(kv));
-    std::memcpy(key.data() + sizeof(kv), &P, sizeof(OpParams));
+    const std::vector<char> key = capture_key(
+        h, {(double)(uintptr_t)S.nbuf, (double)(uintptr_t)S.nsmall, (double)m, (double)sizeof(TV),
+            o->krylov.rtol, o->krylov.atol, (double)o->krylov.max_it, (double)o->max_it,
+            o->armijo_c, (double)o->max_backtracks, (double)per_setup});
     if (!S.nexec || S.nkey != key) {
       if (S.nexec) { cudaGraphExecDestroy(S.nexec); S.nexec = nullptr; }
       double* q = S.dsmall;

@@ -157,3 +157,99 @@ def test_continuation_rejects_bad_options():
     with pytest.raises(enp.EnpError) as ei:
         op.newton_continuation(u, [[1.0, 0, 0, 0]], step0=0.5, step_max=0.25)
     assert ei.value.status == enp.ENP_ERR_INVALID_ARG
+
+
+def _graph_case(enp, change):
+    """(problem, prepare(op), alter(op, new)): the state a first graph solve runs in,
+    and what makes it that of the second (new: of a handle without the first)."""
+    if change == "phi_app":
+        P = W.config("reactor_n1_p2")
+        alter = lambda op, new: op.set_phi_app(np.array([[20.0, 0, 0, 0]]))  # noqa: E731
+    elif change == "dirichlet":
+        P = W.config("cube_n2_p3")
+        P = dataclasses.replace(P, tags=[np.full_like(t, W.DIRICHLET) for t in P.tags])
+        alter = lambda op, new: op.set_sources(None, _cuda(W.random_dirichlet(P, 4)))  # noqa: E731
+    elif change == "arithmetic":
+        P = W.config("cube_n3_p2")
+        alter = lambda op, new: op.set_arithmetic(enp.ARITH_DF32)  # noqa: E731
+    else:   # captured between the switch and the setup that makes the sweep ready
+        P = W.config("cube_n3_p2")
+        alter = lambda op, new: op.set_sweep(1) if new else None  # noqa: E731
+
+    def prepare(op):
+        ud = _cuda(W.random_state(P, 2))
+        if change != "sweep":
+            op.block_jacobi_setup(ud, enp.BJ_F64)
+            return
+        op.set_sweep(1)
+        op.block_jacobi_setup(ud, enp.BJ_F64)
+        op.set_sweep(0)
+        op.set_sweep(1)
+    return P, prepare, alter
+
+
+def _graph_solve(op, u, b, restart=10, graph=True, rtol=1e-8, max_it=2000):
+    import torch
+    x = torch.zeros_like(b)
+    st = op.fgmres_solve(u, b, x, restart=restart, max_it=max_it, rtol=rtol, graph=graph,
+                         raise_on_fail=False)
+    return x.cpu().numpy(), st["iterations"], st["converged"]
+
+
+@pytest.mark.parametrize("change", ["phi_app", "dirichlet", "arithmetic", "sweep"])
+def test_graph_cycle_is_captured_again_after(change):
+    """A cycle captured before something it bakes in was changed is not replayed
+    after: the solve equals a fresh handle's bit for bit."""
+    enp = _enp()
+    P, prepare, alter = _graph_case(enp, change)
+    u, b = _cuda(W.random_state(P, 2)), _cuda(W.random_vector(P, 6))
+    op, fresh = enp.Operator(P), enp.Operator(P)
+    prepare(op)
+    _graph_solve(op, u, b)
+    res = []
+    for o in (op, fresh):
+        alter(o, o is fresh)
+        o.block_jacobi_setup(u, enp.BJ_F64)
+        res.append(_graph_solve(o, u, b))
+    assert res[0][1:] == res[1][1:] and res[1][2] == 1
+    np.testing.assert_array_equal(res[0][0], res[1][0])
+
+
+def test_graph_cycle_is_captured_again_when_its_partial_sums_move():
+    """An eager solve that needs more Krylov vectors than any before enlarges the
+    buffer of partial sums that a captured cycle writes."""
+    enp = _enp()
+    P = W.config("cube_n3_p2")
+    u, b = _cuda(W.random_state(P, 2)), _cuda(W.random_vector(P, 6))
+    op, fresh = enp.Operator(P), enp.Operator(P)
+    for o in (op, fresh):
+        o.block_jacobi_setup(u, enp.BJ_F64)
+    _graph_solve(op, u, b, restart=60, graph=False, rtol=0.5)      # all other workspace
+    _graph_solve(op, u, b)
+    _graph_solve(op, u, b, restart=60, graph=False, rtol=1e-10)
+    got, ref = _graph_solve(op, u, b), _graph_solve(fresh, u, b)
+    assert got[1:] == ref[1:] and ref[2] == 1
+    np.testing.assert_array_equal(got[0], ref[0])
+
+
+def test_graph_cycle_is_captured_again_when_the_coarse_solve_changes():
+    """A coarsest matrix singular at the first state (potentials so high that no
+    electrode holds them, no oxidant) is smoothed, one regular at the second is
+    applied as its inverse."""
+    enp = _enp()
+    P = W.config("channel_n1", p=2)
+    assert P.bv_oxidant == P.m - 1 and P.z[0] == -P.z[1]   # c_1 = c_2: no oxidant
+    s = np.ones((P.n_fields, P.E, P.Np))
+    s[0] = 40.0 * P.RT / (P.bv_alpha1 * P.bv_n * P.F)
+    u0, u, b = _cuda(s.reshape(-1)), _cuda(W.random_state(P, 2)), _cuda(W.random_vector(P, 6))
+    op, fresh = enp.Operator(P), enp.Operator(P)
+    res = []
+    for o in (op, fresh):
+        o.set_preconditioner(1)
+        if o is op:
+            o.block_jacobi_setup(u0, enp.BJ_F64)
+            _graph_solve(o, u0, b, max_it=10)
+        o.block_jacobi_setup(u, enp.BJ_F64)
+        res.append(_graph_solve(o, u, b))
+    assert res[0][1:] == res[1][1:] and res[1][2] == 1
+    np.testing.assert_array_equal(res[0][0], res[1][0])
