@@ -121,6 +121,7 @@ static cudaError_t launch_3d_op(const OpParams& prm, const io_t<R>* u, const io_
     const long long nf = prm.foff[3], per_block = (long long)warps * FW;
     const dim3 fgrid((unsigned)((nf + per_block - 1) / per_block), batch);
     fk<<<fgrid, warps * 32, warps * per_warp, stream>>>(prm, u, v);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     constexpr int EG = tile_elems<P, R>();
     const int groups = (eb + EG - 1) / EG;
     const dim3 grid((prm.E + groups * EG - 1) / (groups * EG), batch);
@@ -141,7 +142,7 @@ static cudaError_t launch_3d_op(const OpParams& prm, const io_t<R>* u, const io_
     cfg.stream = stream;
     cfg.attrs = &early;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, prm, u, v, out);
+    return launch_status(cudaLaunchKernelEx(&cfg, kern, prm, u, v, out));
   } else {
     auto kern = param3d_kernel<P, NF, R>;
     cudaError_t e = raise_smem_limit(attr, kern, (size_t)max_eb<P, NF, MODE, R>() * per_el);

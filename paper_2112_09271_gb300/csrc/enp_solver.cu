@@ -2266,15 +2266,15 @@ static cudaError_t bj_launch(enp_handle h, const TV* x, TV* y, bool beside) {
     const int rg = n / v, sets = std::max(1, std::min(256 / rg, 8));
     cfg.blockDim = dim3(rg * sets);
     cfg.dynamicSmemBytes = sizeof(TA) * n * (1 + sets);
-    return cudaLaunchKernelEx(&cfg, enp::bj_apply_rows_kernel<TS, TA, TV, v>, B, x, y, n, P.Np, EN,
-                              P.batch_stride, S.pc_shared_built);
+    return enp::launch_status(cudaLaunchKernelEx(&cfg, enp::bj_apply_rows_kernel<TS, TA, TV, v>, B, x, y,
+                                                 n, P.Np, EN, P.batch_stride, S.pc_shared_built));
   };
   if (n >= 96 && n % W == 0) return rows(std::integral_constant<int, W>());
   if (n >= 96 && n % 2 == 0) return rows(std::integral_constant<int, 2>());
   cfg.blockDim = dim3(std::min(256, ((n + 31) / 32) * 32));
   cfg.dynamicSmemBytes = sizeof(TA) * n;
-  return cudaLaunchKernelEx(&cfg, enp::bj_apply_kernel<TS, TA, TV>, B, x, y, n, P.NF, P.Np, EN,
-                            P.batch_stride, S.pc_shared_built);
+  return enp::launch_status(cudaLaunchKernelEx(&cfg, enp::bj_apply_kernel<TS, TA, TV>, B, x, y, n, P.NF,
+                                               P.Np, EN, P.batch_stride, S.pc_shared_built));
 }
 
 template <class TV>

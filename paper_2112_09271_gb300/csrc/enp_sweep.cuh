@@ -319,8 +319,8 @@ static cudaError_t launch_sweep_typed(const OpParams& prm, const void* binv, con
   cfg.stream = stream;
   cfg.attrs = &early;
   cfg.numAttrs = beside ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kern, prm, static_cast<const TS*>(binv), x, z, upc, a, dir,
-                            shared_blocks);
+  return launch_status(cudaLaunchKernelEx(&cfg, kern, prm, static_cast<const TS*>(binv), x, z, upc, a,
+                                          dir, shared_blocks));
 }
 template <int P, int NF, class TV>
 static cudaError_t launch_sweep_pn(const OpParams& prm, const void* binv, int storage, const TV* x,

@@ -272,3 +272,29 @@ def test_unsupported_and_invalid_inputs_raise():
     with pytest.raises(enp.EnpError) as ei:
         enp.Operator(dataclasses.replace(P, coords=bad))
     assert ei.value.status == enp.ENP_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("kernel", ["fpb3d_set", "eb3d_set"])
+def test_failed_launch_is_reported_once(kernel):
+    """The operator is two launches, of the face kernel and of the element kernel.
+    One that the runtime refuses (a block of more threads than there are) is
+    reported although the other succeeds, and not again by the next call."""
+    import ctypes
+    import torch
+    enp = _enp()
+    P = W.config("cube_n2_p2")
+    op = enp.Operator(P)
+    u = torch.tensor(W.random_state(P, 1), device="cuda")
+    ref = op.residual(u).cpu().numpy()
+    # enp::fpb3d_set<double>, enp::eb3d_set<double>: faces, elements per block
+    shape = getattr(enp.load(), "_ZN3enp%d%sIdEEviiii" % (len(kernel), kernel))
+    shape.argtypes, shape.restype = [ctypes.c_int] * 4, None
+    shape(P.p, P.n_fields, 0, 4096)
+    try:
+        with pytest.raises(enp.EnpError) as ei:
+            op.residual(u)
+        assert ei.value.status == enp.ENP_ERR_CUDA
+        op.recover_cm(u)
+    finally:
+        shape(P.p, P.n_fields, 0, 0)
+    np.testing.assert_array_equal(op.residual(u).cpu().numpy(), ref)
