@@ -41,7 +41,7 @@ elim_invert_kernel(float* blocks, long long stride, long long offset, long long 
   constexpr int NP4 = (n + 3) / 4 * 4;
   static_assert(NR >= n, "rows");
   __shared__ __align__(16) float prow[W > 1 ? 2 : 1][W][NP4];   // per warp: its candidate row
-  __shared__ float cand[W > 1 ? 2 : 1][W];
+  __shared__ unsigned cand[W > 1 ? 2 : 1][W];
   __shared__ int candi[W > 1 ? 2 : 1][W];
   __shared__ int piv[n], stepof[NR];
   __shared__ float wmax[W];
@@ -96,7 +96,7 @@ elim_invert_kernel(float* blocks, long long stride, long long offset, long long 
     const unsigned who = __ballot_sync(0xffffffffu, key == top);
     const int owner = __ffs(who) - 1;
     if (lane == owner) {
-      cand[buf][w] = __uint_as_float(top);
+      cand[buf][w] = top;
       candi[buf][w] = slot;
       float4* o = reinterpret_cast<float4*>(prow[buf][w]);
 #pragma unroll
@@ -110,19 +110,19 @@ elim_invert_kernel(float* blocks, long long stride, long long offset, long long 
         }
     }
     int pw = 0;
-    float best;
+    unsigned btop = top;
     if (W > 1) {
       __syncthreads();
-      best = cand[buf][0];
+      btop = cand[buf][0];
 #pragma unroll
       for (int q = 1; q < W; ++q) {
-        const float c = cand[buf][q];
-        if (!(c <= best)) { best = c; pw = q; }     // a NaN wins and is caught below
+        const unsigned c = cand[buf][q];
+        if (c > btop) { btop = c; pw = q; }         // as bits: a NaN of any warp wins
       }
     } else {
       __syncwarp();
-      best = __uint_as_float(top);
     }
+    const float best = __uint_as_float(btop);
     if (!(best > thr) || !isfinite(best)) { bad = true; break; }   // the same in every thread
     const bool mine = (W == 1 || pw == w) && lane == owner;
     const float4* pr = reinterpret_cast<const float4*>(prow[buf][pw]);

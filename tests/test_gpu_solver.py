@@ -287,3 +287,107 @@ def test_shared_block_inverses(storage):
     assert _rel(sols[1], sols[0]) < 1e-7
     with pytest.raises(enp.EnpError):
         op.set_shared_blocks(B)
+
+
+def _field_pivot(A):
+    """The smallest pivot of A, rounded to FP32, over its largest entry (Gauss-Jordan
+    with the pivot searched in each column)."""
+    A = A.astype(np.float32)
+    top, free, least = np.abs(A).max(), np.ones(len(A), bool), np.inf
+    for k in range(len(A)):
+        r = int(np.where(free, np.abs(A[:, k]), -1).argmax())
+        free[r] = False
+        least = min(least, abs(A[r, k]) / top)
+        f = A[:, k] / A[r, k]
+        f[r] = 0
+        A -= np.outer(f, A[r])
+    return least
+
+
+def _unsafe_state(P, s):
+    """A potential of size s that drives the first species into the middle of three
+    elements through its interior faces, walls on its other sides: of its own block
+    only the diffusive penalty, 1/s of the rest, keeps the constants out of the left
+    kernel. Concentrations of the same size keep the whole block regular."""
+    from numpy.polynomial import legendre as L
+    top = np.zeros(P.p + 1)
+    top[P.p] = 1.0
+    g = (np.concatenate([[-1.0], np.sort(L.legroots(L.legder(top)).real), [1.0]]) + 1) / 2
+    X, Y, Z = [(c[:-1, None] + np.diff(c)[:, None] * g - c[-1] / 2) / c[-1] for c in P.coords]
+    X, Y, Z = X[:, None, None, :], Y[0][None, None, :, None], Z[0][None, :, None, None]
+    u = np.empty((P.n_fields, P.E, P.Np))
+    u[0] = (X * X * (1 + 0.5 * Y + 0.3 * Z) + 0.4 * Y * Y - 0.3 * Z * Z + 0.3 * Y * Z + 0.2 * Y
+            + 0.15 * Z * Y * Y).reshape(P.E, -1)
+    u[1:] = 1 + 0.3 * np.random.RandomState(3).rand(P.n_fields - 1, P.E, P.Np)
+    return s * u.reshape(-1)
+
+
+@pytest.mark.parametrize("storage", [1, 2])
+@pytest.mark.parametrize("fields", [2, 3])
+@pytest.mark.parametrize("p", [2, 3, 4])
+def test_block_without_a_safe_species_pivot_is_inverted_whole(p, fields, storage):
+    """FP32 and BF16 setups eliminate the species; where a species block of any
+    operating point has no safe pivot, all points are inverted whole. Two points, a
+    regular state and one whose middle element has none: both inverses against the
+    oracle's blocks, the entries of every field block off by 8 FP32 roundings of its
+    largest, and by the storage's rounding (BF16)."""
+    import dataclasses
+    enp = _enp()
+    P = W.config("cube_n2_p2" if fields == 2 else "channel_n1", p=p)
+    n = [3, 1, 1]
+    coords = [c[-1] * np.linspace(0, 1, k + 1) for c, k in zip(P.coords, n)]
+    tags = W.box_tags(3, n, coords, W.WALL)
+    tags[0][:] = tags[1][:] = W.DIRICHLET
+    P = dataclasses.replace(P, n_el=n, coords=coords, tags=tags, vel_kind=W.VEL_CONSTANT,
+                            vel_params=[0.0] * 8)
+    us = [W.random_state(P, 2), _unsafe_state(P, 1e9)]
+    x = [W.random_vector(P, 5), W.random_vector(P, 6)]
+    blocks = [oracle.Oracle(P).block_diagonal(u) for u in us]
+    Np = P.Np
+    species = lambda B: [B[k * Np:(k + 1) * Np, k * Np:(k + 1) * Np] for k in range(1, fields)]  # noqa: E731
+    assert min(_field_pivot(A) for B in blocks[0] for A in species(B)) > 1e-4
+    assert _field_pivot(species(blocks[1][1])[0]) < 5e-7
+
+    op = enp.Operator(P, batch=2)
+    op.set_sweep(0)
+    op.block_jacobi_setup(_cuda(np.concatenate(us)), storage)
+    z = op.block_jacobi_apply(_cuda(np.concatenate(x))).cpu().numpy().reshape(2, fields, P.E, Np)
+    assert np.isfinite(z).all()
+    alone = enp.Operator(P)     # eliminated: not the same bits
+    alone.set_sweep(0)
+    alone.block_jacobi_setup(_cuda(us[0]), storage)
+    za = alone.block_jacobi_apply(_cuda(x[0])).cpu().numpy().reshape(fields, P.E, Np)
+    assert (za != z[0]).any()
+    # (the regular point's elements; of the other, whose whole blocks lose digits with
+    # the degree and the fields, the middle one at two fields and p <= 3)
+    for b, e in [(0, 0), (0, 1), (0, 2)] + ([(1, 1)] if fields == 2 and p < 4 else []):
+        B = blocks[b][e]
+        inv, xe = np.linalg.inv(B), x[b].reshape(fields, P.E, Np)[:, e].reshape(-1)
+        ref = inv @ xe
+        big = np.abs(B).reshape(fields, Np, fields, Np).max(axis=(1, 3)).repeat(Np, 0).repeat(Np, 1)
+        bound = 8 * 2.0 ** -24 * np.abs(inv) @ (big @ np.abs(ref))
+        if storage == 2:
+            bound = bound + 2.0 ** -9 * np.abs(inv) @ np.abs(xe)
+        assert np.linalg.norm(bound) < 0.1 * np.linalg.norm(ref)
+        for got in [z[b]] + ([za] if b == 0 else []):
+            assert np.linalg.norm(got[:, e].reshape(-1) - ref) <= np.linalg.norm(bound), (b, e)
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+@pytest.mark.parametrize("storage", [1, 2])
+@pytest.mark.parametrize("p", [1, 2, 3, 4])
+def test_nonfinite_block_is_reported_by_every_inversion(p, storage, value):
+    """FP32 and BF16 setups: rejected by the elimination (p >= 2; one, one and four
+    warps a field block), then by the whole inversion; the next setup is not touched
+    by it."""
+    enp = _enp()
+    P = W.config("cube_n2_p2", p=p)
+    u = W.random_state(P, 2)
+    bad = u.reshape(P.n_fields, P.E, P.Np).copy()
+    bad[0, 3, 5] = value
+    op = enp.Operator(P)
+    with pytest.raises(enp.EnpError) as ei:
+        op.block_jacobi_setup(_cuda(bad.reshape(-1)), storage)
+    assert ei.value.status == enp.ENP_ERR_NONFINITE
+    op.block_jacobi_setup(_cuda(u), storage)
+    assert np.isfinite(op.block_jacobi_apply(_cuda(W.random_vector(P, 5))).cpu().numpy()).all()
