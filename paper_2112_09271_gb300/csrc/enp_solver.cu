@@ -663,7 +663,7 @@ __global__ void coarse_dense(const double* __restrict__ A, int nx, int ny, int n
 // the V-cycle of 192 x 48 x 16 cells took 170 us, 125 in this form (a cluster for
 // that many cells too: 220, eight SMs are too few).
 constexpr int kTailCells = 32768;
-constexpr int kTailCtas = 8;
+constexpr int kTailCtas = 8;        // blocks of a cluster, at most
 constexpr int kTailThreads = 1024;
 constexpr int kSoloCells = 2048;
 constexpr int kSoloFloats = 4 * kSoloCells;   // x and b of the solo levels (each at most half the one above)
@@ -714,14 +714,14 @@ __device__ __forceinline__ void vcycle_up(const LevelDev& L, const LevelDev& C, 
     }
 }
 
-__global__ void __cluster_dims__(kTailCtas, 1, 1) __launch_bounds__(kTailThreads)
+__global__ void __launch_bounds__(kTailThreads)
 coarse_vcycle_tail(const VcycleTail T) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   __shared__ float solo[kSoloFloats];
   asm volatile("griddepcontrol.launch_dependents;");   // see wait_for_launch_before
   const int b = blockIdx.y, rank = (int)cluster.block_rank();
-  const int ct = rank * kTailThreads + threadIdx.x, cn = kTailCtas * kTailThreads;
+  const int ct = rank * kTailThreads + threadIdx.x, cn = (int)gridDim.x * kTailThreads;
   auto csync = [&] { cluster.sync(); };
   int s0 = T.l0;      // first solo level: every level below it fits as well
   while (s0 < T.nl - 1 && T.L[s0].n > kSoloCells) ++s0;
@@ -1623,6 +1623,7 @@ struct SolverState {
   struct Level { int nx, ny, nz, n; double* A; float *A32, *x, *b; };  // A: FP64 stencil
   std::vector<Level> levels;      // level 0: the element grid
   bool coarse_direct = false;     // coarsest level solved by its dense inverse
+  int tail_ctas = 1;              // blocks per point of the V-cycle's tail kernel
   double* cdense = nullptr;       // [B][n][n] coarsest matrix
   float* cinv = nullptr;          // [B][n][n] its inverse, transposed, in FP32
   size_t cdense_count = 0, cinv_count = 0;
@@ -1780,6 +1781,19 @@ namespace {
 
 constexpr int kCoarsestSweeps = 100;
 
+// The launch of the V-cycle's tail, a cluster of ctas blocks per operating point.
+cudaLaunchConfig_t tail_config(enp_handle h, int ctas, cudaLaunchAttribute* cluster) {
+  cluster->id = cudaLaunchAttributeClusterDimension;
+  cluster->val.clusterDim = {(unsigned)ctas, 1, 1};
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(ctas, h->batch);
+  cfg.blockDim = dim3(enp::kTailThreads);
+  cfg.stream = h->stream;
+  cfg.attrs = cluster;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
 cudaError_t coarse_levels(enp_handle h) {
   SolverState& S = state_of(h);
   const OpParams& P = h->prm;
@@ -1796,6 +1810,19 @@ cudaError_t coarse_levels(enp_handle h) {
     if (e != cudaSuccess) return e;
     if (L.n <= enp::kCoarsestCells) break;
     nx = (nx + 1) / 2; ny = (ny + 1) / 2; nz = (nz + 1) / 2;
+  }
+  // blocks per operating point: the most with which the clusters of all points run at
+  // once. Three V-cycles on 16^3 cells, p = 1: 32 points 298 us with eight blocks each,
+  // in turns, 196 with four; 64 points 514 and 300 (with two). One block where all
+  // levels are solo (seven would only wait): 8^3 cells, 64 points 152 and 80 us.
+  S.tail_ctas = enp::kTailCtas;
+  for (int active = 0; S.tail_ctas > 1; S.tail_ctas /= 2) {
+    cudaLaunchAttribute cluster{};
+    const cudaLaunchConfig_t cfg = tail_config(h, S.tail_ctas, &cluster);
+    cudaError_t e;
+    if ((e = cudaOccupancyMaxActiveClusters(&active, enp::coarse_vcycle_tail, &cfg)) != cudaSuccess)
+      return e;
+    if (active >= B) break;
   }
   return cudaSuccess;
 }
@@ -1897,7 +1924,9 @@ void vcycle(enp_handle h, size_t l, BESIDE beside) {
     T.smooth = S.coarse_smooth;
     T.omega = S.coarse_omega;
     T.coarsest_sweeps = kCoarsestSweeps;
-    enp::coarse_vcycle_tail<<<dim3(enp::kTailCtas, B), enp::kTailThreads, 0, h->stream>>>(T);
+    cudaLaunchAttribute cluster{};
+    cudaLaunchConfig_t cfg = tail_config(h, L.n <= enp::kSoloCells ? 1 : S.tail_ctas, &cluster);
+    cudaLaunchKernelEx(&cfg, enp::coarse_vcycle_tail, T);   // (coarse_apply reads the status)
     beside();
     return;
   }
@@ -2577,7 +2606,7 @@ static std::vector<char> capture_key(enp_handle h, std::initializer_list<double>
       (double)(uintptr_t)S.V, (double)(uintptr_t)S.dsmall, (double)(uintptr_t)S.part,
       (double)(uintptr_t)S.kcount, (double)(uintptr_t)S.binv, (double)S.storage, (double)S.nb,
       (double)S.pc_gen, (double)S.pc_shared_built, (double)S.potential_only, (double)S.sweep_ready,
-      (double)S.coarse, (double)S.coarse_ready, (double)S.coarse_direct};
+      (double)S.coarse, (double)S.coarse_ready, (double)S.coarse_direct, (double)S.tail_ctas};
   kv.insert(kv.end(), own);
   const size_t nkv = sizeof(double) * kv.size();
   std::vector<char> key(nkv + sizeof(OpParams));

@@ -346,3 +346,30 @@ def test_coarse_right_hand_side_is_summed_in_fp64(values, total):
     others = np.arange(P.E) != K
     assert (np.abs(z[1][0, others]).max() > 0) == (total != 0)
     np.testing.assert_array_equal(z[0][:, others], z[1][:, others])
+
+
+@pytest.mark.parametrize("batch", [9, 20, 40, 80])
+@pytest.mark.parametrize("n", [(6, 6, 6), (13, 13, 13)])
+def test_vcycle_of_many_points_equals_each_alone(n, batch):
+    """The blocks that share a point's V-cycle are as many as run at once for the whole
+    batch (one to eight), and do not change a bit of any point's correction."""
+    import dataclasses
+    enp = _enp()
+    base = W.config("cube_n2_p2", p=1)
+    coords = [np.linspace(0.0, 1.0, k + 1) for k in n]
+    tags = W.box_tags(3, list(n), coords, W.WALL)
+    tags[0][:], tags[1][:] = W.INLET, W.OUTLET
+    tags[2][:] = W.ELECTRODE0
+    P = dataclasses.replace(base, n_el=list(n), coords=coords, tags=tags)
+    us = [W.random_state(P, 2 + i % 5) for i in range(batch)]
+    rs = [W.random_vector(P, 3 + i % 7) for i in range(batch)]
+
+    def corrections(u, r, b):
+        op = enp.Operator(P, batch=b)
+        op.set_preconditioner(1)
+        op.block_jacobi_setup(_cuda(u), enp.BJ_F32)
+        return op.block_jacobi_apply_f32(_cuda(r).float()).cpu().numpy().reshape(b, -1)
+
+    z = corrections(np.concatenate(us), np.concatenate(rs), batch)
+    for i in (0, 1, batch // 2, batch - 1):
+        np.testing.assert_array_equal(z[i], corrections(us[i], rs[i], 1)[0])
