@@ -14,8 +14,9 @@
 //   3. z_e = Binv_e t, with the inverse stored transposed (BT[c][r]).
 // A chain is bound by latency, so nothing on it waits on memory: the next
 // element's state on the face, its x and its geometry are loaded into registers
-// while this one is worked on; its inverse is started towards L2 a step ahead and
-// read into registers (a column piece per thread) during the face stages. One launch per
+// while this one is worked on; its inverse is started towards L2 a step ahead (where
+// few lines run: the inverses of many would not fit L2) and its first columns are read
+// into registers during the face stages. One launch per
 // element plane took 9.5 us a plane whatever its size (192 x 48 x 16 elements,
 // p = 2: 1.8 ms an application, 0.37 now; the inverses alone are 0.26 ms
 // of HBM).
@@ -26,19 +27,23 @@
 
 namespace enp {
 
-// Rows of a block padded to whole warps, times COLS column pieces per row.
-template <int P, int NF>
+// Rows of a block padded to whole warps, times COLS column pieces per row: a thread
+// each (WIDE), or one after the other by the row's thread, in the same order of sums.
+template <int P, int NF, bool WIDE>
 struct SweepShape {
   static constexpr int N = P + 1, Q = P + 2, QP = Rows<P>::QP, FN = N * N, FQ = Q * Q;
   static constexpr int NX = N % 2 ? N : N + 1;
   static constexpr int nb = NF * N * N * N;
   static constexpr int RP = (nb + 31) / 32 * 32;
   static constexpr int COLS = nb <= 64 ? 1 : (nb <= 128 ? 2 : (nb <= 192 ? 4 : (nb <= 256 ? 3 : 2)));
-  static constexpr int NT = RP * COLS;
-  static constexpr int CC = (nb + COLS - 1) / COLS;        // columns per thread
+  static constexpr int NT = WIDE ? RP * COLS : RP;
+  static constexpr int CC = (nb + COLS - 1) / COLS;        // columns per piece
+  // Blocks per SM the registers are sized for (0: the compiler's choice, which gives 768
+  // threads 40 registers with FP64 vectors, and spills 650 bytes).
+  static constexpr int MINB = WIDE ? (NT > 256 ? 1 : 0) : (RP <= 128 ? 5 : (RP <= 192 ? 4 : (RP <= 256 ? 3 : 2)));
   // Columns of the inverse held in registers (the others stream from L2).
   template <class TS> __host__ __device__ static constexpr int ahead() {
-    constexpr int most = (NT > 256 ? 40 : 64) / (sizeof(TS) == 8 ? 2 : 1);
+    constexpr int most = (!WIDE ? 8 : (NT > 256 ? 40 : 64)) / (sizeof(TS) == 8 ? 2 : 1);
     return CC < most ? CC : most;
   }
   static constexpr int NTR = 2 * (NF + 1) + 2 * NF;        // traces: both states, upstream tangent
@@ -49,25 +54,25 @@ struct SweepShape {
   static constexpr int kB = max2(NTR * N * QP, 2 * NF * Q * QP);
   static_assert((2 + NF) * FN <= NT && FQ <= NT, "one trace item, one face point per thread");
 };
-template <int P, int NF, class TV, class TA>
+template <int P, int NF, bool WIDE, class TV, class TA>
 struct SweepSmem {
-  using S = SweepShape<P, NF>;
+  using S = SweepShape<P, NF, WIDE>;
   static constexpr size_t z_off = (size_t)(S::kA + S::kB) * sizeof(TV);
   static constexpr size_t t_off = (z_off + S::nb * sizeof(TV) + 15) / 16 * 16;
   static constexpr size_t p_off = t_off + (size_t)S::RP * sizeof(TA);
-  static constexpr size_t bytes = p_off + (S::COLS > 1 ? (size_t)S::NT * sizeof(TA) : 0);
+  static constexpr size_t bytes = p_off + (WIDE && S::COLS > 1 ? (size_t)S::NT * sizeof(TA) : 0);
 };
 
 // TS: type of the stored inverses (FP64 accumulated in FP64, FP32 and BF16 in
 // FP32). upc: the linearisation point. dir = +1: flow along +e_a, -1: along -e_a.
-template <int P, int NF, class TV, class TS>
-__global__ void __launch_bounds__(SweepShape<P, NF>::NT)
+template <int P, int NF, bool WIDE, class TV, class TS>
+__global__ void __launch_bounds__(SweepShape<P, NF, WIDE>::NT, SweepShape<P, NF, WIDE>::MINB)
 sweep_line_kernel(const OpParams prm, const TS* __restrict__ binv, const TV* __restrict__ x,
                   TV* __restrict__ z, const TV* __restrict__ upc, int a, int dir,
                   int shared_blocks) {
   using TA = typename std::conditional<sizeof(TS) == 8, double, float>::type;
-  using S = SweepShape<P, NF>;
-  using M = SweepSmem<P, NF, TV, TA>;
+  using S = SweepShape<P, NF, WIDE>;
+  using M = SweepSmem<P, NF, WIDE, TV, TA>;
   using TO = TabOff<P>;
   constexpr int N = S::N, Q = S::Q, QP = S::QP, NX = S::NX, FN = S::FN, FQ = S::FQ, NN = N * FN;
   constexpr int nb = S::nb, NT = S::NT, CC = S::CC, AH = S::template ahead<TS>();
@@ -173,7 +178,7 @@ sweep_line_kernel(const OpParams prm, const TS* __restrict__ binv, const TV* __r
   if (nk > 1) { load_state(1); load_geo(1); }
 #pragma unroll 1
   for (int step = 0; step < nk; ++step) {
-    if (step + 1 < nk) prefetch_inverse(step + 1);
+    if (WIDE && step + 1 < nk) prefetch_inverse(step + 1);
     if (step > 0) {
       // layer values and physical normal derivatives along +e_a
       if (state_item || tid < (2 + NF) * FN) {
@@ -262,30 +267,44 @@ sweep_line_kernel(const OpParams prm, const TS* __restrict__ binv, const TV* __r
     if (step + 1 < nk) load_x(step + 1);
     __syncthreads();
     {
-      TA acc[4] = {TA(0), TA(0), TA(0), TA(0)};
+      // a piece's columns in four sums by turns, the pieces added in order
+      const TS* p = BT + elem(step) * (long long)(nb * nb) + rr;
+      auto piece = [&](int from, int n, auto first) {      // columns [from, from + n)
+        constexpr int A0 = decltype(first)::value ? AH : 0;  // of them held in registers
+        TA acc[4] = {TA(0), TA(0), TA(0), TA(0)};
 #pragma unroll
-      for (int i = 0; i < AH; ++i)
-        if (i < cn) acc[i & 3] += (TA)bv[i] * ts[c0 + i];
-      if constexpr (AH < CC) {
-        const TS* p = BT + elem(step) * (long long)(nb * nb) + (long long)c0 * nb + rr;
-        int i = AH;
-        for (; i + 8 <= cn; i += 8) {
-          TS v[8];
+        for (int i = 0; i < A0; ++i)
+          if (i < n) acc[i & 3] += (TA)bv[i] * ts[from + i];
+        if constexpr (A0 < CC) {
+          const TS* pc = p + (long long)from * nb;
+          constexpr int K = WIDE ? 8 : 16;      // loads in flight
+          int i = A0;
+          for (; i + K <= n; i += K) {
+            TS v[K];
 #pragma unroll
-          for (int q = 0; q < 8; ++q) v[q] = p[(long long)(i + q) * nb];
+            for (int q = 0; q < K; ++q) v[q] = pc[(long long)(i + q) * nb];
 #pragma unroll
-          for (int q = 0; q < 8; ++q) acc[q & 3] += (TA)v[q] * ts[c0 + i + q];
+            for (int q = 0; q < K; ++q) acc[q & 3] += (TA)v[q] * ts[from + i + q];
+          }
+#pragma unroll
+          for (int q = 0; q < K; ++q)
+            if (i + q < n) acc[q & 3] += (TA)pc[(long long)(i + q) * nb] * ts[from + i + q];
         }
-        for (; i < cn; ++i) acc[0] += (TA)p[(long long)i * nb] * ts[c0 + i];
-      }
-      TA s = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-      if constexpr (S::COLS > 1) {
+        return (acc[0] + acc[1]) + (acc[2] + acc[3]);
+      };
+      static_assert(AH == CC || AH % 4 == 0, "a column goes to the same sum wherever it is read from");
+      TA s = piece(c0, cn, std::true_type());
+      if constexpr (WIDE && S::COLS > 1) {
         ps[tid] = s;
         __syncthreads();
         if (tid < nb) {
 #pragma unroll
           for (int q = 1; q < S::COLS; ++q) s += ps[q * S::RP + tid];
         }
+      } else if constexpr (S::COLS > 1) {
+#pragma unroll 1
+        for (int q = 1; q < S::COLS; ++q)
+          s += piece(q * CC, q * CC + CC <= nb ? CC : nb - q * CC, std::false_type());
       }
       if (tid < nb) {
         zs[tid] = (TV)s;
@@ -298,13 +317,13 @@ sweep_line_kernel(const OpParams prm, const TS* __restrict__ binv, const TV* __r
 }
 
 // The sweep over every line of elements along axis a, for every operating point.
-template <int P, int NF, class TV, class TS>
-static cudaError_t launch_sweep_typed(const OpParams& prm, const void* binv, const TV* x, TV* z,
+template <int P, int NF, bool WIDE, class TV, class TS>
+static cudaError_t launch_sweep_shape(const OpParams& prm, const void* binv, const TV* x, TV* z,
                                       const TV* upc, int batch, cudaStream_t stream, int a, int dir,
                                       int shared_blocks, bool beside) {
   using TA = typename std::conditional<sizeof(TS) == 8, double, float>::type;
-  constexpr size_t bytes = SweepSmem<P, NF, TV, TA>::bytes;
-  auto kern = sweep_line_kernel<P, NF, TV, TS>;
+  constexpr size_t bytes = SweepSmem<P, NF, WIDE, TV, TA>::bytes;
+  auto kern = sweep_line_kernel<P, NF, WIDE, TV, TS>;
   static SmemAttr attr;
   cudaError_t e = raise_smem_limit(attr, kern, bytes);
   if (e != cudaSuccess) return e;
@@ -314,13 +333,38 @@ static cudaError_t launch_sweep_typed(const OpParams& prm, const void* binv, con
   early.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)lines, (unsigned)batch);
-  cfg.blockDim = dim3(SweepShape<P, NF>::NT);
+  cfg.blockDim = dim3(SweepShape<P, NF, WIDE>::NT);
   cfg.dynamicSmemBytes = bytes;
   cfg.stream = stream;
   cfg.attrs = &early;
   cfg.numAttrs = beside ? 1 : 0;
   return launch_status(cudaLaunchKernelEx(&cfg, kern, prm, static_cast<const TS*>(binv), x, z, upc, a,
                                           dir, shared_blocks));
+}
+// Blocks of 192 rows and more (p = 3 with three fields, p = 4) take 768 threads wide,
+// one line an SM. That is the faster chain, but more lines than SMs then wait for one
+// another, each SM idle on memory during its line's face stages; with a thread per row two
+// to four lines share an SM. 8 elements a line, p = 4, two fields, FP32 inverses and
+// vectors: 80 lines 83 us wide and 108 so, 150 lines 114 and 115, 192 lines 182 and 147,
+// 2,400 lines 1,570 and 1,153; FP64 vectors, whose face stages keep the FP64 pipe busy
+// from one warp only, p = 3, three fields: 80 lines 134 and 108, 2,400 lines 2,060 and 732.
+// Blocks of 128 rows take 256 threads wide, two lines an SM, and gain with FP64 vectors
+// only: 300 lines 123 and 121, 2,400 lines 935 and 575 (FP32 vectors 220 and 319).
+// Both shapes give the same bits.
+constexpr int kSweepWideLines = 152;      // an SM each
+template <int P, int NF, class TV, class TS>
+static cudaError_t launch_sweep_typed(const OpParams& prm, const void* binv, const TV* x, TV* z,
+                                      const TV* upc, int batch, cudaStream_t stream, int a, int dir,
+                                      int shared_blocks, bool beside) {
+  constexpr int rows = SweepShape<P, NF, true>::nb;
+  if constexpr (rows > 128 || (rows == 128 && std::is_same<TV, double>::value)) {
+    const long long lines = (long long)prm.ne[a == 0 ? 1 : 0] * prm.ne[a == 2 ? 1 : 2] * batch;
+    if (lines > (rows > 128 ? 1 : 2) * kSweepWideLines)
+      return launch_sweep_shape<P, NF, false, TV, TS>(prm, binv, x, z, upc, batch, stream, a, dir,
+                                                      shared_blocks, beside);
+  }
+  return launch_sweep_shape<P, NF, true, TV, TS>(prm, binv, x, z, upc, batch, stream, a, dir,
+                                                 shared_blocks, beside);
 }
 template <int P, int NF, class TV>
 static cudaError_t launch_sweep_pn(const OpParams& prm, const void* binv, int storage, const TV* x,

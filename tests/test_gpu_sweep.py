@@ -303,3 +303,30 @@ def test_sweep_every_block_size(p, fields, direction):
         if storage != enp.BJ_F64:
             z = op.block_jacobi_apply_f32(_cuda(r).float()).cpu().numpy()
             assert np.linalg.norm(z - ref) <= tol * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("p,fields,batch", [(3, 3, 8), (4, 2, 8), (4, 3, 8), (3, 2, 16)])
+def test_sweep_of_many_lines_equals_each_point_alone(p, fields, batch):
+    """Large blocks: a line of elements takes several threads per row where few lines
+    run (20 here), one where many do (20 times the batch); the same bits."""
+    enp = _enp()
+    base = W.config("cube_n2_p2" if fields == 2 else "channel_n1", p=p)
+    n = [3, 4, 5]
+    coords = [c[-1] * np.linspace(0, 1, k + 1) ** 1.2 for c, k in zip(base.coords, n)]
+    tags = W.box_tags(3, n, coords, W.WALL)
+    tags[0][:], tags[1][:] = W.INLET, W.OUTLET
+    tags[2][:] = W.ELECTRODE0
+    P = dataclasses.replace(base, n_el=n, coords=coords, tags=tags)
+    u = np.concatenate([W.random_state(P, 2 + b % 3) for b in range(batch)])
+    r = np.concatenate([W.random_vector(P, 5 + b) for b in range(batch)])
+    one, many = enp.Operator(P), enp.Operator(P, batch=batch)
+    for storage in (enp.BJ_F64, enp.BJ_F32, enp.BJ_BF16):
+        z = []
+        for op, k in ((many, batch), (one, 1)):
+            op.set_sweep(1)
+            op.block_jacobi_setup(_cuda(u[:k * P.n_dof]), storage)
+            x = _cuda(r[:k * P.n_dof])
+            z.append([op.block_jacobi_apply(x).cpu().numpy()[:P.n_dof],
+                      op.block_jacobi_apply_f32(x.float()).cpu().numpy()[:P.n_dof]])
+        np.testing.assert_array_equal(z[0][0], z[1][0])
+        np.testing.assert_array_equal(z[0][1], z[1][1])
