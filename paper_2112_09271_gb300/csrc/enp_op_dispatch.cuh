@@ -94,6 +94,15 @@ static int default_eb() {
   }
 }
 
+// FP64 at p = 1: the stages of one element fill 8 to 27 of a warp's 32 lanes, and the FP64
+// pipe takes as long for a part of a warp. Three elements a warp take a third fewer
+// instructions an element, but a longer chain; below this many elements (of all points)
+// there are too few of those to go round. R, two fields: 24 elements 14 us with one and
+// 20 with three, 1,512 elements 39 and 35, 3,072 71 and 68, 196,608 3,676 and 3,019;
+// three fields: 3,072 elements 82 and 86, 7,680 185 and 191, 14,400 340 and 320. The same bits.
+template <int NF>
+constexpr long long few_elements() { return NF == 2 ? 3072 : 10240; }
+
 // Hexahedra: R, J v, J^T w and dR/dtheta (the blocks: enp_assemble.cuh).
 
 }  // namespace enp
@@ -124,12 +133,18 @@ static cudaError_t launch_3d_op(const OpParams& prm, const io_t<R>* u, const io_
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     constexpr int EG = tile_elems<P, R>();
     const int groups = (eb + EG - 1) / EG;
-    const dim3 grid((prm.E + groups * EG - 1) / (groups * EG), batch);
-    auto kern = [] {
+    // FP64 at p = 1: one element a warp while warps are few
+    constexpr bool kFew = EG > 1 && std::is_same<R, double>::value;
+    const bool few = kFew && (long long)prm.E * batch < few_elements<NF>();
+    const int per_group = few ? 1 : EG;
+    const dim3 grid((prm.E + groups * per_group - 1) / (groups * per_group), batch);
+    auto kern = [&] {
       if constexpr (std::is_same<R, float>::value) return lane3d_kernel<P, NF, MODE>;
-      else return tile3d_kernel<P, NF, MODE, R>;
+      else if constexpr (kFew) return few ? tile3d_kernel<P, NF, MODE, R, 1> : tile3d_kernel<P, NF, MODE, R, EG>;
+      else return tile3d_kernel<P, NF, MODE, R, EG>;
     }();
-    e = raise_smem_limit(attr, kern, (size_t)max_eb<P, NF, MODE, R>() * per_el);
+    static SmemAttr few_attr;
+    e = raise_smem_limit(few ? few_attr : attr, kern, (size_t)max_eb<P, NF, MODE, R>() * per_el);
     if (e != cudaSuccess) return e;
     // beside the face kernel: its volume stages need nothing of the faces
     cudaLaunchAttribute early{};
@@ -138,7 +153,7 @@ static cudaError_t launch_3d_op(const OpParams& prm, const io_t<R>* u, const io_
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(groups * tile_threads<P, R>());
-    cfg.dynamicSmemBytes = groups * EG * per_el;
+    cfg.dynamicSmemBytes = groups * per_group * per_el;
     cfg.stream = stream;
     cfg.attrs = &early;
     cfg.numAttrs = 1;

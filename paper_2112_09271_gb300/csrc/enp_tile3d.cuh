@@ -139,8 +139,9 @@ template <int P, class R> __host__ __device__ constexpr int tile_threads() {
   else if constexpr (std::is_same<R, double>::value) return P == 4 ? 64 : 32;
   else return P >= 3 ? 64 : 32;
 }
-// Elements per group (FP32: lane3d_kernel).
+// Elements per group (FP32: lane3d_kernel; FP64 at p = 1: launch_3d_op).
 template <int P, class R> __host__ __device__ constexpr int tile_elems() {
+  if constexpr (std::is_same<R, double>::value) return P == 1 ? 3 : 1;
   return std::is_same<R, float>::value ? (P == 1 ? 3 : (P == 2 ? 2 : (P == 3 ? 1 : 3))) : 1;
 }
 // Faces per warp: as many as fill its lanes with face points (9, 16, 25, 36).
@@ -424,56 +425,80 @@ __device__ __forceinline__ void add_face_terms(const OpParams& prm, const R* fb,
   }
 }
 
-// The pooled stages from the nodal values of one element to the values and
-// reference gradients at its points: region A [NA] values, [NG] z gradients;
-// region B [NG][2] x and y gradients. Ends with a barrier of the group.
-template <int P, int NF, int MODE, class R>
+// Element (of EG in the group) of item w, n items an element; w becomes its own item.
+template <int EG>
+__device__ __forceinline__ int take_elem(int& w, int n) {
+  if constexpr (EG == 1) return 0;
+  const int el = w / n;
+  w -= el * n;
+  return el;
+}
+
+// The pooled stages from the nodal values of a group's EG elements to the values and
+// reference gradients at their points: per element (regions total apart) region A
+// [NA] values, [NG] z gradients; region B [NG][2] x and y gradients. Element el's nodes
+// follow the first's by min(el, last) elements. Ends with a barrier of the group.
+template <int P, int NF, int MODE, class R, int EG = 1>
 __device__ __forceinline__ void tile_points(const io_t<R>* __restrict__ ue,
-                                            const io_t<R>* __restrict__ ve, long long EN, R* A,
-                                            R* Bq, int tid) {
+                                            const io_t<R>* __restrict__ ve, long long EN, R* A0,
+                                            R* B0, int tid, int last = 0) {
   using S = TileE<P, NF, MODE>;
   using SL = Slots<P, NF, MODE>;
   using TO = TabOff<P>;
-  constexpr int N = S::N, Q = S::Q, QP = S::QP, AQ = S::AQ, FN = N * N, FQ = Q * Q;
+  constexpr int N = S::N, Q = S::Q, QP = S::QP, AQ = S::AQ, FN = N * N, FQ = Q * Q, NN = N * FN;
   constexpr int NA = S::NA, NG = S::NG, T = tile_threads<P, R>();
   // x: nodal lines from global memory
 #pragma unroll 1
-  for (int w = tid; w < NA * FN; w += T) {
+  for (int i = tid; i < EG * NA * FN; i += T) {
+    int w = i;
+    const int el = take_elem<EG>(w, NA * FN);
     const int s = w / FN, r = w - s * FN;
-    const io_t<R>* src = (SL::vec(s) ? ve : ue) + SL::field(s) * EN + r * N;
+    const io_t<R>* src = (SL::vec(s) ? ve : ue) + SL::field(s) * EN + min(el, last) * NN + r * N;
     R x[N];
 #pragma unroll
     for (int k = 0; k < N; ++k) x[k] = R(src[k]);
-    R* dst = A + w * QP;
+    R* dst = A0 + el * S::total + w * QP;
     line_rows<P, TO::B, false, N, Q, R>(x, [&](int q, R val) { dst[q] = val; });
   }
   group_sync<tile_lock<P, R>()>();
 #pragma unroll 1
-  for (int w = tid; w < NA * N * Q; w += T) {
+  for (int i = tid; i < EG * NA * N * Q; i += T) {
+    int w = i;
+    const int el = take_elem<EG>(w, NA * N * Q);
     const int g = w / Q, qx = w - g * Q;
-    line<P, TO::B, false, N, Q, R>(A + g * (N * QP) + qx, QP, Bq + g * (Q * QP) + qx, QP);
+    line<P, TO::B, false, N, Q, R>(A0 + el * S::total + g * (N * QP) + qx, QP,
+                                   B0 + el * S::total + g * (Q * QP) + qx, QP);
   }
   group_sync<tile_lock<P, R>()>();
   // z: values of every array, then the z gradients (BD) of the first NG
 #pragma unroll 1
-  for (int w = tid; w < NA * FQ; w += T) {
+  for (int i = tid; i < EG * NA * FQ; i += T) {
+    int w = i;
+    const int el = take_elem<EG>(w, NA * FQ);
     const int s = w / FQ, r = w - s * FQ, o = (r / Q) * QP + r % Q;
-    line<P, TO::B, false, N, Q, R>(Bq + s * (N * Q * QP) + o, Q * QP, A + s * AQ + o, Q * QP);
+    line<P, TO::B, false, N, Q, R>(B0 + el * S::total + s * (N * Q * QP) + o, Q * QP,
+                                   A0 + el * S::total + s * AQ + o, Q * QP);
   }
 #pragma unroll 1
-  for (int w = tid ^ (T > 32 ? 32 : 0); w < NG * FQ; w += T) {
+  for (int i = tid ^ (T > 32 ? 32 : 0); i < EG * NG * FQ; i += T) {
+    int w = i;
+    const int el = take_elem<EG>(w, NG * FQ);
     const int s = w / FQ, r = w - s * FQ, o = (r / Q) * QP + r % Q;
-    line<P, TO::BD, false, N, Q, R>(Bq + s * (N * Q * QP) + o, Q * QP, A + (NA + s) * AQ + o, Q * QP);
+    line<P, TO::BD, false, N, Q, R>(B0 + el * S::total + s * (N * Q * QP) + o, Q * QP,
+                                    A0 + el * S::total + (NA + s) * AQ + o, Q * QP);
   }
   group_sync<tile_lock<P, R>()>();
   // x and y gradients of the first NG arrays, one pool
 #pragma unroll 1
-  for (int w = tid; w < 2 * NG * FQ; w += T) {
+  for (int i = tid; i < EG * 2 * NG * FQ; i += T) {
+    int w = i;
+    const int el = take_elem<EG>(w, 2 * NG * FQ);
     const int d = w >= NG * FQ, t = w - d * (NG * FQ);
     const int s = t / FQ, r = t - s * FQ;
     const int o = d ? (r / Q) * (Q * QP) + r % Q : r * QP;
     const int is = d ? QP : 1;
-    line<P, TO::Dq, false, Q, Q, R>(A + s * AQ + o, is, Bq + (2 * s + d) * AQ + o, is);
+    line<P, TO::Dq, false, Q, Q, R>(A0 + el * S::total + s * AQ + o, is,
+                                    B0 + el * S::total + (2 * s + d) * AQ + o, is);
   }
   group_sync<tile_lock<P, R>()>();
 }
@@ -482,7 +507,7 @@ __device__ __forceinline__ void tile_points(const io_t<R>* __restrict__ ue,
 // FP64 and double-float, whose pencils cost 100 to 300 issue slots: every stage
 // is one pool, so that the lanes stay full (94 % at p = 3) at the price of one
 // index computation per pencil.
-template <int P, int NF, int MODE, class R>
+template <int P, int NF, int MODE, class R, int EG = 1>
 __global__ void __launch_bounds__(kTileThreads, 5)
 tile3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* __restrict__ v,
               io_t<R>* __restrict__ out) {
@@ -490,31 +515,35 @@ tile3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* 
   using SL = Slots<P, NF, MODE>;
   using TO = TabOff<P>;
   constexpr int N = S::N, Q = S::Q, QP = S::QP, AQ = S::AQ, NN = N * N * N, FN = N * N, FQ = Q * Q;
-  constexpr int NA = S::NA, NG = S::NG, T = tile_threads<P, R>();
+  constexpr int NA = S::NA, T = tile_threads<P, R>();
   extern __shared__ __align__(16) unsigned char tile_raw[];
   const int grp = threadIdx.x / T, tid = threadIdx.x % T;
-  const int eraw = blockIdx.x * (blockDim.x / T) + grp;
+  const int eraw = (blockIdx.x * (blockDim.x / T) + grp) * EG;
   if (!tile_lock<P, R>() && eraw >= prm.E) return;
   const bool valid = eraw < prm.E;
-  const int e = valid ? eraw : prm.E - 1;
-  R* A = reinterpret_cast<R*>(tile_raw) + grp * S::total;
-  R* Bq = A + S::kA;
+  const int e0 = valid ? eraw : prm.E - 1;
+  const int last = EG == 1 ? 0 : min(EG, prm.E - e0) - 1;   // elements beyond the mesh shadow it
+  R* A0 = reinterpret_cast<R*>(tile_raw) + grp * (EG * S::total);
+  R* B0 = A0 + S::kA;
   const int bidx = blockIdx.y;
   const long long boff = (long long)bidx * prm.batch_stride;
   const long long EN = (long long)prm.E * NN;
-  const io_t<R>* ue = u + boff + (long long)e * NN;
-  const io_t<R>* ve = SL::JAC ? v + boff + (long long)e * NN : nullptr;
-  tile_points<P, NF, MODE, R>(ue, ve, EN, A, Bq, tid);
+  const io_t<R>* ue = u + boff + (long long)e0 * NN;
+  const io_t<R>* ve = SL::JAC ? v + boff + (long long)e0 * NN : nullptr;
+  tile_points<P, NF, MODE, R, EG>(ue, ve, EN, A0, B0, tid, last);
 
   // point fluxes: those of field f replace x, y in region B slots 2f, 2f + 1, z
   // in region A slot NA + f; the value coefficient (R with sources, J^T w) in
   // region A slot f
-  const ElemGeo<P, R> G(prm, e);
+  const ElemGeo<P, R> G0(prm, e0);     // of the only element (EG 1)
   const bool has_val = MODE == kVjp || (MODE == kResidual && prm.src != nullptr);
   {
     const PhysT<R>& ph = phys<R>(prm);
 #pragma unroll 1
-    for (int pt = tid; pt < Q * FQ; pt += T) {
+    for (int i = tid; i < EG * Q * FQ; i += T) {
+      int pt = i;
+      const int el = take_elem<EG>(pt, Q * FQ), e = e0 + min(el, last);
+      const ElemGeo<P, R> G = EG == 1 ? G0 : ElemGeo<P, R>(prm, e);
       const int kx = pt % Q, ky = (pt / Q) % Q, kz = pt / FQ;
       const int o = kx + QP * (ky + Q * kz);
       const R w = ctab<P, R>(TO::W + kx) * ctab<P, R>(TO::W + ky) * ctab<P, R>(TO::W + kz);
@@ -525,9 +554,9 @@ tile3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* 
         velocity(ph, xp, uv);
         G.factors(w, uv, s2, adv);
       }
-      R* V = A + o;
-      R* Gz = A + NA * AQ + o;
-      R* Gxy = Bq + o;
+      R* V = A0 + el * S::total + o;
+      R* Gz = V + NA * AQ;
+      R* Gxy = B0 + el * S::total + o;
       auto at = [&](int s, int a) -> R& { return a < 2 ? Gxy[(2 * s + a) * AQ] : Gz[s * AQ]; };
       point_flux<NF, MODE, R>(ph, s2, adv, [&](int s) { return V[s * AQ]; },
                               [&](int s, int a) { return at(s, a); },
@@ -543,12 +572,14 @@ tile3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* 
   group_sync<tile_lock<P, R>()>();
   // transposed x and y derivatives, in place, one pool
 #pragma unroll 1
-  for (int w = tid; w < 2 * NF * FQ; w += T) {
+  for (int i = tid; i < EG * 2 * NF * FQ; i += T) {
+    int w = i;
+    const int el = take_elem<EG>(w, 2 * NF * FQ);
     const int d = w >= NF * FQ, t = w - d * (NF * FQ);
     const int f = t / FQ, r = t - f * FQ;
     const int o = d ? (r / Q) * (Q * QP) + r % Q : r * QP;
     const int is = d ? QP : 1;
-    R* p = Bq + (2 * f + d) * AQ + o;
+    R* p = B0 + el * S::total + (2 * f + d) * AQ + o;
     line<P, TO::Dq, true, Q, Q, R>(p, is, p, is);
   }
   group_sync<tile_lock<P, R>()>();
@@ -556,10 +587,13 @@ tile3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* 
   // the line's own values and z fluxes are read before it writes slot f's first
   // N planes, which no other line reads)
 #pragma unroll 1
-  for (int w = tid; w < NF * FQ; w += T) {
+  for (int i = tid; i < EG * NF * FQ; i += T) {
+    int w = i;
+    const int el = take_elem<EG>(w, NF * FQ);
+    R* A = A0 + el * S::total;
     const int f = w / FQ, r = w - f * FQ, o = (r / Q) * QP + r % Q;
     R x[Q], y[Q];
-    const R* hx = Bq + 2 * f * AQ + o;
+    const R* hx = A + S::kA + 2 * f * AQ + o;
 #pragma unroll
     for (int k = 0; k < Q; ++k) {
       x[k] = hx[k * Q * QP] + hx[AQ + k * Q * QP];
@@ -581,25 +615,31 @@ tile3d_kernel(const OpParams prm, const io_t<R>* __restrict__ u, const io_t<R>* 
   group_sync<tile_lock<P, R>()>();
   // y^T into region B [NF][N z][N y][QP]
 #pragma unroll 1
-  for (int w = tid; w < NF * N * Q; w += T) {
+  for (int i = tid; i < EG * NF * N * Q; i += T) {
+    int w = i;
+    const int el = take_elem<EG>(w, NF * N * Q);
     const int g = w / Q, qx = w - g * Q;         // g = f * N + iz
     const int f = g / N, iz = g - f * N;
-    line<P, TO::B, true, Q, N, R>(A + f * AQ + iz * (Q * QP) + qx, QP, Bq + g * (N * QP) + qx, QP);
+    line<P, TO::B, true, Q, N, R>(A0 + el * S::total + f * AQ + iz * (Q * QP) + qx, QP,
+                                  B0 + el * S::total + g * (N * QP) + qx, QP);
   }
   group_sync<tile_lock<P, R>()>();
   wait_for_faces();
   // x^T: one row of N nodes per lane; the six face terms; store
   const R* fb = reinterpret_cast<const R*>(prm.fbuf) + (long long)bidx * prm.fbuf_stride;
 #pragma unroll 1
-  for (int w = tid; w < NF * FN; w += T) {
+  for (int i = tid; i < EG * NF * FN; i += T) {
+    int w = i;
+    const int el = take_elem<EG>(w, NF * FN), e = e0 + min(el, last);
+    const ElemGeo<P, R> G = EG == 1 ? G0 : ElemGeo<P, R>(prm, e);
     const int f = w / FN, r = w - f * FN;        // r = iy + N * iz
     R x[Q];
     Dot<R> acc[N];
 #pragma unroll
-    for (int k = 0; k < Q; ++k) x[k] = Bq[w * QP + k];
+    for (int k = 0; k < Q; ++k) x[k] = B0[el * S::total + w * QP + k];
     line_dots<P, TO::B, true, Q, N, R>(x, acc);
     add_face_terms<P, NF, MODE, R>(prm, fb, G.idx, G.sc, f, r, acc);
-    if (!valid) continue;
+    if (!valid || el > last) continue;
     io_t<R>* o = out + boff + f * EN + (long long)e * NN + r * N;
 #pragma unroll
     for (int n = 0; n < N; ++n) o[n] = to_io(acc[n].get());

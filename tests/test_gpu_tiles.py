@@ -86,3 +86,35 @@ def test_quads(p, fields, n):
     jv = op.jvp_f32(ud.float(), vd.float()).cpu().numpy()
     u32, v32 = (x.float().double().cpu().numpy() for x in (ud, vd))
     assert _rel(jv, orc.jvp(u32, v32), fields) < 2e-5
+
+
+@pytest.mark.parametrize("fields,n,batch", [(2, (5, 4, 3), 64), (3, (5, 4, 4), 150), (2, (16, 16, 13), 1)])
+def test_three_elements_a_warp_equal_one(fields, n, batch):
+    """FP64 at p = 1: many elements are taken three to a warp (the last ones fewer), few
+    one to a warp. A batch of many against its points alone, bit for bit, and a large
+    mesh against the oracle."""
+    import torch
+    import paper_2112_09271_gb300 as enp
+    enp.build()
+    P = _problem(1, fields, n)
+    src = W.random_sources(P, 5)
+
+    def values(u, v, b):
+        op = enp.Operator(P, batch=b)
+        op.set_sources(torch.tensor(src, device="cuda"), None)
+        u, v = (torch.tensor(x, device="cuda") for x in (u, v))
+        return [f.cpu().numpy().reshape(b, -1) for f in (op.residual(u), op.jvp(u, v), op.vjp(u, v))]
+
+    us = [W.random_state(P, 1 + b % 4) for b in range(batch)]
+    vs = [W.random_vector(P, 2 + b % 5) for b in range(batch)]
+    many = values(np.concatenate(us), np.concatenate(vs), batch)
+    if batch > 1:
+        for b in (0, batch // 2, batch - 1):
+            for x, y in zip(many, values(us[b], vs[b], 1)):
+                np.testing.assert_array_equal(x[b], y[0])
+        return
+    orc = oracle.Oracle(P, src=src)
+    ref = (orc.residual(us[0]), orc.jvp(us[0], vs[0]),
+           orc.vjp_entries(us[0], vs[0], np.arange(P.n_dof)))
+    for x, y in zip(many, ref):
+        assert _rel(x[0], y, fields) < 1e-12
