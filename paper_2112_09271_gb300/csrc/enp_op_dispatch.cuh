@@ -97,11 +97,11 @@ static int default_eb() {
 // FP64 at p = 1: the stages of one element fill 8 to 27 of a warp's 32 lanes, and the FP64
 // pipe takes as long for a part of a warp. Three elements a warp take a third fewer
 // instructions an element, but a longer chain; below this many elements (of all points)
-// there are too few of those to go round. R, two fields: 24 elements 14 us with one and
-// 20 with three, 1,512 elements 39 and 35, 3,072 71 and 68, 196,608 3,676 and 3,019;
-// three fields: 3,072 elements 82 and 86, 7,680 185 and 191, 14,400 340 and 320. The same bits.
-template <int NF>
-constexpr long long few_elements() { return NF == 2 ? 3072 : 10240; }
+// there are too few of those to go round. R (J v), two fields: 24 elements 14 us with one
+// and 20 with three, 5,760 elements 125 and 118 (145 and 147), 14,400 283 and 241 (327 and
+// 297), 196,608 3,676 and 3,019; three fields: 7,680 elements 185 and 191 (225 and 224),
+// 14,400 340 and 320 (414 and 403). The same bits.
+constexpr long long kFewElements = 8192;
 
 // Hexahedra: R, J v, J^T w and dR/dtheta (the blocks: enp_assemble.cuh).
 
@@ -135,7 +135,7 @@ static cudaError_t launch_3d_op(const OpParams& prm, const io_t<R>* u, const io_
     const int groups = (eb + EG - 1) / EG;
     // FP64 at p = 1: one element a warp while warps are few
     constexpr bool kFew = EG > 1 && std::is_same<R, double>::value;
-    const bool few = kFew && (long long)prm.E * batch < few_elements<NF>();
+    const bool few = kFew && (long long)prm.E * batch < kFewElements;
     const int per_group = few ? 1 : EG;
     const dim3 grid((prm.E + groups * per_group - 1) / (groups * per_group), batch);
     auto kern = [&] {

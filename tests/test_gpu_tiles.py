@@ -88,7 +88,7 @@ def test_quads(p, fields, n):
     assert _rel(jv, orc.jvp(u32, v32), fields) < 2e-5
 
 
-@pytest.mark.parametrize("fields,n,batch", [(2, (5, 4, 3), 64), (3, (5, 4, 4), 150), (2, (16, 16, 13), 1)])
+@pytest.mark.parametrize("fields,n,batch", [(2, (5, 4, 4), 150), (3, (5, 4, 4), 150), (2, (49, 13, 13), 1)])
 def test_three_elements_a_warp_equal_one(fields, n, batch):
     """FP64 at p = 1: many elements are taken three to a warp (the last ones fewer), few
     one to a warp. A batch of many against its points alone, bit for bit, and a large
