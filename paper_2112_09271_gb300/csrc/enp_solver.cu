@@ -792,38 +792,50 @@ coarse_vcycle_tail(const VcycleTail T) {
   }
 }
 
-// b0[K] = sum over the Phi nodes of element K of r (P^T r), one lane per element,
-// to FP64 accuracy or better. FP64 vectors are summed in FP64. FP32 ones by cascaded
-// TwoSum (Ogita, Rump, Oishi 2005, three terms: 72 bits before the last, FP64
-// additions), off the FP64 pipe: on 147,456 elements, p = 2, an FP64 addition and
-// conversion per entry take 11 us more, a warp per element with an FP64 shuffle
-// tree 77 us in all, 9.1 us here. A sum that leaves FP32's range is formed again in FP64.
-template <class TV>
+// b0[K] = sum over the Phi nodes of element K of r (P^T r), L lanes per element, to FP64
+// accuracy. FP64 vectors are summed in FP64. A lane's FP32 entries by cascaded TwoSum
+// (Ogita, Rump, Oishi 2005, three terms: 72 bits before the FP64 additions), off the
+// FP64 pipe: on 147,456 elements, p = 2, an FP64 addition and conversion per entry take
+// 11 us more, a warp per element with an FP64 shuffle tree 77 us in all, 9.1 us here.
+// Sums that leave FP32's range are formed again in FP64.
+// Four lanes an element from 64 nodes on, where the chain of one lane is long and its
+// loads lie far from the next lane's: an application of the two-level preconditioner on
+// 12 x 10 x 9 elements, p = 4, 62 and 49 us (FP64 vectors), 56 and 47 us (FP32); at p = 2
+// no difference.
+template <class TV, int L>
 __global__ void coarse_from_fine(const TV* __restrict__ r, float* __restrict__ b0, int E, int Np,
                                  long long bstride) {
-  const int b = blockIdx.y;
-  for (int K = blockIdx.x * blockDim.x + threadIdx.x; K < E; K += gridDim.x * blockDim.x) {
-    const TV* row = r + b * bstride + (long long)K * Np;
+  const int b = blockIdx.y, per = blockDim.x / L, sub = threadIdx.x % L;
+  auto over_lanes = [](double v) {
+#pragma unroll
+    for (int k = 1; k < L; k *= 2) v += __shfl_xor_sync(0xffffffffu, v, k);
+    return v;
+  };
+  for (int K0 = blockIdx.x * per; K0 < E; K0 += gridDim.x * per) {
+    const int K = K0 + threadIdx.x / L;
+    const TV* row = r + b * bstride + (long long)min(K, E - 1) * Np;
     double out = 0.0;
-    bool done = false;
+    bool again = true;
     if constexpr (std::is_same<TV, float>::value) {
-      float s = row[0], t = 0.0f, c = 0.0f;
+      float s = row[sub], t = 0.0f, c = 0.0f;
 #pragma unroll 8
-      for (int i = 1; i < Np; ++i) {
+      for (int i = sub + L; i < Np; i += L) {
         float e1, e2;
         two_sum(s, row[i], s, e1);
         two_sum(t, e1, t, e2);
         c = __fadd_rn(c, e2);
       }
-      out = (double)s + ((double)t + (double)c);
-      done = isfinite(out);
+      out = over_lanes((double)s + ((double)t + (double)c));
+      again = __any_sync(0xffffffffu, !isfinite(out));
     }
-    if (!done) {
-      out = (double)row[0];
-#pragma unroll 4
-      for (int i = 1; i < Np; ++i) out += (double)row[i];
+    if (again) {
+      double s = (double)row[sub];
+#pragma unroll 8
+      for (int i = sub + L; i < Np; i += L) s += (double)row[i];
+      s = over_lanes(s);
+      if (std::is_same<TV, double>::value || !isfinite(out)) out = s;
     }
-    b0[(long long)b * E + K] = (float)out;
+    if (K < E && sub == 0) b0[(long long)b * E + K] = (float)out;
   }
 }
 
@@ -1956,8 +1968,10 @@ cudaError_t coarse_apply(enp_handle h, const TV* r, TV* z, BESIDE beside) {
   const OpParams& P = h->prm;
   const int B = h->batch;
   auto& L0 = S.levels[0];
-  enp::coarse_from_fine<TV><<<dim3(grid_for(P.E, 128), B), 128, 0, h->stream>>>(r, L0.b, P.E, P.Np,
-                                                                             P.batch_stride);
+  const int lanes = P.Np >= 64 ? 4 : 1;
+  const dim3 gr(grid_for((long long)P.E * lanes, 128), B);
+  if (lanes == 4) enp::coarse_from_fine<TV, 4><<<gr, 128, 0, h->stream>>>(r, L0.b, P.E, P.Np, P.batch_stride);
+  else enp::coarse_from_fine<TV, 1><<<gr, 128, 0, h->stream>>>(r, L0.b, P.E, P.Np, P.batch_stride);
   vcycle(h, 0, beside);
   if (S.coarse_cycles > 1) {
     // further cycles on the level-0 residual: x += V(b - A0 x); the buffers

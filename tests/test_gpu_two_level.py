@@ -327,12 +327,13 @@ def test_vcycle_of_every_level_size(n, smooth):
 @pytest.mark.parametrize("values,total", [
     ([1.0, 2.0 ** -26, 2.0 ** -52, -1.0, -2.0 ** -26], 2.0 ** -52),
     ([3e38, 3e38, -3e38, -3e38], 0.0)])
-def test_coarse_right_hand_side_is_summed_in_fp64(values, total):
+@pytest.mark.parametrize("cfg", ["cube_n5_p2", "cube_n5_p3"])   # one lane an element, four
+def test_coarse_right_hand_side_is_summed_in_fp64(cfg, values, total):
     """FP32 vectors: P^T r is summed in FP64, so a residual in one element equals, in
     every other element (where the block part is zero), bit for bit the coarse
     correction of a residual that is that sum at one node."""
     enp = _enp()
-    P = W.config("cube_n5_p2")
+    P = W.config(cfg)
     op = enp.Operator(P)
     op.set_preconditioner(1)
     op.set_sweep(0)
@@ -341,7 +342,7 @@ def test_coarse_right_hand_side_is_summed_in_fp64(values, total):
     z = []
     for v in (values, [total]):
         r = np.zeros((P.n_fields, P.E, P.Np), np.float32)
-        r[0, K, :len(v)] = v
+        r[0, K, :4 * len(v):4] = v     # of one lane
         z.append(op.block_jacobi_apply_f32(_cuda(r.reshape(-1))).cpu().numpy().reshape(r.shape))
     others = np.arange(P.E) != K
     assert (np.abs(z[1][0, others]).max() > 0) == (total != 0)
