@@ -330,3 +330,51 @@ def test_sweep_of_many_lines_equals_each_point_alone(p, fields, batch):
                       op.block_jacobi_apply_f32(x.float()).cpu().numpy()[:P.n_dof]])
         np.testing.assert_array_equal(z[0][0], z[1][0])
         np.testing.assert_array_equal(z[0][1], z[1][1])
+
+
+@pytest.mark.parametrize("direction", [1, -1])
+@pytest.mark.parametrize("fields", [2, 3])
+@pytest.mark.parametrize("p", [1, 2, 3, 4])
+def test_sweep_with_bf16_inverses(p, fields, direction):
+    """The lines of test_sweep_every_block_size, BF16 storage, element by element: every
+    z is the stored inverse applied to x minus the oracle's upstream coupling times the
+    z before (the sweep's own), the inverse off by BF16's half unit and the FP32
+    inversion's rounding, sums by FP32's."""
+    enp = _enp()
+    base = W.config("cube_n2_p2" if fields == 2 else "channel_n1", p=p)
+    n = [3, 1, 2]
+    coords = [c[-1] * np.linspace(0, 1, k + 1) ** 1.2 for c, k in zip(base.coords, n)]
+    tags = W.box_tags(3, n, coords, W.WALL)
+    tags[0][:], tags[1][:] = (W.INLET, W.OUTLET) if direction > 0 else (W.OUTLET, W.INLET)
+    tags[2][:] = W.ELECTRODE0
+    vp = list(base.vel_params)
+    vp[4] *= direction
+    P = dataclasses.replace(base, n_el=n, coords=coords, tags=tags, vel_params=vp)
+    u, r = W.random_state(P, 2), W.random_vector(P, 5)
+    orc = oracle.Oracle(P)
+    low = _lower_block_system(orc, P, u, 0, direction)
+    index = np.arange(P.n_dof).reshape(P.n_fields, P.E, P.Np)
+    blocks = orc.block_diagonal(u)
+    op = enp.Operator(P)
+    op.set_sweep(1)
+    op.block_jacobi_setup(_cuda(u), enp.BJ_BF16)
+    for f32 in (False, True):
+        x = _cuda(r).float() if f32 else _cuda(r)
+        z = (op.block_jacobi_apply_f32 if f32 else op.block_jacobi_apply)(x).double().cpu().numpy()
+        for e in range(P.E):
+            rows = index[:, e].reshape(-1)
+            up = e - direction
+            has = 0 <= up < P.E and e // 3 == up // 3
+            c = index[:, up].reshape(-1) if has else rows[:0]
+            L = low[rows][:, c].toarray()
+            t = r[rows] - L @ z[c]
+            inv = np.linalg.inv(blocks[e])
+            # BF16 half unit 2^-9 of every entry; the inverse and t to a few FP32 units
+            # of the terms they are formed from
+            small = 64 * 2.0 ** -24
+            dinv = 2.0 ** -9 * np.abs(inv) + small * np.abs(inv) @ np.abs(blocks[e]) @ np.abs(inv)
+            dt = small * (np.abs(r[rows]) + np.abs(L) @ np.abs(z[c]))
+            tol = np.linalg.norm(dinv @ np.abs(t) + np.abs(inv) @ dt)
+            ref = inv @ t
+            assert tol < 0.1 * np.linalg.norm(ref), (e, tol / np.linalg.norm(ref))
+            assert np.linalg.norm(z[rows] - ref) <= tol, e

@@ -374,3 +374,25 @@ def test_vcycle_of_many_points_equals_each_alone(n, batch):
     z = corrections(np.concatenate(us), np.concatenate(rs), batch)
     for i in (0, 1, batch // 2, batch - 1):
         np.testing.assert_array_equal(z[i], corrections(us[i], rs[i], 1)[0])
+
+
+def test_two_level_fgmres_with_grid_wide_smoothing():
+    """35,937 cells: the finest level's smoothing runs in launches over the whole grid,
+    the levels below in one. FGMRES reaches the tolerance on the oracle's residual, in a
+    number of iterations that block-Jacobi alone does not do with."""
+    import torch
+    enp = _enp()
+    P = W.config("cube_n33_p1")
+    assert P.E > 32768
+    orc = oracle.Oracle(P)
+    u, b = W.random_state(P, 2), W.random_vector(P, 6)
+    op = enp.Operator(P)
+    x, st = _solve(op, u, b, True)
+    assert st["converged"] == 1
+    assert np.linalg.norm(orc.jvp(u, x) - b) <= 1.01e-10 * np.linalg.norm(b)
+    op.set_preconditioner(0)
+    op.block_jacobi_setup(_cuda(u), enp.BJ_F64)
+    y = torch.zeros(b.size, dtype=torch.float64, device="cuda")
+    st = op.fgmres_solve(_cuda(u), _cuda(b), y, restart=60, max_it=st["iterations"], rtol=1e-10,
+                         raise_on_fail=False)
+    assert st["status"] == enp.ENP_ERR_NOT_CONVERGED
