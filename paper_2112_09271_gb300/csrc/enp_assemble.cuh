@@ -24,6 +24,7 @@
 // the products of the 1D tables in constant memory at compile-time indices.
 // Bound by instruction issue, then by the store of the blocks.
 #pragma once
+#include "enp_launch.cuh"
 #include "enp_tile3d.cuh"
 
 namespace enp {

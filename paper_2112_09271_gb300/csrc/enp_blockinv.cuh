@@ -42,7 +42,6 @@ elim_invert_kernel(float* blocks, long long stride, long long offset, long long 
   static_assert(NR >= n, "rows");
   __shared__ __align__(16) float prow[W > 1 ? 2 : 1][W][NP4];   // per warp: its candidate row
   __shared__ unsigned cand[W > 1 ? 2 : 1][W];
-  __shared__ int candi[W > 1 ? 2 : 1][W];
   __shared__ int piv[n], stepof[NR];
   __shared__ float wmax[W];
   extern __shared__ __align__(16) float stage[];   // [n][LD]
@@ -97,7 +96,6 @@ elim_invert_kernel(float* blocks, long long stride, long long offset, long long 
     const int owner = __ffs(who) - 1;
     if (lane == owner) {
       cand[buf][w] = top;
-      candi[buf][w] = slot;
       float4* o = reinterpret_cast<float4*>(prow[buf][w]);
 #pragma unroll
       for (int r = 0; r < RPL; ++r)

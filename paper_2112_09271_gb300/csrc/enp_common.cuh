@@ -160,14 +160,6 @@ template <class R> __device__ __forceinline__ R valof(Tan<R> x) { return x.v; }
 __device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a, b, c); }
 
-// The status of a cudaLaunchKernelEx, and of the launches before it that were not
-// asked for theirs. A failed launch also stays the thread's last error, and the next
-// call to read that would report it as its own: it is taken here.
-static inline cudaError_t launch_status(cudaError_t e) {
-  const cudaError_t last = cudaGetLastError();
-  return e != cudaSuccess ? e : last;
-}
-
 // A kernel launched beside the one before it in the stream (programmatic launch; the
 // earlier kernel lets it start with griddepcontrol.launch_dependents) shares no
 // data with it, and its last block ends only when the earlier kernel has, so that

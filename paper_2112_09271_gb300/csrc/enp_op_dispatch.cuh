@@ -2,38 +2,14 @@
 // For kBlockCol (quads), `batch` is the number of block columns (NF * Np): grid.y
 // runs over the columns.
 #pragma once
-#include <mutex>
-
 #include "enp_internal.h"
+#include "enp_launch.cuh"
 #include "enp_operator.cuh"
 #include "enp_operator3d.cuh"
+#include "enp_quad2d.cuh"
 #include "enp_tile3d.cuh"
 
 namespace enp {
-
-// The dynamic shared-memory limit of a kernel is a per-device attribute: each
-// launch site keeps, per device, whether it has raised the limit (thread-safe).
-struct SmemAttr {
-  std::mutex mu;
-  bool done[64] = {};
-};
-template <class K>
-static cudaError_t raise_smem_limit(SmemAttr& st, K kern, size_t bytes) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64)
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  std::lock_guard<std::mutex> g(st.mu);
-  if (st.done[dev]) return cudaSuccess;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  // shared memory, not L1, bounds the resident blocks of these kernels
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
-  if (e == cudaSuccess) st.done[dev] = true;
-  return e;
-}
 
 // Elements per block of the hexahedral kernel, per (p, fields, mode) and
 // arithmetic type; 0 = the default. One table per
@@ -56,7 +32,7 @@ template <int P, int NF, int MODE, class R>
 static constexpr size_t elem_bytes() {
   if constexpr (MODE <= kVjp && std::is_same<R, float>::value) return (size_t)TileL<P, NF, MODE>::total * sizeof(R);
   else if constexpr (MODE <= kVjp) return (size_t)TileE<P, NF, MODE>::total * sizeof(R);
-  else return (size_t)Smem3<P, NF, tpe3d<P, R>()>::total * sizeof(R);
+  else return (size_t)Smem3<P, NF, tpe3d<P>()>::total * sizeof(R);
 }
 template <int P, int NF, int MODE, class R>
 static constexpr size_t face_bytes() {
@@ -77,7 +53,7 @@ static int max_eb() {
   if constexpr (MODE <= kVjp) {
     return kTileThreads / tile_threads<P, R>() * tile_elems<P, R>();
   } else {
-    int eb = kMaxThreads3D / tpe3d<P, R>();
+    int eb = kMaxThreads3D / tpe3d<P>();
     while (eb > 1 && (size_t)eb * elem_bytes<P, NF, MODE, R>() > 200 * 1024) --eb;
     return eb < 1 ? 1 : eb;
   }
@@ -89,7 +65,7 @@ static int default_eb() {
   } else {  // shared memory near 96 KB
     int eb = (int)((96 * 1024) / elem_bytes<P, NF, MODE, R>());
     eb = eb < 1 ? 1 : eb;
-    while (eb > 1 && eb * tpe3d<P, R>() > kMaxThreads3D) --eb;
+    while (eb > 1 && eb * tpe3d<P>() > kMaxThreads3D) --eb;
     return eb;
   }
 }
@@ -104,11 +80,6 @@ static int default_eb() {
 constexpr long long kFewElements = 8192;
 
 // Hexahedra: R, J v, J^T w and dR/dtheta (the blocks: enp_assemble.cuh).
-
-}  // namespace enp
-#include "enp_quad2d.cuh"
-namespace enp {
-
 template <int P, int NF, int MODE, class R>
 static cudaError_t launch_3d_op(const OpParams& prm, const io_t<R>* u, const io_t<R>* v,
                                 io_t<R>* out, int batch, cudaStream_t stream) {
@@ -163,7 +134,7 @@ static cudaError_t launch_3d_op(const OpParams& prm, const io_t<R>* u, const io_
     cudaError_t e = raise_smem_limit(attr, kern, (size_t)max_eb<P, NF, MODE, R>() * per_el);
     if (e != cudaSuccess) return e;
     const dim3 grid((prm.E + eb - 1) / eb, batch);
-    kern<<<grid, eb * tpe3d<P, R>(), eb * per_el, stream>>>(prm, u, out);
+    kern<<<grid, eb * tpe3d<P>(), eb * per_el, stream>>>(prm, u, out);
   }
   return cudaGetLastError();
 }
@@ -224,7 +195,7 @@ int eb3d_step(int p) {
 template <class R>
 int eb3d_max(int p, int nf, int mode) {
 #define ENP_EBM(PP, NFF, MM) \
-  if (p == PP && nf == NFF && mode == MM && (MM != kParam || !std::is_same<R, df>::value)) return max_eb<PP, NFF, MM, R>();
+  if (p == PP && nf == NFF && mode == MM && (MM != kParam || std::is_same<R, double>::value)) return max_eb<PP, NFF, MM, R>();
 #define ENP_EBM_P(PP) ENP_EBM(PP, 2, 0) ENP_EBM(PP, 2, 1) ENP_EBM(PP, 2, 2) ENP_EBM(PP, 2, 4) \
   ENP_EBM(PP, 3, 0) ENP_EBM(PP, 3, 1) ENP_EBM(PP, 3, 2) ENP_EBM(PP, 3, 4)
   ENP_EBM_P(1) ENP_EBM_P(2) ENP_EBM_P(3) ENP_EBM_P(4)

@@ -7,7 +7,7 @@
 //    FMA operands, no loads);
 //  * each stage runs over all fields and vectors of the element at once, so a
 //    stage costs one __syncthreads;
-//  * the pointwise physics (volume and faces) is the one op_kernel uses.
+//  * the pointwise physics (volume and faces) is that of enp_operator.cuh.
 #pragma once
 #include <type_traits>
 
@@ -79,44 +79,15 @@ __device__ __forceinline__ void pencil_rows(const R* __restrict__ src, int is, R
   for (int k = 0; k < COLS; ++k) x[k] = src[k * is];
 #pragma unroll
   for (int r = 0; r < ROWS; ++r) {
-    if constexpr (std::is_same<R, df>::value) {
-      // double-float dot product: the leading parts summed with TwoSum, the
-      // product errors, cross terms and sum errors gathered in one binary32
-      // term, one renormalisation per output
-      float s = 0.f, t = 0.f;
-      if (ACC) { s = dst[r * os].hi; t = dst[r * os].lo; }
+    R acc = ACC ? dst[r * os] : R(0);
 #pragma unroll
-      for (int k = 0; k < COLS; ++k) {
-        int idx;
-        if (TAB == 0) idx = T::B + (TRANS ? k * T::N + r : r * T::N + k);
-        else idx = T::Dq + (TRANS ? k * T::Q + r : r * T::Q + k);
-        const float2 m = c_tab[P].df[idx];
-        const float p = __fmul_rn(m.x, x[k].hi);
-        float e = __fmaf_rn(m.x, x[k].hi, -p);
-        e = __fmaf_rn(m.x, x[k].lo, e);
-        e = __fmaf_rn(m.y, x[k].hi, e);
-        if (!ACC && k == 0) {
-          s = p;
-          t = e;
-        } else {
-          float s2, err;
-          two_sum(s, p, s2, err);
-          s = s2;
-          t = __fadd_rn(t, __fadd_rn(err, e));
-        }
-      }
-      dst[r * os] = fast_two_sum(s, t);
-    } else {
-      R acc = ACC ? dst[r * os] : R(0);
-#pragma unroll
-      for (int k = 0; k < COLS; ++k) {
-        int idx;
-        if (TAB == 0) idx = T::B + (TRANS ? k * T::N + r : r * T::N + k);
-        else idx = T::Dq + (TRANS ? k * T::Q + r : r * T::Q + k);
-        acc = mad(ctab<P, R>(idx), x[k], acc);
-      }
-      dst[r * os] = acc;
+    for (int k = 0; k < COLS; ++k) {
+      int idx;
+      if (TAB == 0) idx = T::B + (TRANS ? k * T::N + r : r * T::N + k);
+      else idx = T::Dq + (TRANS ? k * T::Q + r : r * T::Q + k);
+      acc = mad(ctab<P, R>(idx), x[k], acc);
     }
+    dst[r * os] = acc;
   }
 }
 
@@ -232,14 +203,9 @@ __device__ PhysT<Tan<R>> seed_phys(const PhysT<R>& p, int m, int j) {
   return q;
 }
 
-// Threads per element of the hexahedral kernel: Q x Q (one per pencil) for
-// FP64, whose issue rate the FP64 pipe bounds; more for FP32, which is
-// latency-bound and needs more warps in flight for the same shared memory.
-template <int P, class R>
-__host__ __device__ constexpr int tpe3d() {
-  if constexpr (std::is_same<R, double>::value) return (P + 2) * (P + 2);
-  else return P <= 1 ? 32 : (P == 2 ? 64 : 128);   // FP32 and double-float: the FP32 pipe
-}
+// Threads per element of param3d_kernel: Q x Q, one per pencil (the FP64 pipe bounds it).
+template <int P>
+__host__ __device__ constexpr int tpe3d() { return (P + 2) * (P + 2); }
 
 template <int P, int NF, int NT>
 struct Smem3 {
@@ -280,11 +246,11 @@ constexpr int kMaxThreads3D = 256;
 template <int P, int NF, class R>
 __global__ void __launch_bounds__(kMaxThreads3D)
 param3d_kernel(const OpParams prm, const R* __restrict__ u, R* __restrict__ out) {
-  using S = Smem3<P, NF, tpe3d<P, R>()>;
+  using S = Smem3<P, NF, tpe3d<P>()>;
   using TO = TabOff<P>;
   constexpr int N = S::N, Q = S::Q, NN = S::NN, NQ = S::NQ, FN = S::FN, FQ = S::FQ;
   constexpr int NX = S::NX, NNP = S::NNP, FNP = S::FNP;
-  constexpr int NA = S::NA, NT = tpe3d<P, R>(), PF = S::kPrefetch;
+  constexpr int NA = S::NA, NT = tpe3d<P>(), PF = S::kPrefetch;
   const PhysT<R>& ph = phys<R>(prm);
   extern __shared__ __align__(16) unsigned char smem3_raw[];
   const int es = threadIdx.x / NT, tid = threadIdx.x % NT;

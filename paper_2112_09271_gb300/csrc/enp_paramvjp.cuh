@@ -14,6 +14,7 @@
 // keep their sums in registers; a fixed grid and order make results reproducible
 // and independent of the batch.
 #pragma once
+#include "enp_launch.cuh"
 #include "enp_reduce.cuh"
 #include "enp_tile3d.cuh"
 

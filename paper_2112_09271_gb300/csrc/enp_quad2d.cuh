@@ -7,6 +7,7 @@
 // problems have (8 x 8 elements, p = 2, residual and J v: 82 us with one array and
 // face after the other, 35 pooled in one warp, 27 so), by the FP64 pipe on large ones.
 #pragma once
+#include "enp_launch.cuh"
 #include "enp_tile3d.cuh"
 
 namespace enp {

@@ -29,6 +29,7 @@
 
 #include "../../include/enp_dg.h"
 #include "enp_internal.h"
+#include "enp_launch.cuh"
 #include "enp_reduce.cuh"
 
 namespace enp {
@@ -2162,25 +2163,25 @@ enp_status enp_block_jacobi_setup(enp_handle h, const double* u, int storage) {
   bool elim = !f64 && enp::elimination_available(P.dim, P.p);
   int flag = 0;
   while (true) {
-  for (int set = 0; set < nsets; ++set) {
-    const int b = shared ? S.pc_shared : set;
-    OpParams Pb = P;
-    if (P.phiapp_batch) Pb.phiapp_batch = P.phiapp_batch + 4 * b;
-    // assemble operating point b's blocks
-    if (f64) {
-      e = element_blocks<double>(h, Pb, u + b * P.batch_stride, S.blocks);
-      if (e != cudaSuccess) return cuda_err(h, e, "element blocks");
-      if (S.potential_only)
-        enp::block_species_identity<double><<<grid_for((long long)(nb - P.Np) * nb * nblk), 256, 0,
-                                              h->stream>>>(S.blocks, nblk, nb, P.Np);
-    } else {
-      e = element_blocks<float>(h, Pb, S.u32 + b * P.batch_stride, S.blocks32);
-      if (e != cudaSuccess) return cuda_err(h, e, "FP32 element blocks");
-      if (S.potential_only)
-        enp::block_species_identity<float><<<grid_for((long long)(nb - P.Np) * nb * nblk), 256, 0,
-                                             h->stream>>>(S.blocks32, nblk, nb, P.Np);
-    }
-    void* out = (char*)S.binv + esz * nn * nblk * set;
+    for (int set = 0; set < nsets; ++set) {
+      const int b = shared ? S.pc_shared : set;
+      OpParams Pb = P;
+      if (P.phiapp_batch) Pb.phiapp_batch = P.phiapp_batch + 4 * b;
+      // assemble operating point b's blocks
+      if (f64) {
+        e = element_blocks<double>(h, Pb, u + b * P.batch_stride, S.blocks);
+        if (e != cudaSuccess) return cuda_err(h, e, "element blocks");
+        if (S.potential_only)
+          enp::block_species_identity<double><<<grid_for((long long)(nb - P.Np) * nb * nblk), 256, 0,
+                                                h->stream>>>(S.blocks, nblk, nb, P.Np);
+      } else {
+        e = element_blocks<float>(h, Pb, S.u32 + b * P.batch_stride, S.blocks32);
+        if (e != cudaSuccess) return cuda_err(h, e, "FP32 element blocks");
+        if (S.potential_only)
+          enp::block_species_identity<float><<<grid_for((long long)(nb - P.Np) * nb * nblk), 256, 0,
+                                               h->stream>>>(S.blocks32, nblk, nb, P.Np);
+      }
+      void* out = (char*)S.binv + esz * nn * nblk * set;
 #define ENP_GJ(T, TS, SM, TB, SRC)                                                              \
   {                                                                                             \
     auto k = enp::gj_invert<T, TS, SM, TB>;                                                     \
@@ -2191,7 +2192,7 @@ enp_status enp_block_jacobi_setup(enp_handle h, const double* u, int storage) {
       e = cudaGetLastError();                                                                   \
     }                                                                                           \
   }
-  // FP32 inversion of blocks up to 192 x 192: the register-resident kernel
+    // FP32 inversion of blocks up to 192 x 192: the register-resident kernel
 #define ENP_GJR(TS, NW, RPW, CPL)                                                                 \
   {                                                                                               \
     auto k = enp::gj_invert_regs<float, TS, NW, RPW, CPL>;                                        \
@@ -2202,7 +2203,7 @@ enp_status enp_block_jacobi_setup(enp_handle h, const double* u, int storage) {
       e = cudaGetLastError();                                                                     \
     }                                                                                             \
   }
-// FP32 inversion of blocks up to 256 x 256: a two-CTA cluster per block
+  // FP32 inversion of blocks up to 256 x 256: a two-CTA cluster per block
 #define ENP_GJC(TS)                                                                               \
   {                                                                                               \
     auto k = enp::gj_invert_cluster<TS>;                                                          \
@@ -2219,37 +2220,37 @@ enp_status enp_block_jacobi_setup(enp_handle h, const double* u, int storage) {
   else if (nb <= 96) ENP_GJR(TS, 8, 12, 3)                       \
   else if (nb <= 128) ENP_GJR(TS, 16, 8, 4)                      \
   else ENP_GJR(TS, 16, 12, 6)
-    const bool regs = !f64 && nb <= 192;
-    const bool clus = !f64 && !regs && nb <= enp::kGjcCols;
-    if (elim) {
-      e = enp::launch_elimination(S.blocks32, out, storage, P.p, P.NF, nblk, S.d_flag, h->stream);
-    } else if (regs) {
-      if (storage == 1) ENP_GJR_ANY(float)
-      else ENP_GJR_ANY(__nv_bfloat16)
-    } else if (clus) {
-      const size_t sm = sizeof(float) * (size_t)((nb + 1) / 2) * nb;
-      if (storage == 1) ENP_GJC(float) else ENP_GJC(__nv_bfloat16)
-    } else if (storage == 0) {
-      if (in_smem) ENP_GJ(double, double, true, double, S.blocks) else ENP_GJ(double, double, false, double, S.blocks)
-    } else if (storage == 1) {
-      if (in_smem) ENP_GJ(float, float, true, float, S.blocks32) else ENP_GJ(float, float, false, float, S.blocks32)
-    } else {
-      if (in_smem) ENP_GJ(float, __nv_bfloat16, true, float, S.blocks32)
-      else ENP_GJ(float, __nv_bfloat16, false, float, S.blocks32)
-    }
+      const bool regs = !f64 && nb <= 192;
+      const bool clus = !f64 && !regs && nb <= enp::kGjcCols;
+      if (elim) {
+        e = enp::launch_elimination(S.blocks32, out, storage, P.p, P.NF, nblk, S.d_flag, h->stream);
+      } else if (regs) {
+        if (storage == 1) ENP_GJR_ANY(float)
+        else ENP_GJR_ANY(__nv_bfloat16)
+      } else if (clus) {
+        const size_t sm = sizeof(float) * (size_t)((nb + 1) / 2) * nb;
+        if (storage == 1) ENP_GJC(float) else ENP_GJC(__nv_bfloat16)
+      } else if (storage == 0) {
+        if (in_smem) ENP_GJ(double, double, true, double, S.blocks) else ENP_GJ(double, double, false, double, S.blocks)
+      } else if (storage == 1) {
+        if (in_smem) ENP_GJ(float, float, true, float, S.blocks32) else ENP_GJ(float, float, false, float, S.blocks32)
+      } else {
+        if (in_smem) ENP_GJ(float, __nv_bfloat16, true, float, S.blocks32)
+        else ENP_GJ(float, __nv_bfloat16, false, float, S.blocks32)
+      }
 #undef ENP_GJ
 #undef ENP_GJC
 #undef ENP_GJR_ANY
 #undef ENP_GJR
-    if (e != cudaSuccess) break;
-  }
-  if (e != cudaSuccess) return cuda_err(h, e, "block inversion");
-  e = cudaMemcpyAsync(&flag, S.d_flag, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return cuda_err(h, e, "block inversion sync");
-  if (!flag || !elim) break;
-  elim = false;
-  cudaMemsetAsync(S.d_flag, 0, sizeof(int), h->stream);
+      if (e != cudaSuccess) break;
+    }
+    if (e != cudaSuccess) return cuda_err(h, e, "block inversion");
+    e = cudaMemcpyAsync(&flag, S.d_flag, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (e != cudaSuccess) return cuda_err(h, e, "block inversion sync");
+    if (!flag || !elim) break;
+    elim = false;
+    cudaMemsetAsync(S.d_flag, 0, sizeof(int), h->stream);
   }
   if (flag) {
     h->err = "singular or non-finite element block";

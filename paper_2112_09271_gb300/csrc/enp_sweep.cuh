@@ -23,6 +23,7 @@
 #pragma once
 #include <cuda_bf16.h>
 
+#include "enp_launch.cuh"
 #include "enp_tile3d.cuh"
 
 namespace enp {

@@ -31,7 +31,7 @@ namespace enp {
 
 // ------------------------------------------------------------ accumulators
 // Sum of products: fused multiply-adds, or in double-float the leading parts by
-// TwoSum with every error term gathered in one binary32 (as pencil_rows), one
+// TwoSum with every error term gathered in one binary32, one
 // renormalisation at the end.
 template <class R>
 struct Dot {
@@ -1152,7 +1152,7 @@ __device__ __forceinline__ void face_point(const OpParams& prm, const FaceAt& F,
   using TO = TabOff<P>;
   constexpr int Q = P + 2;
   const PhysT<R>& ph = phys<R>(prm);
-  const int a = F.a, b0 = a == 0 ? 1 : 0, b1 = a == 2 ? 1 : 2;
+  const int a = F.a, b0 = a == 0 ? 1 : 0;
   const int k1 = pt % Q, k2 = pt / Q;
   const R h0 = G.h0, h1 = G.h1, xa = G.xa, hL = G.hL, hU = G.hU;
   const R hh = h0 * h0 + h1 * h1;
