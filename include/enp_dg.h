@@ -107,8 +107,8 @@ typedef struct {
 /* Create an operator handle. Uploads the mesh, tags and basis tables, using
  * stream (a cudaStream_t, may be 0) for every later call. Synchronises once.
  * On hexahedral meshes the handle also owns the face buffer through which the
- * face kernel hands each face's terms to the element kernel: faces x 4 x m x
- * (p+1)^2 x batch doubles (about 3 E of the faces; 154 MB per operating point
+ * face kernel hands each face's terms to the element kernel: faces x 3 x m x
+ * (p+1)^2 x batch doubles (about 3 E of the faces; 117 MB per operating point
  * for 64x32x16 elements at p = 3, m = 3). Calls on one handle share it and the
  * solver workspace, so they must not overlap on the GPU (use one handle per
  * concurrent stream). Errors: INVALID_ARG (bad descriptor), UNSUPPORTED (p, q,
@@ -144,10 +144,10 @@ enp_status enp_set_phi_app(enp_handle h, const double* phi_app);
 enp_status enp_quadrature_points(enp_handle h, double* xq, double* xbq);
 
 /* Arithmetic of the FP64 operator on hexahedral meshes: enp_residual,
- * enp_jvp, enp_vjp, enp_block_diagonal (and the FP64 block-Jacobi setup), and
- * the FP64 residual and J v inside the Newton and FGMRES solvers; vectors stay
- * FP64 in and out either way. dR/dtheta and the sweep's face terms always use
- * the FP64 kernels.
+ * enp_jvp, enp_vjp, and the FP64 residual and J v inside the Newton and FGMRES
+ * solvers and the FP64 coarse operator; vectors stay FP64 in and out either way.
+ * The element blocks (enp_block_diagonal, the FP64 block-Jacobi setup), dR/dtheta
+ * and the sweep's face terms on FP64 vectors are always formed in FP64.
  *   ENP_ARITH_F64  (default): native FP64 arithmetic. GB300 issues 2 FP64
  *                  fused multiply-adds per clock per SM, so this path is bound
  *                  by the FP64 pipe.
@@ -198,11 +198,15 @@ enp_status enp_inner_product(enp_handle h, const double* x, const double* y, dou
  * nb = m * Np, row/column index f * Np + i. */
 enp_status enp_block_diagonal(enp_handle h, const double* u, double* blocks);
 
-/* Assemble and invert the element-diagonal blocks of J(u) (Gauss-Jordan with
- * partial pivoting) and keep the inverses in handle-owned memory, stored as
- * 0 = FP64, 1 = FP32, 2 = BF16. Storage 0 assembles and inverts in FP64; 1 and 2
- * assemble (with the FP32 operator) and invert in FP32: the preconditioner of
- * a flexible Krylov method need not be exact. Synchronises.
+/* Assemble and invert the element-diagonal blocks of J(u) and keep the inverses
+ * in handle-owned memory, stored as 0 = FP64, 1 = FP32, 2 = BF16. Storage 0
+ * assembles and inverts in FP64; 1 and 2 assemble and invert in FP32: the
+ * preconditioner of a flexible Krylov method need not be exact. Whole blocks are
+ * inverted by Gauss-Jordan with partial pivoting; in FP32 on hexahedra, p >= 2,
+ * the species are eliminated first (the blocks of one species among themselves
+ * and with the potential are the only ones that are not zero) and the pivots
+ * searched within a field's block, unless one of any element is below 1e-5 of
+ * its block's largest entry: all are then inverted whole. Synchronises.
  * Errors: NONFINITE if a block is singular or not finite. */
 enp_status enp_block_jacobi_setup(enp_handle h, const double* u, int storage);
 
@@ -240,7 +244,7 @@ enp_status enp_set_shared_blocks(enp_handle h, int point);
  * multigrid V-cycle on it (2 x 2 x 2 Galerkin aggregation, red-black
  * Gauss-Seidel, 2 + 2 sweeps per level, prolongation over-corrected by 1.8; the coarsest grid, of at most 128
  * cells, solved with its dense inverse, or by 100 sweeps if it is singular to
- * working accuracy; the levels of at most 8192 cells run in one launch). A0 is
+ * working accuracy; the levels of at most 32768 cells run in one launch). A0 is
  * assembled with the FP64 operator when the block inverses are stored in FP64,
  * else with the FP32 one; the V-cycle runs in FP32 (it only preconditions). The Schur-complement-like stiffness of the potential
  * equation (Sec. 3.3) is what block-Jacobi alone cannot reduce.
@@ -266,16 +270,18 @@ enp_status enp_set_coarse_options(enp_handle h, int cycles, int smooth, double o
  * z = (D + L)^-1 r, D the element-diagonal blocks of the last setup and L the
  * coupling of every element to its upstream neighbour along the flow axis (the
  * plate-flow axis in the sign of its mean speed, or the largest component of a
- * constant velocity, in its direction). The element planes across that axis
- * are solved in flow order, one launch per plane: each element evaluates the
- * face term of J(u) z between it and its upstream neighbour (the face kernel's
- * arithmetic, at the u of the last setup, z of the plane solved before) and
- * applies its block inverse. With upwind advection dominating, this carries
+ * constant velocity, in its direction). The lines of elements along that axis
+ * are independent of one another and solved in one launch, each element after
+ * its upstream neighbour: it evaluates the face term of J(u) z between the two
+ * (the face kernel's arithmetic, at the u of the last setup, z of the neighbour)
+ * and applies its block inverse. With upwind advection dominating, this carries
  * information along the whole channel in one application, where block-Jacobi
  * moves it one element per Krylov iteration (Pe = 1e4 in the plate reactor of
- * Sec. 5.2); it costs about 9 us per plane, so it pays on long channels (on the
- * plate reactor: 1.5x faster linear solves at 192 elements along the flow,
- * slower at 96 and below, hence the automatic threshold). Combines with the
+ * Sec. 5.2). An iteration takes longer than with block-Jacobi (plate reactor,
+ * p = 2: by 2 % at 192 elements along the flow, by 28 to 37 % at 24 to 96). The
+ * automatic threshold dates from a sweep in one launch per plane, some five
+ * times slower, which made linear solves 1.5x faster at 192 elements along the
+ * flow and slower at 96 and below. Combines with the
  * two-level correction (added after the sweep). Takes effect at the next
  * enp_block_jacobi_setup, which then also keeps a copy of u.
  * Errors: INVALID_ARG, UNSUPPORTED (on = 1 on a 2D mesh). */

@@ -382,7 +382,7 @@ enp_status enp_dg_create(enp_handle* out, const enp_mesh_desc* mesh, const enp_p
       off += (long long)(P.ne[a] + 1) * P.ne[b0] * P.ne[b1];
     }
     P.foff[3] = off;
-    P.fbuf_stride = off * 2 * 2 * P.NF * (long long)P.n * P.n;
+    P.fbuf_stride = off * 3 * P.NF * (long long)P.n * P.n;   // J^T w; R, J v: 2 NF + 1 slots
     e = cudaMalloc(&h->d_fbuf, sizeof(double) * P.fbuf_stride * P.batch);
     if (e != cudaSuccess) { enp_status s = cuda_fail(h, e, "cudaMalloc face buffer"); enp_dg_destroy(h); return s; }
     P.fbuf = h->d_fbuf;

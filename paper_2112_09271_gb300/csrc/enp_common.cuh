@@ -27,8 +27,8 @@ enum OpMode : int { kResidual = 0, kJvp = 1, kVjp = 2, kBlockCol = 3, kParam = 4
 
 enum FaceTag : int { kInterior = 0, kWall = 1, kInlet = 2, kOutlet = 3, kDirichlet = 4, kElectrode0 = 5 };
 
-// Arithmetic of the FP64-accurate operator (R, J v, J^T w, block columns,
-// dR/dtheta on hexahedra): native FP64, or double-float on the FP32 pipe.
+// Arithmetic of the FP64-accurate operator (R, J v and J^T w on hexahedra; the element
+// blocks and dR/dtheta stay FP64): native FP64, or double-float on the FP32 pipe.
 enum Arith : int { kArithF64 = 0, kArithDF = 1 };
 
 // Physical coefficients in the arithmetic type T of a kernel, converted once on

@@ -2,9 +2,13 @@
 //
 //  * block setup: the element-diagonal blocks of J(u) (volume terms plus this
 //    element's own-side face terms, all fields coupled; enp_assemble.cuh), then
-//    batched Gauss-Jordan inversion with partial pivoting; the inverse is stored transposed in FP64, FP32 or BF16.
+//    their inverses: in FP32 on hexahedra by elimination of the species
+//    (enp_blockinv.cuh), else, or where a species block has no safe pivot, of the
+//    whole blocks by batched Gauss-Jordan with partial pivoting; stored transposed
+//    in FP64, FP32 or BF16.
 //  * block apply: y_e = B_e^{-1} x_e, one thread block per element, threads over
-//    rows, reading the stored inverse once (an HBM-bound batched GEMV).
+//    rows, or over groups of rows and sets of columns (96 rows and more), reading
+//    the stored inverse once (an HBM-bound batched GEMV).
 //  * FGMRES(m) with right preconditioning (flexible: the preconditioner may
 //    change between iterations), classical Gram-Schmidt applied twice, dot
 //    products reduced on the device in a fixed order (warp shuffles, then one
@@ -667,7 +671,9 @@ constexpr int kTailCells = 32768;
 constexpr int kTailCtas = 8;        // blocks of a cluster, at most
 constexpr int kTailThreads = 1024;
 constexpr int kSoloCells = 2048;
-constexpr int kSoloFloats = 4 * kSoloCells;   // x and b of the solo levels (each at most half the one above)
+// x and b of the solo levels: a level has half the cells of the one above, rounded up, or
+// fewer, so at most 2,048 + 1,024 + 512 + 256 + 128 = 3,968 of 4,096 cells.
+constexpr int kSoloFloats = 4 * kSoloCells;
 constexpr int kMaxLevels = 32;      // 2^30 cells in a row have 24
 
 struct LevelDev {
@@ -2023,8 +2029,10 @@ void enp_solver_free(enp_handle h) {
 }
 
 // Elements along the flow axis from which the automatic mode uses the sweep:
-// on the plate reactor (Pe = 1e4) block-Jacobi is faster at 96 elements along
-// the flow and the sweep 1.5x faster at 192 (one FP32 linear solve).
+// on the plate reactor (Pe = 1e4) block-Jacobi was faster at 96 elements along
+// the flow and the sweep 1.5x faster at 192 (one FP32 linear solve), with a sweep
+// in one launch per plane; in one launch for all an FGMRES iteration takes 1.41 ms
+// against 1.38 (block-Jacobi) at 192 elements, 0.332 against 0.259 at 96 (p = 2).
 constexpr int kSweepAutoElements = 128;
 
 // Whether the next setup builds the sweep, and along which axis and direction:

@@ -155,6 +155,7 @@ struct Slots {
   static constexpr int NG = JAC ? NF + 1 : NA;                 // of them with gradients (listed first)
   // face coefficient arrays (none for <w, dR/dtheta>, kParam, which sums at the points)
   static constexpr int NSL = MODE == kParam ? 0 : (MODE == kVjp ? 3 * NF : 2 * NF + 1);
+  static_assert(NSL <= 3 * NF, "the face buffer holds 3 NF arrays a face");
   // array s: vector (0 u, 1 v) and field
   __device__ static __forceinline__ int vec(int s) {
     return MODE == kParam ? s >= NF : (JAC && s >= 1 && s <= NF ? 1 : 0);
