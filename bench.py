@@ -62,13 +62,14 @@ DF32_PEAK_TFLOPS = 152 * 128 * 2.07e9 / 12 * 2 / 1e12
 # of the sources that kernel is built from (stale -> reported null): the
 # operator kernels from the operator headers, the block apply from the solver.
 TRAFFIC = {
-    ("e4205d55fbb1", "jvp_df32", "channel64_p3"): 538.70e6,  # face + element kernel
-    ("e4205d55fbb1", "jvp_f32", "channel64_p3"): 166.23e6,   # face + element kernel
-    ("90522817d8ea", "bj_apply_f32", "channel64_p3"): 4931.24e6,
+    ("8e8b4a309428", "jvp_df32", "channel64_p3"): 539.25e6,  # face + element kernel
+    ("8e8b4a309428", "jvp_f32", "channel64_p3"): 169.34e6,   # face + element kernel
+    ("fdf15a387b2f", "bj_apply_f32", "channel64_p3"): 4933.35e6,
 }
 
 KERNEL_SOURCES = {
-    "operator": ("enp_operator.cuh", "enp_tile3d.cuh", "enp_common.cuh"),
+    "operator": ("enp_operator.cuh", "enp_operator3d.cuh", "enp_tile3d.cuh", "enp_common.cuh",
+                 "enp_df.cuh", "enp_launch.cuh", "enp_op_dispatch.cuh"),
 }
 
 

@@ -666,7 +666,9 @@ __global__ void coarse_dense(const double* __restrict__ A, int nx, int ny, int n
 // barrier. A step of the level reads its stencils (32 bytes a cell) from L2 and
 // costs a launch or a barrier: with one launch per half-sweep above 8192 cells
 // the V-cycle of 192 x 48 x 16 cells took 170 us, 125 in this form (a cluster for
-// that many cells too: 220, eight SMs are too few).
+// that many cells too: 220, eight SMs are too few). Where the line lies, one point, p = 1,
+// an application with its blocks, launches and cluster: 13,824 cells 72 and 64 us, 20,384
+// 78 and 78, 31,744 80 and 86, 38,880 83 and 97.
 constexpr int kTailCells = 32768;
 constexpr int kTailCtas = 8;        // blocks of a cluster, at most
 constexpr int kTailThreads = 1024;
@@ -2311,7 +2313,9 @@ static cudaError_t bj_launch(enp_handle h, const TV* x, TV* y, bool beside) {
   cfg.attrs = &early;
   cfg.numAttrs = beside ? 1 : 0;
   constexpr int W = 16 / sizeof(TS);     // rows of a 16-byte load
-  // blocks of 96 rows and more, whose columns fill several warps' wide loads;
+  // blocks of 96 rows and more, whose columns fill several warps' wide loads (19,200
+  // blocks of 54 rows, FP32: 57 us with a row per thread, 68 with two and column sets;
+  // 4,096 of 128 60 and 47, of 192 122 and 98);
   // the inverses' base is cudaMalloc's, so n alone decides the alignment
   auto rows = [&](auto V) {
     constexpr int v = decltype(V)::value;
