@@ -1821,6 +1821,14 @@ cudaError_t coarse_levels(enp_handle h) {
   if (!S.levels.empty()) return cudaSuccess;
   int nx = P.ne[0], ny = P.ne[1], nz = P.ne[2];
   const int B = h->batch;
+  // a hierarchy is whole or absent: the next setup starts over
+  auto drop = [&](cudaError_t er) {
+    for (auto& L : S.levels) {
+      cudaFree(L.A); cudaFree(L.A32); cudaFree(L.x); cudaFree(L.b);
+    }
+    S.levels.clear();
+    return er;
+  };
   while (true) {
     SolverState::Level L{nx, ny, nz, nx * ny * nz, nullptr, nullptr, nullptr, nullptr};
     cudaError_t e = cudaMalloc(&L.A, sizeof(double) * 7 * (size_t)L.n * B);
@@ -1828,7 +1836,7 @@ cudaError_t coarse_levels(enp_handle h) {
     if (e == cudaSuccess) e = cudaMalloc(&L.x, sizeof(float) * (size_t)L.n * B);
     if (e == cudaSuccess) e = cudaMalloc(&L.b, sizeof(float) * (size_t)L.n * B);
     S.levels.push_back(L);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) return drop(e);
     if (L.n <= enp::kCoarsestCells) break;
     nx = (nx + 1) / 2; ny = (ny + 1) / 2; nz = (nz + 1) / 2;
   }
@@ -1842,7 +1850,7 @@ cudaError_t coarse_levels(enp_handle h) {
     const cudaLaunchConfig_t cfg = tail_config(h, S.tail_ctas, &cluster);
     cudaError_t e;
     if ((e = cudaOccupancyMaxActiveClusters(&active, enp::coarse_vcycle_tail, &cfg)) != cudaSuccess)
-      return e;
+      return drop(e);
     if (active >= B) break;
   }
   return cudaSuccess;
@@ -2127,6 +2135,7 @@ enp_status enp_block_jacobi_setup(enp_handle h, const double* u, int storage) {
     cudaFree(S.binv);
     S.binv = nullptr;
     S.binv_sets = 0;
+    S.storage = -1;   // no preconditioner if this setup fails before it has one
     e = cudaMalloc(&S.binv, esz * nn * nblk * nsets);
     if (e != cudaSuccess) return cuda_err(h, e, "cudaMalloc block inverses");
     S.binv_sets = nsets;
